@@ -208,3 +208,109 @@ def tolerance(case):
     Decisions are whole numbers and agree unless a uniform falls on a threshold or on the edge of a cell of the inverse
     CDF."""
     return {"rel": 2e-6, "max": 1e-5, "differ": 0.01}
+
+
+def _f32(T):
+    """The temperature as the library takes it, a float32, in 64 bits."""
+    return float(torch.tensor(T, dtype=torch.float32))
+
+
+def _g(u, K):
+    """1 - (1 - u)^K without cancellation, u clamped to [0, 1]."""
+    return -torch.expm1(K * torch.log1p(-u.clamp(0.0, 1.0)))
+
+
+def _exact_block(zq, zp, tok, T, K_exp):
+    """h (Eq. 2, Eq. 3) and residual masses of one batch row: zq [K,gamma+1,V], zp [K,gamma,V], tok [K,gamma]."""
+    gamma = zp.shape[1]
+    lq = torch.log_softmax(zq[:, :gamma].double() / T, -1)
+    lp = torch.log_softmax(zp.double() / T, -1)
+    at = tok.long().unsqueeze(-1)
+    zero = torch.zeros_like(lq[:, :1, 0])
+    la = torch.cat([zero, lq.gather(-1, at)[..., 0].cumsum(-1)], -1)        # [K,gamma+1]
+    lb = torch.cat([zero, lp.gather(-1, at)[..., 0].cumsum(-1)], -1)
+    c = (lb - la)[:, :gamma].exp()
+    q = lq.exp_()
+    t = torch.where(q > 0, c.unsqueeze(-1) * lp.exp_() / q, 1.0)
+    R = (q * (1.0 - t).clamp(min=0.0) ** K_exp).sum(-1)                     # [K,gamma]
+    a, b = la.exp(), lb.exp()
+    gb_a = _g(b, K_exp) / a
+    num = (R - (1.0 - c).clamp(min=0.0) ** K_exp).clamp(min=0.0)
+    den = num + (gb_a[:, :gamma] - _g(c, K_exp)).clamp(min=0.0)
+    sub = torch.where(den > 1e-12 * (gb_a[:, :gamma] + 1.0), num / den, 1.0)  # 0/0: accepted
+    c_end = (lb - la)[:, gamma].exp()
+    full = (a[:, gamma] * _g(c_end, K_exp) / _g(b[:, gamma], K_exp)).unsqueeze(-1)
+    return torch.cat([sub[:, 1:], full], -1).clamp(0.0, 1.0), a[:, :gamma] * R
+
+
+def _exact_kseq(st):
+    """rho per position and the acceptance probabilities of the tried tokens, NaN where nothing was tried."""
+    T, K = _f32(st["T"]), st["K"]
+    B, _, g1, _ = st["target"].shape
+    gamma = g1 - 1
+    rho_out = torch.full((B, gamma), math.nan, dtype=torch.float64)
+    acc_out = torch.full((B, K, gamma), math.nan, dtype=torch.float64)
+    tok, u = st["tokens"].cpu(), st["u"].cpu()
+    for b in range(B):
+        kept = list(range(K))
+        for i in range(gamma):
+            lq = torch.log_softmax(st["target"][b, kept[0], i].double() / T, -1)
+            lp = torch.log_softmax(st["draft"][b, kept[0], i].double() / T, -1)
+            q, p, n = lq.exp(), lp.exp(), len(kept)
+            rho = torch.ones((), dtype=torch.float64, device=DEVICE)
+            if n > 1:
+                lo, hi = rho.clone(), rho * n
+                for _ in range(52):
+                    mid = 0.5 * (lo + hi)
+                    beta = torch.minimum(p, q / mid).sum()
+                    up = _g(beta, n) - mid * beta > 0
+                    lo, hi = torch.where(up, mid, lo), torch.where(up, hi, mid)
+                rho = 0.5 * (lo + hi)
+            rho = float(rho)
+            rho_out[b, i] = rho
+            hit = None
+            for k in kept:
+                x = int(tok[b, k, i])
+                acc_out[b, k, i] = min(1.0, math.exp(float(lq[x] - lp[x])) / rho)
+                if float(u[b, k * gamma + i]) < float(acc_out[b, k, i]):
+                    hit = x
+                    break
+            if hit is None:
+                break
+            kept = [k for k in kept if int(tok[b, k, i]) == hit]
+    return rho_out, acc_out
+
+
+def exact(case, seed):
+    """The weights, masses and acceptance probabilities in 64 bits.  Tokens are drawn by inverse CDF, where an entry's
+    cell can be narrower than the rounding of any 32-bit sum, so what follows from the drawn token (its log-probability)
+    has no value of its own here."""
+    kind, K = case["kind"], case["K"]
+    if kind == "draw":
+        return None
+    st = prepare(case, seed)
+    T = _f32(st["T"])
+    if kind == "kseq":
+        if case["B"] * case["gamma"] > 1600:
+            return None                       # tens of seconds
+        rho, acc = _exact_kseq(st)
+        return [None, None, rho, acc, None]
+    if kind == "modify":
+        q = torch.softmax(st["target"].double() / T, -1)
+        p = torch.softmax(st["draft"].double() / T, -1)
+        c = (st["log_b"] - st["log_a"]).exp().unsqueeze(-1)
+        t = torch.where(q > 0, c * p / q, 1.0)
+        return [None, None, None, (q * (1.0 - t).clamp(min=0.0) ** K).sum(-1), None]
+    if kind == "shard":                       # the state holds one rank's range: the whole rows again
+        del st
+        inp = workloads.make_inputs(_config(case, seed), device=DEVICE)
+        zq, zp, tok = inp.target_logits, inp.draft_logits, inp.draft_tokens
+    else:
+        zq, zp, tok = st["target"], st["draft"], st["tokens"]
+    if kind == "gbv":
+        zq, zp, tok = zq.unsqueeze(1), zp.unsqueeze(1), tok.unsqueeze(1)
+    rows = [_exact_block(zq[b], zp[b], tok[b], T, K) for b in range(case["B"])]
+    h, S = (torch.stack([r[n] for r in rows]) for n in (0, 1))
+    if kind == "gbv":
+        return [None, None, h, None]
+    return [None, None, None, h, S, None]
