@@ -82,6 +82,19 @@ __device__ __forceinline__ float ld_logit<uint16_t>(const uint16_t *p, size_t i)
     return __uint_as_float(((uint32_t)__ldg(p + i)) << 16);
 }
 
+// 2^x, results below 2^-126 flushed to 0.
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
+
 // exp((z - m)/T) as 2^((z-m)*scale).
 __device__ __forceinline__ float expo(float z, float m, float scale) { return exp2f((z - m) * scale); }
 

@@ -31,6 +31,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "sgbv_cluster.cuh"
 #include "sgbv_common.cuh"
 
 namespace sgbv {
@@ -67,7 +68,6 @@ struct FusedParams {
 };
 
 // ---- PTX wrappers ------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // mbarrier operations take the barrier's 32-bit shared-memory address
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -124,17 +124,6 @@ __device__ __forceinline__ void issue_cell(uint32_t dst, const void *zq, const v
         "l"(zq), "l"(zp), "r"(bytes), "r"(bar), "r"(pred), "r"(half)
         : "memory");
 }
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_arrive() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // Asynchronous store of 16 bytes into the shared memory of CTA `rank` of this cluster, at the
 // address that `local` has in this CTA; its completion is counted (16 bytes) on the receiver's
 // mbarrier that sits where `local_bar` sits here.
@@ -145,11 +134,6 @@ __device__ __forceinline__ void push_f4(void *local, uint32_t local_bar, uint32_
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1,%2,%3,%4}, [%5];" ::"r"(dst),
                  "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
                  : "memory");
-}
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
 }
 __device__ __forceinline__ float rcp(float x) {
     float y;
@@ -248,13 +232,6 @@ __device__ __forceinline__ float warp_max_redux(float v) {
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
-__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
-
 // r^K for both halves of r, r in [0,1]; KT > 1 is a compile-time K, KT = 0 takes K at run time.
 template <int KT>
 __device__ __forceinline__ float2 ipow2(float2 r, int K) {

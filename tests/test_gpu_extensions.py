@@ -173,3 +173,40 @@ def test_draft_token_draw_matches_the_oracle(N, V, dtype, T):
     zbad[0, 3] = float("nan")
     tok2, _, st2 = binding.sgbv_draw_tokens(zbad, u, T)
     assert tok2[0].item() == -1 and st2[0].item() & binding.STATUS_NONFINITE_LOGIT
+
+
+@pytest.mark.parametrize("N,V,dtype", [(1, 40000, "fp32"), (37, 8192, "bf16"), (74, 16385, "fp32"), (75, 20011, "bf16"),
+                                       (149, 270000, "bf16"), (2, 2048, "fp32")])
+def test_draws_shared_out_over_the_ctas_of_a_row(N, V, dtype):
+    """Few rows are drawn by clusters of 2 to 8 CTAs, many by one CTA each (with more tiles than shared memory holds for
+    the longest): finite entries in one CTA's share only, the smallest and largest uniforms, a row that starts off a
+    16-byte boundary, NaN, +inf and no finite entry at all.  Tokens as the oracle's unless a uniform is within 1e-6 of an
+    edge of the drawn cell; log-probabilities to 2e-5 (float32 sums)."""
+    g = torch.Generator().manual_seed(N * V)
+    z = (2.0 * torch.randn(N, V, generator=g)).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    u = torch.rand(N, generator=g)
+    u[0] = 0.0
+    u[N - 1] = 1.0 - 2.0 ** -24
+    last = z[N // 2, -200:].clone()
+    z[N // 2] = float("-inf")              # all the mass at the end of the row
+    z[N // 2, -200:] = last
+    if N > 2:
+        first = z[1, :5].clone()
+        z[1] = float("-inf")               # ... at its start
+        z[1, :5] = first
+    buf = torch.empty(N * V + 1, dtype=z.dtype, device="cuda")
+    for view in (buf[:-1].view(N, V), buf[1:].view(N, V)):
+        view.copy_(z)
+        tok, lp, st = (t.cpu().numpy() for t in binding.sgbv_draw_tokens(view, u.cuda(), 0.9))
+        rtok, rlp, margin = oracle.draw_tokens(z.float().numpy(), u.numpy(), 0.9)
+        assert (st == 0).all()
+        near = margin < 1e-6
+        assert (tok[~near] == rtok[~near]).all() and ((tok >= 0) & (tok < V)).all()
+        same = tok == rtok
+        np.testing.assert_allclose(lp[same], rlp[same], atol=2e-5)
+    for value, at in ((float("nan"), V - 1), (float("inf"), 0), (float("-inf"), slice(None))):
+        bad = z.clone()
+        bad[N - 1, at] = value
+        tok, lp, st = (t.cpu().numpy() for t in binding.sgbv_draw_tokens(bad.cuda(), u.cuda(), 0.9))
+        assert tok[N - 1] == -1 and np.isnan(lp[N - 1]) and st[N - 1] == binding.STATUS_NONFINITE_LOGIT
+        assert (st[:N - 1] == 0).all()
