@@ -1,237 +1,428 @@
 // Comparison verifiers of Section 3 of the paper, behind the same boundary as the block verifier:
 // SpecTr's position-wise K-SEQ (Section 3.2) and, as its one-draft case, token-level speculative sampling
 // (Section 3.1).  They exist so that the verification cost of the methods can be compared on one machine
-// (the paper's Table 2); they are written for correctness and reasonable speed, not tuned like the block
-// verifier's streaming kernel.
+// (the paper's Table 2).
 //
-// One CTA per batch row walks the positions i = 0..gamma-1 in order.  At a position the drafts that still match
-// the accepted prefix ("retained", n of them) are the candidates; they share the rows of that prefix, and the
+// One cluster of C CTAs per batch row walks the positions i = 0..gamma-1 in order.  At a position the drafts that still
+// match the accepted prefix ("retained", n of them) are the candidates; they share the rows of that prefix, and the
 // rows of the first retained draft are read:
-//   1. row maxima and normalisers of the target and draft rows (two passes over the rows, from L2);
-//   2. rho in [1, n]: root of 1 - (1 - beta(rho))^n = rho beta(rho), beta(rho) = sum_x min{p(x), q(x)/rho}, by
-//      bisection, one pass over the rows per step (n = 1: rho = 1);
+//   1. every CTA reads its share of the target and the draft row ONCE into shared memory; row maxima, then the
+//      exponentials in place and their sums, both exchanged within the cluster;
+//   2. rho in [1, n]: root of 1 - (1 - beta(rho))^n = rho beta(rho), beta(rho) = sum_x min{p(x), q(x)/rho}, by Newton's
+//      method from the exponentials in shared memory, inside a bracket that every step shrinks (a step that would leave
+//      it bisects it).  rho beta(rho) = S1 + rho S2 with S1 = sum of q where q < rho p, S2 = sum of p elsewhere, so one
+//      sweep gives the value and the slope (n = 1: rho = 1);
 //   3. the retained drafts are tried in order, draft k's token x is accepted if eta < min{1, q(x)/(rho p(x))};
 //      the first accepted token extends the prefix, the drafts with that token stay retained;
 //   4. if none is accepted: y from norm(max{q - rho p, 0}) by inverse CDF over per-tile sums, and the row is done.
-// After gamma accepted positions y is drawn from the target row that follows the block.
+// After gamma accepted positions y is drawn from the target row that follows the block.  All decisions are taken by every
+// CTA of the cluster from the same numbers.
+//
+// What bounds it is the serial chain: positions one after the other, some six sweeps and as many cluster exchanges each.
+// Rows stay on chip between the sweeps (a CTA holds up to kCapTiles tiles; the rest of a longer share is read again in
+// every sweep), and a row is spread over as many CTAs as the batch leaves free.  64 prompts, K = 3, gamma = 12, 32256
+// float32: 99 us, against 424 us of one CTA of 1024 threads per prompt that read the rows from L2 in two sweeps for the
+// statistics and one for each of 34 bisections.  (Two prompts in three stop at the first or second position; the time is
+// that of the longest walk.)
+#include <atomic>
+
 #include "sgbv_sample.cuh"
 
 namespace sgbv {
 
 namespace {
 
-constexpr int kKseqThreads = 1024;
-constexpr int kBisections = 34;  // interval n 2^-34: far below float32 resolution of beta
+constexpr int kThreads = 512;        // two CTAs per SM
+constexpr int kWarpsPerCta = kThreads / 32;
+constexpr int kSlots = 2 * 148;      // CTAs the device holds
+constexpr int kCapTiles = 104;       // tiles of both rows in one CTA's shared memory (208 KB)
+constexpr int kMaxSteps = 60;        // bisection alone reaches float64's resolution of rho in that many
 
-// 1 - (1-u)^n as a geometric sum (all terms positive).
-__device__ __forceinline__ double gfun_n(double u, int n) {
-    if (u >= 1.0) return 1.0;
-    if (!(u > 0.0)) return 0.0;
-    const double v = 1.0 - u;
-    double sum = 1.0;
-    for (int j = 1; j < n; ++j) sum = fma(sum, v, 1.0);
-    return u * sum;
+// 1 - (1-u)^n as a geometric sum (all terms positive), and its derivative n (1-u)^(n-1).
+__device__ __forceinline__ double gfun_n(double u, int n, double &slope) {
+    const double v = u >= 1.0 ? 0.0 : u > 0.0 ? 1.0 - u : 1.0;
+    double sum = 1.0, pw = 1.0;
+    for (int j = 1; j < n; ++j) {
+        sum = fma(sum, v, 1.0);
+        pw *= v;
+    }
+    slope = (double)n * pw;
+    return u >= 1.0 ? 1.0 : u > 0.0 ? u * sum : 0.0;
 }
 
-// Sum of a double over the CTA (every thread gets it).  All threads must call.
-__device__ __forceinline__ double block_sum(double v, double *sh_warp) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    v = warp_sum(v);
-    __syncthreads();  // (sh_warp may still be read from the previous use)
-    if (lane == 0) sh_warp[wid] = v;
+struct KseqScratch {
+    double part[2][kWarpsPerCta];
+    double slots[2][kMaxRowCtas][2];   // by parity of the exchange: every CTA's pair of values
+    DrawScratch draw;
+    float tiles[2][kCapTiles];
+    int kept[kMaxK];
+    int n, accepted;
+};
+
+// Two values per thread combined over the cluster (sum, or maximum); every thread of every CTA gets the results, and
+// slots[par][r] keeps CTA r's share until the exchange after the next one.  All threads must call.
+template <bool kMaximum>
+__device__ __forceinline__ void exchange(double &a, double &b, KseqScratch &sc, int rank, int C, int &par) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    auto op = [](double x, double y) { return kMaximum ? fmax(x, y) : x + y; };
+    auto all = [&](double v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+        return v;
+    };
+    a = all(a);
+    b = all(b);
+    if (lane == 0) {
+        sc.part[0][wid] = a;
+        sc.part[1][wid] = b;
+    }
     __syncthreads();
-    return warp_sum(lane < nwarps ? sh_warp[lane] : 0.0);
+    par ^= 1;
+    if (wid == 0) {
+        const double none = kMaximum ? -INFINITY : 0.0;
+        a = all(lane < kWarpsPerCta ? sc.part[0][lane] : none);
+        b = all(lane < kWarpsPerCta ? sc.part[1][lane] : none);
+        if (lane < C) {
+            st_peer(&sc.slots[par][rank][0], lane, a);
+            st_peer(&sc.slots[par][rank][1], lane, b);
+        }
+    }
+    cluster_arrive();
+    cluster_wait();
+    a = sc.slots[par][0][0];
+    b = sc.slots[par][0][1];
+    for (int r = 1; r < C; ++r) {  // (rank order: the same on every CTA)
+        a = op(a, sc.slots[par][r][0]);
+        b = op(b, sc.slots[par][r][1]);
+    }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kKseqThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const int32_t *__restrict__ tok_all,
-            const float *__restrict__ u_all, Shape s, float *__restrict__ tile_scratch, int32_t *__restrict__ out_tau,
-            int32_t *__restrict__ out_tokens, double *__restrict__ out_rho, double *__restrict__ out_acc,
+            const float *__restrict__ u_all, Shape s, int C, float *__restrict__ tile_scratch, int32_t *__restrict__ out_tau,
+            int32_t *out_tokens, double *__restrict__ out_rho, double *__restrict__ out_acc,
             int32_t *__restrict__ out_status) {
-    __shared__ SampleScratch sc;
-    __shared__ int kept[kMaxK];
-    __shared__ int sh_n, sh_accepted, sh_flags;
-    __shared__ float sh_max[2][kSampleMaxWarps];
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int nthreads = blockDim.x, nwarps = nthreads >> 5;
+    extern __shared__ __align__(16) float rows_s[];  // exponentials of this CTA's tiles: target row, then draft row
+    __shared__ KseqScratch sc;
+    const int rank = (int)cluster_ctarank();
+    cluster_arrive();
+    const int b = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int K = s.K, g = s.gamma, V = s.V;
     const int32_t *tok = tok_all + (size_t)b * K * g;
     const float *u = u_all + (size_t)b * (K * g + 1);
-    float *tile_s = tile_scratch + (size_t)b * 2 * s.ntiles, *tile_m = tile_s + s.ntiles;
-
-    for (int n = tid; n <= g; n += nthreads) out_tokens[(size_t)b * (g + 1) + n] = -1;
-    if (out_rho)
-        for (int n = tid; n < g; n += nthreads) out_rho[(size_t)b * g + n] = NAN;
-    if (out_acc)
-        for (int n = tid; n < K * g; n += nthreads) out_acc[(size_t)b * K * g + n] = NAN;
-    if (tid == 0) {
-        sh_n = K;
-        sh_flags = 0;
+    const int per = (s.ntiles + C - 1) / C, t0 = min(s.ntiles, rank * per), t1 = min(s.ntiles, t0 + per);
+    const int held = min(t1 - t0, kCapTiles);        // tiles in shared memory
+    const int rest0 = (t0 + held) * kTile, rest1 = min(V, t1 * kTile);  // entries that are read again in every sweep
+    float *eq_s = rows_s, *ep_s = rows_s + (size_t)min(per, kCapTiles) * kTile;
+    // per-tile sums: in shared memory, or for long shares in global scratch
+    float *tile_s = sc.tiles[0], *tile_m = sc.tiles[1];
+    if (per > kCapTiles) {
+        tile_s = tile_scratch + (size_t)b * 2 * s.ntiles + t0;
+        tile_m = tile_s + s.ntiles;
     }
-    for (int k = tid; k < K; k += nthreads) kept[k] = k;
-    __syncthreads();
+    const bool lead = rank == 0 && tid == 0;
+
+    if (rank == 0) {
+        for (int n = tid; n <= g; n += kThreads) out_tokens[(size_t)b * (g + 1) + n] = -1;
+        if (out_rho)
+            for (int n = tid; n < g; n += kThreads) out_rho[(size_t)b * g + n] = NAN;
+        if (out_acc)
+            for (int n = tid; n < K * g; n += kThreads) out_acc[(size_t)b * K * g + n] = NAN;
+    }
+    if (tid == 0) sc.n = K;
+    for (int k = tid; k < K; k += kThreads) sc.kept[k] = k;
     bool range = false;
-    for (int n = tid; n < K * g; n += nthreads) range |= tok[n] < 0 || tok[n] >= V;
-    if (__syncthreads_or(range)) {
-        if (tid == 0) {
+    for (int n = tid; n < K * g; n += kThreads) range |= tok[n] < 0 || tok[n] >= V;
+    range = __syncthreads_or(range);
+    cluster_wait();  // every CTA of the cluster is running
+    if (range) {
+        if (lead) {
             out_tau[b] = -1;
             out_status[b] = SGBV_STATUS_TOKEN_RANGE;
         }
         return;
     }
 
-    int tau = 0, y = -1, flags = 0;
+    int tau = 0, flags = 0, par = 0;
     bool stopped = false;
     for (int i = 0; i < g && !stopped; ++i) {
-        const int k0 = kept[0], nk = sh_n;
+        const int k0 = sc.kept[0], nk = sc.n;
         const T *zq = zq_all + (((size_t)b * K + k0) * (g + 1) + i) * V;
         const T *zp = zp_all + (((size_t)b * K + k0) * g + i) * V;
-        // ---- 1. maxima (NaN / +inf detection on the way), then normalisers ---------------------------------
-        float mq = -INFINITY, mp = -INFINITY;
-        bool bad = false;
-        for (int x = tid; x < V; x += nthreads) {
-            const float a = ld_logit(zq, x), c = ld_logit(zp, x);
-            bad |= (a != a) | (c != c) | (a == INFINITY) | (c == INFINITY);
-            mq = fmaxf(mq, a);
-            mp = fmaxf(mp, c);
+        // the logits of the retained drafts' tokens, fetched ahead (first warp, two drafts per lane)
+        float zqx[2] = {0.0f, 0.0f}, zpx[2] = {0.0f, 0.0f};
+        int tokx[2] = {-1, -1};
+        if (wid == 0)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (lane + 32 * e < nk) {
+                    tokx[e] = tok[sc.kept[lane + 32 * e] * g + i];
+                    zqx[e] = ld_logit(zq, tokx[e]);
+                    zpx[e] = ld_logit(zp, tokx[e]);
+                }
+        // ---- 1. logits to shared memory, maxima; exponentials, normalisers ---------------------------------
+        const bool pieces = (reinterpret_cast<uintptr_t>(zq) % 16 == 0) && (reinterpret_cast<uintptr_t>(zp) % 16 == 0) &&
+                            (V % (16 / (int)sizeof(T)) == 0);
+        float mqf = -INFINITY, mpf = -INFINITY;
+        for (int t = wid; t < held; t += 2 * kWarpsPerCta) {  // two tiles of both rows in flight per warp
+            float a[2][kTile / 32], c[2][kTile / 32];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int tt = t + q * kWarpsPerCta;
+                if (pieces) {
+                    load_tile_pieces<T>(zq, t0 + tt, tt < held, V, lane, a[q]);
+                    load_tile_pieces<T>(zp, t0 + tt, tt < held, V, lane, c[q]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < kTile / 32; ++e) {
+                        const int x = (t0 + tt) * kTile + lane + 32 * e;
+                        a[q][e] = tt < held && x < V ? ld_logit(zq, x) : -INFINITY;
+                        c[q][e] = tt < held && x < V ? ld_logit(zp, x) : -INFINITY;
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int tt = t + q * kWarpsPerCta;
+                if (tt >= held) break;
+#pragma unroll
+                for (int e = 0; e < kTile / 32; ++e) {
+                    mqf = fmaxf(mqf, a[q][e]);
+                    mpf = fmaxf(mpf, c[q][e]);
+                }
+                float *dq = eq_s + tt * kTile, *dp = ep_s + tt * kTile;
+                if (pieces) {
+                    // where load_tile_pieces takes a lane's entries from
+                    const int xa = sizeof(T) == 4 ? lane * 4 : lane * 8, xb = sizeof(T) == 4 ? kTile / 2 + lane * 4 : lane * 8 + 4;
+                    *reinterpret_cast<float4 *>(dq + xa) = make_float4(a[q][0], a[q][1], a[q][2], a[q][3]);
+                    *reinterpret_cast<float4 *>(dq + xb) = make_float4(a[q][4], a[q][5], a[q][6], a[q][7]);
+                    *reinterpret_cast<float4 *>(dp + xa) = make_float4(c[q][0], c[q][1], c[q][2], c[q][3]);
+                    *reinterpret_cast<float4 *>(dp + xb) = make_float4(c[q][4], c[q][5], c[q][6], c[q][7]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < kTile / 32; ++e) {
+                        dq[lane + 32 * e] = a[q][e];
+                        dp[lane + 32 * e] = c[q][e];
+                    }
+                }
+            }
         }
-        mq = warp_max(mq);
-        mp = warp_max(mp);
-        if (lane == 0) {
-            sh_max[0][wid] = mq;
-            sh_max[1][wid] = mp;
+        for (int x = rest0 + tid; x < rest1; x += kThreads) {
+            mqf = fmaxf(mqf, ld_logit(zq, x));
+            mpf = fmaxf(mpf, ld_logit(zp, x));
         }
-        bad = __syncthreads_or(bad);
-        mq = warp_max(lane < nwarps ? sh_max[0][lane] : -INFINITY);
-        mp = warp_max(lane < nwarps ? sh_max[1][lane] : -INFINITY);
-        if (bad || !(mq > -INFINITY) || !(mp > -INFINITY)) {
+        double mqd = (double)mqf, mpd = (double)mpf;
+        exchange<true>(mqd, mpd, sc, rank, C, par);
+        const float mq = (float)mqd, mp = (float)mpd;
+        const float nmq = mq > -INFINITY ? -mq : 0.0f, nmp = mp > -INFINITY ? -mp : 0.0f;
+        auto eqof = [&](float z) { return ex2((z + nmq) * s.scale); };
+        auto epof = [&](float z) { return ex2((z + nmp) * s.scale); };
+        float4 *const eq4 = reinterpret_cast<float4 *>(eq_s), *const ep4 = reinterpret_cast<float4 *>(ep_s);
+        const int n4 = held * (kTile / 4);
+        float sq = 0.0f, sp = 0.0f;
+        for (int j = tid; j < n4; j += kThreads) {
+            float4 a = eq4[j], c = ep4[j];
+            a = make_float4(eqof(a.x), eqof(a.y), eqof(a.z), eqof(a.w));
+            c = make_float4(epof(c.x), epof(c.y), epof(c.z), epof(c.w));
+            eq4[j] = a;
+            ep4[j] = c;
+            sq += (a.x + a.y) + (a.z + a.w);
+            sp += (c.x + c.y) + (c.z + c.w);
+        }
+        for (int x = rest0 + tid; x < rest1; x += kThreads) {
+            sq += eqof(ld_logit(zq, x));
+            sp += epof(ld_logit(zp, x));
+        }
+        double Zq = (double)sq, Zp = (double)sp;
+        exchange<false>(Zq, Zp, sc, rank, C, par);
+        // NaN entries end up in the sums; +inf is its row's maximum and gives inf - inf there
+        if (!(mq > -INFINITY) || !(mp > -INFINITY) || Zq != Zq || Zp != Zp) {
             flags |= SGBV_STATUS_NONFINITE_LOGIT;
             break;
         }
-        float sq = 0.0f, sp = 0.0f;
-        for (int x = tid; x < V; x += nthreads) {
-            sq += expo(ld_logit(zq, x), mq, s.scale);
-            sp += expo(ld_logit(zp, x), mp, s.scale);
-        }
-        const double Zq = block_sum((double)sq, sc.warp), Zp = block_sum((double)sp, sc.warp);
-        const float inv_Zq = (float)(1.0 / Zq), inv_Zp = (float)(1.0 / Zp);
-        // ---- 2. rho -----------------------------------------------------------------------------------------
+        // ---- 2. rho (the same on every thread of the cluster) ----------------------------------------------
         double rho = 1.0;
         if (nk > 1) {
             double lo = 1.0, hi = (double)nk;
-            for (int it = 0; it < kBisections; ++it) {
-                const double mid = 0.5 * (lo + hi);
-                const float q_scale = (float)(1.0 / (Zq * mid));
-                float acc = 0.0f;
-                for (int x = tid; x < V; x += nthreads) {
-                    const float qx = expo(ld_logit(zq, x), mq, s.scale) * q_scale;
-                    const float px = expo(ld_logit(zp, x), mp, s.scale) * inv_Zp;
-                    acc += fminf(px, qx);
+            for (int it = 0; it < kMaxSteps; ++it) {
+                const float thr = (float)(rho * (Zq / Zp));
+                float s1 = 0.0f, s2 = 0.0f;
+                // (added up in the order of the normalisers, so that equal rows give S2 = 1 and with it rho = 1 exactly: the
+                // root is n-fold there, and a rounding error e in S2 would move it by e^(1/n))
+                auto q_of = [&](float a, float c) { return a < thr * c ? a : 0.0f; };
+                auto p_of = [&](float a, float c) { return a < thr * c ? 0.0f : c; };
+                for (int j = tid; j < n4; j += kThreads) {
+                    const float4 a = eq4[j], c = ep4[j];
+                    s1 += (q_of(a.x, c.x) + q_of(a.y, c.y)) + (q_of(a.z, c.z) + q_of(a.w, c.w));
+                    s2 += (p_of(a.x, c.x) + p_of(a.y, c.y)) + (p_of(a.z, c.z) + p_of(a.w, c.w));
                 }
-                const double beta = block_sum((double)acc, sc.warp);
-                const double f = gfun_n(beta, nk) - mid * beta;  // (the same on every thread)
-                if (f > 0.0) lo = mid;
-                else hi = mid;
+                for (int x = rest0 + tid; x < rest1; x += kThreads) {
+                    const float a = eqof(ld_logit(zq, x)), c = epof(ld_logit(zp, x));
+                    s1 += q_of(a, c);
+                    s2 += p_of(a, c);
+                }
+                double S1 = (double)s1, S2 = (double)s2;
+                exchange<false>(S1, S2, sc, rank, C, par);
+                S1 /= Zq;
+                S2 /= Zp;
+                const double beta = S1 / rho + S2;
+                double gs;
+                const double f = gfun_n(beta, nk, gs) - (S1 + rho * S2);
+                if (f > 0.0) lo = rho;
+                else hi = rho;
+                if (hi <= lo) break;  // (f <= 0 at 1: the root is 1)
+                const double df = -gs * S1 / (rho * rho) - S2;
+                double next = rho - f / df;
+                if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
+                const double step = fabs(next - rho);
+                rho = next;
+                if (step <= 1e-10 * rho) break;
             }
-            rho = 0.5 * (lo + hi);
         }
-        // ---- 3. the retained drafts, in order -----------------------------------------------------------------
-        if (tid == 0) {
-            if (out_rho) out_rho[(size_t)b * g + i] = rho;
-            int accepted = -1;
-            for (int j = 0; j < nk && accepted < 0; ++j) {
-                const int k = kept[j];
-                const int x = tok[k * g + i];
-                const float zpx = ld_logit(zp, x);
-                double acc = 1.0;
-                if (zpx > -INFINITY) {
-                    const double lq = ((double)ld_logit(zq, x) - (double)mq) * s.inv_T - log(Zq);
-                    const double lp = ((double)zpx - (double)mp) * s.inv_T - log(Zp);
-                    acc = exp(lq - lp) / rho;
-                    if (!(acc < 1.0)) acc = 1.0;
+        // ---- 3. the retained drafts, in order (first warp of every CTA) -----------------------------------------
+        if (wid == 0) {
+            if (lead && out_rho) out_rho[(size_t)b * g + i] = rho;
+            const double lZq = log(Zq), lZp = log(Zp);
+            double acc[2];
+            unsigned pass[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int j = lane + 32 * e;
+                acc[e] = 1.0;
+                if (j < nk && zpx[e] > -INFINITY) {
+                    const double lq = ((double)zqx[e] - (double)mq) * s.inv_T - lZq;
+                    const double lp = ((double)zpx[e] - (double)mp) * s.inv_T - lZp;
+                    acc[e] = exp(lq - lp) / rho;
+                    if (!(acc[e] < 1.0)) acc[e] = 1.0;
                 }
-                if (out_acc) out_acc[((size_t)b * K + k) * g + i] = acc;
-                if ((double)u[k * g + i] < acc) accepted = k;
+                pass[e] = __ballot_sync(0xffffffffu, j < nk && (double)u[(j < nk ? sc.kept[j] : 0) * g + i] < acc[e]);
             }
-            sh_accepted = accepted;
-            if (accepted >= 0) {
-                const int x = tok[accepted * g + i];
-                int m = 0;
-                for (int j = 0; j < nk; ++j)
-                    if (tok[kept[j] * g + i] == x) kept[m++] = kept[j];
-                sh_n = m;
-                out_tokens[(size_t)b * (g + 1) + i] = x;
+            const int first = pass[0] ? __ffs(pass[0]) - 1 : pass[1] ? 31 + __ffs(pass[1]) : -1;  // among the retained
+            const int x = first < 0 ? -1 : __shfl_sync(0xffffffffu, first < 32 ? tokx[0] : tokx[1], first & 31);
+            int stay[2], m = 0;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int j = lane + 32 * e, k = j < nk ? sc.kept[j] : 0;
+                if (rank == 0 && out_acc && j < nk && (first < 0 || j <= first)) out_acc[((size_t)b * K + k) * g + i] = acc[e];
+                const unsigned same = __ballot_sync(0xffffffffu, first >= 0 && j < nk && tokx[e] == x);
+                stay[e] = (same >> lane) & 1u ? m + __popc(same & ((1u << lane) - 1u)) : -1;
+                tokx[e] = k;  // (the draft)
+                m += __popc(same);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                if (stay[e] >= 0) sc.kept[stay[e]] = tokx[e];
+            if (lane == 0) {
+                sc.accepted = first;
+                if (first >= 0) {
+                    sc.n = m;
+                    if (rank == 0) out_tokens[(size_t)b * (g + 1) + i] = x;
+                }
             }
         }
         __syncthreads();
-        if (sh_accepted >= 0) {
+        if (sc.accepted >= 0) {
             tau = i + 1;
             continue;
         }
         // ---- 4. nothing accepted: y from norm(max{q - rho p, 0}) ------------------------------------------------
-        const float rho_p = (float)rho * inv_Zp;
-        auto wfun = [&](int x) {
-            const float qx = expo(ld_logit(zq, x), mq, s.scale) * inv_Zq;
-            const float px = expo(ld_logit(zp, x), mp, s.scale) * rho_p;
-            return fmaxf(qx - px, 0.0f);
+        stopped = true;
+        const float iZq = (float)(1.0 / Zq), rho_p = (float)rho * (float)(1.0 / Zp);
+        auto wof = [&](float a, float c) { return fmaxf(a * iZq - c * rho_p, 0.0f); };
+        auto entry = [&](int x) {
+            const int j = x - t0 * kTile;
+            return j < held * kTile ? wof(eq_s[j], ep_s[j]) : wof(eqof(ld_logit(zq, x)), epof(ld_logit(zp, x)));
         };
-        double wtot = 0.0;
-        for (int t = wid; t < s.ntiles; t += nwarps) {  // one warp per 256-entry tile
+        for (int t = wid; t < t1 - t0; t += kWarpsPerCta) {  // one warp per tile
             float acc = 0.0f;
-            for (int x = t * kTile + lane; x < min(V, (t + 1) * kTile); x += 32) acc += wfun(x);
+#pragma unroll
+            for (int e = 0; e < kTile / 32; ++e) {
+                const int x = (t0 + t) * kTile + lane + 32 * e;
+                if (x < V) acc += entry(x);
+            }
             acc = warp_sum(acc);
             if (lane == 0) tile_s[t] = acc;
-            wtot += (double)acc;
         }
-        const double W = block_sum(lane == 0 ? wtot : 0.0, sc.warp);
+        __syncthreads();
+        double W = 0.0, unused = 0.0;
+        for (int t = tid; t < t1 - t0; t += kThreads) W += (double)tile_s[t];
+        exchange<false>(W, unused, sc, rank, C, par);
         const double us = (double)u[K * g];
         if (W > 0.0) {
-            locate_tile(tile_s, nullptr, s.ntiles, us * W, false, sc.i, sc.d, sc.warp);
-            const int sel = sc.i[2];
-            Pick pk = pick_in_tile(sel * kTile, min(V, (sel + 1) * kTile), sc.d[0], sc.d[1], wfun, sc.warp, sc.pick);
-            y = (pk.first != INT_MAX) ? pk.first : pk.last;
+            // the CTA whose share the target falls into draws
+            const double target = us * W;
+            double run = 0.0, before = 0.0;
+            int owner = -1, last = -1;
+            for (int r = 0; r < C; ++r) {
+                const double v = sc.slots[par][r][0];
+                if (v > 0.0) last = r;
+                if (owner < 0 && run + v > target) owner = r;
+                if (r < rank) before += v;
+                run += v;
+            }
+            if (rank == (owner < 0 ? last : owner) && wid == 0) {
+                auto weight = [&](int t) { return (double)tile_s[t]; };
+                const int y = warp_draw(weight, t1 - t0, t0, V, owner < 0 ? INFINITY : target - before, entry);
+                if (lane == 0) out_tokens[(size_t)b * (g + 1) + i] = y;
+            }
         } else {  // q <= rho p everywhere: the draw comes from q itself
             flags |= SGBV_STATUS_DEGENERATE_RESIDUAL;
-            bool bad_row = false;
-            y = draw_from_row<T>(zq, s, us, tile_s, tile_m, &sc, bad_row);
-            if (bad_row) flags |= SGBV_STATUS_NONFINITE_LOGIT;
+            const Drawn d = draw_row<T>(zq, s, us, rank, C, tile_s, tile_m, &sc.draw);
+            if (tid == 0 && d.y >= 0) out_tokens[(size_t)b * (g + 1) + i] = d.y;
         }
-        stopped = true;
     }
     if (!stopped && !(flags & SGBV_STATUS_NONFINITE_LOGIT)) {  // every position accepted: bonus token
-        const T *zq = zq_all + (((size_t)b * K + kept[0]) * (g + 1) + g) * V;
-        bool bad_row = false;
-        y = draw_from_row<T>(zq, s, (double)u[K * g], tile_s, tile_m, &sc, bad_row);
-        if (bad_row) flags |= SGBV_STATUS_NONFINITE_LOGIT;
+        const T *zq = zq_all + (((size_t)b * K + sc.kept[0]) * (g + 1) + g) * V;
+        const Drawn d = draw_row<T>(zq, s, (double)u[K * g], rank, C, tile_s, tile_m, &sc.draw);
+        if (wid == 0 && d.bad) flags |= SGBV_STATUS_NONFINITE_LOGIT;  // (the first warps know)
+        if (tid == 0 && d.y >= 0) out_tokens[(size_t)b * (g + 1) + g] = d.y;
     }
-    __syncthreads();
-    const bool failed = (flags & SGBV_STATUS_NONFINITE_LOGIT) != 0;
-    if (failed) {
-        for (int n = tid; n <= g; n += nthreads) out_tokens[(size_t)b * (g + 1) + n] = -1;
-    } else if (tid == 0) {
-        out_tokens[(size_t)b * (g + 1) + tau] = y;
+    if (rank == 0 && wid == 0) {
+        const bool failed = (flags & SGBV_STATUS_NONFINITE_LOGIT) != 0;
+        if (failed)
+            for (int n = lane; n <= g; n += 32) out_tokens[(size_t)b * (g + 1) + n] = -1;
+        if (lane == 0) {
+            out_tau[b] = failed ? -1 : tau;
+            out_status[b] = flags;
+        }
     }
-    if (tid == 0) {
-        out_tau[b] = failed ? -1 : tau;
-        out_status[b] = flags;
+}
+
+template <typename T>
+int run(const Launch &L, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status) {
+    const Shape &s = L.s;
+    int dev = 0;
+    static std::atomic<bool> attr_done[64];
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SGBV_ERR_CUDA;
+    if (!attr_done[dev]) {
+        if (cudaFuncSetAttribute(kseq_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * kCapTiles * kTile * (int)sizeof(float)) != cudaSuccess)
+            return SGBV_ERR_CUDA;
+        attr_done[dev] = true;
     }
+    // as few CTAs as hold a row on chip; more while the device has room for all of the batch's and a CTA keeps a tile for
+    // every other warp
+    int C = 1;
+    while (C < kMaxRowCtas && (s.ntiles > C * kCapTiles ||
+                               ((long)s.B * 2 * C <= kSlots && s.ntiles >= 2 * C * (kWarpsPerCta / 2))))
+        C *= 2;
+    const int per = (s.ntiles + C - 1) / C;
+    const size_t smem = 2 * (size_t)(per < kCapTiles ? per : kCapTiles) * kTile * sizeof(float);
+    if (launch_clusters(kseq_kernel<T>, (unsigned)s.B * (unsigned)C, kThreads, smem, C, L.stream, (const T *)L.zq,
+                        (const T *)L.zp, L.tok, L.u, s, C, tile_scratch, L.out_tau, L.out_tokens, out_rho, out_acc,
+                        out_status) == cudaSuccess)
+        return 1;
+    cudaGetLastError();
+    return SGBV_ERR_CUDA;
 }
 
 }  // namespace
 
 int launch_kseq(const Launch &L, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status) {
-    const Shape &s = L.s;
-    if (L.dtype == SGBV_DTYPE_BF16)
-        kseq_kernel<uint16_t><<<s.B, kKseqThreads, 0, L.stream>>>((const uint16_t *)L.zq, (const uint16_t *)L.zp, L.tok, L.u, s,
-                                                                  tile_scratch, L.out_tau, L.out_tokens, out_rho, out_acc,
-                                                                  out_status);
-    else
-        kseq_kernel<float><<<s.B, kKseqThreads, 0, L.stream>>>((const float *)L.zq, (const float *)L.zp, L.tok, L.u, s,
-                                                               tile_scratch, L.out_tau, L.out_tokens, out_rho, out_acc,
-                                                               out_status);
-    if (cudaGetLastError() != cudaSuccess) return SGBV_ERR_CUDA;
-    return 1;
+    return L.dtype == SGBV_DTYPE_BF16 ? run<uint16_t>(L, tile_scratch, out_rho, out_acc, out_status)
+                                      : run<float>(L, tile_scratch, out_rho, out_acc, out_status);
 }
 
 }  // namespace sgbv

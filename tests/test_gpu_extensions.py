@@ -117,6 +117,34 @@ def test_kseq_matches_the_oracle(B, K, gamma, V, dtype, T, alpha):
     assert binding.last_main_kernel() == "kseq_kernel"
 
 
+@pytest.mark.parametrize("B,K,gamma,V,dtype,T,alpha,shift", [
+    (1, 4, 6, 50257, "bf16", 0.6, 0.95, 0),     # eight CTAs per row, rows that start anywhere
+    (40, 2, 3, 8191, "fp32", 0.9, 0.8, 1),      # four, off a 16-byte boundary
+    (80, 3, 2, 9000, "fp32", 0.5, 0.9, 0),      # two
+    (150, 2, 2, 3000, "bf16", 1.0, 0.7, 0),     # one
+    (1, 3, 2, 221000, "bf16", 1.0, 0.9, 0),     # more tiles than the shared memory of eight CTAs holds
+    (3, 64, 2, 2048, "fp32", 0.4, 0.99, 0),     # the most drafts
+])
+def test_kseq_shared_out_over_the_ctas_of_a_row(B, K, gamma, V, dtype, T, alpha, shift):
+    """Rows held by clusters of one to eight CTAs, ragged and unaligned rows, and rows too long for shared memory.  Then
+    with equal models: rho = 1, an n-fold root there, so that a rounding error e in the sums would move it by e^(1/n) (the
+    float64 oracle itself is 2e-5 off at n = 3, hence no comparison with it); every token is accepted."""
+    cfg = workloads.VerifyConfig("kc", B=B, K=K, gamma=gamma, V=V, dtype=dtype, temperature=T, alpha=alpha, seed=77 + V % 83)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t):
+        v = torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape)
+        return v.copy_(t)
+    inp = workloads.VerifyInputs(cfg, moved(inp.target_logits), moved(inp.draft_logits), inp.draft_tokens, inp.uniforms)
+    out, ref = _kseq_compare(inp, T)
+    again = binding.sgbv_verify_kseq(inp.target_logits, inp.draft_logits, inp.draft_tokens, inp.uniforms, T)
+    assert torch.equal(out.tokens, again.tokens) and torch.equal(out.rho.nan_to_num(-1), again.rho.nan_to_num(-1))
+    equal = inp.target_logits[:, :, :gamma].contiguous()
+    same = binding.sgbv_verify_kseq(inp.target_logits, equal, inp.draft_tokens, inp.uniforms, T)
+    np.testing.assert_allclose(same.rho.cpu().numpy(), 1.0, atol=1e-6)
+    assert (same.accept_len == gamma).all() and ((same.tokens >= 0) & (same.tokens < V)).all() and (same.status == 0).all()
+
+
 def test_kseq_flags():
     cfg = workloads.VerifyConfig("ksf", B=4, K=2, gamma=2, V=300, alpha=0.8, seed=9)
     inp = workloads.make_inputs(cfg, device="cuda")
