@@ -45,6 +45,8 @@ constexpr int kCtasPerSm = 1;              // CTAs that share an SM (1 or 2): tw
 constexpr int kWarps = 32;                 // warps per CTA (16 warps of 128 registers measured a third slower)
 constexpr int kCtaCells = 128 / kCtasPerSm;  // cells of a row per CTA: 16 tensor-memory columns per cell in each of the 4
                                            // lane quarters, 512 columns per SM: 128 cells = 32,768 entries per SM
+constexpr int kSlack = 16;  // extra bytes per cell and tensor in a slot when rows start anywhere: a copy then begins at the
+                           // 16-byte boundary before the cell and ends behind it
 constexpr int kTmemCols = 512 / kCtasPerSm;  // this CTA's share of the SM's tensor memory
 constexpr int kMaxCluster = 8 * kCtasPerSm;  // CTAs per cluster (beyond 8 the size is not portable, which sm_100 allows)
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about one second of SM clock
@@ -219,9 +221,21 @@ __device__ __forceinline__ void read_cell<uint16_t>(const unsigned char *cell_ba
     v[2] = make_float2(__uint_as_float(a.z << 16), __uint_as_float(a.z & 0xffff0000u));
     v[3] = make_float2(__uint_as_float(a.w << 16), __uint_as_float(a.w & 0xffff0000u));
 }
-// Offset (in elements, within the 256-element cell) of this lane's e-th element.
+// The same from a slot whose cell begins at any multiple of the element size behind the slot's start: a lane takes every
+// 32nd entry, so that the 32 lanes of a load read 32 neighbours.
 template <typename T>
+__device__ __forceinline__ void read_cell_at(const unsigned char *cell_base, int lane, float2 (&v)[4]) {
+    const T *p = reinterpret_cast<const T *>(cell_base) + lane;
+    auto at = [&](int e) {
+        return sizeof(T) == 4 ? __uint_as_float((uint32_t)reinterpret_cast<const uint32_t *>(p)[32 * e]) : __uint_as_float((uint32_t)p[32 * e] << 16);
+    };
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = make_float2(at(2 * e), at(2 * e + 1));
+}
+// Offset (in elements, within the 256-element cell) of this lane's e-th element.
+template <typename T, bool kAny>
 __device__ __forceinline__ int cell_offset(int lane, int e) {
+    if (kAny) return lane + 32 * e;
     if (sizeof(T) == 4) return (e < 4) ? lane * 4 + e : 128 + lane * 4 + (e - 4);
     return lane * 8 + e;
 }
@@ -288,26 +302,49 @@ struct RowScalars {
     float c;      // c_i
 };
 
-// First sweep of one cell, first half: the lane's 8 target and 8 draft logits from the ring slot (entries past the
-// end of the row read as -inf), and their maxima.
-template <typename T>
-__device__ __forceinline__ void first_sweep_fetch(const unsigned char *slot, int lane, bool is_tail, int tail_valid,
-                                                  float2 (&eq)[4], float2 (&ep)[4], float &m1, float &m2) {
-    read_cell<T>(slot, lane, eq);
-    read_cell<T>(slot + kCell * (int)sizeof(T), lane, ep);
-    if (is_tail) {  // the row ends inside this cell
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (cell_offset<T>(lane, 2 * e) >= tail_valid) eq[e].x = ep[e].x = -INFINITY;
-            if (cell_offset<T>(lane, 2 * e + 1) >= tail_valid) eq[e].y = ep[e].y = -INFINITY;
-        }
-    }
+__device__ __forceinline__ void cell_maxima(const float2 (&eq)[4], const float2 (&ep)[4], float &m1, float &m2) {
     m1 = m2 = -INFINITY;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         m1 = max3(m1, eq[e].x, eq[e].y);
         m2 = max3(m2, ep[e].x, ep[e].y);
     }
+}
+// First sweep of one cell, first half: the lane's 8 target and 8 draft logits from the ring slot (entries past the
+// end of the row read as -inf), and their maxima.
+template <typename T, bool kAny>
+__device__ __forceinline__ void first_sweep_fetch(const unsigned char *slot, uint32_t off_q, uint32_t off_p, int lane, bool is_tail,
+                                                  int tail_valid, float2 (&eq)[4], float2 (&ep)[4], float &m1, float &m2) {
+    if (kAny) {
+        read_cell_at<T>(slot + off_q, lane, eq);
+        read_cell_at<T>(slot + kCell * (int)sizeof(T) + kSlack + off_p, lane, ep);
+    } else {
+        read_cell<T>(slot, lane, eq);
+        read_cell<T>(slot + kCell * (int)sizeof(T), lane, ep);
+    }
+    if (is_tail) {  // the row ends inside this cell
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (cell_offset<T, kAny>(lane, 2 * e) >= tail_valid) eq[e].x = ep[e].x = -INFINITY;
+            if (cell_offset<T, kAny>(lane, 2 * e + 1) >= tail_valid) eq[e].y = ep[e].y = -INFINITY;
+        }
+    }
+    cell_maxima(eq, ep, m1, m2);
+}
+// A cell that no copy can bring (its 16-byte pieces reach past an end of a tensor): straight from global memory.
+template <typename T>
+__device__ __forceinline__ void first_sweep_direct(const unsigned char *q, const unsigned char *p, int lane, int valid,
+                                                   float2 (&eq)[4], float2 (&ep)[4], float &m1, float &m2) {
+    auto at = [&](const unsigned char *base, int e) {
+        const int x = lane + 32 * e;
+        return x < valid ? ld_logit(reinterpret_cast<const T *>(base), x) : -INFINITY;
+    };
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        eq[e] = make_float2(at(q, 2 * e), at(q, 2 * e + 1));
+        ep[e] = make_float2(at(p, 2 * e), at(p, 2 * e + 1));
+    }
+    cell_maxima(eq, ep, m1, m2);
 }
 // Second half: exponentials relative to the thread's own maxima of the cell (0 if it saw only -inf; the maximum
 // itself maps to exactly 1, so point-mass rows stay exact) into tensor memory, and their sums.
@@ -411,10 +448,25 @@ __device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, float fmq
     }
 }
 
+template <bool kWide>
+struct Sum {
+    typedef float type;
+};
+template <>
+struct Sum<true> {
+    typedef double type;
+};
+
+// kAny: rows that do not all start on 16-byte boundaries (odd vocabularies, unaligned buffers).  A copy then brings the
+// 16-byte pieces that hold the cell, and the reads from shared memory start at the remainder.  The few cells at the ends of the
+// tensors whose pieces reach past them are loaded directly.
+// Such rows used to take the two-sweep path (three scalar reads of every logit, four kernels): 16 prompts, K = 4, gamma = 4,
+// V = 50257 bfloat16 113 -> 66 us, one prompt at V = 32001 float32 73 -> 19, 64 prompts, K = 2 at V = 128255 float32 527 -> 195.
+// Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4.
 // W warps per CTA; NS ring slots per warp (the cells per warp and row, kCtaCells / W, are a multiple of it, so
 // that cell j of a row always sits in slot j % NS); KT: the number of drafts K when it has a specialised
 // second sweep (1, 2, 3, 4, 8), else 0 (any K, loops).
-template <typename T, bool kRow, int W, int NS, int KT>
+template <typename T, bool kRow, int W, int NS, int KT, bool kAny>
 __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const FusedParams p) {
     constexpr int kFWarps = W, kFThreads = W * 32, kCellsPerWarp = kCtaCells / W;
     static_assert(kCellsPerWarp % NS == 0, "cell j of a row must always land in slot j % NS");
@@ -427,7 +479,8 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     const int cid = blockIdx.x / C;
     const int G = gridDim.x / C;
     constexpr int kHalfBytes = kCell * (int)sizeof(T);  // one tensor's cell
-    constexpr int kSlotBytes = 2 * kHalfBytes;          // the cell of zq, then the same cell of zp
+    constexpr int kHalfSlot = kHalfBytes + (kAny ? kSlack : 0);
+    constexpr int kSlotBytes = 2 * kHalfSlot;           // the cell of zq, then the same cell of zp
     constexpr int kStrideBytes = kFWarps * kHalfBytes;  // from one cell of a warp to its next, in a row
     constexpr int kRingBytes = kFWarps * NS * kSlotBytes;
     // [rings][full barriers][draft factors of every thread's cells][Control]
@@ -541,12 +594,38 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     const unsigned char *const zp_warp = reinterpret_cast<const unsigned char *>(p.zp) + (size_t)first_cell * kHalfBytes;
     const uint32_t is_lane0 = lane == 0 ? 1u : 0u;
     uint32_t pending = 0, phases = 0;
-#define SGBV_ISSUE(QROW, PROW, JJ, SLOT)                                                                                \
+    // kAny: where a copy starts (the 16-byte boundary at or before the cell) and how long it is (a constant for all full
+    // cells: always one piece more)
+    auto floor16 = [](const unsigned char *a) {
+        return kAny ? reinterpret_cast<const unsigned char *>(reinterpret_cast<uintptr_t>(a) & ~(uintptr_t)15) : a;
+    };
+    auto rest16 = [](const unsigned char *a) { return (uint32_t)reinterpret_cast<uintptr_t>(a) & 15u; };
+    constexpr uint32_t kCopyBytes = (uint32_t)kHalfSlot;
+    const uint32_t tail_bytes = kAny ? (((uint32_t)(tail_valid * (int)sizeof(T)) + 15u) & ~15u) + kSlack : (uint32_t)(tail_valid * (int)sizeof(T));
+    const unsigned char *const zq_begin = reinterpret_cast<const unsigned char *>(p.zq), *const zp_begin = reinterpret_cast<const unsigned char *>(p.zp);
+    // whether copies of [a, a + bytes) of both tensors would leave them
+    auto outside = [&](const unsigned char *q, const unsigned char *pp, size_t bytes) {
+        return floor16(q) < zq_begin || floor16(pp) < zp_begin ||
+               floor16(q) + bytes > zq_begin + (size_t)p.nchains * s.zq_rows * row_bytes ||
+               floor16(pp) + bytes > zp_begin + (size_t)p.nchains * s.gamma * row_bytes;
+    };
+    // rows that may hold such cells (q, pp: this warp's first cells of the row)
+    auto edge_row = [&](const unsigned char *q, const unsigned char *pp) {
+        if (!kAny) return false;
+        const size_t ahead = (size_t)first_cell * kHalfBytes;
+        return outside(q - ahead, pp - ahead, row_bytes + 48);
+    };
+#define SGBV_DIRECT(QROW, PROW, JJ, EDGE)                                                                               \
+    (kAny && (EDGE) &&                                                                                                 \
+     outside((QROW) + (size_t)(JJ) * kStrideBytes, (PROW) + (size_t)(JJ) * kStrideBytes, (JJ) == tail_j ? tail_bytes : kCopyBytes))
+#define SGBV_ISSUE(QROW, PROW, JJ, SLOT, EDGE)                                                                          \
     do {                                                                                                               \
-        const uint32_t bytes_ = ((JJ) == tail_j) ? (uint32_t)(tail_valid * (int)sizeof(T)) : (uint32_t)kHalfBytes;      \
-        issue_cell(ring_u32 + (uint32_t)((SLOT) * kSlotBytes), (QROW) + (size_t)(JJ) * kStrideBytes,                    \
-                   (PROW) + (size_t)(JJ) * kStrideBytes, bytes_, full_u32 + 8u * (uint32_t)(SLOT), is_lane0, kHalfBytes); \
-        pending |= 1u << (SLOT);                                                                                       \
+        if (!SGBV_DIRECT(QROW, PROW, JJ, EDGE)) {                                                                       \
+            issue_cell(ring_u32 + (uint32_t)((SLOT) * kSlotBytes), floor16((QROW) + (size_t)(JJ) * kStrideBytes),       \
+                       floor16((PROW) + (size_t)(JJ) * kStrideBytes), (JJ) == tail_j ? tail_bytes : kCopyBytes,         \
+                       full_u32 + 8u * (uint32_t)(SLOT), is_lane0, kHalfSlot);                                          \
+            pending |= 1u << (SLOT);                                                                                   \
+        }                                                                                                              \
     } while (0)
     // First sweep of cell J of the row whose cells start at (QROW, PROW); the slot is refilled from the same row
     // or, past this warp's last cell, from the row that follows (QNXT, PNXT; only if MORE).
@@ -559,13 +638,18 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             pending ^= 1u << slot_;                                                                                    \
         }                                                                                                              \
         float2 eq_[4], ep_[4];                                                                                         \
-        first_sweep_fetch<T>(ring + slot_ * kSlotBytes, lane, (J) == tail_j, tail_valid, eq_, ep_, mq[J], mp[J]);      \
+        if (SGBV_DIRECT(QROW, PROW, J, edge_b))                                                                        \
+            first_sweep_direct<T>((QROW) + (size_t)(J) * kStrideBytes, (PROW) + (size_t)(J) * kStrideBytes, lane,      \
+                                  (J) == tail_j ? tail_valid : kCell, eq_, ep_, mq[J], mp[J]);                         \
+        else                                                                                                           \
+            first_sweep_fetch<T, kAny>(ring + slot_ * kSlotBytes, rest16(QROW), rest16(PROW), lane, (J) == tail_j,     \
+                                       tail_valid, eq_, ep_, mq[J], mp[J]);                                            \
         /* every lane holds its share of the slot in registers now: refill it */                                       \
         __syncwarp();                                                                                                  \
         if ((J) + NS < ncw) {                                                                                          \
-            if (!timed_out) SGBV_ISSUE(QROW, PROW, (J) + NS, slot_);                                                   \
+            if (!timed_out) SGBV_ISSUE(QROW, PROW, (J) + NS, slot_, edge_b);                                           \
         } else if (MORE) {                                                                                             \
-            SGBV_ISSUE(QNXT, PNXT, slot_, slot_);                                                                      \
+            SGBV_ISSUE(QNXT, PNXT, slot_, slot_, edge_d);                                                              \
         }                                                                                                              \
         first_sweep_store(taddr + 16u * (uint32_t)(J), s.scale, eq_, ep_, mq[J], mp[J], sq[J], sp[J]);                 \
     } while (0)
@@ -577,10 +661,11 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     int i_b = row_mode ? cid % s.gamma : 0;
     const unsigned char *q_b = zq_warp + ((size_t)bk_b * s.zq_rows + i_b) * row_bytes;  // this warp's first cell of row B
     const unsigned char *p_b = zp_warp + ((size_t)bk_b * s.gamma + i_b) * row_bytes;
+    bool edge_b = nrows > 0 && edge_row(q_b, p_b);
     if (nrows > 0) {
 #pragma unroll
         for (int k = 0; k < NS; ++k)
-            if (k < ncw) SGBV_ISSUE(q_b, p_b, k, k);
+            if (k < ncw) SGBV_ISSUE(q_b, p_b, k, k, edge_b);
     }
 
     // The last warp of this CTA combines the partials, carries c_i and fetches the token logits of a row while its
@@ -608,6 +693,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         const bool more = has_d && !timed_out;
         const unsigned char *q_d = zq_warp + ((size_t)bk_d * s.zq_rows + i_d) * row_bytes;
         const unsigned char *p_d = zp_warp + ((size_t)bk_d * s.gamma + i_d) * row_bytes;
+        const bool edge_d = has_d && edge_row(q_d, p_d);
         const size_t r_a = (size_t)bk_a * s.gamma + i_a, r_b = (size_t)bk_b * s.gamma + i_b;
 
         // ---- combining warp: the logits of row B's draft token ------------------------------------------
@@ -641,7 +727,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         // whose plain numerator would cancel, a few per cent: here they slow every row with c < 1, and with it the
         // whole cluster, by more than half, which is worth two more launches only when the step is long.
         const bool aux_row = p.aux_here && rs.c < 1.0f;
-        const bool steady = ncw == kCellsPerWarp && has_a && more && tail_j < 0 && !aux_row;
+        const bool steady = ncw == kCellsPerWarp && has_a && more && tail_j < 0 && !aux_row && !edge_b && !edge_d;
         if (steady) {
 #pragma unroll
             for (int j = 0; j < kCellsPerWarp; ++j) {
@@ -652,16 +738,17 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 mbar_wait(full_u32 + 8u * slot, (phases >> slot) & 1u, timed_out);
                 phases ^= 1u << slot;
                 float2 eq_[4], ep_[4];
-                first_sweep_fetch<T>(ring + slot * kSlotBytes, lane, false, tail_valid, eq_, ep_, mq[j], mp[j]);
+                first_sweep_fetch<T, kAny>(ring + slot * kSlotBytes, rest16(q_b), rest16(p_b), lane, false, tail_valid, eq_, ep_,
+                                           mq[j], mp[j]);
                 __syncwarp();  // every lane holds its share of the slot in registers now: refill it
                 if (j + NS < kCellsPerWarp)
-                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), q_b + (size_t)(j + NS) * kStrideBytes,
-                               p_b + (size_t)(j + NS) * kStrideBytes, kHalfBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
-                               kHalfBytes);
+                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), floor16(q_b) + (size_t)(j + NS) * kStrideBytes,
+                               floor16(p_b) + (size_t)(j + NS) * kStrideBytes, kCopyBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
+                               kHalfSlot);
                 else
-                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), q_d + (size_t)slot * kStrideBytes,
-                               p_d + (size_t)slot * kStrideBytes, kHalfBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
-                               kHalfBytes);
+                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), floor16(q_d) + (size_t)slot * kStrideBytes,
+                               floor16(p_d) + (size_t)slot * kStrideBytes, kCopyBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
+                               kHalfSlot);
                 first_sweep_store(taddr + 16u * (uint32_t)j, s.scale, eq_, ep_, mq[j], mp[j], sq[j], sp[j]);
             }
         } else if (has_a && aux_row) {  // the rare kind of row: two more sums per cell
@@ -760,10 +847,12 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             const float4 v = lane < kFWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
             float bq_row = warp_max_redux(v.x), bp_row = warp_max_redux(v.z);
             float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-            float Zq = warp_sum(v.x > -INFINITY ? v.y * ex2((v.x - rq_row) * s.scale) : 0.0f);
-            float Zp = warp_sum(v.z > -INFINITY ? v.w * ex2((v.z - rp_row) * s.scale) : 0.0f);
+            // (kAny: in float64, as the two-sweep path does that such rows took before)
+            typedef typename Sum<kAny>::type Z;
+            Z Zq = warp_sum(v.x > -INFINITY ? (Z)v.y * (Z)ex2((v.x - rq_row) * s.scale) : (Z)0);
+            Z Zp = warp_sum(v.z > -INFINITY ? (Z)v.w * (Z)ex2((v.z - rp_row) * s.scale) : (Z)0);
             if (C > 1) {  // the same once more over the CTAs of the cluster
-                if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, make_float4(bq_row, Zq, bp_row, Zp));
+                if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, make_float4(bq_row, (float)Zq, bp_row, (float)Zp));
                 mbar_wait(xbar, xph, timed_out);
                 timed_out = __any_sync(0xffffffffu, timed_out != 0);
                 const float4 cv = lane < C ? ctl->slots[par][lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
@@ -771,8 +860,8 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 bp_row = warp_max_redux(cv.z);
                 rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f;
                 rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-                Zq = warp_sum(cv.x > -INFINITY ? cv.y * ex2((cv.x - rq_row) * s.scale) : 0.0f);
-                Zp = warp_sum(cv.z > -INFINITY ? cv.w * ex2((cv.z - rp_row) * s.scale) : 0.0f);
+                Zq = warp_sum(cv.x > -INFINITY ? (Z)cv.y * (Z)ex2((cv.x - rq_row) * s.scale) : (Z)0);
+                Zp = warp_sum(cv.z > -INFINITY ? (Z)cv.w * (Z)ex2((cv.z - rp_row) * s.scale) : (Z)0);
             }
             // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
             // NEXT row needs it, so it is worked out after the other warps have been released.
@@ -852,7 +941,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             if (lane == 0 && rank == 0) {
                 // nonfinite logits: NaN poisons Z, +inf shows up as an infinite maximum, a row of
                 // -inf only has Z = 0
-                const bool bad = !(Zq > 0.0f) || !(Zp > 0.0f) || !(Zq < INFINITY) || !(Zp < INFINITY) ||
+                const bool bad = !(Zq > 0.0f) || !(Zp > 0.0f) || !(Zq < (Z)INFINITY) || !(Zp < (Z)INFINITY) ||
                                  !(bq_row < INFINITY) || !(bp_row < INFINITY);
                 RowInfo ri;
                 ri.flags = bad ? SGBV_STATUS_NONFINITE_LOGIT : 0;
@@ -882,6 +971,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         i_b = i_d;
         q_b = q_d;
         p_b = p_d;
+        edge_b = edge_d;
     }
     // a warp that gave up may still have copies under way: they must land before the shared memory goes
     if (timed_out) {
@@ -897,6 +987,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     __syncthreads();  // every warp of this CTA is done with the tensor memory
     if (warp == 0) tmem_dealloc(ctl->tmem_base, kTmemCols);
 #undef SGBV_ISSUE
+#undef SGBV_DIRECT
 #undef SGBV_FIRST_SWEEP_CELL
 #undef SGBV_C0
 }
@@ -922,19 +1013,19 @@ constexpr int kCtaSlots = 148 * kCtasPerSm;  // CTAs the device holds
 // ring slots per warp: half a row's cells for float32 (128 KB of copies under way per SM), all of them for bfloat16
 template <typename T>
 constexpr int slots_for() { return (sizeof(T) == 4 ? 2 : 4) * 32 / kWarps / kCtasPerSm; }
-template <typename T>
+template <typename T, bool kAny>
 constexpr size_t smem_bytes() {
-    return (size_t)kWarps * slots_for<T>() * (2 * kCell * sizeof(T) + 8) + (size_t)(kCtaCells / kWarps) * kWarps * 32 * 4 + sizeof(Control);
+    return (size_t)kWarps * slots_for<T>() * (2 * (kCell * sizeof(T) + (kAny ? kSlack : 0)) + 8) + (size_t)(kCtaCells / kWarps) * kWarps * 32 * 4 + sizeof(Control);
 }
 int slice_cells_of(int cells, int C) { return (cells + C - 1) / C; }
 
-template <typename T, bool kRow, int KT>
+template <typename T, bool kRow, int KT, bool kAny>
 cudaError_t prepare(int dev) {
     static bool attr_done[kDevices];
     if (!attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
+        cudaError_t e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
@@ -942,14 +1033,14 @@ cudaError_t prepare(int dev) {
 }
 
 // Clusters of C CTAs of this kernel that the device runs side by side (queried once per configuration).
-template <typename T, bool kRow, int KT>
+template <typename T, bool kRow, int KT, bool kAny>
 int resident_clusters(int dev, int C) {
     static int cached[kDevices][kMaxCluster + 1];
     int &slot = cached[dev][C];
     if (slot == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.blockDim = dim3(kWarps * 32);
-        cfg.dynamicSmemBytes = smem_bytes<T>();
+        cfg.dynamicSmemBytes = smem_bytes<T, kAny>();
         cfg.gridDim = dim3(C * (kCtaSlots / C));
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -959,7 +1050,7 @@ int resident_clusters(int dev, int C) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nmax = 0;
-        if (cudaOccupancyMaxActiveClusters(&nmax, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT>, &cfg) != cudaSuccess || nmax < 1) {
+        if (cudaOccupancyMaxActiveClusters(&nmax, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, &cfg) != cudaSuccess || nmax < 1) {
             cudaGetLastError();
             return 0;
         }
@@ -968,7 +1059,7 @@ int resident_clusters(int dev, int C) {
     return slot;
 }
 
-template <typename T, bool kRow, int KT>
+template <typename T, bool kRow, int KT, bool kAny>
 int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, bool aux_here) {
     FusedParams fp;
     fp.zq = L.zq;
@@ -988,7 +1079,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
 
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kWarps * 32);
-    cfg.dynamicSmemBytes = smem_bytes<T>();
+    cfg.dynamicSmemBytes = smem_bytes<T, kAny>();
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1009,7 +1100,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
         cudaMemsetAsync(L.ws.ratio, 0xff, (size_t)fp.nchains * L.s.gamma * sizeof(double), L.stream) != cudaSuccess)
         return SGBV_ERR_CUDA;
     if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT>, fp);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, fp);
     if (L.ev_end) cudaEventRecord(L.ev_end, L.stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1019,14 +1110,14 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
 }
 
 // Chooses the cluster size and the walk, then launches.  Returns launches, 0 if declined, or < 0.
-template <typename T, int KT>
+template <typename T, int KT, bool kAny>
 int plan_and_launch(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart) {
     const Shape &s = L.s;
     const int cells = s.ntiles;
     const long nchains = (long)s.B * s.cpr, units = nchains * s.gamma;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return SGBV_ERR_CUDA;
-    if (prepare<T, false, KT>(dev) != cudaSuccess || prepare<T, true, KT>(dev) != cudaSuccess) {
+    if (prepare<T, false, KT, kAny>(dev) != cudaSuccess || prepare<T, true, KT, kAny>(dev) != cudaSuccess) {
         cudaGetLastError();
         return SGBV_ERR_CUDA;
     }
@@ -1035,7 +1126,7 @@ int plan_and_launch(const Launch &L, int *error_flag, bool *walked_rows, bool *a
     if (Cmin > kMaxCluster) return 0;
     auto fits = [&](int C) { return C >= Cmin && C <= kMaxCluster; };
     auto resident = [&](int C, bool row) {
-        return row ? resident_clusters<T, true, KT>(dev, C) : resident_clusters<T, false, KT>(dev, C);
+        return row ? resident_clusters<T, true, KT, kAny>(dev, C) : resident_clusters<T, false, KT, kAny>(dev, C);
     };
     // Few units of work: spread each over more CTAs (at least half the warps keep a cell) while all of them
     // still run side by side.
@@ -1070,8 +1161,8 @@ int plan_and_launch(const Launch &L, int *error_flag, bool *walked_rows, bool *a
     // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed)
     const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1));
     *aux_apart = !aux_here;
-    return plan.row_mode ? launch_as<T, true, KT>(L, plan, error_flag, clusters, true)
-                         : launch_as<T, false, KT>(L, plan, error_flag, clusters, aux_here);
+    return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true)
+                         : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here);
 }
 
 }  // namespace
@@ -1086,23 +1177,18 @@ void fused_set_options(int cluster, int max_clusters, int walk, int poll_us, int
     g_opt_poll_us = poll_us;
 }
 
-// Whether the fused path can take this call: rows must be 16-byte aligned for the bulk copies and a
-// row must fit the tensor memory of a cluster (8 CTAs x 32,768 entries).
-bool fused_supported(const Launch &L) {
-    const size_t esz = L.dtype == SGBV_DTYPE_BF16 ? 2 : 4;
-    if (((uintptr_t)L.zq % 16) || ((uintptr_t)L.zp % 16) || (((size_t)L.s.V * esz) % 16)) return false;
-    return L.s.ntiles <= kMaxCluster * kCtaCells;
-}
+// Whether the fused path can take this call: a row must fit the tensor memory of a cluster (8 CTAs x 32,768 entries).
+bool fused_supported(const Launch &L) { return L.s.ntiles <= kMaxCluster * kCtaCells; }
 
-template <typename T>
+template <typename T, bool kAny>
 int dispatch_k(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart) {
     switch (L.s.K) {
-        case 1: return plan_and_launch<T, 1>(L, error_flag, walked_rows, aux_apart);
-        case 2: return plan_and_launch<T, 2>(L, error_flag, walked_rows, aux_apart);
-        case 3: return plan_and_launch<T, 3>(L, error_flag, walked_rows, aux_apart);
-        case 4: return plan_and_launch<T, 4>(L, error_flag, walked_rows, aux_apart);
-        case 8: return plan_and_launch<T, 8>(L, error_flag, walked_rows, aux_apart);
-        default: return plan_and_launch<T, 0>(L, error_flag, walked_rows, aux_apart);
+        case 1: return plan_and_launch<T, 1, kAny>(L, error_flag, walked_rows, aux_apart);
+        case 2: return plan_and_launch<T, 2, kAny>(L, error_flag, walked_rows, aux_apart);
+        case 3: return plan_and_launch<T, 3, kAny>(L, error_flag, walked_rows, aux_apart);
+        case 4: return plan_and_launch<T, 4, kAny>(L, error_flag, walked_rows, aux_apart);
+        case 8: return plan_and_launch<T, 8, kAny>(L, error_flag, walked_rows, aux_apart);
+        default: return plan_and_launch<T, 0, kAny>(L, error_flag, walked_rows, aux_apart);
     }
 }
 
@@ -1110,8 +1196,14 @@ int launch_fused(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_
     *walked_rows = false;
     *aux_apart = false;
     std::lock_guard<std::mutex> lock(g_plan_mu);
-    return L.dtype == SGBV_DTYPE_BF16 ? dispatch_k<uint16_t>(L, error_flag, walked_rows, aux_apart)
-                                      : dispatch_k<float>(L, error_flag, walked_rows, aux_apart);
+    // rows that all start on 16-byte boundaries?
+    const size_t esz = L.dtype == SGBV_DTYPE_BF16 ? 2 : 4;
+    const bool any = ((uintptr_t)L.zq % 16) || ((uintptr_t)L.zp % 16) || (((size_t)L.s.V * esz) % 16);
+    if (L.dtype == SGBV_DTYPE_BF16)
+        return any ? dispatch_k<uint16_t, true>(L, error_flag, walked_rows, aux_apart)
+                   : dispatch_k<uint16_t, false>(L, error_flag, walked_rows, aux_apart);
+    return any ? dispatch_k<float, true>(L, error_flag, walked_rows, aux_apart)
+               : dispatch_k<float, false>(L, error_flag, walked_rows, aux_apart);
 }
 
 }  // namespace sgbv

@@ -317,6 +317,38 @@ def test_unaligned_views_and_repeated_calls_are_deterministic():
         assert torch.equal(a.h, b.h) and torch.equal(a.resmass, b.resmass)
 
 
+@pytest.mark.parametrize("B,K,gamma,V,dtype,walk", [
+    (2, 2, 3, 32003, "bf16", 0),      # row walk
+    (40, 3, 4, 8191, "fp32", 0),      # chain walk, chains cut between clusters
+    (20, 8, 4, 33025, "bf16", 1),     # clusters of two, a last cell of one entry
+    (3, 1, 2, 131071, "fp32", 1),     # one draft, four CTAs
+    (2, 5, 2, 1023, "bf16", 1),       # a draft count without a specialised kernel
+    (4, 2, 3, 777, "bf16", 0),        # a few cells
+])
+def test_rows_that_start_anywhere(B, K, gamma, V, dtype, walk):
+    """The fused kernel on rows that do not start on 16-byte boundaries, with the two tensors off theirs by different
+    amounts and each ending where its allocation ends: parity with the oracle, and the same bits wherever the tensors lie."""
+    cfg = workloads.VerifyConfig(f"any_{V}", B=B, K=K, gamma=gamma, V=V, dtype=dtype, temperature=0.8, alpha=0.85, seed=V)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t, shift):
+        return torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape).copy_(t)
+    binding.set_option("walk", walk)
+    try:
+        outs = []
+        for sq, sp in ((0, 0), (1, 3), (3, 2)):
+            rep, out, _ = run_both(workloads.VerifyInputs(cfg, moved(inp.target_logits, sq), moved(inp.draft_logits, sp),
+                                                          inp.draft_tokens, inp.uniforms))
+            assert binding.last_main_kernel() == "fused_chain_kernel"
+            assert_parity(rep)
+            outs.append(out)
+    finally:
+        binding.set_option("walk", 0)
+    for o in outs[1:]:
+        assert torch.equal(o.tokens, outs[0].tokens) and torch.equal(o.status, outs[0].status)
+        assert torch.equal(o.h, outs[0].h) and torch.equal(o.resmass, outs[0].resmass)
+
+
 def test_degenerate_and_flagged_rows():
     cfg = workloads.VerifyConfig("flags", B=6, K=2, gamma=2, V=300, alpha=0.8, seed=7)
     inp = workloads.make_inputs(cfg, device="cuda")
