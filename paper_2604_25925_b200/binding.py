@@ -6,6 +6,7 @@ missing library or a non-CUDA tensor raises.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 from dataclasses import dataclass
@@ -31,6 +32,19 @@ EXPORTS = ("sgbv_workspace_bytes", "sgbv_verify", "sgbv_verify_bf16", "sgbv_veri
            "sgbv_shard_stats", "sgbv_shard_sums", "sgbv_shard_decide", "sgbv_shard_draw")
 
 _lib = None
+_HERE = contextlib.nullcontext()
+
+
+def _on(dev: torch.device):
+    """Makes `dev` the current device for a call; nothing to do where it already is (entering and leaving
+    ``torch.cuda.device`` costs 1.4 us)."""
+    here = dev.type == "cuda" and torch.cuda.current_device() == dev.index
+    return _HERE if here else torch.cuda.device(dev)
+
+
+def _stream(dev: torch.device) -> int:
+    """Handle of the current stream of `dev` (0.1 us; 2.2 us through a ``torch.cuda.Stream`` object)."""
+    return torch._C._cuda_getCurrentRawStream(dev.index)
 
 
 class SgbvError(RuntimeError):
@@ -192,10 +206,10 @@ def sgbv_verify(target_logits, draft_logits, draft_tokens, uniforms, temperature
                            torch.empty(B, dtype=torch.int32, device=dev),
                            torch.empty((B, gamma + 1), dtype=torch.int32, device=dev))
     fn = load().sgbv_verify if _dtype_code(target_logits) == DTYPE_F32 else load().sgbv_verify_bf16
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = fn(target_logits.data_ptr(), draft_logits.data_ptr(), draft_tokens.data_ptr(),
                 uniforms.data_ptr(), B, K, gamma, V, float(temperature), out.accept_len.data_ptr(),
-                out.draft_idx.data_ptr(), out.tokens.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
+                out.draft_idx.data_ptr(), out.tokens.data_ptr(), _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -219,7 +233,7 @@ def sgbv_verify_ex(target_logits, draft_logits, draft_tokens, uniforms, temperat
         out.status = torch.empty(B, dtype=torch.int32, device=dev)
     ws_ptr, ws_bytes = (workspace.data_ptr(), workspace.numel() * workspace.element_size()) \
         if workspace is not None else (None, 0)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_verify_ex(
             target_logits.data_ptr(), draft_logits.data_ptr(), _dtype_code(target_logits),
             draft_tokens.data_ptr(), uniforms.data_ptr(), B, K, gamma, V, float(temperature),
@@ -227,7 +241,7 @@ def sgbv_verify_ex(target_logits, draft_logits, draft_tokens, uniforms, temperat
             out.h.data_ptr() if out.h is not None else None,
             out.resmass.data_ptr() if out.resmass is not None else None,
             out.status.data_ptr() if out.status is not None else None,
-            torch.cuda.current_stream(dev).cuda_stream)
+            _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -255,7 +269,7 @@ def sgbv_verify_static(target_logits, draft_logits, draft_tokens, uniforms, temp
                            torch.empty((B, K, gamma), dtype=torch.float64, device=dev),
                            torch.empty((B, K, gamma), dtype=torch.float64, device=dev),
                            torch.empty(B, dtype=torch.int32, device=dev))
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_verify_static(
             target_logits.data_ptr(), draft_logits.data_ptr(), _dtype_code(target_logits),
             draft_tokens.data_ptr(), uniforms.data_ptr(), B, K, gamma, V, float(temperature),
@@ -263,7 +277,7 @@ def sgbv_verify_static(target_logits, draft_logits, draft_tokens, uniforms, temp
             out.h.data_ptr() if out.h is not None else None,
             out.resmass.data_ptr() if out.resmass is not None else None,
             out.status.data_ptr() if out.status is not None else None,
-            torch.cuda.current_stream(dev).cuda_stream)
+            _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -321,12 +335,12 @@ def sgbv_modify(target_logits, draft_logits, log_a, log_b, uniforms, K: int, tem
                        torch.empty(B, dtype=torch.int32, device=dev))
     ws_ptr, ws_bytes = (workspace.data_ptr(), workspace.numel() * workspace.element_size()) \
         if workspace is not None else (None, 0)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_modify(target_logits.data_ptr(), draft_logits.data_ptr(), _dtype_code(target_logits),
                                 log_a.data_ptr(), log_b.data_ptr(), uniforms.data_ptr(), B, int(K), V,
                                 float(temperature), out.token.data_ptr(), out.log_a.data_ptr(), out.log_b.data_ptr(),
                                 out.resmass.data_ptr(), out.status.data_ptr(), ws_ptr, ws_bytes,
-                                torch.cuda.current_stream(dev).cuda_stream)
+                                _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -350,12 +364,12 @@ def sgbv_verify_kseq(target_logits, draft_logits, draft_tokens, uniforms, temper
                              torch.empty((B, gamma), dtype=torch.float64, device=dev),
                              torch.empty((B, K, gamma), dtype=torch.float64, device=dev),
                              torch.empty(B, dtype=torch.int32, device=dev))
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_verify_kseq(target_logits.data_ptr(), draft_logits.data_ptr(), _dtype_code(target_logits),
                                      draft_tokens.data_ptr(), uniforms.data_ptr(), B, K, gamma, V, float(temperature),
                                      out.accept_len.data_ptr(), out.tokens.data_ptr(), out.rho.data_ptr(),
                                      out.accept_prob.data_ptr(), out.status.data_ptr(), None, 0,
-                                     torch.cuda.current_stream(dev).cuda_stream)
+                                     _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -372,11 +386,11 @@ def _single_draft(name, target_logits, draft_logits, draft_tokens, uniforms, tem
                              torch.empty((B, gamma + 1), dtype=torch.int32, device=dev), None,
                              torch.empty((B, 1, gamma), dtype=torch.float64, device=dev),
                              torch.empty(B, dtype=torch.int32, device=dev))
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = getattr(load(), name)(target_logits.data_ptr(), draft_logits.data_ptr(), _dtype_code(target_logits),
                                    draft_tokens.data_ptr(), uniforms.data_ptr(), B, gamma, V, float(temperature),
                                    out.accept_len.data_ptr(), out.tokens.data_ptr(), out.accept_prob.data_ptr(),
-                                   out.status.data_ptr(), None, 0, torch.cuda.current_stream(dev).cuda_stream)
+                                   out.status.data_ptr(), None, 0, _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -404,10 +418,10 @@ def sgbv_draw_tokens(logits, uniforms, temperature: float = 1.0):
     tok = torch.empty(N, dtype=torch.int32, device=dev)
     lp = torch.empty(N, dtype=torch.float64, device=dev)
     st = torch.empty(N, dtype=torch.int32, device=dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_draw_tokens(logits.data_ptr(), _dtype_code(logits), uniforms.data_ptr(), N, V, float(temperature),
                                      tok.data_ptr(), lp.data_ptr(), st.data_ptr(), None, 0,
-                                     torch.cuda.current_stream(dev).cuda_stream)
+                                     _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return tok, lp, st
@@ -438,10 +452,10 @@ def sgbv_shard_stats(target_shard, draft_shard, draft_tokens, v_begin: int, V: i
     B, K, gamma, Vs = _shard_shapes(target_shard, draft_shard)
     dev = target_shard.device
     out = torch.empty((B, K, gamma + 1, 8), dtype=torch.float32, device=dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_shard_stats(target_shard.data_ptr(), draft_shard.data_ptr(), _dtype_code(target_shard),
                                      draft_tokens.data_ptr(), B, K, gamma, Vs, int(v_begin), int(V), float(temperature),
-                                     out.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
+                                     out.data_ptr(), _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -454,11 +468,11 @@ def sgbv_shard_sums(target_shard, draft_shard, temperature: float, stats_all, wo
     if tuple(stats_all.shape[1:]) != (B, K, gamma + 1, 8) or stats_all.dtype != torch.float32 or not stats_all.is_contiguous():
         raise ValueError("stats_all must be contiguous float32 [n_ranks,B,K,gamma+1,8]")
     out = torch.empty((B, K, gamma, 3), dtype=torch.float64, device=dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_shard_sums(target_shard.data_ptr(), draft_shard.data_ptr(), _dtype_code(target_shard), B, K, gamma,
                                     Vs, float(temperature), stats_all.data_ptr(), int(stats_all.shape[0]),
                                     workspace.data_ptr(), workspace.numel(), out.data_ptr(),
-                                    torch.cuda.current_stream(dev).cuda_stream)
+                                    _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -478,13 +492,13 @@ def sgbv_shard_decide(draft_tokens, uniforms, shard_V: int, temperature: float, 
                        torch.empty((B, K, gamma), dtype=torch.float64, device=dev),
                        torch.empty((B, K, gamma), dtype=torch.float64, device=dev),
                        torch.empty(B, dtype=torch.int32, device=dev))
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_shard_decide(draft_tokens.data_ptr(), uniforms.data_ptr(), B, K, gamma, int(shard_V),
                                       float(temperature), stats_all.data_ptr(), sums_all.data_ptr(), int(stats_all.shape[0]),
                                       workspace.data_ptr(), workspace.numel(), out.accept_len.data_ptr(),
                                       out.draft_idx.data_ptr(), out.tokens.data_ptr(), out.h.data_ptr(),
                                       out.resmass.data_ptr(), out.status.data_ptr(),
-                                      torch.cuda.current_stream(dev).cuda_stream)
+                                      _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
     return out
@@ -494,9 +508,9 @@ def sgbv_shard_draw(target_shard, draft_shard, v_begin: int, temperature: float,
     """The owning rank writes the extra token's global id into tokens[b, accept_len] (in place)."""
     B, K, gamma, Vs = _shard_shapes(target_shard, draft_shard)
     dev = target_shard.device
-    with torch.cuda.device(dev):
+    with _on(dev):
         rc = load().sgbv_shard_draw(target_shard.data_ptr(), draft_shard.data_ptr(), _dtype_code(target_shard), B, K, gamma,
                                     Vs, int(v_begin), float(temperature), int(rank), workspace.data_ptr(), workspace.numel(),
-                                    tokens.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
+                                    tokens.data_ptr(), _stream(dev))
     if rc != OK:
         raise SgbvError(rc)
