@@ -158,6 +158,13 @@ __device__ __forceinline__ double exp2_short(double x) {
 // e^x through the same short chain.
 __device__ __forceinline__ double exp_short(double x) { return exp2_short(x * 1.4426950408889634074); }
 
+// A value that is the same in all lanes of a warp, said so to the compiler: lane 0's.  Behind a branch or an early return on a
+// value that it cannot prove to be uniform (anything read from memory) the warp's lanes ran apart in the finishing and the
+// K-SEQ kernel, and every later shuffle took some 300 cycles instead of 25.
+template <typename V>
+__device__ __forceinline__ V uniform(V v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int warp_index() { return uniform((int)(threadIdx.x >> 5)); }
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

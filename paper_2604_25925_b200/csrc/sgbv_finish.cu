@@ -15,7 +15,6 @@ namespace {
 
 constexpr int kMaxThreads = 1024;  // CTA size when few batch rows leave most SMs idle (the kernel is a
 constexpr int kMinThreads = 256;   // chain of memory latencies, so more warps per row help); else 512 or 256
-constexpr int kMaxWarps = kMaxThreads / 32;
 constexpr int kTilesInSmem = 4096;  // rows up to 2^20 entries keep the bonus row's tile sums in shared memory
 static_assert(kMinThreads >= kTile, "one thread per element of a tile");
 
@@ -43,7 +42,6 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
                                                : ws.bonus + (size_t)blockIdx.x * 2 * s.ntiles;  // [ntiles]
     float *tile_m = tile_s + s.ntiles;                                        // [ntiles]
     __shared__ SampleScratch sc;
-    __shared__ unsigned sh_or[2];
     __shared__ int sh_flags;
     double *sh_warp = sc.warp;
     int *sh_pick = sc.pick, *sh_i = sc.i;
@@ -54,7 +52,7 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     // Only for small batches, where this grid leaves most SMs idle.
     if (s.B <= kChainedLaunchMaxB) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int nthreads = blockDim.x, nwarps = nthreads / 32;
     const int32_t *tok = tok_all + (size_t)b * KG;
     const float *u = u_all + (size_t)b * (KG + 1);
@@ -69,7 +67,7 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     // before touching the row records and cell sums.
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();  // the staged tokens and uniforms are read by other threads than those that fetched them
-    const bool lost = *ws.error != 0;  // a bounded wait expired upstream: nothing can be trusted
+    const bool lost = uniform(*ws.error) != 0;  // a bounded wait expired upstream: nothing can be trusted
     // the streaming kernel has consumed the "not published yet" pattern of this batch row's ratio words:
     // put it back, so that the next call on this scratch area need not clear them first
     if (ws.ratio_used)
@@ -143,7 +141,7 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     // block-wide OR of the flags (rarely any), then the barrier after the loop
     if (myflags) atomicOr(&sh_flags, myflags);
     __syncthreads();
-    const int status_in = sh_flags & (SGBV_STATUS_TOKEN_RANGE | SGBV_STATUS_NONFINITE_LOGIT);
+    const int status_in = uniform(sh_flags) & (SGBV_STATUS_TOKEN_RANGE | SGBV_STATUS_NONFINITE_LOGIT);
     const bool invalid = lost || status_in != 0;
     // la_s/lb_s[k][i+1] now hold log q_i(x_k^i), log p_i(x_k^i); every user below adds up the terms it needs
     // itself, in the order of a running sum (at most gamma additions, and no pass and barrier of its own)
@@ -172,13 +170,13 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
         ws.resmass[(size_t)b * KG + n] = invalid ? NAN : S;
         if (i >= 1) {
             const double hv = weight_sub(la, lb, R, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, below, exact_s[n] != 0);
-            if ((double)u_s[k * g + i - 1] < hv) atomicOr(&pass_s[k], 1ull << (i - 1));
+            if ((double)u_s[k * g + i - 1] < hv) set_bit(&pass_s[k], i - 1);
             ws.h[(size_t)b * KG + k * g + i - 1] = invalid ? NAN : hv;
         }
     }
     for (int k = tid; k < K; k += nthreads) {  // the first threads, while the last ones do Eq. 2
         const double hv = weight_full(prefix(la_s + k * (g + 1), g), prefix(lb_s + k * (g + 1), g), K);
-        if ((double)u_s[k * g + g - 1] < hv) atomicOr(&pass_s[k], 1ull << (g - 1));
+        if ((double)u_s[k * g + g - 1] < hv) set_bit(&pass_s[k], g - 1);
         ws.h[(size_t)b * KG + k * g + g - 1] = invalid ? NAN : hv;
     }
     // longest common prefix of every pair of drafts (for the membership test in H)
@@ -203,14 +201,14 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     // ---- 2. scan (Algorithm 1), warp 0 ---------------------------------------------------------
     if (wid == 0) {
         int tau, f;
-        scan_block(pass_s, lcp_s, K, g, sh_or, tau, f);
+        scan_block(pass_s, lcp_s, K, g, tau, f);
         if (lane == 0) {
             sh_i[0] = tau;
             sh_i[1] = f;
         }
     }
     __syncthreads();
-    const int tau = sh_i[0], f = sh_i[1];
+    const int tau = uniform(sh_i[0]), f = uniform(sh_i[1]);
     const int kk = (tau == 0) ? 0 : f;
     const double us = (double)u_s[KG];
 
@@ -221,7 +219,7 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     bool from_q = (tau == g);
     if (!from_q) {
         const size_t r = ((size_t)b * K + kk) * g + tau;
-        const double W = W_s[kk * g + tau];
+        const double W = uniform(W_s[kk * g + tau]);
         if (W > 0.0) {
             const float *wp = ws.wpart + r * s.ntiles;
             const RowInfo ri = ws.rows[r];  // fetched while the tile is being located
@@ -275,19 +273,19 @@ modify_finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all,
                      Workspace ws, const double *carry_loga, const double *carry_logb, int32_t *__restrict__ out_token,
                      double *out_loga, double *out_logb, double *__restrict__ out_resmass, int32_t *__restrict__ out_status) {
     __shared__ SampleScratch sc;
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int nthreads = blockDim.x, nwarps = nthreads / 32;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // (launched behind the streaming kernel)
-    const bool lost = *ws.error != 0;
+    const bool lost = uniform(*ws.error) != 0;
     const RowInfo ri = ws.rows[b];
-    const int status_in = (ri.flags | (ws.prestatus ? ws.prestatus[b] : 0)) & SGBV_STATUS_NONFINITE_LOGIT;
+    const int status_in = uniform((ri.flags | (ws.prestatus ? ws.prestatus[b] : 0)) & SGBV_STATUS_NONFINITE_LOGIT);
     const float *wp = ws.wpart + (size_t)b * s.ntiles;
     double local = 0.0;
     for (int t = tid; t < s.ntiles; t += nthreads) local += (double)wp[t];
     local = warp_sum(local);
     if (lane == 0) sc.warp[wid] = local;
     __syncthreads();
-    const double W = warp_sum(lane < nwarps ? sc.warp[lane] : 0.0);
+    const double W = uniform(warp_sum(lane < nwarps ? sc.warp[lane] : 0.0));
     __syncthreads();
     const double la = carry_loga[b], lb = carry_logb[b];
     if (lost || status_in) {

@@ -21,7 +21,7 @@
 // What bounds it is the serial chain: positions one after the other, some six sweeps and as many cluster exchanges each.
 // Rows stay on chip between the sweeps (a CTA holds up to kCapTiles tiles; the rest of a longer share is read again in
 // every sweep), and a row is spread over as many CTAs as the batch leaves free.  64 prompts, K = 3, gamma = 12, 32256
-// float32: 99 us, against 424 us of one CTA of 1024 threads per prompt that read the rows from L2 in two sweeps for the
+// float32: 71 us, against 424 us of one CTA of 1024 threads per prompt that read the rows from L2 in two sweeps for the
 // statistics and one for each of 34 bisections.  (Two prompts in three stop at the first or second position; the time is
 // that of the longest walk.)
 #include <atomic>
@@ -63,7 +63,7 @@ struct KseqScratch {
 // slots[par][r] keeps CTA r's share until the exchange after the next one.  All threads must call.
 template <bool kMaximum>
 __device__ __forceinline__ void exchange(double &a, double &b, KseqScratch &sc, int rank, int C, int &par) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = warp_index();
     auto op = [](double x, double y) { return kMaximum ? fmax(x, y) : x + y; };
     auto all = [&](double v) {
 #pragma unroll
@@ -107,7 +107,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
     __shared__ KseqScratch sc;
     const int rank = (int)cluster_ctarank();
     cluster_arrive();
-    const int b = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int b = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int K = s.K, g = s.gamma, V = s.V;
     const int32_t *tok = tok_all + (size_t)b * K * g;
     const float *u = u_all + (size_t)b * (K * g + 1);
@@ -147,7 +147,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
     int tau = 0, flags = 0, par = 0;
     bool stopped = false;
     for (int i = 0; i < g && !stopped; ++i) {
-        const int k0 = sc.kept[0], nk = sc.n;
+        const int k0 = uniform(sc.kept[0]), nk = uniform(sc.n);
         const T *zq = zq_all + (((size_t)b * K + k0) * (g + 1) + i) * V;
         const T *zp = zp_all + (((size_t)b * K + k0) * g + i) * V;
         // the logits of the retained drafts' tokens, fetched ahead (first warp, two drafts per lane)
@@ -237,7 +237,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         double Zq = (double)sq, Zp = (double)sp;
         exchange<false>(Zq, Zp, sc, rank, C, par);
         // NaN entries end up in the sums; +inf is its row's maximum and gives inf - inf there
-        if (!(mq > -INFINITY) || !(mp > -INFINITY) || Zq != Zq || Zp != Zp) {
+        if (uniform((int)(!(mq > -INFINITY) || !(mp > -INFINITY) || Zq != Zq || Zp != Zp))) {
             flags |= SGBV_STATUS_NONFINITE_LOGIT;
             break;
         }
@@ -271,13 +271,13 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
                 const double f = gfun_n(beta, nk, gs) - (S1 + rho * S2);
                 if (f > 0.0) lo = rho;
                 else hi = rho;
-                if (hi <= lo) break;  // (f <= 0 at 1: the root is 1)
+                if (uniform((int)(hi <= lo))) break;  // (f <= 0 at 1: the root is 1)
                 const double df = -gs * S1 / (rho * rho) - S2;
                 double next = rho - f / df;
                 if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
                 const double step = fabs(next - rho);
                 rho = next;
-                if (step <= 1e-10 * rho) break;
+                if (uniform((int)(step <= 1e-10 * rho))) break;
             }
         }
         // ---- 3. the retained drafts, in order (first warp of every CTA) -----------------------------------------
@@ -323,7 +323,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
             }
         }
         __syncthreads();
-        if (sc.accepted >= 0) {
+        if (uniform(sc.accepted) >= 0) {
             tau = i + 1;
             continue;
         }
@@ -350,7 +350,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         for (int t = tid; t < t1 - t0; t += kThreads) W += (double)tile_s[t];
         exchange<false>(W, unused, sc, rank, C, par);
         const double us = (double)u[K * g];
-        if (W > 0.0) {
+        if (uniform((int)(W > 0.0))) {
             // the CTA whose share the target falls into draws
             const double target = us * W;
             double run = 0.0, before = 0.0;
@@ -362,7 +362,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
                 if (r < rank) before += v;
                 run += v;
             }
-            if (rank == (owner < 0 ? last : owner) && wid == 0) {
+            if (rank == uniform(owner < 0 ? last : owner) && wid == 0) {
                 auto weight = [&](int t) { return (double)tile_s[t]; };
                 const int y = warp_draw(weight, t1 - t0, t0, V, owner < 0 ? INFINITY : target - before, entry);
                 if (lane == 0) out_tokens[(size_t)b * (g + 1) + i] = y;

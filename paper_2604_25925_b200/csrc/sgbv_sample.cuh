@@ -31,7 +31,7 @@ struct Pick {
 // weight before the tile. All threads must call.
 template <typename F>
 __device__ Pick pick_in_tile(int x0, int x1, double base, double target, F wfun, double *sh_warp, int *sh_pick) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     float w[kEpt];
     double local = 0.0;
 #pragma unroll
@@ -81,7 +81,7 @@ __device__ Pick pick_in_tile(int x0, int x1, double base, double target, F wfun,
 // sh_d[1] = target.
 static __device__ void locate_tile(const float *partials, const float *scale, int ntiles, double target, bool relative,
                             int *sh_i, double *sh_d, double *sh_warp) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int nthreads = blockDim.x;
     const int per = (ntiles + nthreads - 1) / nthreads;
     const int t0 = min(ntiles, tid * per), t1 = min(ntiles, t0 + per);
@@ -180,7 +180,7 @@ __device__ __forceinline__ void load_tile_pieces<uint16_t>(const uint16_t *zq, i
 // out warp by warp, so that every warp has one before any has two; kNT of them are in flight per warp.
 template <typename T>
 __device__ __forceinline__ bool row_tile_stats(const T *zq, const Shape &s, int t0, int t1, float *tile_s, float *tile_m) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wid = warp_index(), nwarps = blockDim.x >> 5;
     bool bad = false;
     constexpr int kNT = 4;
     static_assert(kTile == 256, "a lane takes 8 entries of a tile");
@@ -264,8 +264,8 @@ __device__ __forceinline__ int warp_draw(W weight, int ntiles, int first_tile, i
 #pragma unroll 4
     for (int t = t0; t < t1; ++t) local += weight(t);
     double incl = warp_scan(local, lane);
-    unsigned hit = __ballot_sync(kAll, local > 0.0 && incl > target);
-    unsigned any = __ballot_sync(kAll, local > 0.0);
+    unsigned hit = uniform(__ballot_sync(kAll, local > 0.0 && incl > target));
+    unsigned any = uniform(__ballot_sync(kAll, local > 0.0));
     if (any == 0u) return -1;
     int owner = hit ? __ffs(hit) - 1 : 31 - __clz(any);
     double base = __shfl_sync(kAll, incl - local, owner);
@@ -274,8 +274,8 @@ __device__ __forceinline__ int warp_draw(W weight, int ntiles, int first_tile, i
     for (int c0 = r0; c0 < r1 && tile < 0; c0 += 32) {
         const double v = c0 + lane < r1 ? weight(c0 + lane) : 0.0;
         incl = warp_scan(v, lane);
-        hit = __ballot_sync(kAll, v > 0.0 && base + incl > target);
-        any = __ballot_sync(kAll, v > 0.0);
+        hit = uniform(__ballot_sync(kAll, v > 0.0 && base + incl > target));
+        any = uniform(__ballot_sync(kAll, v > 0.0));
         if (any) last = c0 + 31 - __clz(any);
         owner = hit ? __ffs(hit) - 1 : 31;
         if (hit) tile = c0 + owner;
@@ -303,7 +303,7 @@ __device__ __forceinline__ int warp_draw(W weight, int ntiles, int first_tile, i
             if (first < 0 && crossed && cum > target) first = x0 + e;
         }
     }
-    hit = __ballot_sync(kAll, first >= 0);
+    hit = uniform(__ballot_sync(kAll, first >= 0));
     if (hit) return __shfl_sync(kAll, first, __ffs(hit) - 1);
     any = __ballot_sync(kAll, last >= 0);
     return any ? __shfl_sync(kAll, last, 31 - __clz(any)) : -1;
@@ -332,7 +332,7 @@ struct Drawn {
 template <typename T>
 __device__ __forceinline__ Drawn draw_row(const T *zq, const Shape &s, double us, int rank, int C, float *tile_s, float *tile_m,
                                           DrawScratch *sc) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = warp_index();
     const int per = (s.ntiles + C - 1) / C, t0 = min(s.ntiles, rank * per), t1 = min(s.ntiles, t0 + per);
     const bool mybad = row_tile_stats<T>(zq, s, t0, t1, tile_s, tile_m);
     const bool anybad = __syncthreads_or(mybad);
@@ -380,11 +380,14 @@ __device__ __forceinline__ Drawn draw_row(const T *zq, const Shape &s, double us
             run += v;
         }
         o.bad = bad || !(o.m > -INFINITY);
+        owner = uniform(owner);
+        last = uniform(last);
+        o.bad = uniform((int)o.bad) != 0;
         if (o.bad || rank != (owner < 0 ? last : owner)) return o;
         if (owner < 0) before = -INFINITY;  // no share crosses: its last entry with positive weight
     } else {
         o.total = S;
-        o.bad = bad || !(o.m > -INFINITY);
+        o.bad = uniform((int)(bad || !(o.m > -INFINITY))) != 0;
         if (o.bad) return o;
     }
     auto weight = [&](int t) { return tile_m[t] > -INFINITY ? (double)tile_s[t] * (double)expo(tile_m[t], m, s.scale) : 0.0; };
@@ -402,7 +405,7 @@ __device__ __forceinline__ Drawn draw_row(const T *zq, const Shape &s, double us
 template <typename T>
 __device__ int draw_from_row(const T *zq, const Shape &s, double us, float *tile_s, float *tile_m, SampleScratch *sc,
                              bool &bad_out, float *row_max_out = nullptr) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int nthreads = blockDim.x, nwarps = nthreads / 32;
     bool bad = false;
     float m = -INFINITY;

@@ -374,11 +374,10 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
     int32_t *tok_s = reinterpret_cast<int32_t *>(pass_s + K);
     float *u_s = reinterpret_cast<float *>(tok_s + KG);
     unsigned char *lcp_s = reinterpret_cast<unsigned char *>(u_s + KG + 1);
-    __shared__ unsigned sh_or[2];
     __shared__ int sh_i[2];
     __shared__ int sh_flags;
 
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const size_t NR = (size_t)s.B * KG;
     const int32_t *tok = tok_all + (size_t)b * KG;
     for (int n = tid; n <= KG; n += kThreads) u_s[n] = u_all[(size_t)b * (KG + 1) + n];
@@ -406,7 +405,7 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
     }
     if (myflags) atomicOr(&sh_flags, myflags);
     __syncthreads();
-    const int status_in = sh_flags & (SGBV_STATUS_TOKEN_RANGE | SGBV_STATUS_NONFINITE_LOGIT);
+    const int status_in = uniform(sh_flags) & (SGBV_STATUS_TOKEN_RANGE | SGBV_STATUS_NONFINITE_LOGIT);
     const bool invalid = status_in != 0;
     auto prefix = [&](const double *row, int len) {
         double acc = 0.0;
@@ -423,13 +422,13 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
         if (out_resmass) out_resmass[(size_t)b * KG + n] = invalid ? NAN : exp_short(la) * Rr;
         if (i >= 1) {
             const double hv = weight_sub(la, lb, Rr, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, ri.c < 1.0f, true);
-            if ((double)u_s[k * g + i - 1] < hv) atomicOr(&pass_s[k], 1ull << (i - 1));
+            if ((double)u_s[k * g + i - 1] < hv) set_bit(&pass_s[k], i - 1);
             if (out_h) out_h[(size_t)b * KG + k * g + i - 1] = invalid ? NAN : hv;
         }
     }
     for (int k = tid; k < K; k += kThreads) {
         const double hv = weight_full(prefix(la_s + k * (g + 1), g), prefix(lb_s + k * (g + 1), g), K);
-        if ((double)u_s[k * g + g - 1] < hv) atomicOr(&pass_s[k], 1ull << (g - 1));
+        if ((double)u_s[k * g + g - 1] < hv) set_bit(&pass_s[k], g - 1);
         if (out_h) out_h[(size_t)b * KG + k * g + g - 1] = invalid ? NAN : hv;
     }
     for (int n = tid; n < K * K; n += kThreads) {
@@ -441,7 +440,7 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
     __syncthreads();
     if (wid == 0 && !invalid) {
         int tau, f;
-        scan_block(pass_s, lcp_s, K, g, sh_or, tau, f);
+        scan_block(pass_s, lcp_s, K, g, tau, f);
         if (lane == 0) {
             sh_i[0] = tau;
             sh_i[1] = f;
@@ -530,11 +529,11 @@ shard_draw_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Sh
     __shared__ SampleScratch sc;
     const int b = blockIdx.x;
     const Plan pl = plan[b];
-    if (pl.owner != rank) return;
+    if (uniform(pl.owner) != rank) return;
     const int K = s.K, g = s.gamma;
     const T *zq = zq_all + (((size_t)b * K + pl.k) * (g + 1) + pl.i) * s.V;
     int y = -1;
-    if (pl.mode == 0) {
+    if (uniform(pl.mode) == 0) {
         const size_t r = ((size_t)b * K + pl.k) * g + pl.i;
         const RowInfo ri = rows[r];
         const T *zp = zp_all + r * s.V;
