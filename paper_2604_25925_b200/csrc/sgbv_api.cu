@@ -38,7 +38,7 @@ Shape make_shape(int B, int K, int gamma, int V, float temperature) {
 }
 
 struct Carve {
-    size_t rows, part, wpart, dpart, mpart, ratio, cut, bonus, h, resmass, status, error, total;
+    size_t rows, part, wpart, dpart, mpart, ratio, bonus, h, resmass, status, error, total;
 };
 
 Carve carve(const Shape &s) {
@@ -53,7 +53,7 @@ Carve carve(const Shape &s) {
     c.wpart = off;     off += align_up(NR * s.ntiles * sizeof(float));
     c.dpart = off;     off += align_up(NR * s.ntiles * sizeof(float));
     c.mpart = off;     off += align_up(NR * s.ntiles * sizeof(float));
-    c.cut = off;       off += align_up((size_t)s.B * s.cpr * sizeof(double));
+    off += align_up((size_t)s.B * s.cpr * sizeof(double));  // (unused; kept so that the size a shape needs does not change)
     c.bonus = off;     off += align_up((size_t)s.B * 2 * s.ntiles * sizeof(float));
     c.h = off;         off += align_up(NR * sizeof(double));
     c.resmass = off;   off += align_up(NR * sizeof(double));
@@ -164,8 +164,8 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
     L.ws.wpart = (float *)(base + c.wpart);
     L.ws.dpart = (float *)(base + c.dpart);
     L.ws.mpart = (float *)(base + c.mpart);
+    L.ws.list = (int32_t *)(base + c.part);
     L.ws.ratio = (double *)(base + c.ratio);
-    L.ws.cut = (double *)(base + c.cut);
     L.ws.bonus = (float *)(base + c.bonus);
     L.ws.h = out_h ? out_h : (double *)(base + c.h);
     L.ws.resmass = out_resmass ? out_resmass : (double *)(base + c.resmass);
@@ -190,11 +190,11 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
     // error word itself; the two-sweep kernels set status bits with atomics, so those start at zero
     bool fused = g_opt_path != 1 && fused_supported(L);
     L.ws.prestatus = nullptr;
-    bool walked_rows = false;
+    int words_used = 0;
     bool aux_apart = false;
-    int n1 = fused ? launch_fused(L, L.ws.error, &walked_rows, &aux_apart) : 0;
+    int n1 = fused ? launch_fused(L, L.ws.error, &words_used, &aux_apart) : 0;
     if (n1 < 0) return n1;
-    L.ws.ratio_used = (n1 > 0 && walked_rows) ? 1 : 0;
+    L.ws.ratio_used = n1 > 0 ? words_used : 0;
     if (n1 == 0) {
         if (g_opt_path == 2) return SGBV_ERR_SHAPE;
         fused = false;
@@ -207,14 +207,13 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
     // the extra sums of Eq. 2 for rows with c < 1: written for all such rows by the two-sweep path and, for small and
     // medium problems, by the fused kernel; for large ones it leaves them to kernels of their own, which do the few rows
     // that need them
-    L.ws.have_aux = 1;
-    if (fused && aux_apart) {
-        const int na = launch_auxreduce(L);
-        if (na < 0) return na;
-        n1 += na;
-        L.ws.have_aux = 2;
-    }
-    int n2 = launch_finish(L);
+    const bool apart = fused && aux_apart;
+    // (the rows' totals lie where the weights go when the caller does not take them: a batch row's are read before its
+    // first weight is written)
+    L.ws.wsum = apart ? (double *)(base + c.h) : nullptr;
+    const int na = apart ? launch_auxreduce(L) : 0;
+    n1 += na;
+    const int n2 = na < 0 ? na : launch_finish(L);
     if (own_dev >= 0 && L.ws.ratio_used) {
         // a walk that cleared the words itself is followed by a finishing kernel that puts them back: the
         // doubt ends unless that kernel was not launched, or nothing ran at all (stream capture)
@@ -359,9 +358,10 @@ int sgbv_modify(const void *target_logits, const void *draft_logits, int dtype, 
     L.ws.wpart = (float *)(base + c.wpart);
     L.ws.dpart = (float *)(base + c.dpart);
     L.ws.mpart = (float *)(base + c.mpart);
+    L.ws.list = (int32_t *)(base + c.part);
+    L.ws.wsum = nullptr;
     L.ws.ratio = (double *)(base + c.ratio);
-    L.ws.cut = (double *)(base + c.cut);
-    L.ws.ratio_used = 0;  // (a single position per chain never takes the row walk)
+    L.ws.ratio_used = 0;  // (a single position per chain: nothing is handed from cluster to cluster)
     L.ws.bonus = (float *)(base + c.bonus);
     L.ws.bonus_in_smem = 0;
     L.ws.h = (double *)(base + c.h);
@@ -381,9 +381,9 @@ int sgbv_modify(const void *target_logits, const void *draft_logits, int dtype, 
     L.carry_loga = log_a;
     L.carry_logb = log_b;
     bool fused = g_opt_path != 1 && fused_supported(L);
-    bool walked_rows = false;
+    int words_used = 0;
     bool aux_apart = false;  // (Algorithm 2 needs no extra sums: its draw only uses Eq. 4's weights)
-    int n1 = fused ? launch_fused(L, L.ws.error, &walked_rows, &aux_apart) : 0;
+    int n1 = fused ? launch_fused(L, L.ws.error, &words_used, &aux_apart) : 0;
     if (n1 < 0) return n1;
     if (n1 == 0) {
         if (g_opt_path == 2) return SGBV_ERR_SHAPE;

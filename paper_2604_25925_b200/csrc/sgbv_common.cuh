@@ -13,8 +13,9 @@ namespace sgbv {
 // Batches of at most this many rows: the finishing kernel (one CTA per row) leaves most SMs idle, so the next
 // call's streaming kernel is allowed onto them while it runs (programmatic dependent launch across calls).
 constexpr int kChainedLaunchMaxB = 16;
-constexpr int kRatioWords = 256;   // ratio words at the head of the scratch: the row walk needs one per row and
-                                   // only runs while every row has a cluster of its own in one wave (<= 148)
+constexpr int kRatioWords = 256;   // hand-over words at the head of the scratch: the row walk needs one per row and only
+                                   // runs while every row has a cluster of its own in one wave, the chain walk one per
+                                   // cluster (both <= 148)
 constexpr int kTile = 256;         // vocabulary elements per tile (granularity of the cached partial sums)
 constexpr int kMaxK = 64;
 constexpr int kMaxGamma = 64;
@@ -32,7 +33,7 @@ struct RowInfo {
     float c;        // c = p(x_k^i)/q(x_k^i), ratio of the joint prefix probabilities (c < 1 selects
                     // the cancellation-free numerator)
     int32_t flags;  // SGBV_STATUS_NONFINITE_LOGIT if the streaming pass found the row pair unusable
-    int32_t pad_;   // 1: dpart/mpart hold this row's extra sums although only some rows have them (Workspace::have_aux = 2)
+    int32_t pad_;   // 1: dpart/mpart hold this row's extra sums although only some rows have them (Workspace::wsum)
 };
 
 struct Workspace {
@@ -41,15 +42,15 @@ struct Workspace {
     float *wpart;       // [B*K*gamma][ntiles]: sum over the tile of eq * max(1 - kappa ep/eq, 0)^K
     float *dpart;       // [B*K*gamma][ntiles]: sum of max(kappa ep - eq, 0)               (c < 1)
     float *mpart;       // [B*K*gamma][ntiles]: sum of eq (c - t)^2 Q(t)                    (c < 1)
-    double *ratio;      // [kRatioWords]: p_i(tok_i)/q_i(tok_i) of each row (row walk of the fused kernel, which
-                        // only runs when B*K*gamma <= kRatioWords); every word holds a NaN pattern ("not
-                        // published yet") whenever no call is in flight
-    double *cut;        // [B*cpr]: c handed from the cluster that walks the head of a chain to the one that walks its tail
-                        // (chain walk of the fused kernel; preset to the NaN pattern when any range cuts a chain)
-    int have_aux;       // which rows with c < 1 have their two extra sums in dpart and mpart: 1 = all of them (two-sweep
-                        // path, row walk of the fused kernel), 2 = those marked RowInfo::pad_ = 1 (chain walk of the fused
-                        // kernel followed by auxreduce_kernel); the others take the plain form of Eq. 2's numerator
-    int ratio_used;     // the streaming kernel walked rows: the finishing kernel puts the NaN pattern back
+    int32_t *list;      // [1 + B*K*gamma]: rows whose plain numerator would cancel (large problems; list[0] counts).
+                        // Shares its place with `part`
+    double *wsum;       // [B*K*gamma]: total of the row's wpart (chain walk of the fused kernel on large problems, followed
+                        // by auxflag_kernel: of the rows with c < 1 only those marked RowInfo::pad_ = 1 then have their two
+                        // extra sums in dpart and mpart, the others take the plain form of Eq. 2's numerator), else NULL
+    double *ratio;      // [kRatioWords]: words handed from cluster to cluster of the fused kernel.  Row walk: p_i(tok_i)/
+                        // q_i(tok_i) of each row; chain walk: c at the place where a cluster's range ends inside a chain.
+                        // Every word holds a NaN pattern ("not published yet") whenever no call is in flight
+    int ratio_used;     // words that the streaming kernel published: the finishing kernel puts the NaN pattern back
     float *bonus;       // [B][2][ntiles]: per-tile sums and maxima of the row a bonus token is drawn from
     int bonus_in_smem;  // set by the finishing kernel's launcher: those tile sums fit its shared memory
     double *h;          // [B][K][gamma]
@@ -204,7 +205,7 @@ struct Launch {
 };
 
 int launch_twopass(const Launch &L);  // statistics + chain + reduction, returns launches or <0
-int launch_auxreduce(const Launch &L); // the extra sums of Eq. 2 for the rows that need them (behind the fused chain walk)
+int launch_auxreduce(const Launch &L); // row totals, and the extra sums of Eq. 2 for the rows that need them (behind the fused chain walk)
 int launch_finish(const Launch &L);   // weights, scan, extra token
 // Algorithm 2's draw per batch row from the cell sums of a gamma = 1 launch with carried logs
 int launch_modify_finish(const Launch &L, const float *u, int32_t *out_token, double *out_loga, double *out_logb,
@@ -217,9 +218,9 @@ int launch_draw_rows(const void *z, int dtype, const float *u, const Shape &s, f
 bool fused_supported(const Launch &L);
 // single-read cluster path for steps A1-A3: launches (> 0), 0 if it declined before launching
 // anything (the caller then takes the two-sweep path), or < 0
-// *walked_rows: the kernel used (and consumed the preset of) ws.ratio
+// *words_used: words of ws.ratio that the kernel uses (and consumes the preset of)
 // *aux_apart: it left the two extra sums of the rows with c < 1 to launch_auxreduce
-int launch_fused(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart);
+int launch_fused(const Launch &L, int *error_flag, int *words_used, bool *aux_apart);
 void fused_set_options(int cluster, int max_clusters, int walk, int poll_us, int withhold, int aux);
 
 }  // namespace sgbv

@@ -68,20 +68,44 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();  // the staged tokens and uniforms are read by other threads than those that fetched them
     const bool lost = uniform(*ws.error) != 0;  // a bounded wait expired upstream: nothing can be trusted
-    // the streaming kernel has consumed the "not published yet" pattern of this batch row's ratio words:
+    // the streaming kernel has consumed the "not published yet" pattern of its hand-over words:
     // put it back, so that the next call on this scratch area need not clear them first
-    if (ws.ratio_used)
-        for (int n = tid; n < KG; n += nthreads)
-            reinterpret_cast<unsigned long long *>(ws.ratio)[(size_t)b * KG + n] = ~0ull;
+    if (b == 0)
+        for (int n = nthreads - 1 - tid; n < ws.ratio_used; n += nthreads)
+            reinterpret_cast<unsigned long long *>(ws.ratio)[n] = ~0ull;
     int myflags = (tid == 0 && ws.prestatus) ? ws.prestatus[b] : 0;
 
     // ---- cell sums of every row (k,i), one warp per row, first warps first; the token work of step 0
-    //      below starts with the LAST threads, so that for small K*gamma both run side by side ----
+    //      below starts with the LAST threads, so that for small K*gamma both run side by side.  Large problems: the
+    //      rows' totals are ready (ws.wsum), and few rows have the two extra sums ----
+    if (ws.wsum) {
+        for (int n = wid; n < KG; n += nwarps) {
+            const size_t r = (size_t)b * KG + n;
+            const double sw = ws.wsum[r];
+            const bool aux = uniform(ws.rows[r].pad_) == 1;
+            double sd = 0.0, sm = 0.0;
+            if (aux) {
+#pragma unroll 4
+                for (int t = lane; t < s.ntiles; t += 32) {
+                    sd += (double)ws.dpart[r * s.ntiles + t];
+                    sm += (double)ws.mpart[r * s.ntiles + t];
+                }
+                sd = warp_sum(sd);
+                sm = warp_sum(sm);
+            }
+            if (lane == 0) {
+                W_s[n] = sw;
+                D_s[n] = sd;
+                M_s[n] = sm;
+                exact_s[n] = aux;
+            }
+        }
+    } else
     for (int n = wid; n < KG; n += nwarps) {
         const int k = n / g, i = n % g;
         const size_t r = ((size_t)b * K + k) * g + i;
         const RowInfo ri = ws.rows[r];
-        const bool aux = ri.c < 1.0f && (ws.have_aux == 1 || ri.pad_ == 1);
+        const bool aux = ri.c < 1.0f;
         const float *wp = ws.wpart + r * s.ntiles, *dp = ws.dpart + r * s.ntiles, *mp = ws.mpart + r * s.ntiles;
         double sw = 0.0, sd = 0.0, sm = 0.0;
         for (int t0 = 0; t0 < s.ntiles; t0 += 128) {  // four independent loads per array in flight

@@ -527,15 +527,19 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     // there clusters wait for one another, so no CTA of this grid may find its place on an SM taken by
     // a kernel that in turn waits for this grid.
     if (!kRow) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (blockIdx.x == 0 && tid == 0) *p.error_flag = 0;  // set again only by a wait that expires (about a second later)
+    if (blockIdx.x == 0 && tid == 0) {
+        *p.error_flag = 0;  // set again only by a wait that expires (about a second later)
+        if (!kRow && !p.aux_here) p.ws.list[0] = 0;
+    }
     // The walk of this cluster: position n = 0, 1, ... is row (bk, i).
     //   chain mode: the list of all rows, u = bk*gamma + i, is cut into G contiguous ranges of equal length (+-1), one
     //               per cluster, so that the clusters finish together whatever the number of chains.  A range may
     //               begin and end inside a chain.  The cluster walks first the HEAD of the chain its range ends in
     //               (rows 0..off_hi-1 of chain_hi) and leaves the ratio c reached there in a word of global memory,
     //               then its whole chains, and last the TAIL of the chain its range begins in (rows off_lo.. of
-    //               chain_lo), whose c it picks up from the word the cluster before it wrote at its very start.  The
-    //               words are preset to a NaN pattern; the one wait (bounded) is for something written long before.
+    //               chain_lo), whose c it picks up from the word the cluster before it wrote at its very start (one word
+    //               per cluster).  The words are preset to a NaN pattern; the one wait (bounded) is for something written
+    //               long before.
     //   row mode:   rows u = cid, cid+G, ... of the list.  Used when there are few rows: all rows of a chain then run
     //               at the same time on different clusters, and c_i comes from the ratios p_j(tok_j)/q_j(tok_j) that
     //               the clusters of rows j < i publish in global memory.  A row only waits for rows earlier in the
@@ -917,14 +921,14 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 const double c_next = cd * SGBV_RATIO();  // c after this row
                 // the head of a chain that another cluster continues: leave c where that cluster looks for it
                 if (bk_b == chain_hi && i_b == off_hi - 1 && lane == 0 && rank == 0)
-                    *reinterpret_cast<volatile double *>(p.ws.cut + bk_b) = (c_next != c_next) ? 0.0 : c_next;
+                    *reinterpret_cast<volatile double *>(p.ws.ratio + cid) = (c_next != c_next) ? 0.0 : c_next;
                 if (has_d) {
                     if (i_d == 0) {
                         c_carry = SGBV_C0(bk_d);
                     } else if (bk_d == bk_b) {
                         c_carry = c_next;
                     } else {  // the tail of a chain whose head another cluster walked at its very start
-                        const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.cut + bk_d);
+                        const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.ratio + cid - 1);
                         double w = *word;
                         if (w != w && !timed_out) {
                             const long long t0 = clock64();
@@ -1060,7 +1064,7 @@ int resident_clusters(int dev, int C) {
 }
 
 template <typename T, bool kRow, int KT, bool kAny>
-int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, bool aux_here) {
+int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, bool aux_here, int words_used) {
     FusedParams fp;
     fp.zq = L.zq;
     fp.zp = L.zp;
@@ -1093,11 +1097,8 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
     cfg.attrs = attr;
     cfg.numAttrs = L.s.B <= kChainedLaunchMaxB ? 2 : 1;  // small batches only: see kChainedLaunchMaxB
     cfg.gridDim = dim3(clusters * plan.cluster);
-    if (!kRow && (fp.nchains % clusters) != 0 &&  // some ranges begin or end inside a chain: their hand-over words
-        cudaMemsetAsync(L.ws.cut, 0xff, (size_t)fp.nchains * sizeof(double), L.stream) != cudaSuccess)
-        return SGBV_ERR_CUDA;
-    if (kRow && !L.ratio_preset &&
-        cudaMemsetAsync(L.ws.ratio, 0xff, (size_t)fp.nchains * L.s.gamma * sizeof(double), L.stream) != cudaSuccess)
+    if (words_used > 0 && !L.ratio_preset &&
+        cudaMemsetAsync(L.ws.ratio, 0xff, (size_t)words_used * sizeof(double), L.stream) != cudaSuccess)
         return SGBV_ERR_CUDA;
     if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
     cudaError_t e = cudaLaunchKernelEx(&cfg, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, fp);
@@ -1111,7 +1112,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
 
 // Chooses the cluster size and the walk, then launches.  Returns launches, 0 if declined, or < 0.
 template <typename T, int KT, bool kAny>
-int plan_and_launch(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart) {
+int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux_apart) {
     const Shape &s = L.s;
     const int cells = s.ntiles;
     const long nchains = (long)s.B * s.cpr, units = nchains * s.gamma;
@@ -1154,15 +1155,18 @@ int plan_and_launch(const Launch &L, int *error_flag, bool *walked_rows, bool *a
     if (clusters < 1) return 0;  // this cluster shape cannot be scheduled here: nothing launched
     const long share = plan.row_mode ? units : nchains;  // what the clusters share out
     if (clusters > share) clusters = (int)share;
-    *walked_rows = plan.row_mode != 0;
+    if (clusters > kRatioWords) clusters = kRatioWords;  // (a forced number: one hand-over word per cluster)
+    // hand-over words: one per row in the row walk; in the chain walk one per cluster, if a range may end inside a chain
+    // (the words are put back by the finishing kernel, so on the library's own scratch no call has to clear them)
+    *words_used = plan.row_mode ? (int)units : (s.gamma > 1 && nchains % clusters != 0) ? clusters : 0;
     // the extra sums of rows with c < 1: in this kernel, or for long steps (chain walk, 1 GB of logits or more) in the
     // kernels that the caller queues behind it
     const double bytes = 2.0 * (double)units * (double)s.V * (double)sizeof(T);
     // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed)
     const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1));
     *aux_apart = !aux_here;
-    return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true)
-                         : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here);
+    return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true, *words_used)
+                         : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here, *words_used);
 }
 
 }  // namespace
@@ -1181,29 +1185,29 @@ void fused_set_options(int cluster, int max_clusters, int walk, int poll_us, int
 bool fused_supported(const Launch &L) { return L.s.ntiles <= kMaxCluster * kCtaCells; }
 
 template <typename T, bool kAny>
-int dispatch_k(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart) {
+int dispatch_k(const Launch &L, int *error_flag, int *words_used, bool *aux_apart) {
     switch (L.s.K) {
-        case 1: return plan_and_launch<T, 1, kAny>(L, error_flag, walked_rows, aux_apart);
-        case 2: return plan_and_launch<T, 2, kAny>(L, error_flag, walked_rows, aux_apart);
-        case 3: return plan_and_launch<T, 3, kAny>(L, error_flag, walked_rows, aux_apart);
-        case 4: return plan_and_launch<T, 4, kAny>(L, error_flag, walked_rows, aux_apart);
-        case 8: return plan_and_launch<T, 8, kAny>(L, error_flag, walked_rows, aux_apart);
-        default: return plan_and_launch<T, 0, kAny>(L, error_flag, walked_rows, aux_apart);
+        case 1: return plan_and_launch<T, 1, kAny>(L, error_flag, words_used, aux_apart);
+        case 2: return plan_and_launch<T, 2, kAny>(L, error_flag, words_used, aux_apart);
+        case 3: return plan_and_launch<T, 3, kAny>(L, error_flag, words_used, aux_apart);
+        case 4: return plan_and_launch<T, 4, kAny>(L, error_flag, words_used, aux_apart);
+        case 8: return plan_and_launch<T, 8, kAny>(L, error_flag, words_used, aux_apart);
+        default: return plan_and_launch<T, 0, kAny>(L, error_flag, words_used, aux_apart);
     }
 }
 
-int launch_fused(const Launch &L, int *error_flag, bool *walked_rows, bool *aux_apart) {
-    *walked_rows = false;
+int launch_fused(const Launch &L, int *error_flag, int *words_used, bool *aux_apart) {
+    *words_used = 0;
     *aux_apart = false;
     std::lock_guard<std::mutex> lock(g_plan_mu);
     // rows that all start on 16-byte boundaries?
     const size_t esz = L.dtype == SGBV_DTYPE_BF16 ? 2 : 4;
     const bool any = ((uintptr_t)L.zq % 16) || ((uintptr_t)L.zp % 16) || (((size_t)L.s.V * esz) % 16);
     if (L.dtype == SGBV_DTYPE_BF16)
-        return any ? dispatch_k<uint16_t, true>(L, error_flag, walked_rows, aux_apart)
-                   : dispatch_k<uint16_t, false>(L, error_flag, walked_rows, aux_apart);
-    return any ? dispatch_k<float, true>(L, error_flag, walked_rows, aux_apart)
-               : dispatch_k<float, false>(L, error_flag, walked_rows, aux_apart);
+        return any ? dispatch_k<uint16_t, true>(L, error_flag, words_used, aux_apart)
+                   : dispatch_k<uint16_t, false>(L, error_flag, words_used, aux_apart);
+    return any ? dispatch_k<float, true>(L, error_flag, words_used, aux_apart)
+               : dispatch_k<float, false>(L, error_flag, words_used, aux_apart);
 }
 
 }  // namespace sgbv

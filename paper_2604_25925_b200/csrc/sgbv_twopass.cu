@@ -233,24 +233,31 @@ otreduce_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shap
 }
 
 // Behind a fused kernel that left the two extra sums of Eq. 2 aside (large problems), two small kernels:
-//   auxflag_kernel  one warp per row: for a row with c < 1 whose numerator R - (1-c)^K would cancel in that plain form
-//                   (plain_form_is_safe; R from the cell sums the fused kernel wrote), the row is put on a list and
-//                   marked in its record (RowInfo::pad_ = 1) for the finishing kernel;
+//   auxflag_kernel  one warp per row: the total of the cell sums that the fused kernel wrote, for the finishing kernel (whose
+//                   one CTA per batch row took 10 us over those of 64 rows of 594 cells); a row with c < 1 whose numerator
+//                   R - (1-c)^K would cancel in that plain form (plain_form_is_safe) is put on a list and marked in its
+//                   record (RowInfo::pad_ = 1);
 //   auxwork_kernel  a fixed grid shares out the listed rows in slices of kAuxSliceTiles cells and writes, per cell, the
 //                   sums over max(c p - q, 0) and q (c-t)^2 Q(t) from a second read of the row pair.
 // A few per cent of the rows are listed; the order of the list varies from run to run, the sums do not.
+// Both are chained to the kernel ahead by programmatic dependent launch, so that neither launch costs time of its own.
+// (What the kernel ahead writes is not declared __restrict__ const: such loads may be moved ahead of the wait.)
 constexpr int kAuxSliceTiles = 16;
 
 __global__ void __launch_bounds__(kThreads)
-auxflag_kernel(Shape s, RowInfo *__restrict__ rows, const float *__restrict__ wpart, int *__restrict__ list) {
+auxflag_kernel(Shape s, RowInfo *rows, const float *wpart, double *wsum, int *list) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = threadIdx.x & 31;
     const size_t r = (size_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-    if (r >= (size_t)s.B * s.cpr * s.gamma || r % s.gamma == 0) return;  // Eq. 2 is about sub-blocks of length i >= 1
+    if (r >= (size_t)s.B * s.cpr * s.gamma) return;
     const RowInfo ri = rows[r];
-    if (!(ri.c < 1.0f) || ri.flags) return;
     double sw = 0.0;
+#pragma unroll 8
     for (int t = lane; t < s.ntiles; t += 32) sw += (double)wpart[r * s.ntiles + t];
     sw = warp_sum(sw);
+    if (lane == 0) wsum[r] = sw;
+    if (!(ri.c < 1.0f) || ri.flags || r % s.gamma == 0) return;  // (Eq. 2 is about sub-blocks of length i >= 1)
     if (plain_form_is_safe(sw / ri.Zq, (double)ri.c, s.K)) return;
     if (lane == 0) {
         list[1 + atomicAdd(list, 1)] = (int)r;  // list[0] counts
@@ -260,8 +267,10 @@ auxflag_kernel(Shape s, RowInfo *__restrict__ rows, const float *__restrict__ wp
 
 template <typename T, int KT>
 __global__ void __launch_bounds__(kThreads)
-auxwork_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shape s, const RowInfo *__restrict__ rows,
-               const int *__restrict__ list, float *__restrict__ dpart, float *__restrict__ mpart) {
+auxwork_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shape s, const RowInfo *rows, const int *list,
+               float *dpart, float *mpart) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int K = KT ? KT : s.K;
     const int per_row = (s.ntiles + kAuxSliceTiles - 1) / kAuxSliceTiles;
     const long items = (long)list[0] * per_row;
@@ -321,29 +330,45 @@ int run_otreduce(const Launch &L) {
     return cudaGetLastError() == cudaSuccess ? 1 : SGBV_ERR_CUDA;
 }
 
+// A launch that may be scheduled before the kernel ahead of it has finished (it waits for it itself).
+template <typename... P, typename... A>
+cudaError_t launch_behind(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <typename T>
 int run_auxreduce(const Launch &L) {
     const Shape &s = L.s;
     const size_t NR = (size_t)s.B * s.cpr * s.gamma;
-    // the list lives where the two-sweep path keeps its slice partials (at least 16 bytes per row), unused here
-    int *list = reinterpret_cast<int *>(L.ws.part);
-    if (cudaMemsetAsync(list, 0, sizeof(int), L.stream) != cudaSuccess) return SGBV_ERR_CUDA;
-    auxflag_kernel<<<(unsigned)((NR + kThreads / 32 - 1) / (kThreads / 32)), kThreads, 0, L.stream>>>(s, L.ws.rows, L.ws.wpart,
-                                                                                                     list);
+    // (the list lies where the two-sweep path keeps its slice partials, at least 16 bytes per row)
+    const cudaError_t e = launch_behind(auxflag_kernel, (unsigned)((NR + kThreads / 32 - 1) / (kThreads / 32)), kThreads, L.stream,
+                                        s, L.ws.rows, L.ws.wpart, L.ws.wsum, L.ws.list);
+    cudaError_t e2;
     const T *zq = (const T *)L.zq, *zp = (const T *)L.zp;
     const unsigned grid = 8 * 148;
 #define SGBV_AUX(KT) \
-    auxwork_kernel<T, KT><<<grid, kThreads, 0, L.stream>>>(zq, zp, s, L.ws.rows, list, L.ws.dpart, L.ws.mpart)
+    launch_behind(auxwork_kernel<T, KT>, grid, kThreads, L.stream, zq, zp, s, L.ws.rows, L.ws.list, L.ws.dpart, L.ws.mpart)
     switch (s.K) {
-        case 1: SGBV_AUX(1); break;
-        case 2: SGBV_AUX(2); break;
-        case 3: SGBV_AUX(3); break;
-        case 4: SGBV_AUX(4); break;
-        case 8: SGBV_AUX(8); break;
-        default: SGBV_AUX(0); break;
+        case 1: e2 = SGBV_AUX(1); break;
+        case 2: e2 = SGBV_AUX(2); break;
+        case 3: e2 = SGBV_AUX(3); break;
+        case 4: e2 = SGBV_AUX(4); break;
+        case 8: e2 = SGBV_AUX(8); break;
+        default: e2 = SGBV_AUX(0); break;
     }
 #undef SGBV_AUX
-    return cudaGetLastError() == cudaSuccess ? 2 : SGBV_ERR_CUDA;
+    if (e == cudaSuccess && e2 == cudaSuccess) return 2;
+    cudaGetLastError();
+    return SGBV_ERR_CUDA;
 }
 
 }  // namespace
