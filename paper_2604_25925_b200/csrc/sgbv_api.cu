@@ -79,11 +79,23 @@ struct DeviceBuffers {
     void *idx = nullptr;        // accepted-draft indices that sgbv_verify_gbv has no output for
     size_t idx_bytes = 0;
     // the ratio words at the head of the scratch may not hold the "not published yet" pattern (a call
-    // failed between the kernel that consumes them and the one that puts them back)
+    // failed between the kernel that publishes them and the one that puts them back)
     bool ratio_dirty = false;
 };
 DeviceBuffers g_buf[kMaxDevices];
 std::mutex g_mu;
+
+// Puts the pattern back into all hand-over words, in stream order.  *dirty ends with it, unless the stream is only being
+// captured (nothing has run then).
+int clear_words(double *words, cudaStream_t stream, bool *dirty) {
+    if (cudaMemsetAsync(words, 0xff, kRatioWords * sizeof(double), stream) != cudaSuccess) {
+        cudaGetLastError();
+        return SGBV_ERR_CUDA;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) *dirty = false;
+    return SGBV_OK;
+}
 
 // Grows a per-device buffer.  preset_head: the first bytes of a new buffer get the 0xff pattern of unpublished
 // ratio words before anyone uses it (the device is idle then).
@@ -153,11 +165,14 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
         if (rc != SGBV_OK) return rc;
         base = (unsigned char *)g_buf[dev].scratch;
         own_dev = dev;
-        // The row walk of the fused kernel needs its ratio words preset.  They sit at a fixed place, are preset
-        // when the buffer is allocated, and every finishing kernel puts the pattern back after use: whatever the
-        // order of eager calls and graph replays, a call finds them ready.  Only a call that failed half-way
-        // leaves them in doubt; the next row walk then clears them itself.
-        L.ratio_preset = !g_buf[dev].ratio_dirty;
+        // The fused kernel needs its hand-over words preset.  They sit at a fixed place, are preset when the buffer is
+        // allocated, and every finishing kernel puts the pattern back after use: whatever the order of eager calls and
+        // graph replays, a call finds them ready.  Only a call that failed half-way leaves them in doubt, all of them and
+        // not just as many as the next call uses: they are cleared before anything reads them again.
+        if (g_buf[dev].ratio_dirty) {
+            if (clear_words((double *)(base + c.ratio), stream, &g_buf[dev].ratio_dirty) != SGBV_OK) return SGBV_ERR_CUDA;
+        }
+        L.ratio_preset = true;
     }
     L.ws.rows = (RowInfo *)(base + c.rows);
     L.ws.part = (float *)(base + c.part);
@@ -214,14 +229,11 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
     const int na = apart ? launch_auxreduce(L) : 0;
     n1 += na;
     const int n2 = na < 0 ? na : launch_finish(L);
-    if (own_dev >= 0 && L.ws.ratio_used) {
-        // a walk that cleared the words itself is followed by a finishing kernel that puts them back: the
-        // doubt ends unless that kernel was not launched, or nothing ran at all (stream capture)
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        const bool capturing = cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (n2 < 0 && own_dev >= 0 && L.ws.ratio_used) {
+        // the words have been published (or will be, when a captured graph runs) and nothing puts them back
         std::lock_guard<std::mutex> lock(g_mu);
-        if (n2 < 0) g_buf[own_dev].ratio_dirty = true;
-        else if (!capturing) g_buf[own_dev].ratio_dirty = false;
+        g_buf[own_dev].ratio_dirty = true;
+        clear_words(L.ws.ratio, stream, &g_buf[own_dev].ratio_dirty);
     }
     if (n2 < 0) return n2;
     t_last_launches = n1 + n2;
