@@ -191,6 +191,7 @@ struct Control {
     // row parity, of every CTA of the cluster (pushed by their owners)
     float4 wslots[kMaxWarps];
     float4 slots[2][kMaxCluster];
+    float4 low[2][kMaxCluster];          // rows that start anywhere: what the sums in `slots` were rounded by (y, w)
     float4 rs;                           // the row's scalars for the second sweep: rq, rp, kappa, c
     uint32_t tmem_base;                  // address of the allocated tensor memory
 };
@@ -456,6 +457,16 @@ template <>
 struct Sum<true> {
     typedef double type;
 };
+// 2^((m - row) scale), the factor that moves a sum from units of the maximum m to units of the row's, in the precision of
+// the sum.
+template <typename Z>
+__device__ __forceinline__ Z unit_factor(float m, float row, float scale);
+template <>
+__device__ __forceinline__ float unit_factor<float>(float m, float row, float scale) { return ex2((m - row) * scale); }
+template <>
+__device__ __forceinline__ double unit_factor<double>(float m, float row, float scale) {
+    return exp2_short(((double)m - (double)row) * (double)scale);
+}
 
 // kAny: rows that do not all start on 16-byte boundaries (odd vocabularies, unaligned buffers).  A copy then brings the
 // 16-byte pieces that hold the cell, and the reads from shared memory start at the remainder.  The few cells at the ends of the
@@ -583,7 +594,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             }
         }
     };
-    const uint32_t xbytes = (uint32_t)(C * sizeof(float4));  // one partial from every CTA of the cluster
+    const uint32_t xbytes = (uint32_t)(C * (kAny ? 2 : 1) * sizeof(float4));  // one partial from every CTA of the cluster
     uint32_t timed_out = 0;
 
     // ---- this warp's copy ring --------------------------------------------------------------------
@@ -851,12 +862,18 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             const float4 v = lane < kFWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
             float bq_row = warp_max_redux(v.x), bp_row = warp_max_redux(v.z);
             float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-            // (kAny: in float64, as the two-sweep path does that such rows took before)
+            // (kAny: factors and sums from here on in float64, as on the two-sweep path that takes such rows otherwise)
             typedef typename Sum<kAny>::type Z;
-            Z Zq = warp_sum(v.x > -INFINITY ? (Z)v.y * (Z)ex2((v.x - rq_row) * s.scale) : (Z)0);
-            Z Zp = warp_sum(v.z > -INFINITY ? (Z)v.w * (Z)ex2((v.z - rp_row) * s.scale) : (Z)0);
+            Z Zq = warp_sum(v.x > -INFINITY ? (Z)v.y * unit_factor<Z>(v.x, rq_row, s.scale) : (Z)0);
+            Z Zp = warp_sum(v.z > -INFINITY ? (Z)v.w * unit_factor<Z>(v.z, rp_row, s.scale) : (Z)0);
             if (C > 1) {  // the same once more over the CTAs of the cluster
-                if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, make_float4(bq_row, (float)Zq, bp_row, (float)Zp));
+                const float zq_hi = (float)Zq, zp_hi = (float)Zp;
+                if (lane < C) {
+                    push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, make_float4(bq_row, zq_hi, bp_row, zp_hi));
+                    if (kAny)
+                        push_f4(&ctl->low[par][rank], xbar, (uint32_t)lane,
+                                make_float4(0.0f, (float)(Zq - (Z)zq_hi), 0.0f, (float)(Zp - (Z)zp_hi)));
+                }
                 mbar_wait(xbar, xph, timed_out);
                 timed_out = __any_sync(0xffffffffu, timed_out != 0);
                 const float4 cv = lane < C ? ctl->slots[par][lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
@@ -864,8 +881,13 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 bp_row = warp_max_redux(cv.z);
                 rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f;
                 rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-                Zq = warp_sum(cv.x > -INFINITY ? (Z)cv.y * (Z)ex2((cv.x - rq_row) * s.scale) : (Z)0);
-                Zp = warp_sum(cv.z > -INFINITY ? (Z)cv.w * (Z)ex2((cv.z - rp_row) * s.scale) : (Z)0);
+                Z cq = (Z)cv.y, cp = (Z)cv.w;
+                if (kAny && lane < C) {
+                    cq += (Z)ctl->low[par][lane].y;
+                    cp += (Z)ctl->low[par][lane].w;
+                }
+                Zq = warp_sum(cv.x > -INFINITY ? cq * unit_factor<Z>(cv.x, rq_row, s.scale) : (Z)0);
+                Zp = warp_sum(cv.z > -INFINITY ? cp * unit_factor<Z>(cv.z, rp_row, s.scale) : (Z)0);
             }
             // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
             // NEXT row needs it, so it is worked out after the other warps have been released.
@@ -1162,8 +1184,9 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
     // the extra sums of rows with c < 1: in this kernel, or for long steps (chain walk, 1 GB of logits or more) in the
     // kernels that the caller queues behind it
     const double bytes = 2.0 * (double)units * (double)s.V * (double)sizeof(T);
-    // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed)
-    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1));
+    // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed; rows that start
+    // anywhere have the cancellation-free numerator at every size, as on the two-sweep path)
+    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1 || kAny));
     *aux_apart = !aux_here;
     return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true, *words_used)
                          : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here, *words_used);

@@ -349,6 +349,52 @@ def test_rows_that_start_anywhere(B, K, gamma, V, dtype, walk):
         assert torch.equal(o.h, outs[0].h) and torch.equal(o.resmass, outs[0].resmass)
 
 
+@pytest.mark.parametrize("V,dtype,d,T", [(20001, "fp32", 9.375, 1.0), (70001, "fp32", 10.75, 0.9), (70001, "bf16", 10.75, 1.0),
+                                        (151937, "fp32", 11.5, 0.7)])
+def test_normalisers_of_rows_that_start_anywhere_are_combined_in_float64(V, dtype, d, T):
+    """One target entry at 0 that only one warp sees, the others' maxima d below it, all of their exponentials 1 in their own
+    units: the residual mass is 1 / Z with Z = 1 + n 2^(-d scale), and all that can be inexact in it are the factors between the
+    warps' and the CTAs' units.  scale is the float32 that the kernels are given; 1e-13 covers a dozen float64 roundings."""
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    zq = torch.full((V,), -d)
+    zp = torch.zeros(V)
+    for cell in (0, 32, 64, 96):            # the first CTA's first warp
+        zq[cell * 256:(cell + 1) * 256] = float("-inf")
+        zp[cell * 256:(cell + 1) * 256] = float("-inf")
+    n = int(torch.isfinite(zq).sum())
+    zq[5] = 0.0
+    target = torch.stack([zq, zq]).to(dt).view(1, 1, 2, V).cuda()
+    draft = zp.to(dt).view(1, 1, 1, V).cuda()
+    binding.set_option("path", 2)
+    try:
+        out = binding.sgbv_verify_ex(target, draft, torch.full((1, 1, 1), V - 1, dtype=torch.int32, device="cuda"),
+                                     torch.full((1, 2), 0.5, device="cuda"), T)
+    finally:
+        binding.set_option("path", 0)
+    scale = np.float64(np.float32(np.float64(np.float32(1.4426950408889634)) / np.float64(np.float32(T))))
+    want = 1.0 / (1.0 + n * np.exp2(-np.float64(d) * scale))
+    np.testing.assert_allclose(out.resmass.item(), want, rtol=1e-13)
+
+
+def test_long_steps_on_rows_that_start_anywhere_keep_the_cancellation_free_numerator():
+    """1 GB of logits in rows of an odd length, two models close to one another: the same bits as with the extra sums forced
+    into the streaming kernel."""
+    B, K, gamma, V = 64, 4, 5, 105001       # 1.08 GB
+    g = torch.Generator(device="cuda").manual_seed(3)
+    target = 2.0 * torch.randn((B, K, gamma + 1, V), device="cuda", generator=g)
+    draft = target[:, :, :gamma] + 1e-3 * torch.randn((B, K, gamma, V), device="cuda", generator=g)
+    tok = torch.randint(0, V, (B, K, gamma), device="cuda", generator=g, dtype=torch.int32)
+    u = torch.rand((B, K * gamma + 1), device="cuda", generator=g)
+    got = binding.sgbv_verify_ex(target, draft, tok, u, 0.9)
+    assert binding.last_launch_count() == 2
+    binding.set_option("aux", 1)
+    try:
+        want = binding.sgbv_verify_ex(target, draft, tok, u, 0.9)
+    finally:
+        binding.set_option("aux", 0)
+    assert torch.equal(got.h, want.h) and torch.equal(got.tokens, want.tokens)
+
+
 def test_degenerate_and_flagged_rows():
     cfg = workloads.VerifyConfig("flags", B=6, K=2, gamma=2, V=300, alpha=0.8, seed=7)
     inp = workloads.make_inputs(cfg, device="cuda")
