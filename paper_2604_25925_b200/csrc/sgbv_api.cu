@@ -203,7 +203,7 @@ int verify_device(const void *zq, const void *zp, int dtype, const int32_t *tok,
     }
     // the fused kernel needs nothing cleared: it reports through the row records and zeroes the
     // error word itself; the two-sweep kernels set status bits with atomics, so those start at zero
-    bool fused = g_opt_path != 1 && fused_supported(L);
+    bool fused = g_opt_path != 1 && fused_supported(L) && (g_opt_path == 2 || !fused_outrun(L));
     L.ws.prestatus = nullptr;
     int words_used = 0;
     bool aux_apart = false;
@@ -392,7 +392,7 @@ int sgbv_modify(const void *target_logits, const void *draft_logits, int dtype, 
     L.stream = stream;
     L.carry_loga = log_a;
     L.carry_logb = log_b;
-    bool fused = g_opt_path != 1 && fused_supported(L);
+    bool fused = g_opt_path != 1 && fused_supported(L) && (g_opt_path == 2 || !fused_outrun(L));
     int words_used = 0;
     bool aux_apart = false;  // (Algorithm 2 needs no extra sums: its draw only uses Eq. 4's weights)
     int n1 = fused ? launch_fused(L, L.ws.error, &words_used, &aux_apart) : 0;

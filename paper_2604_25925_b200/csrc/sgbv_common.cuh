@@ -216,6 +216,7 @@ int launch_kseq(const Launch &L, float *tile_scratch, double *out_rho, double *o
 int launch_draw_rows(const void *z, int dtype, const float *u, const Shape &s, float *tile_scratch, int32_t *out_token,
                      double *out_logp, int32_t *out_status, cudaStream_t stream);
 bool fused_supported(const Launch &L);
+bool fused_outrun(const Launch &L);   // ... and would be the slower one
 // single-read cluster path for steps A1-A3: launches (> 0), 0 if it declined before launching
 // anything (the caller then takes the two-sweep path), or < 0
 // *words_used: words of ws.ratio that the kernel uses (and consumes the preset of)

@@ -1204,8 +1204,35 @@ void fused_set_options(int cluster, int max_clusters, int walk, int poll_us, int
     g_opt_poll_us = poll_us;
 }
 
+// Whether all rows of this call start on 16-byte boundaries.
+bool rows_aligned(const Launch &L) {
+    const size_t esz = L.dtype == SGBV_DTYPE_BF16 ? 2 : 4;
+    return (uintptr_t)L.zq % 16 == 0 && (uintptr_t)L.zp % 16 == 0 && ((size_t)L.s.V * esz) % 16 == 0;
+}
+
 // Whether the fused path can take this call: a row must fit the tensor memory of a cluster (8 CTAs x 32,768 entries).
 bool fused_supported(const Launch &L) { return L.s.ntiles <= kMaxCluster * kCtaCells; }
+
+// Whether the two-sweep kernels are the faster ones: many short rows that start anywhere.  A row costs a cluster some 2.5 us
+// however short it is, and a cluster walks its rows one after the other, where the two-sweep kernels run all rows side by side
+// and pay by the entry (three scalar reads, and the power of Eq. 2 in a loop where K has no kernel of its own).  Two sweeps :
+// streaming, us, bfloat16 (float32): 1024 rows (64 x 4 x 4) of 4 cells 40 : 43 (38 : 43), of 17 cells 50 : 47 (47 : 45); 8192 rows
+// (256 x 8 x 4) of 4 cells 82 : 222 (82 : 220), 17 cells 182 : 247 (189 : 245), 25 cells 243 : 264 (257 : 261), 32 cells 308 : 295
+// (327 : 285).  One position (1024 x 1 x 1): 4 cells 40 : 51 (41 : 49), 17 cells 49 : 54 (48 : 52), 29 cells 58 : 58 (60 : 57);
+// 512 rows (64 x 8 x 1) of 4 cells 32 : 33 (30 : 33), of 13 cells 36 : 34 (34 : 34).  K = 5, 3840 rows of 7 cells 85 : 119
+// (87 : 117), of 13 cells 106 : 124 (152 : 129).  Rows on the boundaries (16-byte reads) stay with the streaming kernel at any
+// length, as before.
+bool fused_outrun(const Launch &L) {
+    const Shape &s = L.s;
+    std::lock_guard<std::mutex> lock(g_plan_mu);
+    if (rows_aligned(L) || g_opt_cluster || g_opt_max_clusters || g_opt_walk || g_opt_aux) return false;
+    const long rows = (long)s.B * s.cpr * s.gamma;
+    const bool own_kernel = s.K <= 4 || s.K == 8;
+    if (s.gamma == 1 && rows < 6 * 148) return rows >= 3 * 148 && s.ntiles <= 9 && own_kernel;
+    if (rows < 6 * 148) return false;
+    if (!own_kernel) return s.ntiles <= 9;
+    return s.ntiles <= (rows >= 12 * 148 || s.gamma == 1 ? 24 : 12);
+}
 
 template <typename T, bool kAny>
 int dispatch_k(const Launch &L, int *error_flag, int *words_used, bool *aux_apart) {
@@ -1223,9 +1250,7 @@ int launch_fused(const Launch &L, int *error_flag, int *words_used, bool *aux_ap
     *words_used = 0;
     *aux_apart = false;
     std::lock_guard<std::mutex> lock(g_plan_mu);
-    // rows that all start on 16-byte boundaries?
-    const size_t esz = L.dtype == SGBV_DTYPE_BF16 ? 2 : 4;
-    const bool any = ((uintptr_t)L.zq % 16) || ((uintptr_t)L.zp % 16) || (((size_t)L.s.V * esz) % 16);
+    const bool any = !rows_aligned(L);
     if (L.dtype == SGBV_DTYPE_BF16)
         return any ? dispatch_k<uint16_t, true>(L, error_flag, words_used, aux_apart)
                    : dispatch_k<uint16_t, false>(L, error_flag, words_used, aux_apart);

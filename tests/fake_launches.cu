@@ -80,6 +80,7 @@ char __cudaInitModule(void **) { return 0; }
 
 namespace sgbv {
 bool fused_supported(const Launch &) { return true; }
+bool fused_outrun(const Launch &) { return false; }
 void fused_set_options(int, int, int, int, int, int) {}
 // As many words as batch rows; cleared first where nobody vouches for them, as the real launcher does.
 int launch_fused(const Launch &L, int *, int *words_used, bool *aux_apart) {

@@ -376,6 +376,39 @@ def test_normalisers_of_rows_that_start_anywhere_are_combined_in_float64(V, dtyp
     np.testing.assert_allclose(out.resmass.item(), want, rtol=1e-13)
 
 
+@pytest.mark.parametrize("B,K,gamma,V,dtype,kernel", [
+    (256, 4, 4, 777, "bf16", "otreduce_kernel"),      # 4096 rows of 4 cells
+    (512, 1, 4, 6143, "fp32", "otreduce_kernel"),     # 2048 of 24: the longest rows that many of them take two sweeps for
+    (512, 1, 4, 6145, "fp32", "fused_chain_kernel"),  # 25
+    (56, 4, 4, 3071, "bf16", "otreduce_kernel"),      # 896 of 12
+    (55, 4, 4, 3071, "bf16", "fused_chain_kernel"),   # 880
+    (56, 4, 4, 3073, "bf16", "fused_chain_kernel"),   # 896 of 13
+    (64, 8, 1, 777, "fp32", "otreduce_kernel"),       # one position: 512 rows
+    (40, 8, 1, 777, "fp32", "fused_chain_kernel"),    # 320
+    (64, 6, 4, 2303, "fp32", "otreduce_kernel"),      # a draft count without a kernel of its own: 9 cells at most
+    (64, 6, 4, 2305, "fp32", "fused_chain_kernel"),
+    (256, 4, 4, 776, "bf16", "fused_chain_kernel"),   # rows on the boundaries never do
+])
+def test_many_short_rows_that_start_anywhere_take_two_sweeps(B, K, gamma, V, dtype, kernel):
+    """Both sides of the rule, each with parity and against the other path (twice the tolerance).  Residual masses: where the
+    draft covers nearly all of the target, S / a = sum of max(q - c p, 0)^K q^(1-K) is a small remainder of terms that each carry
+    the float32 rounding of q and c p, 4 of 2^-24 in all, so that S is good to 2.4e-7 a and no better."""
+    cfg = workloads.VerifyConfig(f"short_{B}_{V}", B=B, K=K, gamma=gamma, V=V, dtype=dtype, temperature=0.8, alpha=0.85, seed=V)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    _, out, ref = run_both(inp)
+    assert binding.last_main_kernel() == kernel
+    assert_parity(compare(ref, *(t.cpu().numpy() for t in (out.accept_len, out.draft_idx, out.tokens, out.h, out.resmass,
+                                                           out.status)), S_atol_rel_a=2.4e-7))
+    binding.set_option("path", 1 if kernel == "fused_chain_kernel" else 2)
+    try:
+        other = binding.sgbv_verify_ex(inp.target_logits, inp.draft_logits, inp.draft_tokens, inp.uniforms, cfg.temperature)
+        assert binding.last_main_kernel() != kernel
+    finally:
+        binding.set_option("path", 0)
+    torch.testing.assert_close(out.h, other.h, rtol=2e-5, atol=2e-9)
+    torch.testing.assert_close(out.resmass, other.resmass, rtol=2e-5, atol=5e-7)   # a <= 1
+
+
 def test_long_steps_on_rows_that_start_anywhere_keep_the_cancellation_free_numerator():
     """1 GB of logits in rows of an odd length, two models close to one another: the same bits as with the extra sums forced
     into the streaming kernel."""
