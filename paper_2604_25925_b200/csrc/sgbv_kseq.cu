@@ -61,7 +61,7 @@ struct KseqScratch {
 
 // Two values per thread combined over the cluster (sum, or maximum); every thread of every CTA gets the results, and
 // slots[par][r] keeps CTA r's share until the exchange after the next one.  All threads must call.
-template <bool kMaximum>
+template <bool kMaximum, bool kHeld>
 __device__ __forceinline__ void exchange(double &a, double &b, KseqScratch &sc, int rank, int C, int &par) {
     const int lane = threadIdx.x & 31, wid = warp_index();
     auto op = [](double x, double y) { return kMaximum ? fmax(x, y) : x + y; };
@@ -87,8 +87,12 @@ __device__ __forceinline__ void exchange(double &a, double &b, KseqScratch &sc, 
             st_peer(&sc.slots[par][rank][1], lane, b);
         }
     }
-    cluster_arrive();
-    cluster_wait();
+    if (kHeld || C > 1) {
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        __syncthreads();
+    }
     a = sc.slots[par][0][0];
     b = sc.slots[par][0][1];
     for (int r = 1; r < C; ++r) {  // (rank order: the same on every CTA)
@@ -97,7 +101,49 @@ __device__ __forceinline__ void exchange(double &a, double &b, KseqScratch &sc, 
     }
 }
 
-template <typename T>
+// f(8 target logits, 8 draft logits) over the entries of tiles t0..t1-1 of a pair of rows, by the whole CTA (-inf in the places
+// past the end): in 16-byte pieces, two tiles of both rows in flight per warp, where the rows can be read so.
+template <typename T, typename F>
+__device__ __forceinline__ void for_entries(const T *zq, const T *zp, int t0, int t1, int V, bool pieces, F f) {
+    constexpr int kPer = kTile / 32;
+    if (!pieces) {
+        const int end = min(V, t1 * kTile);
+        int x = t0 * kTile + threadIdx.x;
+        float a[kPer], c[kPer];
+        for (; x + (kPer - 1) * kThreads < end; x += kPer * kThreads) {
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) {
+                a[e] = ld_logit(zq, x + e * kThreads);
+                c[e] = ld_logit(zp, x + e * kThreads);
+            }
+            f(a, c);
+        }
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const bool in = x + e * kThreads < end;
+            a[e] = in ? ld_logit(zq, x + e * kThreads) : -INFINITY;
+            c[e] = in ? ld_logit(zp, x + e * kThreads) : -INFINITY;
+        }
+        f(a, c);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    for (int t = t0 + warp_index(); t < t1; t += 2 * kWarpsPerCta) {
+        float a[2][kPer], c[2][kPer];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int tt = t + q * kWarpsPerCta;
+            load_tile_pieces<T>(zq, tt, tt < t1, V, lane, a[q]);
+            load_tile_pieces<T>(zp, tt, tt < t1, V, lane, c[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) f(a[q], c[q]);
+    }
+}
+
+// kHeld: the CTA keeps the exponentials of its tiles in shared memory.  Without it (one draft: nothing but the normalisers is
+// added up, so a row is gone through twice and, once per prompt, a third time) it has none, and two CTAs share an SM at any length.
+template <typename T, bool kHeld>
 __global__ void __launch_bounds__(kThreads, 2)
 kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const int32_t *__restrict__ tok_all,
             const float *__restrict__ u_all, Shape s, int C, float *__restrict__ tile_scratch, int32_t *__restrict__ out_tau,
@@ -112,7 +158,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
     const int32_t *tok = tok_all + (size_t)b * K * g;
     const float *u = u_all + (size_t)b * (K * g + 1);
     const int per = (s.ntiles + C - 1) / C, t0 = min(s.ntiles, rank * per), t1 = min(s.ntiles, t0 + per);
-    const int held = min(t1 - t0, kCapTiles);        // tiles in shared memory
+    const int held = kHeld ? min(t1 - t0, kCapTiles) : 0;  // tiles in shared memory
     const int rest0 = (t0 + held) * kTile, rest1 = min(V, t1 * kTile);  // entries that are read again in every sweep
     float *eq_s = rows_s, *ep_s = rows_s + (size_t)min(per, kCapTiles) * kTile;
     // per-tile sums: in shared memory, or for long shares in global scratch
@@ -208,12 +254,22 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
                 }
             }
         }
-        for (int x = rest0 + tid; x < rest1; x += kThreads) {
-            mqf = fmaxf(mqf, ld_logit(zq, x));
-            mpf = fmaxf(mpf, ld_logit(zp, x));
+        if (kHeld) {
+            for (int x = rest0 + tid; x < rest1; x += kThreads) {
+                mqf = fmaxf(mqf, ld_logit(zq, x));
+                mpf = fmaxf(mpf, ld_logit(zp, x));
+            }
+        } else {
+            for_entries<T>(zq, zp, t0, t1, V, pieces, [&](const float (&a)[8], const float (&c)[8]) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    mqf = fmaxf(mqf, a[e]);
+                    mpf = fmaxf(mpf, c[e]);
+                }
+            });
         }
         double mqd = (double)mqf, mpd = (double)mpf;
-        exchange<true>(mqd, mpd, sc, rank, C, par);
+        exchange<true, kHeld>(mqd, mpd, sc, rank, C, par);
         const float mq = (float)mqd, mp = (float)mpd;
         const float nmq = mq > -INFINITY ? -mq : 0.0f, nmp = mp > -INFINITY ? -mp : 0.0f;
         auto eqof = [&](float z) { return ex2((z + nmq) * s.scale); };
@@ -230,12 +286,23 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
             sq += (a.x + a.y) + (a.z + a.w);
             sp += (c.x + c.y) + (c.z + c.w);
         }
-        for (int x = rest0 + tid; x < rest1; x += kThreads) {
-            sq += eqof(ld_logit(zq, x));
-            sp += epof(ld_logit(zp, x));
+        if (kHeld) {
+            for (int x = rest0 + tid; x < rest1; x += kThreads) {
+                sq += eqof(ld_logit(zq, x));
+                sp += epof(ld_logit(zp, x));
+            }
+        } else {
+            // (eight at a time, in a tree: short chains of float32 additions)
+            auto sum8 = [](float a, float b, float c, float d, float e, float f, float g, float h) {
+                return ((a + b) + (c + d)) + ((e + f) + (g + h));
+            };
+            for_entries<T>(zq, zp, t0, t1, V, pieces, [&](const float (&a)[8], const float (&c)[8]) {
+                sq += sum8(eqof(a[0]), eqof(a[1]), eqof(a[2]), eqof(a[3]), eqof(a[4]), eqof(a[5]), eqof(a[6]), eqof(a[7]));
+                sp += sum8(epof(c[0]), epof(c[1]), epof(c[2]), epof(c[3]), epof(c[4]), epof(c[5]), epof(c[6]), epof(c[7]));
+            });
         }
         double Zq = (double)sq, Zp = (double)sp;
-        exchange<false>(Zq, Zp, sc, rank, C, par);
+        exchange<false, kHeld>(Zq, Zp, sc, rank, C, par);
         // NaN entries end up in the sums; +inf is its row's maximum and gives inf - inf there
         if (uniform((int)(!(mq > -INFINITY) || !(mp > -INFINITY) || Zq != Zq || Zp != Zp))) {
             flags |= SGBV_STATUS_NONFINITE_LOGIT;
@@ -243,7 +310,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         }
         // ---- 2. rho (the same on every thread of the cluster) ----------------------------------------------
         double rho = 1.0;
-        if (nk > 1) {
+        if (kHeld && nk > 1) {
             double lo = 1.0, hi = (double)nk;
             for (int it = 0; it < kMaxSteps; ++it) {
                 const float thr = (float)(rho * (Zq / Zp));
@@ -263,7 +330,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
                     s2 += p_of(a, c);
                 }
                 double S1 = (double)s1, S2 = (double)s2;
-                exchange<false>(S1, S2, sc, rank, C, par);
+                exchange<false, kHeld>(S1, S2, sc, rank, C, par);
                 S1 /= Zq;
                 S2 /= Zp;
                 const double beta = S1 / rho + S2;
@@ -348,7 +415,7 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         __syncthreads();
         double W = 0.0, unused = 0.0;
         for (int t = tid; t < t1 - t0; t += kThreads) W += (double)tile_s[t];
-        exchange<false>(W, unused, sc, rank, C, par);
+        exchange<false, kHeld>(W, unused, sc, rank, C, par);
         const double us = (double)u[K * g];
         if (uniform((int)(W > 0.0))) {
             // the CTA whose share the target falls into draws
@@ -390,32 +457,52 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
     }
 }
 
-template <typename T>
-int run(const Launch &L, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status) {
+template <typename T, bool kHeld>
+int run_as(const Launch &L, int C, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status) {
     const Shape &s = L.s;
     int dev = 0;
     static std::atomic<bool> attr_done[64];
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SGBV_ERR_CUDA;
-    if (!attr_done[dev]) {
-        if (cudaFuncSetAttribute(kseq_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (kHeld && !attr_done[dev]) {
+        if (cudaFuncSetAttribute(kseq_kernel<T, kHeld>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  2 * kCapTiles * kTile * (int)sizeof(float)) != cudaSuccess)
             return SGBV_ERR_CUDA;
         attr_done[dev] = true;
     }
+    const int per = (s.ntiles + C - 1) / C;
+    const size_t smem = kHeld ? 2 * (size_t)(per < kCapTiles ? per : kCapTiles) * kTile * sizeof(float) : 0;
+    if (launch_clusters(kseq_kernel<T, kHeld>, (unsigned)s.B * (unsigned)C, kThreads, smem, C, L.stream, (const T *)L.zq,
+                        (const T *)L.zp, L.tok, L.u, s, C, tile_scratch, L.out_tau, L.out_tokens, out_rho, out_acc,
+                        out_status) == cudaSuccess)
+        return 1;
+    cudaGetLastError();
+    return SGBV_ERR_CUDA;
+}
+
+template <typename T>
+int run(const Launch &L, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status) {
+    const Shape &s = L.s;
     // as few CTAs as hold a row on chip; more while the device has room for all of the batch's and a CTA keeps a tile for
     // every other warp
     int C = 1;
     while (C < kMaxRowCtas && (s.ntiles > C * kCapTiles ||
                                ((long)s.B * 2 * C <= kSlots && s.ntiles >= 2 * C * (kWarpsPerCta / 2))))
         C *= 2;
+    // One draft has no sums to add up again and again: holding its rows only pays while the CTAs are all resident (one per SM where
+    // a share is longer than half of kCapTiles), and a row of a few tiles is done before a cluster has met.  Else nothing is
+    // held: one CTA for 128 KB of a row, two for 256, four beyond, more while the device has room for the batch's and a CTA
+    // keeps 28 tiles.  us, gamma = 4, held : not held (one CTA of 1024 threads per prompt and no cluster): 1024 prompts of 128256
+    // bfloat16 1563 : 656 (915), 148 of them 258 : 127 (215); 148 of 50257 110 : 71 (81), float32 108 : 82 (96); 400 of 32256 float32
+    // 149 : 131 (146); 148 of 8192 33 : 27 (31).
     const int per = (s.ntiles + C - 1) / C;
-    const size_t smem = 2 * (size_t)(per < kCapTiles ? per : kCapTiles) * kTile * sizeof(float);
-    if (launch_clusters(kseq_kernel<T>, (unsigned)s.B * (unsigned)C, kThreads, smem, C, L.stream, (const T *)L.zq,
-                        (const T *)L.zp, L.tok, L.u, s, C, tile_scratch, L.out_tau, L.out_tokens, out_rho, out_acc,
-                        out_status) == cudaSuccess)
-        return 1;
-    cudaGetLastError();
-    return SGBV_ERR_CUDA;
+    const bool resident = per <= kCapTiles / 2 || (long)s.B * C <= (C == kMaxRowCtas ? 3 * kSlots / 4 : kSlots / 2);
+    if (s.K == 1 && (s.ntiles <= 32 || s.B > kSlots / 2 || !resident)) {
+        const size_t bytes = (size_t)s.V * sizeof(T);
+        C = bytes <= 128 * 1024 ? 1 : bytes <= 256 * 1024 ? 2 : 4;
+        while (C < kMaxRowCtas && (long)s.B * 2 * C <= kSlots && s.ntiles >= 2 * C * 28) C *= 2;
+        return run_as<T, false>(L, C, tile_scratch, out_rho, out_acc, out_status);
+    }
+    return run_as<T, true>(L, C, tile_scratch, out_rho, out_acc, out_status);
 }
 
 }  // namespace

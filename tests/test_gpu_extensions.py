@@ -145,6 +145,46 @@ def test_kseq_shared_out_over_the_ctas_of_a_row(B, K, gamma, V, dtype, T, alpha,
     assert (same.accept_len == gamma).all() and ((same.tokens >= 0) & (same.tokens < V)).all() and (same.status == 0).all()
 
 
+@pytest.mark.parametrize("B,V,dtype,shift", [
+    (600, 777, "fp32", 0),       # one CTA per prompt, a few tiles
+    (150, 32000, "bf16", 0),     # one, pieces of 16 bytes
+    (100, 32001, "fp32", 0),     # two, rows that start anywhere
+    (60, 40000, "bf16", 1),      # four, off a 16-byte boundary
+    (20, 151936, "fp32", 0),     # eight
+    (50, 221001, "bf16", 0),     # four, more tiles than have a place in shared memory
+])
+def test_one_draft_on_rows_that_are_not_held(B, V, dtype, shift):
+    """Token-level verification of batches: parity, then a NaN in the target row of the first position, +inf in the draft row,
+    nothing finite in a row, a token out of range, and equal rows with a token that the target excludes, so that nothing is left
+    of q - p and the draw comes from q."""
+    cfg = workloads.VerifyConfig("one", B=B, K=1, gamma=3, V=V, dtype=dtype, temperature=0.8, alpha=0.85, seed=V)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t):
+        v = torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape)
+        return v.copy_(t)
+    zq, zp, tok, u = moved(inp.target_logits), moved(inp.draft_logits), inp.draft_tokens.clone(), inp.uniforms
+    good, _ = _kseq_compare(workloads.VerifyInputs(cfg, zq, zp, tok, u), cfg.temperature)
+    zq[1, 0, 0, V - 1] = float("nan")
+    zp[2, 0, 0, V // 2] = float("inf")
+    zq[3, 0, 0] = float("-inf")
+    tok[4, 0, 2] = V
+    zp[5, 0, 0] = zq[5, 0, 0] = 0.0
+    zq[5, 0, 0, 7] = float("-inf")
+    zp[5, 0, 0, 7] = -100.0                        # e^-125: beside V ones it adds nothing to the normaliser
+    zp[5, 0, 0, 8] = float("-inf")                 # (as many ones in both rows)
+    zq[5, 0, 0, 8] = float("-inf")
+    tok[5, 0, 0] = 7
+    out = binding.sgbv_verify_kseq(zq, zp, tok, u, cfg.temperature)
+    st = out.status.cpu().numpy()
+    bad, rng = binding.STATUS_NONFINITE_LOGIT, binding.STATUS_TOKEN_RANGE
+    assert st[1] == bad and st[2] == bad and st[3] == bad and st[4] == rng and st[5] == binding.STATUS_DEGENERATE_RESIDUAL
+    assert (out.accept_len[1:5] == -1).all() and (out.tokens[1:5] == -1).all() and out.accept_len[5].item() == 0
+    assert 0 <= out.tokens[5, 0].item() < V and out.tokens[5, 0].item() not in (7, 8)
+    same = [0] + list(range(6, B))
+    assert torch.equal(out.tokens[same], good.tokens[same]) and (st[same] == good.status.cpu().numpy()[same]).all()
+
+
 def test_kseq_flags():
     cfg = workloads.VerifyConfig("ksf", B=4, K=2, gamma=2, V=300, alpha=0.8, seed=9)
     inp = workloads.make_inputs(cfg, device="cuda")
