@@ -8,10 +8,10 @@
 // rows of the first retained draft are read:
 //   1. every CTA reads its share of the target and the draft row ONCE into shared memory; row maxima, then the
 //      exponentials in place and their sums, both exchanged within the cluster;
-//   2. rho in [1, n]: root of 1 - (1 - beta(rho))^n = rho beta(rho), beta(rho) = sum_x min{p(x), q(x)/rho}, by Newton's
-//      method from the exponentials in shared memory, inside a bracket that every step shrinks (a step that would leave
-//      it bisects it).  rho beta(rho) = S1 + rho S2 with S1 = sum of q where q < rho p, S2 = sum of p elsewhere, so one
-//      sweep gives the value and the slope (n = 1: rho = 1);
+//   2. rho in [1, n]: root of 1 - (1 - beta(rho))^n = rho beta(rho), beta(rho) = sum_x min{p(x), q(x)/rho}.  With the excess
+//      E(rho) = sum_x max{q(x) - rho p(x), 0} it reads E = (1 - beta)^n, 1 - beta = (E + rho - 1) / rho: nothing cancels however
+//      close the rows are.  Newton's method from the exponentials in shared memory, inside a bracket that every step shrinks;
+//      one sweep gives E and the slope (n = 1: rho = 1);
 //   3. the retained drafts are tried in order, draft k's token x is accepted if eta < min{1, q(x)/(rho p(x))};
 //      the first accepted token extends the prefix, the drafts with that token stay retained;
 //   4. if none is accepted: y from norm(max{q - rho p, 0}) by inverse CDF over per-tile sums, and the row is done.
@@ -36,19 +36,8 @@ constexpr int kThreads = 512;        // two CTAs per SM
 constexpr int kWarpsPerCta = kThreads / 32;
 constexpr int kSlots = 2 * 148;      // CTAs the device holds
 constexpr int kCapTiles = 104;       // tiles of both rows in one CTA's shared memory (208 KB)
-constexpr int kMaxSteps = 60;        // bisection alone reaches float64's resolution of rho in that many
-
-// 1 - (1-u)^n as a geometric sum (all terms positive), and its derivative n (1-u)^(n-1).
-__device__ __forceinline__ double gfun_n(double u, int n, double &slope) {
-    const double v = u >= 1.0 ? 0.0 : u > 0.0 ? 1.0 - u : 1.0;
-    double sum = 1.0, pw = 1.0;
-    for (int j = 1; j < n; ++j) {
-        sum = fma(sum, v, 1.0);
-        pw *= v;
-    }
-    slope = (double)n * pw;
-    return u >= 1.0 ? 1.0 : u > 0.0 ? u * sum : 0.0;
-}
+constexpr int kNewtonSteps = 40;     // sweeps that may follow Newton's method; then
+constexpr int kMaxSteps = 80;        // as many that halve the bracket: n 2^-40 is left of it in any case
 
 struct KseqScratch {
     double part[2][kWarpsPerCta];
@@ -313,38 +302,43 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         if (kHeld && nk > 1) {
             double lo = 1.0, hi = (double)nk;
             for (int it = 0; it < kMaxSteps; ++it) {
-                const float thr = (float)(rho * (Zq / Zp));
-                float s1 = 0.0f, s2 = 0.0f;
-                // (added up in the order of the normalisers, so that equal rows give S2 = 1 and with it rho = 1 exactly: the
-                // root is n-fold there, and a rounding error e in S2 would move it by e^(1/n))
-                auto q_of = [&](float a, float c) { return a < thr * c ? a : 0.0f; };
-                auto p_of = [&](float a, float c) { return a < thr * c ? 0.0f : c; };
+                const double r = rho * (Zq / Zp);
+                const float thr = (float)r;
+                float e = 0.0f, s2 = 0.0f;  // sums over the entries with q > rho p: of q - thr p and of p
+                auto excess = [&](float a, float c) { return fmaxf(fmaf(-thr, c, a), 0.0f); };
+                auto p_of = [&](float d, float c) { return d > 0.0f ? c : 0.0f; };
                 for (int j = tid; j < n4; j += kThreads) {
                     const float4 a = eq4[j], c = ep4[j];
-                    s1 += (q_of(a.x, c.x) + q_of(a.y, c.y)) + (q_of(a.z, c.z) + q_of(a.w, c.w));
-                    s2 += (p_of(a.x, c.x) + p_of(a.y, c.y)) + (p_of(a.z, c.z) + p_of(a.w, c.w));
+                    const float dx = excess(a.x, c.x), dy = excess(a.y, c.y), dz = excess(a.z, c.z), dw = excess(a.w, c.w);
+                    e += (dx + dy) + (dz + dw);
+                    s2 += (p_of(dx, c.x) + p_of(dy, c.y)) + (p_of(dz, c.z) + p_of(dw, c.w));
                 }
                 for (int x = rest0 + tid; x < rest1; x += kThreads) {
-                    const float a = eqof(ld_logit(zq, x)), c = epof(ld_logit(zp, x));
-                    s1 += q_of(a, c);
-                    s2 += p_of(a, c);
+                    const float c = epof(ld_logit(zp, x)), d = excess(eqof(ld_logit(zq, x)), c);
+                    e += d;
+                    s2 += p_of(d, c);
                 }
-                double S1 = (double)s1, S2 = (double)s2;
-                exchange<false, kHeld>(S1, S2, sc, rank, C, par);
-                S1 /= Zq;
+                double E = (double)e, S2 = (double)s2;
+                exchange<false, kHeld>(E, S2, sc, rank, C, par);
+                E = fmax(E - (r - (double)thr) * S2, 0.0) / Zq;  // (thr is the float32 next to r)
                 S2 /= Zp;
-                const double beta = S1 / rho + S2;
-                double gs;
-                const double f = gfun_n(beta, nk, gs) - (S1 + rho * S2);
+                const double miss = fmax(E + (rho - 1.0), 0.0) / rho;  // 1 - beta
+                double pw = 1.0;
+                for (int j = 1; j < nk; ++j) pw *= miss;
+                const double f = E - pw * miss;
                 if (f > 0.0) lo = rho;
                 else hi = rho;
                 if (uniform((int)(hi <= lo))) break;  // (f <= 0 at 1: the root is 1)
-                const double df = -gs * S1 / (rho * rho) - S2;
+                const double S1 = fmax(1.0 - E - rho * S2, 0.0);
+                const double df = -(double)nk * pw * S1 / (rho * rho) - S2;
                 double next = rho - f / df;
-                if (!(next > lo && next < hi)) next = 0.5 * (lo + hi);
-                const double step = fabs(next - rho);
-                rho = next;
-                if (uniform((int)(step <= 1e-10 * rho))) break;
+                // (right of the largest q / p nothing is left of E, and Newton's method would creep back)
+                const bool creeps = it >= kNewtonSteps || !(S2 > 0.0);
+                // the last step: below the resolution of the float32 sums (asked before the bracket is: the step may be 0)
+                const bool last = !creeps && fabs(next - rho) <= 1e-8 * rho;
+                if (!last && (creeps || !(next > lo && next < hi))) next = 0.5 * (lo + hi);
+                rho = fmin(fmax(next, lo), hi);
+                if (uniform((int)(last || hi - lo <= 1e-8 * rho))) break;
             }
         }
         // ---- 3. the retained drafts, in order (first warp of every CTA) -----------------------------------------

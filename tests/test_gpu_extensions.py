@@ -145,6 +145,29 @@ def test_kseq_shared_out_over_the_ctas_of_a_row(B, K, gamma, V, dtype, T, alpha,
     assert (same.accept_len == gamma).all() and ((same.tokens >= 0) & (same.tokens < V)).all() and (same.status == 0).all()
 
 
+@pytest.mark.parametrize("K,V,eps", [(2, 32256, 1e-4), (3, 32256, 1e-5), (4, 128256, 1e-3), (8, 32256, 1e-3), (8, 50257, 1e-2), (64, 8192, 0.1)])
+def test_kseq_rho_of_rows_close_to_one_another(K, V, eps):
+    """Draft logits = target logits + eps noise: both sides of the equation of rho are 1 up to eps there, and rho lies near the
+    largest q / p.  Reference: the equation in the form that does not cancel, E = (1 - beta)^n with E = sum max(q - rho p, 0) and
+    1 - beta = (E + rho - 1) / rho, bisected in float64.  1e-5, as for all rho: the exponentials of logits 20 below the
+    maximum carry 20 * 2^-24 of relative error, 1.2e-6 each."""
+    g = torch.Generator(device="cuda").manual_seed(K)
+    B = 3
+    target = (3.0 * torch.randn((B, 1, 2, V), device="cuda", generator=g)).expand(B, K, 2, V).contiguous()
+    draft = (target[:, :1, :1] + eps * torch.randn((B, 1, 1, V), device="cuda", generator=g)).expand(B, K, 1, V).contiguous()
+    tok = torch.zeros((B, K, 1), dtype=torch.int32, device="cuda")
+    u = torch.full((B, K + 1), 0.5, device="cuda")
+    rho = binding.sgbv_verify_kseq(target, draft, tok, u, 1.0).rho[:, 0]
+    q, p = torch.softmax(target[:, 0, 0].double(), -1), torch.softmax(draft[:, 0, 0].double(), -1)
+    lo, hi = torch.ones(B, 1, dtype=torch.float64, device="cuda"), torch.full((B, 1), float(K), dtype=torch.float64, device="cuda")
+    for _ in range(60):
+        mid = 0.5 * (lo + hi)
+        E = (q - mid * p).clamp(min=0.0).sum(-1, keepdim=True)
+        up = E > ((E + mid - 1.0) / mid) ** K
+        lo, hi = torch.where(up, mid, lo), torch.where(up, hi, mid)
+    np.testing.assert_allclose(rho.cpu().numpy(), (0.5 * (lo + hi))[:, 0].cpu().numpy(), rtol=1e-5)
+
+
 @pytest.mark.parametrize("B,V,dtype,shift", [
     (600, 777, "fp32", 0),       # one CTA per prompt, a few tiles
     (150, 32000, "bf16", 0),     # one, pieces of 16 bytes
