@@ -392,24 +392,39 @@ kseq_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const in
         stopped = true;
         const float iZq = (float)(1.0 / Zq), rho_p = (float)rho * (float)(1.0 / Zp);
         auto wof = [&](float a, float c) { return fmaxf(a * iZq - c * rho_p, 0.0f); };
+        // (exp2f: ex2 flushes what lies below 2^-126 of the row's maximum to 0)
+        auto eq_full = [&](int x) { return exp2f((ld_logit(zq, x) + nmq) * s.scale); };
+        auto ep_full = [&](int x) { return exp2f((ld_logit(zp, x) + nmp) * s.scale); };
         auto entry = [&](int x) {
             const int j = x - t0 * kTile;
-            return j < held * kTile ? wof(eq_s[j], ep_s[j]) : wof(eqof(ld_logit(zq, x)), epof(ld_logit(zp, x)));
+            return j < held * kTile ? wof(eq_s[j], ep_s[j]) : wof(eq_full(x), ep_full(x));
         };
-        for (int t = wid; t < t1 - t0; t += kWarpsPerCta) {  // one warp per tile
-            float acc = 0.0f;
+        double W = 0.0;
+        for (bool full = !kHeld;; full = true) {
+            for (int t = wid; t < t1 - t0; t += kWarpsPerCta) {  // one warp per tile
+                float acc = 0.0f;
 #pragma unroll
-            for (int e = 0; e < kTile / 32; ++e) {
-                const int x = (t0 + t) * kTile + lane + 32 * e;
-                if (x < V) acc += entry(x);
+                for (int e = 0; e < kTile / 32; ++e) {
+                    const int x = (t0 + t) * kTile + lane + 32 * e;
+                    if (x < V) acc += entry(x);
+                }
+                acc = warp_sum(acc);
+                if (lane == 0) tile_s[t] = acc;
             }
-            acc = warp_sum(acc);
-            if (lane == 0) tile_s[t] = acc;
+            __syncthreads();
+            double unused = 0.0;
+            W = 0.0;
+            for (int t = tid; t < t1 - t0; t += kThreads) W += (double)tile_s[t];
+            exchange<false, kHeld>(W, unused, sc, rank, C, par);
+            if (full || uniform((int)(W > 0x1p-90))) break;
+            // next to no mass: what was flushed may be all there is of q - rho p, so the held exponentials are made again
+            for (int j = tid; j < held * kTile; j += kThreads)
+                if (t0 * kTile + j < V) {
+                    eq_s[j] = eq_full(t0 * kTile + j);
+                    ep_s[j] = ep_full(t0 * kTile + j);
+                }
+            __syncthreads();
         }
-        __syncthreads();
-        double W = 0.0, unused = 0.0;
-        for (int t = tid; t < t1 - t0; t += kThreads) W += (double)tile_s[t];
-        exchange<false, kHeld>(W, unused, sc, rank, C, par);
         const double us = (double)u[K * g];
         if (uniform((int)(W > 0.0))) {
             // the CTA whose share the target falls into draws

@@ -168,6 +168,23 @@ def test_kseq_rho_of_rows_close_to_one_another(K, V, eps):
     np.testing.assert_allclose(rho.cpu().numpy(), (0.5 * (lo + hi))[:, 0].cpu().numpy(), rtol=1e-5)
 
 
+@pytest.mark.parametrize("B,K,V", [(2, 1, 300), (2, 3, 9000), (1, 2, 50257), (160, 1, 9000)])
+def test_kseq_residual_of_entries_far_below_the_maximum(B, K, V):
+    """Equal rows (four ones each: exact normalisers) but for an entry at 2^-130 that the draft excludes and, at 2^-128, the
+    drafted token that the target excludes: the token is rejected, and all that is left of q - rho p is the first of them."""
+    zq = torch.full((B, K, 2, V), float("-inf"))
+    zq[..., 10:14] = 0.0
+    zp = zq[:, :, :1].clone()
+    zq[:, :, 0, V - 3] = -130.0 * float(np.log(2.0))
+    zp[:, :, 0, 20] = -128.0 * float(np.log(2.0))
+    tok = torch.full((B, K, 1), 20, dtype=torch.int32)
+    u = torch.full((B, K + 1), 0.5)
+    out = binding.sgbv_verify_kseq(zq.cuda(), zp.cuda(), tok.cuda(), u.cuda(), 1.0)
+    ref = oracle.kseq_verify(zq.numpy(), zp.numpy(), tok.numpy(), u.numpy(), 1.0)
+    assert (ref.tokens[:, 0] == V - 3).all() and (ref.status == 0).all()
+    assert (out.tokens[:, 0].cpu().numpy() == ref.tokens[:, 0]).all() and (out.status == 0).all() and (out.accept_len == 0).all()
+
+
 @pytest.mark.parametrize("B,V,dtype,shift", [
     (600, 777, "fp32", 0),       # one CTA per prompt, a few tiles
     (150, 32000, "bf16", 0),     # one, pieces of 16 bytes
