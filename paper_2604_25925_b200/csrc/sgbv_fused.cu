@@ -457,15 +457,22 @@ template <>
 struct Sum<true> {
     typedef double type;
 };
-// 2^((m - row) scale), the factor that moves a sum from units of the maximum m to units of the row's, in the precision of
-// the sum.
+// 2^((m - row) scale), m <= row: the factor that moves a sum from units of the maximum m to units of the row's, in the
+// precision of the sum.
 template <typename Z>
 __device__ __forceinline__ Z unit_factor(float m, float row, float scale);
 template <>
 __device__ __forceinline__ float unit_factor<float>(float m, float row, float scale) { return ex2((m - row) * scale); }
 template <>
 __device__ __forceinline__ double unit_factor<double>(float m, float row, float scale) {
-    return exp2_short(((double)m - (double)row) * (double)scale);
+    // e^(f ln 2), |f| <= 1/2, by its Taylor series to degree 11 (remainder below 7e-15), in pairs and without a branch: behind
+    // exp2_short's the lanes ran apart and the shuffles of the sums took 1.1 us more per row
+    const double x = fmax(((double)m - (double)row) * (double)scale, -1000.0);
+    const double n = rint(x), t = (x - n) * 0.6931471805599453094, t2 = t * t, t4 = t2 * t2;
+    const double c0 = 1.0 + t, c1 = fma(t, 1.0 / 6.0, 0.5), c2 = fma(t, 1.0 / 120.0, 1.0 / 24.0), c3 = fma(t, 1.0 / 5040.0, 1.0 / 720.0);
+    const double c4 = fma(t, 1.0 / 362880.0, 1.0 / 40320.0), c5 = fma(t, 1.0 / 39916800.0, 1.0 / 3628800.0);
+    const double lo = fma(t2, c1, c0), mid = fma(t2, c3, c2), hi = fma(t2, c5, c4);
+    return fma(t4, fma(t4, hi, mid), lo) * __longlong_as_double((long long)((int)n + 1023) << 52);
 }
 
 // kAny: rows that do not all start on 16-byte boundaries (odd vocabularies, unaligned buffers).  A copy then brings the
@@ -864,8 +871,9 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
             // (kAny: factors and sums from here on in float64, as on the two-sweep path that takes such rows otherwise)
             typedef typename Sum<kAny>::type Z;
-            Z Zq = warp_sum(v.x > -INFINITY ? (Z)v.y * unit_factor<Z>(v.x, rq_row, s.scale) : (Z)0);
-            Z Zp = warp_sum(v.z > -INFINITY ? (Z)v.w * unit_factor<Z>(v.z, rp_row, s.scale) : (Z)0);
+            const Z fq = (Z)v.y * unit_factor<Z>(v.x, rq_row, s.scale), fp = (Z)v.w * unit_factor<Z>(v.z, rp_row, s.scale);
+            Z Zq = warp_sum(v.x > -INFINITY ? fq : (Z)0);
+            Z Zp = warp_sum(v.z > -INFINITY ? fp : (Z)0);
             if (C > 1) {  // the same once more over the CTAs of the cluster
                 const float zq_hi = (float)Zq, zp_hi = (float)Zp;
                 if (lane < C) {
@@ -886,8 +894,10 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                     cq += (Z)ctl->low[par][lane].y;
                     cp += (Z)ctl->low[par][lane].w;
                 }
-                Zq = warp_sum(cv.x > -INFINITY ? cq * unit_factor<Z>(cv.x, rq_row, s.scale) : (Z)0);
-                Zp = warp_sum(cv.z > -INFINITY ? cp * unit_factor<Z>(cv.z, rp_row, s.scale) : (Z)0);
+                cq *= unit_factor<Z>(cv.x, rq_row, s.scale);
+                cp *= unit_factor<Z>(cv.z, rp_row, s.scale);
+                Zq = warp_sum(cv.x > -INFINITY ? cq : (Z)0);
+                Zp = warp_sum(cv.z > -INFINITY ? cp : (Z)0);
             }
             // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
             // NEXT row needs it, so it is worked out after the other warps have been released.
@@ -1185,8 +1195,9 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
     // kernels that the caller queues behind it
     const double bytes = 2.0 * (double)units * (double)s.V * (double)sizeof(T);
     // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed; rows that start
-    // anywhere have the cancellation-free numerator at every size, as on the two-sweep path)
-    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1 || kAny));
+    // anywhere included: error of the weights against 64 bits with the sums here / apart 4.1e-8 / 5.7e-8 at 64 x 8 x 6 x 50257
+    // bfloat16, 5.9e-8 / 1.0e-7 at 64 x 2 x 12 x 100003, where the two-sweep path has 1.6e-7 and 4.0e-7)
+    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1));
     *aux_apart = !aux_here;
     return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true, *words_used)
                          : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here, *words_used);

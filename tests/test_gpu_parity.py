@@ -409,25 +409,6 @@ def test_many_short_rows_that_start_anywhere_take_two_sweeps(B, K, gamma, V, dty
     torch.testing.assert_close(out.resmass, other.resmass, rtol=2e-5, atol=5e-7)   # a <= 1
 
 
-def test_long_steps_on_rows_that_start_anywhere_keep_the_cancellation_free_numerator():
-    """1 GB of logits in rows of an odd length, two models close to one another: the same bits as with the extra sums forced
-    into the streaming kernel."""
-    B, K, gamma, V = 64, 4, 5, 105001       # 1.08 GB
-    g = torch.Generator(device="cuda").manual_seed(3)
-    target = 2.0 * torch.randn((B, K, gamma + 1, V), device="cuda", generator=g)
-    draft = target[:, :, :gamma] + 1e-3 * torch.randn((B, K, gamma, V), device="cuda", generator=g)
-    tok = torch.randint(0, V, (B, K, gamma), device="cuda", generator=g, dtype=torch.int32)
-    u = torch.rand((B, K * gamma + 1), device="cuda", generator=g)
-    got = binding.sgbv_verify_ex(target, draft, tok, u, 0.9)
-    assert binding.last_launch_count() == 2
-    binding.set_option("aux", 1)
-    try:
-        want = binding.sgbv_verify_ex(target, draft, tok, u, 0.9)
-    finally:
-        binding.set_option("aux", 0)
-    assert torch.equal(got.h, want.h) and torch.equal(got.tokens, want.tokens)
-
-
 def test_degenerate_and_flagged_rows():
     cfg = workloads.VerifyConfig("flags", B=6, K=2, gamma=2, V=300, alpha=0.8, seed=7)
     inp = workloads.make_inputs(cfg, device="cuda")
