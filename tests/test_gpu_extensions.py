@@ -225,6 +225,37 @@ def test_one_draft_on_rows_that_are_not_held(B, V, dtype, shift):
     assert torch.equal(out.tokens[same], good.tokens[same]) and (st[same] == good.status.cpu().numpy()[same]).all()
 
 
+@pytest.mark.parametrize("V,dtype", [(9000, "fp32"), (50257, "bf16")])
+def test_kseq_flags_with_several_ctas_per_row(V, dtype):
+    """Every way out of the walk by clusters of four (V = 9000) and eight CTAs: a token out of range, NaN in the first and second
+    position, a row without a finite entry, a bonus row with +inf, a residual without mass.  The other rows keep their bits."""
+    B, K, gamma = 8, 2, 2
+    cfg = workloads.VerifyConfig("kfl", B=B, K=K, gamma=gamma, V=V, dtype=dtype, temperature=0.8, alpha=0.85, seed=V)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    zq, zp, tok, u = inp.target_logits.clone(), inp.draft_logits.clone(), inp.draft_tokens.clone(), inp.uniforms.clone()
+    good, _ = _kseq_compare(inp, cfg.temperature)
+    tok[1, 1, 1] = V
+    zq[2, :, 0, V - 1] = float("nan")
+    zp[3, :, :, :] = zq[3, :, :gamma]                # all accepted up to the NaN of the second position
+    zp[3, :, 1, V // 3] = float("nan")
+    zq[4, :, 0] = float("-inf")
+    zp[5] = zq[5, :, :gamma]                         # all accepted, then a bonus row that cannot be drawn from
+    zq[5, :, gamma, 0] = float("inf")
+    zp[6, :, 0] = zq[6, :, 0] = 0.0                  # equal rows but for a token that the target excludes
+    zq[6, :, 0, 7] = zq[6, :, 0, 8] = zp[6, :, 0, 8] = float("-inf")
+    zp[6, :, 0, 7] = -100.0                          # e^-125: beside V ones it adds nothing to the normaliser
+    tok[6, :, 0] = 7
+    out = binding.sgbv_verify_kseq(zq, zp, tok, u, cfg.temperature)
+    st = out.status.cpu().numpy()
+    bad, rng = binding.STATUS_NONFINITE_LOGIT, binding.STATUS_TOKEN_RANGE
+    assert st.tolist() == [good.status[0].item(), rng, bad, bad, bad, bad, binding.STATUS_DEGENERATE_RESIDUAL, good.status[7].item()]
+    assert (out.accept_len[1:6] == -1).all() and (out.tokens[1:6] == -1).all() and out.accept_len[6].item() == 0
+    assert 0 <= out.tokens[6, 0].item() < V and out.tokens[6, 0].item() not in (7, 8)
+    for b in (0, 7):
+        assert torch.equal(out.tokens[b], good.tokens[b])
+        assert torch.equal(out.accept_prob[b].nan_to_num(-1), good.accept_prob[b].nan_to_num(-1))
+
+
 def test_kseq_flags():
     cfg = workloads.VerifyConfig("ksf", B=4, K=2, gamma=2, V=300, alpha=0.8, seed=9)
     inp = workloads.make_inputs(cfg, device="cuda")

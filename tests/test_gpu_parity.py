@@ -409,6 +409,86 @@ def test_many_short_rows_that_start_anywhere_take_two_sweeps(B, K, gamma, V, dty
     torch.testing.assert_close(out.resmass, other.resmass, rtol=2e-5, atol=5e-7)   # a <= 1
 
 
+@pytest.mark.parametrize("V,dtype,walk,shift", [(8191, "fp32", 1, 0), (8191, "bf16", 2, 1), (40001, "bf16", 1, 3), (40001, "fp32", 2, 1),
+                                               (151937, "bf16", 1, 0)])
+def test_flagged_and_masked_rows_that_start_anywhere(V, dtype, walk, shift):
+    """NaN, +inf and missing rows where rows start anywhere, among them the entries at the two ends of the tensors, which no copy
+    brings; masked halves; equal rows; a token out of range.  The ordinary rows keep their bits."""
+    B = 9
+    cfg = workloads.VerifyConfig("anyflags", B=B, K=2, gamma=2, V=V, dtype=dtype, alpha=0.85, seed=V)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t):
+        return torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape).copy_(t)
+    zq, zp = moved(inp.target_logits), moved(inp.draft_logits)
+    tok, u = inp.draft_tokens.clone(), inp.uniforms.clone()
+    ninf = float("-inf")
+    tok[5] %= V // 2
+    tok[6] = V // 2 + tok[6] % (V - V // 2)
+    zq[5, :, :, V // 2:] = zp[5, :, :, V // 2:] = ninf       # masked: the second half, and the first
+    zq[6, :, :, :V // 2] = zp[6, :, :, :V // 2] = ninf
+    zp[7] = zq[7, :, :2]                                     # p == q: no residual mass
+    u[7, :4] = 0.999
+    binding.set_option("walk", walk)
+    binding.set_option("path", 2)
+    try:
+        rep, good, _ = run_both(workloads.VerifyInputs(cfg, zq, zp, tok, u))
+        assert_parity(rep)
+        zq[0, 0, 0, 0] = float("nan")                        # the first entry of the target tensor
+        zp[B - 1, 1, 1, V - 1] = float("nan")                # the last one of the draft tensor
+        zq[1, 1, 0, V // 2] = float("inf")
+        zp[2, 0, 1] = ninf                                   # a row without a finite entry
+        zq[3, 0, 1, V - 1] = float("nan")
+        tok[4, 1, 1] = V
+        out = binding.sgbv_verify_ex(zq, zp, tok, u, cfg.temperature)
+    finally:
+        binding.set_option("walk", 0)
+        binding.set_option("path", 0)
+    st = out.status.cpu().numpy()
+    assert (st[[0, 1, 2, 3, 8]] == binding.STATUS_NONFINITE_LOGIT).all() and st[4] == binding.STATUS_TOKEN_RANGE
+    bad = [0, 1, 2, 3, 4, 8]
+    assert (out.tokens[bad] == -1).all() and (out.accept_len[bad] == -1).all() and out.h[bad].isnan().all()
+    for b in (5, 6, 7):
+        assert torch.equal(out.tokens[b], good.tokens[b]) and torch.equal(out.h[b], good.h[b]) and out.status[b] == good.status[b]
+    assert st[7] & binding.STATUS_DEGENERATE_RESIDUAL
+
+
+@pytest.mark.parametrize("K,dtype,alpha", [(2, "bf16", 0.9), (8, "fp32", 0.95), (5, "bf16", 0.99), (3, "fp32", 0.9995)])
+def test_extra_sums_in_kernels_of_their_own_on_rows_that_start_anywhere(K, dtype, alpha):
+    """As the test on aligned rows, for an odd vocabulary; and the plain entry point, which takes no weights: the rows' totals
+    then lie where the weights go."""
+    cfg = workloads.VerifyConfig(f"auxany_{K}", B=20, K=K, gamma=4, V=20225, dtype=dtype, temperature=0.8, alpha=alpha, seed=K)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    res = {}
+    for aux in (2, 1):
+        binding.set_option("walk", 1)
+        binding.set_option("aux", aux)
+        try:
+            rep, res[aux], _ = run_both(inp)
+            assert_parity(rep)
+            for _ in range(2):
+                plain = binding.sgbv_verify(inp.target_logits, inp.draft_logits, inp.draft_tokens, inp.uniforms, cfg.temperature)
+                assert binding.last_launch_count() == (4 if aux == 2 else 2)
+                assert torch.equal(plain.tokens, res[aux].tokens) and torch.equal(plain.accept_len, res[aux].accept_len)
+                assert torch.equal(plain.draft_idx, res[aux].draft_idx)
+        finally:
+            binding.set_option("walk", 0)
+            binding.set_option("aux", 0)
+    np.testing.assert_allclose(res[2].h.cpu().numpy(), res[1].h.cpu().numpy(), rtol=2e-5, atol=1e-9)
+
+
+@pytest.mark.parametrize("V,dtype,shift", [(8 * 32768 + 1, "fp32", 0), (8 * 32768 + 4099, "bf16", 0), (8 * 32768 + 8, "bf16", 1)])
+def test_vocabulary_beyond_the_fused_kernel_capacity_on_rows_that_start_anywhere(V, dtype, shift):
+    cfg = workloads.VerifyConfig("biganyv", B=2, K=2, gamma=2, V=V, dtype=dtype, alpha=0.85, seed=608)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t):
+        return torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape).copy_(t)
+    rep, _, _ = run_both(workloads.VerifyInputs(cfg, moved(inp.target_logits), moved(inp.draft_logits), inp.draft_tokens, inp.uniforms))
+    assert_parity(rep)
+    assert binding.last_main_kernel() == "otreduce_kernel"
+
+
 def test_degenerate_and_flagged_rows():
     cfg = workloads.VerifyConfig("flags", B=6, K=2, gamma=2, V=300, alpha=0.8, seed=7)
     inp = workloads.make_inputs(cfg, device="cuda")
