@@ -210,7 +210,7 @@ int launch_finish(const Launch &L);   // weights, scan, extra token
 // Algorithm 2's draw per batch row from the cell sums of a gamma = 1 launch with carried logs
 int launch_modify_finish(const Launch &L, const float *u, int32_t *out_token, double *out_loga, double *out_logb,
                          double *out_resmass, int32_t *out_status);
-// K-SEQ / token-level verification, one CTA per batch row; tile_scratch: [B][2][ntiles] floats
+// K-SEQ / token-level verification, one to eight CTAs per batch row; tile_scratch: [B][2][ntiles] floats
 int launch_kseq(const Launch &L, float *tile_scratch, double *out_rho, double *out_acc, int32_t *out_status);
 // one token per row of z [s.B, s.V] from softmax(z/T) by inverse CDF; tile_scratch: [s.B][2][ntiles] floats
 int launch_draw_rows(const void *z, int dtype, const float *u, const Shape &s, float *tile_scratch, int32_t *out_token,

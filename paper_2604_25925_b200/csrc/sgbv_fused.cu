@@ -457,14 +457,8 @@ template <>
 struct Sum<true> {
     typedef double type;
 };
-// 2^((m - row) scale), m <= row: the factor that moves a sum from units of the maximum m to units of the row's, in the
-// precision of the sum.
-template <typename Z>
-__device__ __forceinline__ Z unit_factor(float m, float row, float scale);
-template <>
-__device__ __forceinline__ float unit_factor<float>(float m, float row, float scale) { return ex2((m - row) * scale); }
-template <>
-__device__ __forceinline__ double unit_factor<double>(float m, float row, float scale) {
+// 2^((m - row) scale), m <= row: the factor that moves a sum from units of the maximum m to units of the row's, in float64.
+__device__ __forceinline__ double unit_factor(float m, float row, float scale) {
     // e^(f ln 2), |f| <= 1/2, by its Taylor series to degree 11 (remainder below 7e-15), in pairs and without a branch: behind
     // exp2_short's the lanes ran apart and the shuffles of the sums took 1.1 us more per row
     const double x = fmax(((double)m - (double)row) * (double)scale, -1000.0);
@@ -871,17 +865,23 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
             // (kAny: factors and sums from here on in float64, as on the two-sweep path that takes such rows otherwise)
             typedef typename Sum<kAny>::type Z;
-            const Z fq = (Z)v.y * unit_factor<Z>(v.x, rq_row, s.scale), fp = (Z)v.w * unit_factor<Z>(v.z, rp_row, s.scale);
-            Z Zq = warp_sum(v.x > -INFINITY ? fq : (Z)0);
-            Z Zp = warp_sum(v.z > -INFINITY ? fp : (Z)0);
-            if (C > 1) {  // the same once more over the CTAs of the cluster
-                const float zq_hi = (float)Zq, zp_hi = (float)Zp;
-                if (lane < C) {
-                    push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, make_float4(bq_row, zq_hi, bp_row, zp_hi));
-                    if (kAny)
-                        push_f4(&ctl->low[par][rank], xbar, (uint32_t)lane,
-                                make_float4(0.0f, (float)(Zq - (Z)zq_hi), 0.0f, (float)(Zp - (Z)zp_hi)));
+            // the sum over the lanes of z, each moved from units of m to units of `row` (-inf: a lane without a share)
+            auto combine = [&](float m, Z z, float row) {
+                if constexpr (kAny) {
+                    const Z moved = z * unit_factor(m, row, s.scale);
+                    return warp_sum(m > -INFINITY ? moved : (Z)0);
+                } else {
+                    return warp_sum(m > -INFINITY ? z * ex2((m - row) * s.scale) : 0.0f);
                 }
+            };
+            Z Zq = combine(v.x, v.y, rq_row), Zp = combine(v.z, v.w, rp_row);
+            if (C > 1) {  // the same once more over the CTAs of the cluster
+                const float4 mine = make_float4(bq_row, (float)Zq, bp_row, (float)Zp);
+                if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, mine);
+                if constexpr (kAny)
+                    if (lane < C)
+                        push_f4(&ctl->low[par][rank], xbar, (uint32_t)lane,
+                                make_float4(0.0f, (float)(Zq - (Z)mine.y), 0.0f, (float)(Zp - (Z)mine.w)));
                 mbar_wait(xbar, xph, timed_out);
                 timed_out = __any_sync(0xffffffffu, timed_out != 0);
                 const float4 cv = lane < C ? ctl->slots[par][lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
@@ -889,15 +889,14 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 bp_row = warp_max_redux(cv.z);
                 rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f;
                 rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-                Z cq = (Z)cv.y, cp = (Z)cv.w;
-                if (kAny && lane < C) {
-                    cq += (Z)ctl->low[par][lane].y;
-                    cp += (Z)ctl->low[par][lane].w;
+                if constexpr (kAny) {
+                    const float4 low = lane < C ? ctl->low[par][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    Zq = combine(cv.x, (Z)cv.y + (Z)low.y, rq_row);
+                    Zp = combine(cv.z, (Z)cv.w + (Z)low.w, rp_row);
+                } else {
+                    Zq = combine(cv.x, cv.y, rq_row);
+                    Zp = combine(cv.z, cv.w, rp_row);
                 }
-                cq *= unit_factor<Z>(cv.x, rq_row, s.scale);
-                cp *= unit_factor<Z>(cv.z, rp_row, s.scale);
-                Zq = warp_sum(cv.x > -INFINITY ? cq : (Z)0);
-                Zp = warp_sum(cv.z > -INFINITY ? cp : (Z)0);
             }
             // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
             // NEXT row needs it, so it is worked out after the other warps have been released.

@@ -34,7 +34,7 @@ namespace {
 
 constexpr int kThreads = 512;        // two CTAs per SM
 constexpr int kWarpsPerCta = kThreads / 32;
-constexpr int kSlots = 2 * 148;      // CTAs the device holds
+constexpr int kSlots = 2 * 148;      // CTAs the device holds, of up to half of kCapTiles tiles (or none held); longer ones: half as many
 constexpr int kCapTiles = 104;       // tiles of both rows in one CTA's shared memory (208 KB)
 constexpr int kNewtonSteps = 40;     // sweeps that may follow Newton's method; then
 constexpr int kMaxSteps = 80;        // as many that halve the bracket: n 2^-40 is left of it in any case

@@ -3,7 +3,7 @@
 //   chain    (chain_kernel)     per draft: row normalisers, c_i = p(x^i)/q(x^i), kappa_i
 //   sweep 2  (otreduce_kernel)  per-tile sums of the residual weights (and of the two
 //                               non-negative numerator terms when c_i < 1)
-// It reads each needed logit twice, so it is the fallback for rows longer than the fused kernel holds.
+// It reads each needed logit twice: for rows longer than the fused kernel holds, and for many short rows that start anywhere.
 #include "sgbv_sample.cuh"
 #include "sgbv_weights.cuh"
 
