@@ -49,8 +49,10 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
 
     // A kernel launched behind this one with programmatic stream serialisation (the next call's streaming
     // kernel) may be scheduled from now on; it waits for this grid to complete before it touches memory.
-    // Only for small batches, where this grid leaves most SMs idle.
-    if (s.B <= kChainedLaunchMaxB) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Only for small batches, where this grid leaves most SMs idle, and not behind the kernels of a long step's rare rows: this
+    // grid's CTAs then lie scattered over the device, the next streaming kernel's clusters are packed around them, and one
+    // that no longer fits runs behind the others (16 x 8 x 12 x 151936 float32 in a row of calls 459 -> 666 us).
+    if (s.B <= kChainedLaunchMaxB && !ws.wsum) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int b = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const int nthreads = blockDim.x, nwarps = nthreads / 32;

@@ -472,8 +472,9 @@ __device__ __forceinline__ double unit_factor(float m, float row, float scale) {
 // kAny: rows that do not all start on 16-byte boundaries (odd vocabularies, unaligned buffers).  A copy then brings the
 // 16-byte pieces that hold the cell, and the reads from shared memory start at the remainder.  The few cells at the ends of the
 // tensors whose pieces reach past them are loaded directly.
-// Such rows used to take the two-sweep path (three scalar reads of every logit, four kernels): 16 prompts, K = 4, gamma = 4,
-// V = 50257 bfloat16 113 -> 66 us, one prompt at V = 32001 float32 73 -> 19, 64 prompts, K = 2 at V = 128255 float32 527 -> 195.
+// Two sweeps over such rows (three scalar reads of every logit, four kernels) take longer, unless the rows are short and many
+// (fused_outrun): 16 prompts, K = 4, gamma = 4, V = 50257 bfloat16 105 us against 63 here, one prompt at V = 32001 float32 68 and 20,
+// 64 prompts, K = 2 at V = 128255 float32 510 and 200.
 // Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4.
 // W warps per CTA; NS ring slots per warp (the cells per warp and row, kCtaCells / W, are a multiple of it, so
 // that cell j of a row always sits in slot j % NS); KT: the number of drafts K when it has a specialised

@@ -18,12 +18,13 @@
 // After gamma accepted positions y is drawn from the target row that follows the block.  All decisions are taken by every
 // CTA of the cluster from the same numbers.
 //
-// What bounds it is the serial chain: positions one after the other, some six sweeps and as many cluster exchanges each.
-// Rows stay on chip between the sweeps (a CTA holds up to kCapTiles tiles; the rest of a longer share is read again in
-// every sweep), and a row is spread over as many CTAs as the batch leaves free.  64 prompts, K = 3, gamma = 12, 32256
-// float32: 71 us, against 424 us of one CTA of 1024 threads per prompt that read the rows from L2 in two sweeps for the
-// statistics and one for each of 34 bisections.  (Two prompts in three stop at the first or second position; the time is
-// that of the longest walk.)
+// What bounds it is the serial chain: positions one after the other, some seven sweeps and as many cluster exchanges each
+// (five for rho on ordinary rows, up to some 30 where target and draft nearly agree).  Rows stay on chip between the sweeps (a
+// CTA holds up to kCapTiles tiles; the rest of a longer share is read again in every sweep), and a row is spread over as many
+// CTAs as the batch leaves free.  64 prompts, K = 3, gamma = 12, 32256 float32: 66-72 us from machine to machine (two prompts in
+// three stop at the first or second position; the time is that of the longest walk), against 370-480 of one CTA of 1024 threads per
+// prompt that read the rows from L2 in two sweeps for the statistics and one for each of 34 bisections.  With one draft
+// there is no rho, and batches that leave no SM idle hold nothing (kHeld = false; the rule and its figures stand at run()).
 #include <atomic>
 
 #include "sgbv_sample.cuh"
