@@ -1127,7 +1127,13 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = L.s.B <= kChainedLaunchMaxB ? 2 : 1;  // small batches only: see kChainedLaunchMaxB
+    // Small batches only (see kChainedLaunchMaxB), and not where the clusters would be packed around the finishing kernel's
+    // CTAs, one per batch row: if those do not fit on the SMs that the clusters leave idle, some clusters of an odd size find
+    // no room and run behind the others (16 x 8 x 4 x 98304, clusters of three, float32 138 -> 156 us, bfloat16 138 -> 158;
+    // clusters of five with 18 idle SMs gain 5 us of 250, those of two, four, six and eight lost nothing).
+    const bool early = L.s.B <= kChainedLaunchMaxB &&
+                       (kRow || plan.cluster == 1 || plan.cluster % 2 == 0 || clusters * plan.cluster + L.s.B <= kCtaSlots);
+    cfg.numAttrs = early ? 2 : 1;
     cfg.gridDim = dim3(clusters * plan.cluster);
     if (words_used > 0 && !L.ratio_preset &&
         cudaMemsetAsync(L.ws.ratio, 0xff, (size_t)words_used * sizeof(double), L.stream) != cudaSuccess)
