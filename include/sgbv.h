@@ -288,7 +288,9 @@ int sgbv_profile_end(double *out_total_ms, int *out_records);
 
 /*
  * Tuning knobs for experiments (process-wide, not thread-safe; 0 restores the automatic choice):
- *   "path"         1 = always the generic two-sweep kernels, 2 = the fused single-read kernel or fail
+ *   "path"         1 = always the generic two-sweep kernels, 2 = the fused single-read kernel or fail; 0 = the fused one, but
+ *                  two sweeps for rows of more than 262,144 entries and for many short rows that do not start on 16-byte
+ *                  boundaries (unless one of the next four options is set)
  *   "cluster"      CTAs per cluster of the fused kernel (1..8)
  *   "max_clusters" cap on the number of resident clusters it launches
  *   "walk"         1 = a cluster of the fused kernel walks whole draft chains, 2 = single rows
