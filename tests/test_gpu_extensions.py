@@ -61,6 +61,39 @@ def test_modify_flags_and_degenerate_rows():
     assert out.token[2].item() == -1 and (out.token.cpu().numpy()[[0, 1, 3]] == ref.token[[0, 1, 3]]).all()
 
 
+@pytest.mark.parametrize("V,dtype,shift", [(701, "fp32", 0), (40001, "bf16", 1), (40000, "fp32", 3), (151937, "bf16", 0)])
+def test_modify_flags_on_rows_that_start_anywhere(V, dtype, shift):
+    """Among them NaN and +inf in the first and the last entry of a tensor, which no copy brings."""
+    B = 7
+    cfg = workloads.VerifyConfig("modany", B=B, K=1, gamma=1, V=V, dtype=dtype, alpha=0.8, seed=V)
+    zq, zp = _position_rows(cfg)
+
+    def moved(t):
+        return torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape).copy_(t)
+    zq, zp = moved(zq), moved(zp)
+    zq[0, 0] = float("nan")
+    zp[1, V // 2] = float("inf")
+    zp[2] = zq[2]                          # p == q and b >= a: no residual mass, the draw comes from q
+    zq[3, V // 2:] = float("-inf")         # a masked half
+    zq[4] = float("-inf")                  # no finite entry
+    zp[B - 1, V - 1] = float("inf")
+    g = torch.Generator().manual_seed(V)
+    la = -2.0 * torch.rand(B, dtype=torch.float64, generator=g)
+    lb = la - 0.4
+    lb[2] = la[2] + 0.5
+    u = torch.rand(B, generator=g)
+    out = binding.sgbv_modify(zq, zp, la.cuda(), lb.cuda(), u.cuda(), 3, 0.9)
+    ref = oracle.modify(zq.float().cpu().numpy(), zp.float().cpu().numpy(), la.numpy(), lb.numpy(), u.numpy(), 3, 0.9)
+    assert binding.last_main_kernel() == "fused_chain_kernel"
+    st, tok = out.status.cpu().numpy(), out.token.cpu().numpy()
+    bad = binding.STATUS_NONFINITE_LOGIT
+    assert st.tolist() == [bad, bad, binding.STATUS_DEGENERATE_RESIDUAL, 0, bad, 0, bad] and (st == ref.status).all()
+    assert (tok[[0, 1, 4, 6]] == -1).all() and out.log_a[[0, 1, 4, 6]].isnan().all()
+    for b in (2, 3, 5):
+        assert tok[b] == ref.token[b] or ref.margin[b] < 1e-6
+    np.testing.assert_allclose(out.resmass.cpu().numpy()[[3, 5]], ref.R[[3, 5]], rtol=1e-5, atol=1e-9)
+
+
 def test_modify_over_several_positions_follows_the_oracle_chain():
     """A few positions in a row, the carried logs fed back (in place), as a decode loop would do."""
     B, V, K, T = 6, 12000, 3, 0.9
