@@ -2,34 +2,35 @@
 // CTA of 32 warps per SM, the row resident in TENSOR MEMORY between the two sweeps.
 //
 // For every position i = 0..gamma-1 of the chain the cluster
-//   * streams the target row and the draft row from HBM exactly once.  CTA r of the cluster owns a
-//     contiguous slice of the vocabulary, warp w of the CTA the 256-entry cells  w, w+32, w+64, w+96
-//     of that slice.  Every warp runs its own little ring of bulk asynchronous copies
-//     (cp.async.bulk + mbarrier transaction counts; one cell of both tensors per slot): the warp that
-//     consumes a slot refills it itself, so the load path needs no block-wide synchronisation and
-//     runs ahead across rows and chains;
-//   * first sweep: a thread takes 8 (target, draft) pairs of a cell, turns them into exponentials
-//     relative to its own maxima of that cell (the maximum maps to exactly 1) and parks them in
-//     tensor memory (tcgen05.st; each warp owns 64 of the 512 columns of its lane quarter, 256 KB per
-//     SM in all = 32,768 pairs), keeping only the cell's maximum and sum in registers;
-//   * exchanges (max, sum-exp) partials in two levels: the warps of a CTA leave theirs in shared
-//     memory and the last one to arrive combines them and PUSHES one partial per CTA into every
-//     CTA's shared memory with asynchronous distributed-shared-memory stores that complete on the
-//     receiver's mbarrier; a warp goes on as soon as all CTA partials of the row have landed.
-//     There is no block-wide or cluster-wide barrier inside the row loop;
-//   * second sweep: reads the exponentials back from tensor memory (tcgen05.ld) and writes one
-//     partial sum of the coupling terms per cell.  Shared memory is never read twice and the
-//     registers hold no row data between the sweeps, which is what lets 32 warps share the SM.
-// The joint likelihood ratio c_i = p(x^i)/q(x^i) is carried as a running product by one thread per
-// CTA, which computes c_{i+1} right after the statistics of row i and arms the next row's exchange
-// with it, a whole row before it is needed.  The finishing kernel (weights, scan, extra token)
-// consumes the cell sums.
+//   * streams the target row and the draft row from HBM exactly once.  CTA r of the cluster owns a contiguous slice of the
+//     vocabulary, each of its warps one to four 256-entry cells of it.  Every warp runs its own little ring of asynchronous copies
+//     (one cell of both tensors per slot): the warp that consumes a slot refills it itself, so the load path needs no block-wide
+//     synchronisation and runs ahead across rows and chains;
+//   * first sweep: a thread takes 8 (target, draft) pairs of a cell, turns them into exponentials relative to its warp's reference
+//     and parks them in tensor memory (tcgen05.st; each warp owns 64 of the 512 columns of its lane quarter, 256 KB per SM in all =
+//     32,768 pairs) or, every fifth cell, in shared memory; only their sum stays in registers;
+//   * exchanges (reference, sum-exp) partials in two levels: the warps of a CTA leave theirs in shared memory, and the last warp,
+//     which has no cells unless there are more than the others can hold, combines them and PUSHES one partial per CTA into
+//     every CTA's shared memory with asynchronous distributed-shared-memory stores that complete on the receiver's
+//     mbarrier.  The other warps meanwhile sweep the row before for the last time and the row behind for the first;
+//   * second sweep: reads the exponentials back and writes one partial sum of the coupling terms per cell.  Shared memory holds
+//     a copied cell once and the registers no row data between the sweeps, which is what lets 32 warps share the SM.
+// The joint likelihood ratio c_i = p(x^i)/q(x^i) is carried as a running product by the last warp, which works c_{i+1} out
+// right after the release of row i.  The finishing kernel (weights, scan, extra token) consumes the cell sums.
+//
+// What bounds it: the special-function unit (3.1 of its instructions per pair, 62 % of its rate at 16 x 8 x 8 x 151936 float32) and
+// the exchange, during which most of the SM waits; up to there float32 rows, HBM.  Steps, us, before / now (one B200, streaming
+// kernel and the kernels behind it): 64 x 8 x 8 x 151936 float32 1087 / 818, 256 x 8 x 4 x 32000 float32 396 / 360,
+// 32 x 4 x 5 x 128256 bfloat16 169 / 128, 256 x 1 x 4 x 32000 float32 81 / 70.  Warp instructions per 32 pairs 34 / 25.6.
 //
 // Every wait on an mbarrier or on a word in global memory is bounded; on expiry the warp records
 // an error flag and keeps executing the protocol, so a lost copy cannot hang the kernel, and the
 // tensor memory is released on every path.
+#include <float.h>
+
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "sgbv_cluster.cuh"
 #include "sgbv_common.cuh"
@@ -47,8 +48,9 @@ constexpr int kCtaCells = 128 / kCtasPerSm;  // cells of a row per CTA: 16 tenso
                                            // lane quarters, 512 columns per SM: 128 cells = 32,768 entries per SM
 constexpr int kSlack = 16;  // extra bytes per cell and tensor in a slot when rows start anywhere: a copy then begins at the
                            // 16-byte boundary before the cell and ends behind it
+constexpr int kParkBytes = kCell * 2 * (int)sizeof(float);  // the exponentials of one cell of both tensors, a warp's parked first cell
 constexpr int kTmemCols = 512 / kCtasPerSm;  // this CTA's share of the SM's tensor memory
-constexpr int kMaxCluster = 8 * kCtasPerSm;  // CTAs per cluster (beyond 8 the size is not portable, which sm_100 allows)
+constexpr int kMaxCluster = 8;  // CTAs per cluster (beyond 8 the size is not portable, which sm_100 allows)
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about one second of SM clock
 constexpr uint32_t kPollNs = 100u;                    // sleep between two tests of a barrier that is not ready
 static_assert(kTile == 256, "the fused path writes one partial sum per 256-element cell");
@@ -66,6 +68,7 @@ struct FusedParams {
     int *error_flag;  // set to 1 if a bounded wait expired
     long long poll_limit;  // cycles a poll of a published ratio may take (row walk)
     int withhold;     // failure-detection test: the first row of every chain does not publish its ratio
+    float rise;       // kRise in units of logits
     int aux_here;     // rows with c < 1 get their two extra sums in this kernel (else: the kernels that follow it)
 };
 
@@ -143,6 +146,28 @@ __device__ __forceinline__ float rcp(float x) {
     return y;
 }
 
+// 2^x without a flush to 0 below 2^-126.
+__device__ __forceinline__ float ex2_wide(float x) {
+    float y;
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// x y clamped to [0, 1]; NaN gives 0.
+__device__ __forceinline__ float mul_sat(float x, float y) {
+    float r;
+    asm("mul.ftz.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+    return r;
+}
+// This thread's asynchronous copies of 16 bytes, in groups that complete in order.
+template <int kDst, int kSrc>
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global.L2::128B [%0 + %2], [%1 + %3], 16;" ::"r"(dst), "l"(src), "n"(kDst), "n"(kSrc) : "memory");
+}
+__device__ __forceinline__ void copy_group_end() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// Waits until at most N of this thread's groups are under way.
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 // ---- tensor memory --------------------------------------------------------------------------------
 // One warp allocates all columns for the CTA (the address lands in shared memory), every warp then
 // reads and writes only the lanes of its own quarter (warp index mod 4) and its own columns.
@@ -191,7 +216,7 @@ struct Control {
     // row parity, of every CTA of the cluster (pushed by their owners)
     float4 wslots[kMaxWarps];
     float4 slots[2][kMaxCluster];
-    float4 low[2][kMaxCluster];          // rows that start anywhere: what the sums in `slots` were rounded by (y, w)
+    float4 low[2][kMaxCluster];          // what the sums in `slots` were rounded by (y, w)
     float4 rs;                           // the row's scalars for the second sweep: rq, rp, kappa, c
     uint32_t tmem_base;                  // address of the allocated tensor memory
 };
@@ -295,16 +320,42 @@ __device__ __forceinline__ void warp_sum_multi(float (&v)[P], int lane) {
     for (; off > 0; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
 }
 
-// What the second sweep needs of a row from this thread's point of view.
+// Exponentials are relative to ONE logit per warp and tensor of a row, its reference: the maximum of the warp's first cell.  The
+// warp's later cells may reach kRise above it, in units of log2; a logit beyond that becomes the reference from there on (the cells
+// before it keep theirs, see FirstSweep::moved): a few warps per row.  So what carries most of a row's mass is a reference or
+// within 2^kRise of one, the largest entry of a point-mass row maps to exactly 1, and every factor between units is the same for the
+// whole warp.  References per thread and cell, as before, took three exponentials and some 25 instructions per cell.
+constexpr float kRise = 6.0f;
+
+// What the second sweep needs of a row, in units of this warp's references.
 struct RowScalars {
-    float Fq;     // moves sums in units of this thread's row maximum of zq to row-max units (0: the thread saw no finite zq)
-    float KF;     // kappa * Fp / Fq: with the cell's factor ratio it makes c p(x)/q(x) = kt * ep/eq
-    float kFp;    // kappa * Fp (cells whose target share underflows)
+    float Fq;     // moves sums to units of the row's reference
+    float KF;     // kappa * Fp / Fq: c p(x)/q(x) = KF * ep/eq
+    float kFp;    // kappa * Fp (rows with c < 1: where the warp's target share underflows)
     float c;      // c_i
 };
+// What a warp keeps of the row whose first sweep runs.
+struct FirstSweep {
+    float bq, bp;    // references (-FLT_MAX: no finite logit so far, and -inf against it still gives 0)
+    float2 sq, sp;   // this thread's sums of exponentials
+    int moved;       // 0, or the first cell whose references are not in shared memory: references have moved, and the cells before
+                     // it keep theirs
+};
+
+// f(Int<0>()), ..., f(Int<N - 1>()), N <= 4: an unrolled loop whose index is a constant expression.
+template <int I>
+using Int = std::integral_constant<int, I>;
+template <int N, typename F>
+__device__ __forceinline__ void for_each_cell(F f) {
+    f(Int<0>());
+    if constexpr (N > 1) f(Int<1>());
+    if constexpr (N > 2) f(Int<2>());
+    if constexpr (N > 3) f(Int<3>());
+    static_assert(N <= 4, "cells per warp");
+}
 
 __device__ __forceinline__ void cell_maxima(const float2 (&eq)[4], const float2 (&ep)[4], float &m1, float &m2) {
-    m1 = m2 = -INFINITY;
+    m1 = m2 = -FLT_MAX;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         m1 = max3(m1, eq[e].x, eq[e].y);
@@ -347,79 +398,108 @@ __device__ __forceinline__ void first_sweep_direct(const unsigned char *q, const
     }
     cell_maxima(eq, ep, m1, m2);
 }
-// Second half: exponentials relative to the thread's own maxima of the cell (0 if it saw only -inf; the maximum
-// itself maps to exactly 1, so point-mass rows stay exact) into tensor memory, and their sums.
-__device__ __forceinline__ void first_sweep_store(uint32_t taddr_cell, float scale, float2 (&eq)[4], float2 (&ep)[4], float m1,
-                                                  float m2, float &s1, float &s2) {
-    const float bq = (m1 > -INFINITY) ? m1 : 0.0f;
-    const float bp = (m2 > -INFINITY) ? m2 : 0.0f;
-    const float2 nbq = splat(-bq), nbp = splat(-bp), sc2 = splat(scale);
-    float2 sq2 = splat(0.0f), sp2 = splat(0.0f);
+// Before the exponentials of cell j: the warp's references.  m1, m2: this thread's maxima of the cell; refs: the warp's words in
+// shared memory, one pair per cell.
+__device__ __forceinline__ void set_references(FirstSweep &f, int j, float m1, float m2, float scale, float rise, float2 *refs) {
+    if (j == 0) {
+        f.bq = warp_max_redux(m1);
+        f.bp = warp_max_redux(m2);
+        return;
+    }
+    if (!__any_sync(0xffffffffu, m1 > f.bq + rise || m2 > f.bp + rise)) return;
+    if ((threadIdx.x & 31) == 0)
+        for (int i = f.moved; i < j; ++i) refs[i] = make_float2(f.bq, f.bp);
+    f.moved = j;
+    auto raise = [&](float m, float &b, float2 &sum) {
+        m = warp_max_redux(m);
+        if (!(m > b + rise)) return;
+        const float move = ex2((b - m) * scale);
+        sum.x *= move;
+        sum.y *= move;
+        b = m;
+    };
+    raise(m1, f.bq, f.sq);
+    raise(m2, f.bp, f.sp);
+}
+// Second half: the exponentials into tensor memory, or into shared memory (parked), and their sums.
+__device__ __forceinline__ void first_sweep_store(uint32_t taddr_cell, bool parked, float4 *park, float scale, float2 (&eq)[4], float2 (&ep)[4], FirstSweep &f) {
+    const float2 nbq = splat(-f.bq), nbp = splat(-f.bp), sc2 = splat(scale);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const float2 aq = __fmul2_rn(__fadd2_rn(eq[e], nbq), sc2);
         const float2 ap = __fmul2_rn(__fadd2_rn(ep[e], nbp), sc2);
         eq[e] = make_float2(ex2(aq.x), ex2(aq.y));
         ep[e] = make_float2(ex2(ap.x), ex2(ap.y));
-        sq2 = __fadd2_rn(sq2, eq[e]);
-        sp2 = __fadd2_rn(sp2, ep[e]);
+        f.sq = __fadd2_rn(f.sq, eq[e]);
+        f.sp = __fadd2_rn(f.sp, ep[e]);
     }
-    tmem_st_cell(taddr_cell, eq, ep);
-    s1 = sq2.x + sq2.y;
-    s2 = sp2.x + sp2.y;
+    if (parked) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            park[32 * e] = make_float4(eq[2 * e].x, eq[2 * e].y, eq[2 * e + 1].x, eq[2 * e + 1].y);
+            park[32 * e + 64] = make_float4(ep[2 * e].x, ep[2 * e].y, ep[2 * e + 1].x, ep[2 * e + 1].y);
+        }
+    } else {
+        tmem_st_cell(taddr_cell, eq, ep);
+    }
 }
 
-// Second sweep of one cell, read back from tensor memory, two vocabulary entries per instruction (f32x2).
-// eq/ep are exponentials relative to the THREAD's maxima of the cell; fmq moves the cell's target units to the
-// thread's row units, rt is the ratio of the cell's draft and target factors, so that fq = fmq Fq and
-// kt = KF rt.  Returns in row-max units
+// Second sweep of one cell, read back from tensor memory (or shared memory: parked), two vocabulary entries per instruction (f32x2).
+// eq/ep are exponentials relative to the warp's references; with kt = KF c p(x)/q(x) = kt ep/eq.  Returns this thread's sums
 //   w  = sum eq (1 - min{kt ep/eq, 1})^K                    (Eq. 4's weights, Eq. 2's sum)
 //   sd = sum max(kt ep - eq, 0)                             (c < 1 only)
 //   sm = sum eq (c - t)^2 Q(t)                              (c < 1 only)
-// coef: Horner coefficients of Q, (t+1) (1-c)^t, t = 1..K-2.  fmp_stash: this thread's draft factor of the cell
-// in shared memory, read only when its target share underflows in a row with c < 1.
+// tiny: the warp's share of the target row underflows (or nearly so, which would overflow kt): its q is 0 in row units, its weights
+// vanish, and max(c p - q, 0) = c p, in units of the draft (kAux; without the extra sums nothing needs doing: whatever kt is, the
+// clamp below leaves a weight in [0, eq]).
 template <int KT, bool kAux>
-__device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, float fmq, float rt, const RowScalars &rs, int K,
-                                                  const float2 *coef, const float *fmp_stash, float &w, float &sd_out,
+__device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, bool parked, const float4 *park, float kt, float c, bool tiny, int K, float &w, float &sd_out,
                                                   float &sm_out) {
     float2 eq[4], ep[4];
-    tmem_ld_cell(taddr_cell, eq, ep);
-    // thread units -> row units
-    float scale_w = fmq * rs.Fq, scale_d = scale_w;
-    float kt = rs.KF * rt;
-    const float v1 = 1.0f - rs.c;
+    const float v1 = 1.0f - c;
     const float2 nv1 = splat(-v1);
-    tmem_wait_ld(eq, ep);
-    if (kAux) {
-        // A thread whose share of the target row underflows (or nearly so, which would overflow kt): its q
-        // is 0 in row units, its weights vanish, and max(c p - q, 0) = c p.  Without the extra sums nothing
-        // needs doing: an infinite or NaN kt gives a zero weight through the clamps below.
-        const bool tiny = !(scale_w > 1e-30f);
-        if (__any_sync(0xffffffffu, tiny)) {
-            if (tiny) {
+    if (parked) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) eq[e] = splat(0.0f);
-                kt = 1.0f;
-                scale_w = 0.0f;
-                scale_d = rs.kFp * *fmp_stash;
-            }
+        for (int e = 0; e < 2; ++e) {
+            const float4 a = park[32 * e], b = park[32 * e + 64];
+            eq[2 * e] = make_float2(a.x, a.y);
+            eq[2 * e + 1] = make_float2(a.z, a.w);
+            ep[2 * e] = make_float2(b.x, b.y);
+            ep[2 * e + 1] = make_float2(b.z, b.w);
+        }
+    } else {
+        tmem_ld_cell(taddr_cell, eq, ep);
+        tmem_wait_ld(eq, ep);
+    }
+    if (kAux) {
+        if (tiny) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) eq[e] = splat(0.0f);
+            kt = 1.0f;
         }
     }
     const float2 nkt = splat(-kt);
+    float coef[KT > 2 ? KT - 2 : 1];  // Horner coefficients of Q, (t+1) (1-c)^t, t = 1..K-2
+    if (kAux && KT > 2) {
+        float vj = 1.0f;
+#pragma unroll
+        for (int t = 1; t <= KT - 2; ++t) {
+            vj *= v1;
+            coef[t - 1] = (float)(t + 1) * vj;
+        }
+    }
     float2 sw = splat(0.0f), sd = splat(0.0f), sm = splat(0.0f);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const float2 q = eq[e];
         const float2 diff = __ffma2_rn(nkt, ep[e], q);  // q - c p, thread units
-        const float2 pos = make_float2(fmaxf(diff.x, 0.0f), fmaxf(diff.y, 0.0f));
         if (KT == 1) {  // one draft: Q = 0, the second extra sum vanishes and nothing needs the ratio
-            sw = __fadd2_rn(sw, pos);
+            sw = __fadd2_rn(sw, make_float2(fmaxf(diff.x, 0.0f), fmaxf(diff.y, 0.0f)));
             if (kAux) sd = __fadd2_rn(sd, make_float2(fmaxf(-diff.x, 0.0f), fmaxf(-diff.y, 0.0f)));
             continue;
         }
-        // r = 1 - min{c p/q, 1}; q = 0 gives -inf or NaN before the clamp, 0 after it
-        const float2 t = __fmul2_rn(diff, make_float2(rcp(q.x), rcp(q.y)));
-        const float2 r = make_float2(fmaxf(t.x, 0.0f), fmaxf(t.y, 0.0f));
+        // r = 1 - min{c p/q, 1}; q = 0 gives -inf or NaN before the clamp to [0, 1], 0 after it
+        const float2 r = make_float2(mul_sat(diff.x, rcp(q.x)), mul_sat(diff.y, rcp(q.y)));
         if (KT != 1) sw = __ffma2_rn(q, ipow2<KT>(r, K), sw);
         if (kAux) {
             sd = __fadd2_rn(sd, make_float2(fmaxf(-diff.x, 0.0f), fmaxf(-diff.y, 0.0f)));
@@ -428,7 +508,7 @@ __device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, float fmq
                 if (KT >= 2) {
                     acc = splat(1.0f);
 #pragma unroll
-                    for (int u = 0; u < KT - 2; ++u) acc = __ffma2_rn(acc, r, coef[u]);
+                    for (int u = 0; u < KT - 2; ++u) acc = __ffma2_rn(acc, r, splat(coef[u]));
                 }
             } else if (K >= 2) {
                 acc = splat(1.0f);
@@ -442,31 +522,47 @@ __device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, float fmq
             sm = __ffma2_rn(__fmul2_rn(q, __fmul2_rn(ct, ct)), acc, sm);
         }
     }
-    w = (sw.x + sw.y) * scale_w;
+    w = sw.x + sw.y;
     if (kAux) {
-        sd_out = (sd.x + sd.y) * scale_d;
-        sm_out = (sm.x + sm.y) * scale_w;
+        sd_out = sd.x + sd.y;
+        sm_out = sm.x + sm.y;
     }
 }
 
-template <bool kWide>
-struct Sum {
-    typedef float type;
-};
-template <>
-struct Sum<true> {
-    typedef double type;
-};
 // 2^((m - row) scale), m <= row: the factor that moves a sum from units of the maximum m to units of the row's, in float64.
 __device__ __forceinline__ double unit_factor(float m, float row, float scale) {
     // e^(f ln 2), |f| <= 1/2, by its Taylor series to degree 11 (remainder below 7e-15), in pairs and without a branch: behind
     // exp2_short's the lanes ran apart and the shuffles of the sums took 1.1 us more per row
-    const double x = fmax(((double)m - (double)row) * (double)scale, -1000.0);
-    const double n = rint(x), t = (x - n) * 0.6931471805599453094, t2 = t * t, t4 = t2 * t2;
+    // (the nearest integer by an addition that leaves no room for a fraction: it also stands in the low word then)
+    const double x = fmax(((double)m - (double)row) * (double)scale, -1000.0), y = x + 6755399441055744.0;
+    const double t = (x - (y - 6755399441055744.0)) * 0.6931471805599453094, t2 = t * t, t4 = t2 * t2;
     const double c0 = 1.0 + t, c1 = fma(t, 1.0 / 6.0, 0.5), c2 = fma(t, 1.0 / 120.0, 1.0 / 24.0), c3 = fma(t, 1.0 / 5040.0, 1.0 / 720.0);
     const double c4 = fma(t, 1.0 / 362880.0, 1.0 / 40320.0), c5 = fma(t, 1.0 / 39916800.0, 1.0 / 3628800.0);
     const double lo = fma(t2, c1, c0), mid = fma(t2, c3, c2), hi = fma(t2, c5, c4);
-    return fma(t4, fma(t4, hi, mid), lo) * __longlong_as_double((long long)((int)n + 1023) << 52);
+    return fma(t4, fma(t4, hi, mid), lo) * __hiloint2double((__double2loint(y) + 1023) << 20, 0);
+}
+// The same in float32: the difference and the product with what they were rounded by, so that what is left is the error of
+// ex2.approx, 2^-22, in factors other than 1.
+__device__ __forceinline__ float unit_factor_f32(float m, float row, float scale) {
+    const float d = row - m, lost = (row - d) - m, x = d * -scale;
+    const float f = ex2(x);
+    return f > 0.0f ? fmaf(f, (fmaf(d, -scale, -x) - lost * scale) * 0.69314718f, f) : 0.0f;  // (0 x inf where m is -FLT_MAX)
+}
+// Sum over the warp of values in [0, 2^17), rounded to multiples of 2^-28 (of 32 multiples each, which add up exactly): the parts above
+// and below 2^-5 as integers.  NaN if a lane's value is not in the range.
+__device__ __forceinline__ double warp_sum_fixed(float v) {
+    const float hi0 = 1.5f * 262144.0f, lo0 = 1.5f / 32.0f;  // an addition to these leaves the integer in the low bits
+    const float hi = v + hi0, lo = (v - (hi - hi0)) + lo0;
+    const int h = __reduce_add_sync(0xffffffffu, __float_as_int(hi) - __float_as_int(hi0));
+    const int l = __reduce_add_sync(0xffffffffu, __float_as_int(lo) - __float_as_int(lo0));
+    const double sum = fma((double)h, 1.0 / 32.0, (double)l * (1.0 / 268435456.0));
+    return __any_sync(0xffffffffu, !(v < 131072.0f)) ? (double)NAN : sum;
+}
+// 1/x for x in the range of normal float32 numbers: the hardware's float32 reciprocal and one step of Newton's method (relative
+// error below 2e-14).  NaN for 0 and inf.
+__device__ __forceinline__ double reciprocal(double x) {
+    const double r = (double)rcp((float)x);
+    return fma(r, fma(-x, r, 1.0), r);
 }
 
 // kAny: rows that do not all start on 16-byte boundaries (odd vocabularies, unaligned buffers).  A copy then brings the
@@ -475,7 +571,7 @@ __device__ __forceinline__ double unit_factor(float m, float row, float scale) {
 // Two sweeps over such rows (three scalar reads of every logit, four kernels) take longer, unless the rows are short and many
 // (fused_outrun): 16 prompts, K = 4, gamma = 4, V = 50257 bfloat16 105 us against 63 here, one prompt at V = 32001 float32 68 and 20,
 // 64 prompts, K = 2 at V = 128255 float32 510 and 200.
-// Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4.
+// Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4, and mbarriers for its copies.
 // W warps per CTA; NS ring slots per warp (the cells per warp and row, kCtaCells / W, are a multiple of it, so
 // that cell j of a row always sits in slot j % NS); KT: the number of drafts K when it has a specialised
 // second sweep (1, 2, 3, 4, 8), else 0 (any K, loops).
@@ -494,30 +590,47 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     constexpr int kHalfBytes = kCell * (int)sizeof(T);  // one tensor's cell
     constexpr int kHalfSlot = kHalfBytes + (kAny ? kSlack : 0);
     constexpr int kSlotBytes = 2 * kHalfSlot;           // the cell of zq, then the same cell of zp
-    constexpr int kStrideBytes = kFWarps * kHalfBytes;  // from one cell of a warp to its next, in a row
+    constexpr int kStride = kAny ? kFWarps : 1;  // from one cell of a warp to its next, in a row
     constexpr int kRingBytes = kFWarps * NS * kSlotBytes;
-    // [rings][full barriers][draft factors of every thread's cells][Control]
+    // [rings][full barriers][references of the cells][parked first cells][Control]
     const unsigned char *ring = smem + (size_t)warp * NS * kSlotBytes;
     const uint32_t ring_u32 = smem_u32(ring);
+    uint32_t pieces_u32 = ring_u32 + (uint32_t)lane * 16u;
     const uint32_t full_u32 = smem_u32(smem) + (uint32_t)(kRingBytes + warp * NS * 8);
-    float *fmp_stash = reinterpret_cast<float *>(smem + kRingBytes + kFWarps * NS * 8) + tid;  // [cell][thread]
-    Control *ctl = reinterpret_cast<Control *>(smem + kRingBytes + kFWarps * NS * 8 + kCellsPerWarp * kFThreads * 4);
+    float2 *refs = reinterpret_cast<float2 *>(smem + kRingBytes + kFWarps * NS * 8) + warp * kCellsPerWarp;
+    float4 *park = reinterpret_cast<float4 *>(smem + kRingBytes + kFWarps * NS * 8 + kCtaCells * (int)sizeof(float2)) + warp * 128 + lane;  // stride 32
+    Control *ctl = reinterpret_cast<Control *>(smem + kRingBytes + kFWarps * NS * 8 + kCtaCells * (int)sizeof(float2) + kFWarps * kParkBytes);
     const uint32_t xbar_u32 = smem_u32(&ctl->xbar[0]);
 
-    // this CTA's slice of the vocabulary, and this warp's cells in it: warp, warp + W, ...
+    // This CTA's slice of the vocabulary, and this warp's cells in it: a few neighbours each.  The last warp, which does the exchange
+    // of every row, only has those that the others cannot hold (with its share of the cells it kept the whole CTA waiting).
     const int cell_begin = rank * p.slice_cells;
     const int ncells_cta = max(0, min(s.ntiles, cell_begin + p.slice_cells) - cell_begin);
-    const int ncw = ncells_cta > warp ? (ncells_cta - warp + kFWarps - 1) / kFWarps : 0;  // cells of this warp per row
-    const int first_cell = cell_begin + warp;
+    // (In the row walk, where one row is all that most clusters have, the cells are shared out evenly.)
+    const int most = kRow ? (ncells_cta + kFWarps - 1) / kFWarps : kCellsPerWarp;
+    const int rest = max(0, ncells_cta - most * (kFWarps - 1));  // of the last warp
+    const int each = (ncells_cta - rest) / (kFWarps - 1), more_by_one = (ncells_cta - rest) % (kFWarps - 1);
+    // (rows that start anywhere: cells w, w + 32, ... of the slice for warp w; of the last warp's, those that fit go one each to
+    // the first warps that would have one cell fewer than others)
+    const int columns = ncells_cta / kFWarps, odd = ncells_cta % kFWarps, given = odd > 0 ? min(columns, kFWarps - 1 - odd) : 0;
+    const int own_cells = columns + (warp < odd), extra = kAny && warp >= odd && warp < odd + given ? warp - odd : -1;
+    int ncw = !kAny ? (warp == kFWarps - 1 ? rest : each + (warp < more_by_one))  // cells of this warp per row
+                    : warp == kFWarps - 1 ? columns - given : own_cells + (extra >= 0);
+    const int first_cell = cell_begin + (kAny ? (warp == kFWarps - 1 ? warp + given * kFWarps : warp) : warp == kFWarps - 1 ? ncells_cta - rest : warp * each + min(warp, more_by_one));
+    // cell j of this warp, counted from its first one
+    const int extra_j = extra >= 0 ? own_cells : -1, extra_at = kFWarps - 1 + extra * kFWarps - warp;
+    auto cell_at = [&](int j) { return kAny && j == extra_j ? extra_at : j * kStride; };
     // the row's last cell may be a partial one: which of this warp's cells it is (-1: none), and its entries
     const int tail_valid = s.V - (s.ntiles - 1) * kCell;
-    const int tail_j = (tail_valid < kCell && ncw > 0 && first_cell + (ncw - 1) * kFWarps == s.ntiles - 1) ? ncw - 1 : -1;
+    int tail_j = -1;
+    for (int j = 0; j < ncw; ++j)
+        if (tail_valid < kCell && first_cell + cell_at(j) == s.ntiles - 1) tail_j = j;
 
     if (tid == 0) {
         mbar_init(xbar_u32, 1);
         mbar_init(xbar_u32 + 8, 1);
     }
-    if (lane == 0)
+    if (kAny && lane == 0)
         for (int k = 0; k < NS; ++k) mbar_init(full_u32 + 8 * k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncwarp();
@@ -564,62 +677,63 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     const int chain_hi = (int)(range_hi / s.gamma), off_hi = (int)(range_hi % s.gamma);
     const int chain_mid = chain_lo + (off_lo > 0 ? 1 : 0);  // first whole chain of the range
     const int nrows = row_mode ? (int)((total_rows - cid + G - 1) / G) : (int)(range_hi - range_lo);  // rows this cluster walks
-    // the row after (bk, i) in this cluster's walk
-    auto walk_next = [&](int &bk, int &i) {
+    // The first row of the walk: its number in the list and its place in its chain; seg_end: where its segment ends
+    // (a range of gamma rows or more has a head or a whole chain)
+    int r_b = row_mode ? cid : (off_hi > 0 ? chain_hi : chain_mid) * s.gamma;
+    int i_b = row_mode ? cid % s.gamma : 0;
+    int seg_end = row_mode ? 0 : off_hi > 0 ? r_b + off_hi : chain_hi * s.gamma;
+    // From row (r, i) to the row after it in the walk.  Returns the number of chains between them.
+    auto walk_next = [&](int &r, int &i) {
         if (row_mode) {
-            bk += G / s.gamma;
-            i += G % s.gamma;
-            if (i >= s.gamma) {
-                i -= s.gamma;
-                ++bk;
-            }
-            return;
+            const int from = r / s.gamma;
+            r += G;
+            i = r % s.gamma;
+            return r / s.gamma - from;
         }
+        ++r;
         ++i;
-        if (bk == chain_hi) {  // in the head
-            if (i >= off_hi) {
-                if (chain_mid < chain_hi) {
-                    bk = chain_mid;
-                    i = 0;
-                } else {
-                    bk = chain_lo;
-                    i = off_lo;
-                }
-            }
-        } else if (i >= s.gamma && !(bk == chain_lo && off_lo > 0)) {  // a whole chain is done (the tail is the last segment)
-            if (bk + 1 < chain_hi) {
-                ++bk;
+        if (r == seg_end) {
+            const int from = (r - 1) / s.gamma;
+            if (from == chain_hi && chain_mid < chain_hi) {  // from the head to the whole chains
+                r = chain_mid * s.gamma;
                 i = 0;
-            } else {
-                bk = chain_lo;
+                seg_end = chain_hi * s.gamma;
+            } else {  // to the tail
+                r = (int)range_lo;
                 i = off_lo;
+                seg_end = -1;
             }
+            return r / s.gamma - from;
         }
+        if (i < s.gamma) return 0;
+        i = 0;
+        return 1;
     };
-    const uint32_t xbytes = (uint32_t)(C * (kAny ? 2 : 1) * sizeof(float4));  // one partial from every CTA of the cluster
+    const uint32_t xbytes = (uint32_t)(C * 2 * sizeof(float4));  // one partial from every CTA of the cluster
     uint32_t timed_out = 0;
 
     // ---- this warp's copy ring --------------------------------------------------------------------
-    // Cell j of a row lands in slot j % NS.  The warp that has moved a cell from its slot to registers refills
-    // the slot at once with the next cell that maps to it: cell j + NS of the same row, or, past the warp's
-    // last cell, the slot's first cell of the next row of the walk.  So the schedule is fixed at compile time
-    // apart from the number of cells this warp has (ncw); lane 0 starts the copies.  `pending` has bit k set
+    // Cell j of a row lands in slot j % NS.  The warp that has moved a cell from its slot to registers refills the slot at once,
+    // with cell j + NS of the same row or, past the last, of the next row of the walk: the schedule is fixed at compile time.
+    // Rows on 16-byte boundaries: every thread copies the 16-byte pieces that it will read itself (cp.async), one group of copies
+    // per cell, an empty one where the warp has no such cell, and waits for its own groups by their order: no barrier, no
+    // elected lane and hardly any address arithmetic.
+    // kAny: bulk copies on the slot's mbarrier, which may start and end off the cell's boundaries; `pending` has bit k set
     // while a copy into slot k is under way, `phases` bit k is the parity of slot k's barrier.  A warp that has
     // given up on a wait issues no further loads and, before it leaves, waits for those in flight.
     const size_t row_bytes = (size_t)s.V * sizeof(T);
-    const unsigned char *const zq_warp = reinterpret_cast<const unsigned char *>(p.zq) + (size_t)first_cell * kHalfBytes;
-    const unsigned char *const zp_warp = reinterpret_cast<const unsigned char *>(p.zp) + (size_t)first_cell * kHalfBytes;
+    const unsigned char *const zq_begin = reinterpret_cast<const unsigned char *>(p.zq), *const zp_begin = reinterpret_cast<const unsigned char *>(p.zp);
+    const size_t ahead = (size_t)first_cell * kHalfBytes + (kAny ? 0 : lane * 16);  // from the start of a row to this warp's first cell
     const uint32_t is_lane0 = lane == 0 ? 1u : 0u;
     uint32_t pending = 0, phases = 0;
     // kAny: where a copy starts (the 16-byte boundary at or before the cell) and how long it is (a constant for all full
     // cells: always one piece more)
     auto floor16 = [](const unsigned char *a) {
-        return kAny ? reinterpret_cast<const unsigned char *>(reinterpret_cast<uintptr_t>(a) & ~(uintptr_t)15) : a;
+        return reinterpret_cast<const unsigned char *>(reinterpret_cast<uintptr_t>(a) & ~(uintptr_t)15);
     };
     auto rest16 = [](const unsigned char *a) { return (uint32_t)reinterpret_cast<uintptr_t>(a) & 15u; };
     constexpr uint32_t kCopyBytes = (uint32_t)kHalfSlot;
-    const uint32_t tail_bytes = kAny ? (((uint32_t)(tail_valid * (int)sizeof(T)) + 15u) & ~15u) + kSlack : (uint32_t)(tail_valid * (int)sizeof(T));
-    const unsigned char *const zq_begin = reinterpret_cast<const unsigned char *>(p.zq), *const zp_begin = reinterpret_cast<const unsigned char *>(p.zp);
+    const uint32_t tail_bytes = (((uint32_t)(tail_valid * (int)sizeof(T)) + 15u) & ~15u) + kSlack;
     // whether copies of [a, a + bytes) of both tensors would leave them
     auto outside = [&](const unsigned char *q, const unsigned char *pp, size_t bytes) {
         return floor16(q) < zq_begin || floor16(pp) < zp_begin ||
@@ -627,224 +741,388 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                floor16(pp) + bytes > zp_begin + (size_t)p.nchains * s.gamma * row_bytes;
     };
     // rows that may hold such cells (q, pp: this warp's first cells of the row)
-    auto edge_row = [&](const unsigned char *q, const unsigned char *pp) {
-        if (!kAny) return false;
-        const size_t ahead = (size_t)first_cell * kHalfBytes;
-        return outside(q - ahead, pp - ahead, row_bytes + 48);
+    auto edge_row = [&](const unsigned char *q, const unsigned char *pp) { return kAny && outside(q - ahead, pp - ahead, row_bytes + 48); };
+    // cell j of the row whose first cells are q and pp cannot be copied
+    auto direct = [&](const unsigned char *q, const unsigned char *pp, int j, bool edge) {
+        return kAny && edge && outside(q + (size_t)cell_at(j) * kHalfBytes, pp + (size_t)cell_at(j) * kHalfBytes, j == tail_j ? tail_bytes : kCopyBytes);
     };
-#define SGBV_DIRECT(QROW, PROW, JJ, EDGE)                                                                               \
-    (kAny && (EDGE) &&                                                                                                 \
-     outside((QROW) + (size_t)(JJ) * kStrideBytes, (PROW) + (size_t)(JJ) * kStrideBytes, (JJ) == tail_j ? tail_bytes : kCopyBytes))
-#define SGBV_ISSUE(QROW, PROW, JJ, SLOT, EDGE)                                                                          \
-    do {                                                                                                               \
-        if (!SGBV_DIRECT(QROW, PROW, JJ, EDGE)) {                                                                       \
-            issue_cell(ring_u32 + (uint32_t)((SLOT) * kSlotBytes), floor16((QROW) + (size_t)(JJ) * kStrideBytes),       \
-                       floor16((PROW) + (size_t)(JJ) * kStrideBytes), (JJ) == tail_j ? tail_bytes : kCopyBytes,         \
-                       full_u32 + 8u * (uint32_t)(SLOT), is_lane0, kHalfSlot);                                          \
-            pending |= 1u << (SLOT);                                                                                   \
-        }                                                                                                              \
-    } while (0)
-    // First sweep of cell J of the row whose cells start at (QROW, PROW); the slot is refilled from the same row
-    // or, past this warp's last cell, from the row that follows (QNXT, PNXT; only if MORE).
-#define SGBV_FIRST_SWEEP_CELL(J, QROW, PROW, QNXT, PNXT, MORE)                                                          \
-    do {                                                                                                               \
-        const int slot_ = (J) % NS; /* (a constant once the loop is unrolled) */                                       \
-        if (pending & (1u << slot_)) {                                                                                 \
-            mbar_wait(full_u32 + 8u * slot_, (phases >> slot_) & 1u, timed_out);                                       \
-            phases ^= 1u << slot_;                                                                                     \
-            pending ^= 1u << slot_;                                                                                    \
-        }                                                                                                              \
-        float2 eq_[4], ep_[4];                                                                                         \
-        if (SGBV_DIRECT(QROW, PROW, J, edge_b))                                                                        \
-            first_sweep_direct<T>((QROW) + (size_t)(J) * kStrideBytes, (PROW) + (size_t)(J) * kStrideBytes, lane,      \
-                                  (J) == tail_j ? tail_valid : kCell, eq_, ep_, mq[J], mp[J]);                         \
-        else                                                                                                           \
-            first_sweep_fetch<T, kAny>(ring + slot_ * kSlotBytes, rest16(QROW), rest16(PROW), lane, (J) == tail_j,     \
-                                       tail_valid, eq_, ep_, mq[J], mp[J]);                                            \
-        /* every lane holds its share of the slot in registers now: refill it */                                       \
-        __syncwarp();                                                                                                  \
-        if ((J) + NS < ncw) {                                                                                          \
-            if (!timed_out) SGBV_ISSUE(QROW, PROW, (J) + NS, slot_, edge_b);                                           \
-        } else if (MORE) {                                                                                             \
-            SGBV_ISSUE(QNXT, PNXT, slot_, slot_, edge_d);                                                              \
-        }                                                                                                              \
-        first_sweep_store(taddr + 16u * (uint32_t)(J), s.scale, eq_, ep_, mq[J], mp[J], sq[J], sp[J]);                 \
-    } while (0)
+    // Starts the copies of cell j of the row whose first cells are q and pp.  whole: not the partial cell.
+    auto request = [&](const unsigned char *q, const unsigned char *pp, auto cell, bool edge, auto whole) {
+        constexpr bool kWhole = decltype(whole)::value;
+        constexpr int j = decltype(cell)::value, slot = j % NS;
+        if constexpr (kAny) {
+            const unsigned char *qj = q + (size_t)cell_at(j) * kHalfBytes, *pj = pp + (size_t)cell_at(j) * kHalfBytes;
+            if (!direct(q, pp, j, edge)) {
+                issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), floor16(qj), floor16(pj), !kWhole && j == tail_j ? tail_bytes : kCopyBytes,
+                           full_u32 + 8u * (uint32_t)slot, is_lane0, kHalfSlot);
+                pending |= 1u << slot;
+            }
+        } else {
+            auto pieces = [&](auto part) {  // 32 pieces of 16 bytes at a time
+                constexpr int h = decltype(part)::value, to = slot * kSlotBytes + 512 * h, from = j * kHalfBytes + 512 * h;
+                if (!kWhole && j == tail_j && (lane + 32 * h) * (16 / (int)sizeof(T)) >= tail_valid) return;  // past the row's end
+                copy16<to, from>(pieces_u32, q);
+                copy16<to + kHalfSlot, from>(pieces_u32, pp);
+            };
+            pieces(Int<0>());
+            if constexpr (kHalfBytes > 512) pieces(Int<1>());
+        }
+    };
 
-    // rows of the walk: A = the row whose second sweep runs, B = the one after it, whose first sweep runs in the
-    // same loop, D = the one after B, whose cells are requested meanwhile
-    int bk_a = 0, i_a = 0;  // (set when B becomes A)
-    int bk_b = row_mode ? cid / s.gamma : (off_hi > 0 ? chain_hi : chain_mid);  // (a range of gamma rows or more has one of them)
-    int i_b = row_mode ? cid % s.gamma : 0;
-    const unsigned char *q_b = zq_warp + ((size_t)bk_b * s.zq_rows + i_b) * row_bytes;  // this warp's first cell of row B
-    const unsigned char *p_b = zp_warp + ((size_t)bk_b * s.gamma + i_b) * row_bytes;
-    bool edge_b = nrows > 0 && edge_row(q_b, p_b);
-    if (nrows > 0) {
-#pragma unroll
-        for (int k = 0; k < NS; ++k)
-            if (k < ncw) SGBV_ISSUE(q_b, p_b, k, k, edge_b);
-    }
-
-    // The last warp of this CTA combines the partials, carries c_i and fetches the token logits of a row while its
-    // first sweep runs (every lane the same words).
+    // The last warp of this CTA combines the partials, carries c_i and fetches the token logits of a row ahead of its exchange
+    // (every lane the same words).
     const bool combiner = warp == kFWarps - 1;
     // c at the start of chain bk: 1, or exp(log p(s) - log q(s)) of what Algorithm 2 carries in
 #define SGBV_C0(BK) (p.carry_loga ? exp_short(p.carry_logb[BK] - p.carry_loga[BK]) : 1.0)
     double c_carry = 1.0;  // chain walk: c of the row whose exchange comes next (the first row of the walk starts a chain)
-    if (combiner && nrows > 0) c_carry = SGBV_C0(bk_b);
+    if (combiner && nrows > 0) c_carry = SGBV_C0(r_b / s.gamma);
+    // The combining warp: the next row's draft token, fetched a row ahead, and that row's logits of it.
+    int tok_b = combiner && nrows > 0 && p.tok ? __ldg(p.tok + r_b) : 0;
+    float zq_tok = 0.0f, zp_tok = 0.0f;
+    auto prepare_exchange = [&](int pos, int r, int i) {
+        if (C > 1 && lane == 0) mbar_expect_tx(xbar_u32 + 8u * (uint32_t)(pos & 1), xbytes);  // the partials of the cluster's CTAs
+        const int t = tok_b >= 0 && tok_b < s.V ? tok_b : 0;  // (the finishing kernel flags the batch row)
+        zq_tok = ld_logit(reinterpret_cast<const T *>(p.zq) + ((size_t)(r / s.gamma) * s.zq_rows + i) * s.V, t);
+        zp_tok = ld_logit(reinterpret_cast<const T *>(p.zp) + (size_t)r * s.V, t);
+    };
+    // The exchange of row r (position pos of the walk; row nx, at place i_nx of its chain, chains_on chains further, follows if
+    // has_next), by the combining warp.
+    auto exchange = [&](int pos, int r, int i, bool has_next, int nx, int i_nx, int chains_on) {
+        const int par = pos & 1;
+        const uint32_t xph = (uint32_t)(pos >> 1) & 1u;
+        const uint32_t xbar = xbar_u32 + 8u * (uint32_t)par;
+        bar_sync(1, kFThreads);
+        const float4 v = lane < kFWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+        float bq_row = warp_max_redux(v.x), bp_row = warp_max_redux(v.z);
+        float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
+        // The sum over the lanes of z, each moved from units of m to units of `row` (-inf: a lane without a share).  Every cycle from
+        // here to the release is one that most of the SM's warps wait.  Sums and factors in float32 made up half of the error of the
+        // residual masses; all in float64 (rows that start anywhere) took 500 cycles more per level.
+        auto combine = [&](float m, double z, float row) {
+            const double moved = z * unit_factor(m, row, s.scale);
+            return warp_sum(m > -INFINITY ? moved : 0.0);
+        };
+        double Zq, Zp;
+        if constexpr (kAny) {
+            Zq = combine(v.x, v.y, rq_row);
+            Zp = combine(v.z, v.w, rp_row);
+        } else {
+            Zq = warp_sum_fixed(v.x > -INFINITY ? v.y * unit_factor_f32(v.x, rq_row, s.scale) : 0.0f);
+            Zp = warp_sum_fixed(v.z > -INFINITY ? v.w * unit_factor_f32(v.z, rp_row, s.scale) : 0.0f);
+        }
+        if (C > 1) {  // the same once more over the CTAs of the cluster
+            const float4 mine = make_float4(bq_row, (float)Zq, bp_row, (float)Zp);
+            if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, mine);
+            if (lane < C) push_f4(&ctl->low[par][rank], xbar, (uint32_t)lane, make_float4(0.0f, (float)(Zq - (double)mine.y), 0.0f, (float)(Zp - (double)mine.w)));
+            mbar_wait(xbar, xph, timed_out);
+            timed_out = __any_sync(0xffffffffu, timed_out != 0);
+            const float4 cv = lane < C ? ctl->slots[par][lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+            bq_row = warp_max_redux(cv.x);
+            bp_row = warp_max_redux(cv.z);
+            rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f;
+            rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
+            const float4 low = lane < C ? ctl->low[par][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if constexpr (kAny) {
+                Zq = combine(cv.x, (double)cv.y + (double)low.y, rq_row);
+                Zp = combine(cv.z, (double)cv.w + (double)low.w, rp_row);
+            } else {  // (at most eight CTAs)
+                Zq = cv.x > -INFINITY ? ((double)cv.y + (double)low.y) * (double)unit_factor_f32(cv.x, rq_row, s.scale) : 0.0;
+                Zp = cv.z > -INFINITY ? ((double)cv.w + (double)low.w) * (double)unit_factor_f32(cv.z, rp_row, s.scale) : 0.0;
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    Zq += __shfl_xor_sync(0xffffffffu, Zq, o);
+                    Zp += __shfl_xor_sync(0xffffffffu, Zp, o);
+                }
+                Zq = __shfl_sync(0xffffffffu, Zq, 0);
+                Zp = __shfl_sync(0xffffffffu, Zp, 0);
+            }
+        }
+        // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
+        // NEXT row needs it, so it is worked out after the other warps have been released.
+        const double Zratio = Zq * reciprocal(Zp);
+        auto ratio_of_row = [&]() {
+            return exp2_short(((double)zp_tok - (double)rp_row) * (double)s.scale - ((double)zq_tok - (double)rq_row) * (double)s.scale) * Zratio;
+        };
+        double cd;
+        if (row_mode) {
+            const double ratio = ratio_of_row();
+            // Publish this row's ratio for the clusters that walk the later rows of this chain.  The
+            // word itself says "ready": it is preset to a NaN pattern, and a ratio is never stored as
+            // NaN (a row that produces one is flagged invalid anyway).
+            if (lane == 0 && rank == 0 && i + 1 < s.gamma && !(p.withhold && i == 0))
+                *reinterpret_cast<volatile double *>(p.ws.ratio + r) = (ratio != ratio) ? 0.0 : ratio;
+            // c_i = product of the published ratios of rows 0..i-1 of this chain (fixed order: a
+            // butterfly over the lanes).  Those rows are walked by other clusters at about the same
+            // time and publish right after their own statistics, which do not depend on c: no chain of
+            // waits forms.  Every lane polls one of them.  Bounded waits.
+            cd = SGBV_C0(r / s.gamma);
+            const int r0 = r - i;
+            for (int j0 = 0; j0 < i; j0 += 32) {
+                double w = 1.0;
+                if (j0 + lane < i) {
+                    const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.ratio + r0 + j0 + lane);
+                    w = *word;
+                    if (w != w && timed_out) w = 0.0;
+                    if (w != w) {
+                        const long long t0 = clock64();
+                        while ((w = *word) != w) {
+                            if (clock64() - t0 > p.poll_limit) {
+                                timed_out = 1;
+                                w = 0.0;
+                                break;
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) w *= __shfl_xor_sync(0xffffffffu, w, o);
+                cd *= w;
+            }
+            timed_out = __any_sync(0xffffffffu, timed_out != 0);
+        } else {
+            cd = c_carry;  // carried along the chain
+        }
+        const float4 rowv = make_float4(rq_row, rp_row, (float)(cd * Zratio), (float)cd);
+        if (lane == 0) ctl->rs = rowv;
+        __syncwarp();
+        bar_arrive(2, kFThreads);
+        // off the critical path: c of the next row of the chain walk (c_{i+1} = c_i ratio, and 1 at the start of
+        // the next chain), and the row's record for the finishing kernel
+        if (!row_mode) {
+            const double c_next = cd * ratio_of_row();  // c after this row
+            // the head of a chain that another cluster continues: leave c where that cluster looks for it
+            if (r == chain_hi * s.gamma + off_hi - 1 && off_hi > 0 && lane == 0 && rank == 0)
+                *reinterpret_cast<volatile double *>(p.ws.ratio + cid) = (c_next != c_next) ? 0.0 : c_next;
+            if (has_next) {
+                if (i_nx == 0) {
+                    c_carry = SGBV_C0(nx / s.gamma);
+                } else if (chains_on == 0) {
+                    c_carry = c_next;
+                } else {  // the tail of a chain whose head another cluster walked at its very start
+                    const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.ratio + cid - 1);
+                    double w = *word;
+                    if (w != w && !timed_out) {
+                        const long long t0 = clock64();
+                        while ((w = *word) != w)
+                            if (clock64() - t0 > kWaitLimitCycles) {
+                                timed_out = 1;
+                                break;
+                            }
+                    }
+                    c_carry = (w != w) ? 0.0 : w;
+                }
+            }
+        }
+        if (lane == 0 && rank == 0) {
+            // nonfinite logits: NaN poisons Z, +inf shows up as an infinite maximum, a row of
+            // -inf only has Z = 0
+            const bool bad = !(Zq > 0.0f) || !(Zp > 0.0f) || !(Zq < (double)INFINITY) || !(Zp < (double)INFINITY) ||
+                             !(bq_row < INFINITY) || !(bp_row < INFINITY);
+            RowInfo ri;
+            ri.flags = bad ? SGBV_STATUS_NONFINITE_LOGIT : 0;
+            ri.pad_ = 0;
+            ri.Zq = (double)Zq;
+            ri.Zp = (double)Zp;
+            ri.mq = bq_row;
+            ri.mp = bp_row;
+            ri.kappa = rowv.z;
+            ri.c = rowv.w;
+            p.ws.rows[r] = ri;
+        }
+        return rowv;
+    };
+    // Without cells that is all it does.
+    const bool exchange_only = combiner && ncw == 0;
+    if (exchange_only) {
+        if (lane == 0) ctl->wslots[warp] = make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+        __syncwarp();
+        for (int pos = 0, r = r_b, i = i_b; pos < nrows; ++pos) {
+            int nx = r, i_nx = i;
+            const int chains_on = walk_next(nx, i_nx);
+            prepare_exchange(pos, r, i);
+            if (pos + 1 < nrows && p.tok) tok_b = __ldg(p.tok + nx);
+            exchange(pos, r, i, pos + 1 < nrows, nx, i_nx, chains_on);
+            r = nx;
+            i = i_nx;
+        }
+    }
 
-    float fmq[kCellsPerWarp], rt[kCellsPerWarp];  // row A: what the second sweep needs of every cell
-    RowScalars rs;                                 // row A
+    // Rows of the walk: A = the row whose second sweep runs, B = the one after it, whose first sweep runs in the same loop, D = the
+    // one after B, E = the one after D.  A warp's cells take five places in turn, four in tensor memory and one in shared memory: cell j
+    // of the row at position n lies in place (4 n + j) mod 5, so that cell j + 1 of row B goes where cell j of row A has just been
+    // read.  Row B's partial is posted before the last cell of row A has its second sweep and the first cell of row D its first
+    // one: that work runs while row B's partials are exchanged.
+    // this warp's first cells (with cp.async this thread's first pieces) of the row whose cells are requested: the row of a cell
+    // that lies NS cells behind the one that is swept
+    const unsigned char *q_r = zq_begin + ahead + ((size_t)(r_b / s.gamma) * s.zq_rows + i_b) * row_bytes;
+    const unsigned char *p_r = zp_begin + ahead + (size_t)r_b * row_bytes;
+    bool edge_r = nrows > 0 && edge_row(q_r, p_r);
+    const int nwalk = exchange_only ? -1 : nrows;  // rows that this warp sweeps
+    if (nwalk > 0) {
+        for_each_cell<NS>([&](auto cell) {
+            if (cell < ncw) request(q_r, p_r, cell, edge_r, std::false_type());
+            if (!kAny) copy_group_end();
+        });
+    }
+    int r_w = r_b, i_w = i_b, chains_w = 0;  // the row that q_r, p_r go to next, and the chains between it and the one before
+    auto to_next_row = [&]() {
+        const int from = r_w;
+        chains_w = walk_next(r_w, i_w);
+        const int rows = r_w - from;
+        q_r += (long)(rows + chains_w * (s.zq_rows - s.gamma)) * (int)row_bytes;
+        p_r += (long)rows * (int)row_bytes;
+        if (kAny) edge_r = edge_row(q_r, p_r);
+    };
+    FirstSweep f;  // row B, later row D
+    auto fresh_row = [&]() {
+        f.bq = f.bp = -FLT_MAX;
+        f.sq = f.sp = splat(0.0f);
+        f.moved = 0;
+    };
+    // First sweep of a cell of row r (kAny: its remainders and whether it may touch an end of a tensor); the slot is refilled, if
+    // more: the row behind r exists.  steady: more, no partial cell, no end of a tensor.
+    auto first_sweep = [&](auto cell, int place, int r, uint32_t rest_q, uint32_t rest_p, bool edge, bool more, auto steady) {
+        constexpr bool kSteady = decltype(steady)::value;
+        constexpr int j = decltype(cell)::value, slot = j % NS;
+        constexpr bool kSameRow = j + NS < kCellsPerWarp;
+        if constexpr (j + NS == kCellsPerWarp) to_next_row();  // from here on the next row's cells
+        auto refill = [&]() {
+            constexpr int next = (j + NS) % kCellsPerWarp;
+            if (next < ncw && (kSameRow || kSteady || more) && (!kAny || kSteady || !timed_out)) request(q_r, p_r, Int<next>(), edge_r, steady);
+            if (!kAny) copy_group_end();
+        };
+        if (j >= ncw) {
+            refill();
+            return;
+        }
+        float2 eq[4], ep[4];
+        float m1, m2;
+        if constexpr (kAny) {
+            const bool copied = kSteady || (pending & (1u << slot));
+            if (copied) {
+                mbar_wait(full_u32 + 8u * slot, (phases >> slot) & 1u, timed_out);
+                phases ^= 1u << slot;
+                pending &= ~(1u << slot);
+            }
+            if (copied) {
+                first_sweep_fetch<T, kAny>(ring + slot * kSlotBytes, rest_q, rest_p, lane, !kSteady && j == tail_j, tail_valid, eq, ep, m1, m2);
+            } else {
+                const size_t off = ahead + (size_t)cell_at(j) * kHalfBytes;
+                first_sweep_direct<T>(zq_begin + off + (size_t)(r + r / s.gamma * (s.zq_rows - s.gamma)) * row_bytes, zp_begin + off + (size_t)r * row_bytes,
+                                      lane, j == tail_j ? tail_valid : kCell, eq, ep, m1, m2);
+            }
+            __syncwarp();  // every lane holds its share of the slot in registers now
+        } else {
+            copy_wait<NS - 1>();
+            first_sweep_fetch<T, kAny>(ring + slot * kSlotBytes, 0, 0, lane, !kSteady && j == tail_j, tail_valid, eq, ep, m1, m2);
+        }
+        refill();
+        set_references(f, j, m1, m2, s.scale, p.rise, refs);
+        first_sweep_store(taddr + 16u * (uint32_t)place, place == 4, park, s.scale, eq, ep, f);
+    };
+    uint32_t rest_qb = rest16(q_r), rest_pb = rest16(p_r);  // (kAny) row B
+    bool edge_b = edge_r;
+    fresh_row();
+    if (nwalk > 0) first_sweep(Int<0>(), 0, r_b, rest_qb, rest_pb, edge_b, nrows > 1, std::false_type());
+
+    RowScalars rs;         // row A
     rs.Fq = rs.KF = rs.kFp = 0.0f;
     rs.c = 1.0f;
-#pragma unroll
-    for (int j = 0; j < kCellsPerWarp; ++j) fmq[j] = rt[j] = 0.0f;
+    bool moved_a = false;  // row A's cells have references of their own (in this warp)
 
+    int r_a = 0;  // (set when B becomes A)
+    int place = 1;  // of row A's first cell (n = -1: -4 mod 5)
     // n = -1: only the first sweep of row 0; n = nrows - 1: only the second sweep of the last row
-    for (int n = -1; n < nrows; ++n) {
-        const bool has_a = n >= 0, has_b = n + 1 < nrows;
-        // row D, the one after B
-        int bk_d = bk_b, i_d = i_b;
-        walk_next(bk_d, i_d);
-        const bool has_d = n + 2 < nrows;
-        const bool more = has_d && !timed_out;
-        const unsigned char *q_d = zq_warp + ((size_t)bk_d * s.zq_rows + i_d) * row_bytes;
-        const unsigned char *p_d = zp_warp + ((size_t)bk_d * s.gamma + i_d) * row_bytes;
-        const bool edge_d = has_d && edge_row(q_d, p_d);
-        const size_t r_a = (size_t)bk_a * s.gamma + i_a, r_b = (size_t)bk_b * s.gamma + i_b;
-
-        // ---- combining warp: the logits of row B's draft token ------------------------------------------
-        float zq_tok = 0.0f, zp_tok = 0.0f;
-        const int par = (n + 1) & 1;  // of row B's exchange
-        const uint32_t xph = (uint32_t)((n + 1) >> 1) & 1u;
-        const uint32_t xbar = xbar_u32 + 8u * (uint32_t)par;
-        if (combiner && has_b) {
-            if (C > 1 && lane == 0) mbar_expect_tx(xbar, xbytes);  // row B's partials of the cluster's CTAs
-            int t = p.tok ? p.tok[r_b] : 0;
-            if (t < 0 || t >= s.V) t = 0;  // the finishing kernel flags the batch row
-            zq_tok = ld_logit(reinterpret_cast<const T *>(p.zq) + ((size_t)bk_b * s.zq_rows + i_b) * s.V, t);
-            zp_tok = ld_logit(reinterpret_cast<const T *>(p.zp) + r_b * s.V, t);
-        }
+    for (int n = -1; n < nwalk; ++n) {
+        // (what follows from these is worked out where it is needed: hoisted out of the loop it would take more registers than there are)
+        asm volatile("" : "+r"(ncw), "+r"(tail_j), "+r"(pieces_u32));
+        const bool has_a = n >= 0, has_b = n + 1 < nrows, has_d = n + 2 < nrows, has_e = n + 3 < nrows;
+        if (combiner && has_b) prepare_exchange(n + 1, r_b, i_b);
 
         // ---- second sweep of row A from tensor memory, cell by cell, each followed by the first sweep of the
         //      same cell of row B into the columns just read: the exponentials of the one and the sums of the
         //      other keep different pipes busy --------------------------------------------------------------
-        float mq[kCellsPerWarp], mp[kCellsPerWarp], sq[kCellsPerWarp], sp[kCellsPerWarp];  // row B
-        float wsum[kCellsPerWarp];                                                         // row A
+        float wsum[kCellsPerWarp];  // row A; the last one is that of the warp's last cell
 #pragma unroll
-        for (int j = 0; j < kCellsPerWarp; ++j) {
-            mq[j] = mp[j] = -INFINITY;
-            sq[j] = sp[j] = wsum[j] = 0.0f;
-        }
-        float *wp = p.ws.wpart + r_a * s.ntiles + first_cell;
-        // The common case by far has nothing to decide per cell: a warp with all its cells, rows before and after,
-        // no partial cell.  Its loop body is straight-line code.
+        for (int j = 0; j < kCellsPerWarp; ++j) wsum[j] = 0.0f;
+        auto part_of = [&](float *base) { return base + (size_t)r_a * s.ntiles + first_cell; };
         // Rows with c < 1 may need two more sums for Eq. 2.  Small and medium problems work them out here, for all
         // such rows (p.aux_here).  Large ones leave them to two kernels that follow this one and only touch the rows
         // whose plain numerator would cancel, a few per cent: here they slow every row with c < 1, and with it the
         // whole cluster, by more than half, which is worth two more launches only when the step is long.
         const bool aux_row = p.aux_here && rs.c < 1.0f;
-        const bool steady = ncw == kCellsPerWarp && has_a && more && tail_j < 0 && !aux_row && !edge_b && !edge_d;
-        if (steady) {
-#pragma unroll
-            for (int j = 0; j < kCellsPerWarp; ++j) {
-                float unused0, unused1;
-                second_sweep_cell<KT, false>(taddr + 16u * (uint32_t)j, fmq[j], rt[j], rs, s.K, nullptr, nullptr, wsum[j],
-                                             unused0, unused1);
-                const int slot = j % NS;  // (a constant once the loop is unrolled)
-                mbar_wait(full_u32 + 8u * slot, (phases >> slot) & 1u, timed_out);
-                phases ^= 1u << slot;
-                float2 eq_[4], ep_[4];
-                first_sweep_fetch<T, kAny>(ring + slot * kSlotBytes, rest16(q_b), rest16(p_b), lane, false, tail_valid, eq_, ep_,
-                                           mq[j], mp[j]);
-                __syncwarp();  // every lane holds its share of the slot in registers now: refill it
-                if (j + NS < kCellsPerWarp)
-                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), floor16(q_b) + (size_t)(j + NS) * kStrideBytes,
-                               floor16(p_b) + (size_t)(j + NS) * kStrideBytes, kCopyBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
-                               kHalfSlot);
-                else
-                    issue_cell(ring_u32 + (uint32_t)(slot * kSlotBytes), floor16(q_d) + (size_t)slot * kStrideBytes,
-                               floor16(p_d) + (size_t)slot * kStrideBytes, kCopyBytes, full_u32 + 8u * (uint32_t)slot, is_lane0,
-                               kHalfSlot);
-                first_sweep_store(taddr + 16u * (uint32_t)j, s.scale, eq_, ep_, mq[j], mp[j], sq[j], sp[j]);
-            }
-        } else if (has_a && aux_row) {  // the rare kind of row: two more sums per cell
-            float *dp = p.ws.dpart + r_a * s.ntiles + first_cell, *mpp = p.ws.mpart + r_a * s.ntiles + first_cell;
-            float2 coef[KT > 2 ? KT - 2 : 1];
-            if (KT > 2) {
-                float vj = 1.0f;
-#pragma unroll
-                for (int t = 1; t <= KT - 2; ++t) {
-                    vj *= 1.0f - rs.c;
-                    coef[t - 1] = splat((float)(t + 1) * vj);
+        // Second sweep of a cell of row A.  plain: no extra sums, one reference per warp.
+        auto second_sweep = [&](int j, float &w, auto plain) {
+            float aux[2];
+            if constexpr (decltype(plain)::value) {
+                second_sweep_cell<KT, false>(taddr + 16u * (uint32_t)place, place == 4, park, rs.KF, rs.c, false, s.K, w, aux[0], aux[1]);
+            } else {
+                float fq = 1.0f, fp = 1.0f, kt = rs.KF;
+                if (moved_a) {  // 2^(this cell's references - the warp's last ones)
+                    const float2 d = refs[j];
+                    fq = ex2(d.x);
+                    fp = ex2(d.y);
+                    kt = fminf(kt * ex2(d.y - d.x), FLT_MAX);
                 }
-            }
-#pragma unroll
-            for (int j = 0; j < kCellsPerWarp; ++j) {
-                if (j < ncw) {  // warp-uniform
-                    float aux[2];
-                    second_sweep_cell<KT, true>(taddr + 16u * (uint32_t)j, fmq[j], rt[j], rs, s.K, coef,
-                                                fmp_stash + j * kFThreads, wsum[j], aux[0], aux[1]);
-                    warp_sum_multi<2>(aux, lane);  // the two extra sums of the cell leave right away
-                    if ((lane & 15) == 0) ((lane & 16) ? mpp : dp)[j * kFWarps] = aux[0];
-                    if (has_b) SGBV_FIRST_SWEEP_CELL(j, q_b, p_b, q_d, p_d, more);
+                if (aux_row) {  // two more sums per cell, which leave right away
+                    const bool tiny = !(fq * rs.Fq > 1e-30f);
+                    second_sweep_cell<KT, true>(taddr + 16u * (uint32_t)place, place == 4, park, kt, rs.c, tiny, s.K, w, aux[0], aux[1]);
+                    warp_sum_multi<2>(aux, lane);
+                    if ((lane & 15) == 0) part_of((lane & 16) ? p.ws.mpart : p.ws.dpart)[cell_at(j)] = aux[0] * (tiny ? ((lane & 16) ? 0.0f : rs.kFp * fp) : fq * rs.Fq);
+                    if (tiny) w = 0.0f;
+                } else {
+                    second_sweep_cell<KT, false>(taddr + 16u * (uint32_t)place, place == 4, park, kt, rs.c, false, s.K, w, aux[0], aux[1]);
                 }
+                w *= fq;
             }
+        };
+        auto next_place = [&]() { place = place == 4 ? 0 : place + 1; };
+        // The common case by far has next to nothing to decide per cell.
+        const bool plain = has_a && !aux_row && !moved_a && ncw > 0;
+        if (plain && has_d && tail_j < 0 && !(kAny && (edge_b || timed_out))) {
+            for_each_cell<kCellsPerWarp - 1>([&](auto cell) {
+                constexpr int j = decltype(cell)::value;
+                if (j + 1 < ncw) second_sweep(j, wsum[j], std::true_type());
+                first_sweep(Int<j + 1>(), place, r_b, rest_qb, rest_pb, edge_b, true, std::true_type());
+                next_place();
+            });
         } else {
-#pragma unroll
-            for (int j = 0; j < kCellsPerWarp; ++j) {
-                if (j < ncw) {  // warp-uniform
-                    float unused0, unused1;
-                    if (has_a)
-                        second_sweep_cell<KT, false>(taddr + 16u * (uint32_t)j, fmq[j], rt[j], rs, s.K, nullptr, nullptr, wsum[j],
-                                                     unused0, unused1);
-                    if (has_b) SGBV_FIRST_SWEEP_CELL(j, q_b, p_b, q_d, p_d, more);
-                }
-            }
+            for_each_cell<kCellsPerWarp - 1>([&](auto cell) {
+                constexpr int j = decltype(cell)::value;
+                if (has_a && j + 1 < ncw) second_sweep(j, wsum[j], std::false_type());
+                if (has_b) first_sweep(Int<j + 1>(), place, r_b, rest_qb, rest_pb, edge_b, has_d, std::false_type());
+                next_place();
+            });
         }
-        // row A's cell sums: summed over the warp now, stored after the exchange below (a store that is still
-        // under way would hold up the memory fence of the exchange)
-        const int idx = owner_index<kCellsPerWarp>(lane);  // the lane that owns value number idx stores it
-        constexpr int kOwnerMask = 32 / kCellsPerWarp - 1;  // lanes that hold the same total
-        const bool store_w = has_a && (lane & kOwnerMask) == 0 && idx < ncw;
-        if (has_a) warp_sum_multi<kCellsPerWarp>(wsum, lane);
+        auto last_cell = [&]() {
+            const int at = place;  // (of cell kCellsPerWarp - 1, whether or not the warp has it)
+            place = at - (kCellsPerWarp - ncw);
+            if (place < 0) place += 5;
+            if (plain) second_sweep(ncw - 1, wsum[kCellsPerWarp - 1], std::true_type());
+            else if (has_a && ncw > 0) second_sweep(ncw - 1, wsum[kCellsPerWarp - 1], std::false_type());
+            place = at;
+        };
+        // row A's cell sums: summed over the warp, stored by the lane that owns value number idx
+        auto store_sums = [&]() {
+            const int idx = owner_index<kCellsPerWarp>(lane);
+            constexpr int kOwnerMask = 32 / kCellsPerWarp - 1;  // lanes that hold the same total
+            warp_sum_multi<kCellsPerWarp>(wsum, lane);
+            const bool is_last = idx == kCellsPerWarp - 1;
+            if ((lane & kOwnerMask) == 0 && (is_last ? ncw > 0 : idx + 1 < ncw)) part_of(p.ws.wpart)[cell_at(is_last ? ncw - 1 : idx)] = wsum[0] * rs.Fq;
+        };
         if (!has_b) {
-            if (store_w) wp[idx * kFWarps] = wsum[0];
+            last_cell();
+            store_sums();
             break;
         }
-        timed_out = __any_sync(0xffffffffu, timed_out != 0);  // the warp gives up as one
-        tmem_wait_st();
-
-        // ---- this thread's partial of row B: cell sums moved to its maximum over the cells; what the
-        //      second sweep will need of every cell: fmq[j] = cell's target units -> thread's row units,
-        //      rt[j] = ratio of the cell's draft and target factors ------------------------------------
-        float mqt = mq[0], mpt = mp[0];
-#pragma unroll
-        for (int j = 1; j < kCellsPerWarp; ++j) {
-            mqt = fmaxf(mqt, mq[j]);
-            mpt = fmaxf(mpt, mp[j]);
-        }
-        const bool has_q = mqt > -INFINITY, has_p = mpt > -INFINITY;
-        const float bqt = has_q ? mqt : 0.0f, bpt = has_p ? mpt : 0.0f;
-        float sqt = 0.0f, spt = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kCellsPerWarp; ++j) {
-            fmq[j] = rt[j] = 0.0f;
-            if (j < ncw) {  // a cell without a finite entry has sum 0 and factor 2^-inf = 0
-                const float dq = (mq[j] - bqt) * s.scale, dp = (mp[j] - bpt) * s.scale;
-                const float fmp = ex2(dp);
-                fmq[j] = ex2(dq);
-                rt[j] = ex2(dp - dq);  // (NaN or inf where a factor is 0: those cells weigh nothing)
-                sqt = fmaf(sq[j], fmq[j], sqt);
-                spt = fmaf(sp[j], fmp, spt);
-                fmp_stash[j * kFThreads] = fmp;
-            }
-        }
-        // warp partials relative to the warp's maxima
-        const float bqw = warp_max_redux(has_q ? bqt : -INFINITY), bpw = warp_max_redux(has_p ? bpt : -INFINITY);
-        const float rqw = (bqw > -INFINITY) ? bqw : 0.0f, rpw = (bpw > -INFINITY) ? bpw : 0.0f;
-        sqt = warp_sum(has_q ? sqt * ex2((bqt - rqw) * s.scale) : 0.0f);
-        spt = warp_sum(has_p ? spt * ex2((bpt - rpw) * s.scale) : 0.0f);
+        if (kAny) timed_out = __any_sync(0xffffffffu, timed_out != 0);  // the warp gives up as one
+        // (the requests have come to row D)
+        const int r_d = r_w, i_d = i_w, chains_on = chains_w;
+        if (combiner && has_d && p.tok) tok_b = __ldg(p.tok + r_d);
+        const uint32_t rest_qd = rest16(q_r), rest_pd = rest16(p_r);
+        const bool edge_d = edge_r;
+        float part[2] = {f.sq.x + f.sq.y, f.sp.x + f.sp.y};  // the warp's partial of row B: its references, and its sums relative to them
+        warp_sum_multi<2>(part, lane);                       // lanes 0-15: the target's, 16-31: the draft's
         // Exchange.  Every warp leaves its partial in shared memory; the LAST warp of the CTA combines them,
         // trades the CTA's partial with the other CTAs of the cluster (asynchronous distributed-shared-memory
         // stores that complete on the receiver's mbarrier; it alone polls that barrier), works out the row's
@@ -852,169 +1130,55 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         // issue slots: barrier 1 = "all partials are in", barrier 2 = "the row's scalars are in".
         // (a store to shared memory followed by an arrival on the barrier is the producer half of the hardware
         // barrier's producer/consumer pattern: the consumer that syncs on it sees the store)
-        if (lane == 0) ctl->wslots[warp] = make_float4(bqw, sqt, bpw, spt);
+        if ((lane & 15) == 0) reinterpret_cast<float2 *>(&ctl->wslots[warp])[lane >> 4] = make_float2(lane ? f.bp : f.bq, part[0]);
         __syncwarp();
         float4 rowv;  // rq, rp, kappa, c
         if (!combiner) {
             bar_arrive(1, kFThreads);
+        } else {
+            rowv = exchange(n + 1, r_b, i_b, has_d, r_d, i_d, chains_on);
+        }
+        last_cell();
+        moved_a = f.moved != 0;
+        if (moved_a) {  // the cells' references against the warp's last ones, in units of log2
+            __syncwarp();
+            if (lane < ncw) {
+                const float2 own = lane < f.moved ? refs[lane] : make_float2(f.bq, f.bp);
+                refs[lane] = make_float2((own.x - f.bq) * s.scale, (own.y - f.bp) * s.scale);
+            }
+        }
+        const float bq_b = f.bq, bp_b = f.bp;
+        fresh_row();
+        if (has_d) first_sweep(Int<0>(), place, r_d, rest_qd, rest_pd, edge_d, has_e, std::false_type());
+        if (has_a) store_sums();
+        tmem_wait_st();
+        next_place();  // of row B's first cell
+        if (!combiner) {
             bar_sync(2, kFThreads);
             rowv = ctl->rs;  // (the barrier statement is a compiler barrier for memory)
-        } else {
-            bar_sync(1, kFThreads);
-            const float4 v = lane < kFWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
-            float bq_row = warp_max_redux(v.x), bp_row = warp_max_redux(v.z);
-            float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-            // (kAny: factors and sums from here on in float64, as on the two-sweep path that takes such rows otherwise)
-            typedef typename Sum<kAny>::type Z;
-            // the sum over the lanes of z, each moved from units of m to units of `row` (-inf: a lane without a share)
-            auto combine = [&](float m, Z z, float row) {
-                if constexpr (kAny) {
-                    const Z moved = z * unit_factor(m, row, s.scale);
-                    return warp_sum(m > -INFINITY ? moved : (Z)0);
-                } else {
-                    return warp_sum(m > -INFINITY ? z * ex2((m - row) * s.scale) : 0.0f);
-                }
-            };
-            Z Zq = combine(v.x, v.y, rq_row), Zp = combine(v.z, v.w, rp_row);
-            if (C > 1) {  // the same once more over the CTAs of the cluster
-                const float4 mine = make_float4(bq_row, (float)Zq, bp_row, (float)Zp);
-                if (lane < C) push_f4(&ctl->slots[par][rank], xbar, (uint32_t)lane, mine);
-                if constexpr (kAny)
-                    if (lane < C)
-                        push_f4(&ctl->low[par][rank], xbar, (uint32_t)lane,
-                                make_float4(0.0f, (float)(Zq - (Z)mine.y), 0.0f, (float)(Zp - (Z)mine.w)));
-                mbar_wait(xbar, xph, timed_out);
-                timed_out = __any_sync(0xffffffffu, timed_out != 0);
-                const float4 cv = lane < C ? ctl->slots[par][lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
-                bq_row = warp_max_redux(cv.x);
-                bp_row = warp_max_redux(cv.z);
-                rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f;
-                rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
-                if constexpr (kAny) {
-                    const float4 low = lane < C ? ctl->low[par][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    Zq = combine(cv.x, (Z)cv.y + (Z)low.y, rq_row);
-                    Zp = combine(cv.z, (Z)cv.w + (Z)low.w, rp_row);
-                } else {
-                    Zq = combine(cv.x, cv.y, rq_row);
-                    Zp = combine(cv.z, cv.w, rp_row);
-                }
-            }
-            // The ratio p_i(tok_i)/q_i(tok_i) of this row: a chain of float64 operations.  In the chain walk only the
-            // NEXT row needs it, so it is worked out after the other warps have been released.
-#define SGBV_RATIO()                                                                                                     \
-    (exp2_short(((double)zp_tok - (double)rp_row) * (double)s.scale - ((double)zq_tok - (double)rq_row) * (double)s.scale) * \
-     (double)(Zq / Zp))
-            double cd;
-            if (row_mode) {
-                const double ratio = SGBV_RATIO();
-                // Publish this row's ratio for the clusters that walk the later rows of this chain.  The
-                // word itself says "ready": it is preset to a NaN pattern, and a ratio is never stored as
-                // NaN (a row that produces one is flagged invalid anyway).
-                if (lane == 0 && rank == 0 && i_b + 1 < s.gamma && !(p.withhold && i_b == 0))
-                    *reinterpret_cast<volatile double *>(p.ws.ratio + r_b) = (ratio != ratio) ? 0.0 : ratio;
-                // c_i = product of the published ratios of rows 0..i-1 of this chain (fixed order: a
-                // butterfly over the lanes).  Those rows are walked by other clusters at about the same
-                // time and publish right after their own statistics, which do not depend on c: no chain of
-                // waits forms.  Every lane polls one of them.  Bounded waits.
-                cd = SGBV_C0(bk_b);
-                const size_t r0 = (size_t)bk_b * s.gamma;
-                for (int j0 = 0; j0 < i_b; j0 += 32) {
-                    double w = 1.0;
-                    if (j0 + lane < i_b) {
-                        const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.ratio + r0 + j0 + lane);
-                        w = *word;
-                        if (w != w && timed_out) w = 0.0;
-                        if (w != w) {
-                            const long long t0 = clock64();
-                            while ((w = *word) != w) {
-                                if (clock64() - t0 > p.poll_limit) {
-                                    timed_out = 1;
-                                    w = 0.0;
-                                    break;
-                                }
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) w *= __shfl_xor_sync(0xffffffffu, w, o);
-                    cd *= w;
-                }
-                timed_out = __any_sync(0xffffffffu, timed_out != 0);
-            } else {
-                cd = c_carry;  // carried along the chain
-            }
-            rowv = make_float4(rq_row, rp_row, (float)(cd * (double)(Zq / Zp)), (float)cd);
-            if (lane == 0) ctl->rs = rowv;
-            __syncwarp();
-            bar_arrive(2, kFThreads);
-            // off the critical path: c of the next row of the chain walk (c_{i+1} = c_i ratio, and 1 at the start of
-            // the next chain), and the row's record for the finishing kernel
-            if (!row_mode) {
-                const double c_next = cd * SGBV_RATIO();  // c after this row
-                // the head of a chain that another cluster continues: leave c where that cluster looks for it
-                if (bk_b == chain_hi && i_b == off_hi - 1 && lane == 0 && rank == 0)
-                    *reinterpret_cast<volatile double *>(p.ws.ratio + cid) = (c_next != c_next) ? 0.0 : c_next;
-                if (has_d) {
-                    if (i_d == 0) {
-                        c_carry = SGBV_C0(bk_d);
-                    } else if (bk_d == bk_b) {
-                        c_carry = c_next;
-                    } else {  // the tail of a chain whose head another cluster walked at its very start
-                        const volatile double *word = reinterpret_cast<const volatile double *>(p.ws.ratio + cid - 1);
-                        double w = *word;
-                        if (w != w && !timed_out) {
-                            const long long t0 = clock64();
-                            while ((w = *word) != w)
-                                if (clock64() - t0 > kWaitLimitCycles) {
-                                    timed_out = 1;
-                                    break;
-                                }
-                        }
-                        c_carry = (w != w) ? 0.0 : w;
-                    }
-                }
-            }
-            if (lane == 0 && rank == 0) {
-                // nonfinite logits: NaN poisons Z, +inf shows up as an infinite maximum, a row of
-                // -inf only has Z = 0
-                const bool bad = !(Zq > 0.0f) || !(Zp > 0.0f) || !(Zq < (Z)INFINITY) || !(Zp < (Z)INFINITY) ||
-                                 !(bq_row < INFINITY) || !(bp_row < INFINITY);
-                RowInfo ri;
-                ri.flags = bad ? SGBV_STATUS_NONFINITE_LOGIT : 0;
-                ri.pad_ = 0;
-                ri.Zq = (double)Zq;
-                ri.Zp = (double)Zp;
-                ri.mq = bq_row;
-                ri.mp = bp_row;
-                ri.kappa = rowv.z;
-                ri.c = rowv.w;
-                p.ws.rows[r_b] = ri;
-            }
-#undef SGBV_RATIO
         }
-        if (store_w) wp[idx * kFWarps] = wsum[0];
-        // this thread's row units -> row-max units; row B becomes row A
-        const float Fp = has_p ? ex2((bpt - rowv.y) * s.scale) : 0.0f;
-        rs.Fq = has_q ? ex2((bqt - rowv.x) * s.scale) : 0.0f;
-        // equal factors (identical rows above all) must give kappa itself: p = q everywhere then leaves an
-        // exactly zero residual
-        rs.KF = (Fp == rs.Fq) ? rowv.z : rowv.z * Fp * rcp(rs.Fq);
-        rs.kFp = rowv.z * Fp;
+        // this warp's units -> the row's; row B becomes row A
+        const float ref_q = (bq_b - rowv.x) * s.scale, ref_p = (bp_b - rowv.y) * s.scale;
+        rs.Fq = ex2_wide(ref_q);  // (not flushed below 2^-126: the warp's exponentials may be up to 2^kRise)
+        // equal references (identical rows above all) must give kappa itself: p = q everywhere then leaves an
+        // exactly zero residual.  Finite: 0 x inf would take the weight of an entry with p = 0
+        rs.KF = fminf(rowv.z * ex2(ref_p - ref_q), FLT_MAX);
+        rs.kFp = p.aux_here ? rowv.z * ex2(ref_p) : 0.0f;
         rs.c = rowv.w;
-        bk_a = bk_b;
-        i_a = i_b;
-        bk_b = bk_d;
+        r_a = r_b;
+        r_b = r_d;
         i_b = i_d;
-        q_b = q_d;
-        p_b = p_d;
+        rest_qb = rest_qd;
+        rest_pb = rest_pd;
         edge_b = edge_d;
     }
+    if (!kAny) copy_wait<0>();
     // a warp that gave up may still have copies under way: they must land before the shared memory goes
     if (timed_out) {
         uint32_t fresh = 0;
 #pragma unroll
         for (int k = 0; k < NS; ++k)
-            if (pending & (1u << k)) mbar_wait(full_u32 + 8u * k, (phases >> k) & 1u, fresh);
+            if (kAny && (pending & (1u << k))) mbar_wait(full_u32 + 8u * k, (phases >> k) & 1u, fresh);
         if (lane == 0) atomicExch(p.error_flag, 1);
     }
     cluster_arrive();  // no CTA leaves while a neighbour may still write into its slots
@@ -1022,9 +1186,6 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     tmem_fence_before();
     __syncthreads();  // every warp of this CTA is done with the tensor memory
     if (warp == 0) tmem_dealloc(ctl->tmem_base, kTmemCols);
-#undef SGBV_ISSUE
-#undef SGBV_DIRECT
-#undef SGBV_FIRST_SWEEP_CELL
 #undef SGBV_C0
 }
 
@@ -1051,7 +1212,7 @@ template <typename T>
 constexpr int slots_for() { return (sizeof(T) == 4 ? 2 : 4) * 32 / kWarps / kCtasPerSm; }
 template <typename T, bool kAny>
 constexpr size_t smem_bytes() {
-    return (size_t)kWarps * slots_for<T>() * (2 * (kCell * sizeof(T) + (kAny ? kSlack : 0)) + 8) + (size_t)(kCtaCells / kWarps) * kWarps * 32 * 4 + sizeof(Control);
+    return (size_t)kWarps * slots_for<T>() * (2 * (kCell * sizeof(T) + (kAny ? kSlack : 0)) + 8) + (size_t)kCtaCells * sizeof(float2) + (size_t)kWarps * kParkBytes + sizeof(Control);
 }
 int slice_cells_of(int cells, int C) { return (cells + C - 1) / C; }
 
@@ -1111,6 +1272,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
     fp.error_flag = error_flag;
     fp.poll_limit = g_opt_poll_us > 0 ? (long long)g_opt_poll_us * 2000ll : kWaitLimitCycles;
     fp.withhold = g_opt_withhold;
+    fp.rise = kRise / L.s.scale;
     fp.aux_here = aux_here ? 1 : 0;
 
     cudaLaunchConfig_t cfg = {};

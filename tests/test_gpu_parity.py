@@ -293,6 +293,43 @@ def test_extra_sums_in_kernels_of_their_own(K, dtype, alpha, T):
     np.testing.assert_allclose(res[2], res[1], rtol=2e-5, atol=1e-9)
 
 
+@pytest.mark.parametrize("V,K,dtype,kind", [
+    (200, 4, "fp32", "ramp"), (31 * 256, 1, "fp32", "ramp"), (31 * 256 + 1, 3, "bf16", "masked"), (32 * 256 + 8, 8, "bf16", "ramp"),
+    (124 * 256, 4, "fp32", "masked"), (124 * 256 + 4, 2, "fp32", "ramp"), (125 * 256, 1, "bf16", "masked"), (128 * 256, 8, "fp32", "far"),
+    (33025, 3, "fp32", "masked"), (33032, 5, "bf16", "ramp"), (70000, 8, "fp32", "ramp"), (50257, 4, "bf16", "masked"),
+])
+def test_logits_far_from_the_first_ones_of_a_row(V, K, dtype, kind):
+    """Rows whose first entries say little about the rest: rising from cell to cell, masked up to some place (-inf, -1e9 or the type's
+    lowest value) but for an entry here and there, or a million from 0.  Two clusters walk all rows, so that every cell of a warp takes
+    every place it can have, at the sizes where the cells per warp change.  Both tensors get the same offsets, and the
+    draft tokens are entries that they leave likely."""
+    cfg = workloads.VerifyConfig(f"far_{V}_{kind}", B=3, K=K, gamma=4, V=V, dtype=dtype, temperature=0.8, alpha=0.9, seed=V + K)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    x = torch.arange(V, device="cuda")
+    for t in (inp.target_logits, inp.draft_logits):
+        if kind == "ramp":
+            t += (5.0 * (x // 256)).to(t.dtype)
+        elif kind == "far":
+            t += 1.0e6
+        else:
+            for b, value in enumerate((float("-inf"), -1e9, torch.finfo(t.dtype).min)):
+                t[b, :, :, (x < V // 3 * (b + 1) // 2) & (x % 97 != 5)] = value
+    if kind == "ramp":
+        inp.draft_tokens.copy_(V - 1 - inp.draft_tokens % min(V, 150))
+    elif kind == "masked":
+        inp.draft_tokens.copy_((inp.draft_tokens % (V // 97)) * 97 + 5)
+    binding.set_option("walk", 1)
+    binding.set_option("max_clusters", 2)
+    try:
+        rep, _, _ = run_both(inp)
+        assert binding.last_main_kernel() == "fused_chain_kernel"
+    finally:
+        binding.set_option("walk", 0)
+        binding.set_option("max_clusters", 0)
+    assert rep.decision_mismatches == 0 and rep.status_mismatches == 0, rep.detail
+    assert rep.h_violations == 0 and rep.S_violations == 0, rep.detail
+
+
 def test_unaligned_views_and_repeated_calls_are_deterministic():
     cfg = workloads.VerifyConfig("unaligned", B=3, K=2, gamma=3, V=4099, alpha=0.8, seed=99)
     inp = workloads.make_inputs(cfg, device="cuda")
