@@ -159,6 +159,21 @@ __device__ __forceinline__ double exp2_short(double x) {
 // e^x through the same short chain.
 __device__ __forceinline__ double exp_short(double x) { return exp2_short(x * 1.4426950408889634074); }
 
+// 2^x without a branch, so that several of them and what is around them overlap and a warp's lanes stay together: the Taylor series
+// of exp2_short in pairs, the nearest integer by an addition that leaves no room for a fraction, 2^n in two factors.
+__device__ __forceinline__ double exp2_flat(double v) {
+    const double x = fmin(fmax(v, -1100.0), 1100.0), y = x + 6755399441055744.0;
+    const double t = (x - (y - 6755399441055744.0)) * 0.6931471805599453094, t2 = t * t, t4 = t2 * t2;
+    const double p0 = 1.0 + t, p1 = fma(t, 1.0 / 6.0, 0.5), p2 = fma(t, 1.0 / 120.0, 1.0 / 24.0), p3 = fma(t, 1.0 / 5040.0, 1.0 / 720.0);
+    const double p4 = fma(t, 1.0 / 362880.0, 1.0 / 40320.0), p5 = fma(t, 1.0 / 39916800.0, 1.0 / 3628800.0);
+    const double p6 = fma(t, 1.0 / 6227020800.0, 1.0 / 479001600.0);
+    const double lo = fma(t4, fma(t2, p3, p2), fma(t2, p1, p0)), hi = fma(t4, p6, fma(t2, p5, p4));
+    const int n = __double2loint(y), n1 = n >> 1, n2 = n - n1;
+    const double r = fma(t4 * t4, hi, lo) * __hiloint2double((n1 + 1023) << 20, 0) * __hiloint2double((n2 + 1023) << 20, 0);
+    return v != v ? v : r;
+}
+__device__ __forceinline__ double exp_flat(double x) { return exp2_flat(x * 1.4426950408889634074); }
+
 // A value that is the same in all lanes of a warp, said so to the compiler: lane 0's.  Behind a branch or an early return on a
 // value that it cannot prove to be uniform (anything read from memory) the warp's lanes ran apart in the finishing and the
 // K-SEQ kernel, and every later shuffle took some 300 cycles instead of 25.

@@ -64,6 +64,16 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
     for (int n = tid; n < KG; n += nthreads) tok_s[n] = tok[n];
     for (int k = tid; k < K; k += nthreads) pass_s[k] = 0ull;
     if (tid == 0) sh_flags = 0;
+    // the logits of this thread's first draft token (step 0)
+    const int n_first = nthreads - 1 - tid;  // this thread's first (k,i), here and in the weights below
+    float zqt_first = 0.0f, zpt_first = 0.0f;
+    if (n_first < KG) {
+        const int t = tok[n_first];
+        if (t >= 0 && t < s.V) {
+            zqt_first = ld_logit(zq_all, (((size_t)b * K + n_first / g) * (g + 1) + n_first % g) * s.V + t);
+            zpt_first = ld_logit(zp_all, ((size_t)b * KG + n_first) * s.V + t);
+        }
+    }
     // Everything above reads only the caller's inputs.  The kernel may have been scheduled while the
     // streaming kernel was still running (programmatic dependent launch): wait for it to complete
     // before touching the row records and cell sums.
@@ -107,31 +117,25 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
         const int k = n / g, i = n % g;
         const size_t r = ((size_t)b * K + k) * g + i;
         const RowInfo ri = ws.rows[r];
-        const bool aux = ri.c < 1.0f;
-        const float *wp = ws.wpart + r * s.ntiles, *dp = ws.dpart + r * s.ntiles, *mp = ws.mpart + r * s.ntiles;
-        double sw = 0.0, sd = 0.0, sm = 0.0;
-        for (int t0 = 0; t0 < s.ntiles; t0 += 128) {  // four independent loads per array in flight
-            float w4[4], d4[4], m4[4];
+        const bool aux = uniform(ri.c) < 1.0f;
+        // eight independent loads in flight
+        auto total = [&](const float *part) {
+            double sum = 0.0;
+            for (int t0 = 0; t0 < s.ntiles; t0 += 256) {
+                float v[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int t = t0 + lane + 32 * e;
-                const bool in = t < s.ntiles;
-                // the two extra arrays are fetched whether or not the row has them (c < 1), so that the
-                // fetches do not wait for the row's record; what they hold otherwise is dropped below
-                w4[e] = in ? wp[t] : 0.0f;
-                d4[e] = in ? dp[t] : 0.0f;
-                m4[e] = in ? mp[t] : 0.0f;
-            }
+                for (int e = 0; e < 8; ++e) v[e] = t0 + lane + 32 * e < s.ntiles ? part[r * s.ntiles + t0 + lane + 32 * e] : 0.0f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                sw += (double)w4[e];
-                sd += aux ? (double)d4[e] : 0.0;
-                sm += aux ? (double)m4[e] : 0.0;
+                for (int e = 0; e < 8; ++e) sum += (double)v[e];
             }
+            return warp_sum(sum);
+        };
+        const double sw = total(ws.wpart);
+        double sd = 0.0, sm = 0.0;
+        if (aux) {
+            sd = total(ws.dpart);
+            sm = total(ws.mpart);
         }
-        sw = warp_sum(sw);
-        sd = warp_sum(sd);
-        sm = warp_sum(sm);
         if (lane == 0) {
             W_s[n] = sw;
             D_s[n] = sd;
@@ -142,7 +146,6 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
 
     // ---- 0. joint prefix probabilities (logs): token log-probabilities in parallel, then one
     //         running sum per draft ------------------------------------------------------------
-    const int n_first = nthreads - 1 - tid;  // this thread's first (k,i), here and in the weights below
     double inv_Zq_first = 0.0;
     bool below_first = false;
     for (int n = n_first; n < KG; n += nthreads) {
@@ -159,8 +162,8 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
             myflags |= SGBV_STATUS_TOKEN_RANGE;
             t = 0;
         }
-        const float zqt = ld_logit(zq_all, (((size_t)b * K + k) * (g + 1) + i) * s.V + t);
-        const float zpt = ld_logit(zp_all, r * s.V + t);
+        const float zqt = n == n_first ? zqt_first : ld_logit(zq_all, (((size_t)b * K + k) * (g + 1) + i) * s.V + t);
+        const float zpt = n == n_first ? zpt_first : ld_logit(zp_all, r * s.V + t);
         la_s[k * (g + 1) + i + 1] = ((double)zqt - (double)ri.mq) * s.inv_T - log(ri.Zq);
         lb_s[k * (g + 1) + i + 1] = ((double)zpt - (double)ri.mp) * s.inv_T - log(ri.Zp);
     }
@@ -192,10 +195,10 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
         }
         const double R = W_s[n] * inv_Zq;
         const double la = prefix(la_s + k * (g + 1), i), lb = prefix(lb_s + k * (g + 1), i);
-        const double S = exp_short(la) * R;
+        const double a = exp_flat(la), S = a * R;
         ws.resmass[(size_t)b * KG + n] = invalid ? NAN : S;
         if (i >= 1) {
-            const double hv = weight_sub(la, lb, R, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, below, exact_s[n] != 0);
+            const double hv = weight_sub(a, la, lb, R, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, below, exact_s[n] != 0);
             if ((double)u_s[k * g + i - 1] < hv) set_bit(&pass_s[k], i - 1);
             ws.h[(size_t)b * KG + k * g + i - 1] = invalid ? NAN : hv;
         }

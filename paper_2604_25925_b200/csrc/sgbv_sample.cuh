@@ -16,7 +16,6 @@ constexpr int kEpt = 1;              // elements per thread inside one tile (thr
 // Shared-memory scratch of the routines below (one per CTA).
 struct SampleScratch {
     double warp[kSampleMaxWarps];
-    float redf[kSampleMaxWarps];
     int pick[2];
     int i[4];
     double d[2];
@@ -56,14 +55,22 @@ __device__ Pick pick_in_tile(int x0, int x1, double base, double target, F wfun,
     const double wv = lane < (int)(blockDim.x >> 5) ? sh_warp[lane] : 0.0;
     const double off = base + warp_sum(lane < wid ? wv : 0.0);
     double cum = off + incl - local;
+    int first = INT_MAX, last = -1;
 #pragma unroll
     for (int j = 0; j < kEpt; ++j) {
         cum += (double)w[j];
         const int x = x0 + kEpt * tid + j;
         if (w[j] > 0.0f) {
-            atomicMax(&sh_pick[1], x);
-            if (cum > target) atomicMin(&sh_pick[0], x);
+            last = x;
+            if (cum > target) first = min(first, x);
         }
+    }
+    // (one atomic per warp: one per thread, on two words, took a thousand cycles)
+    first = __reduce_min_sync(0xffffffffu, first);
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) {
+        if (last >= 0) atomicMax(&sh_pick[1], last);
+        if (first != INT_MAX) atomicMin(&sh_pick[0], first);
     }
     __syncthreads();
     Pick p{sh_pick[0], sh_pick[1]};
@@ -133,8 +140,11 @@ static __device__ void locate_tile(const float *partials, const float *scale, in
         }
         cum += v;
     }
-    if (first != INT_MAX) atomicMin(&sh_i[2], first);
-    if (lastpos >= 0) atomicMax(&sh_i[3], lastpos);
+    const int first_w = __reduce_min_sync(0xffffffffu, first), last_w = __reduce_max_sync(0xffffffffu, lastpos);
+    if (lane == 0) {
+        if (first_w != INT_MAX) atomicMin(&sh_i[2], first_w);
+        if (last_w >= 0) atomicMax(&sh_i[3], last_w);
+    }
     __syncthreads();
     if (first != INT_MAX && sh_i[2] == first) sh_d[0] = base;  // exactly one thread owns that tile
     __syncthreads();
@@ -404,71 +414,18 @@ __device__ __forceinline__ Drawn draw_row(const T *zq, const Shape &s, double us
 template <typename T>
 __device__ int draw_from_row(const T *zq, const Shape &s, double us, float *tile_s, float *tile_m, SampleScratch *sc,
                              bool &bad_out) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = warp_index();
-    const int nthreads = blockDim.x, nwarps = nthreads / 32;
-    bool bad = false;
-    float m = -INFINITY;
-    constexpr int kNT = 4;  // tiles a warp has in flight
-    static_assert(kTile == 256, "a lane takes 8 entries of a tile");
-    const bool pieces = (reinterpret_cast<uintptr_t>(zq) % 16 == 0) && (s.V % (16 / (int)sizeof(T)) == 0);
-    for (int tb = wid * kNT; tb < s.ntiles; tb += nwarps * kNT) {
-        float z[kNT][kTile / 32];
-        if (pieces) {  // 16-byte loads
-#pragma unroll
-            for (int q = 0; q < kNT; ++q) load_tile_pieces<T>(zq, tb + q, tb + q < s.ntiles, s.V, lane, z[q]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < kNT; ++q)
-#pragma unroll
-                for (int e = 0; e < kTile / 32; ++e) {
-                    const int x = (tb + q) * kTile + lane + 32 * e;
-                    z[q][e] = (tb + q < s.ntiles && x < s.V) ? ld_logit(zq, x) : -INFINITY;
-                }
-        }
-        // the four tiles are reduced side by side (independent shuffle chains)
-        float mt[kNT], acc[kNT];
-#pragma unroll
-        for (int q = 0; q < kNT; ++q) {
-            mt[q] = -INFINITY;
-#pragma unroll
-            for (int e = 0; e < kTile / 32; ++e) {
-                bad |= (z[q][e] != z[q][e]) | (z[q][e] == INFINITY);
-                mt[q] = fmaxf(mt[q], z[q][e]);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < kNT; ++q) mt[q] = fmaxf(mt[q], __shfl_xor_sync(0xffffffffu, mt[q], o));
-#pragma unroll
-        for (int q = 0; q < kNT; ++q) {
-            acc[q] = 0.0f;
-            if (mt[q] > -INFINITY) {
-#pragma unroll
-                for (int e = 0; e < kTile / 32; ++e) acc[q] += expo(z[q][e], mt[q], s.scale);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < kNT; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-#pragma unroll
-        for (int q = 0; q < kNT; ++q) {
-            if (lane == 0 && tb + q < s.ntiles) {
-                tile_s[tb + q] = acc[q];
-                tile_m[tb + q] = mt[q];
-            }
-            m = fmaxf(m, mt[q]);
-        }
-    }
-    if (lane == 0) sc->redf[wid] = m;
-    bad = __syncthreads_or(bad);
-    m = warp_max(lane < nwarps ? sc->redf[lane] : -INFINITY);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int nthreads = blockDim.x;
+    const bool bad = __syncthreads_or(row_tile_stats<T>(zq, s, 0, s.ntiles, tile_s, tile_m));
+    float m = -INFINITY;  // (every warp for itself)
+    for (int t = lane; t < s.ntiles; t += 32) m = fmaxf(m, tile_m[t]);
+    m = warp_max(m);
     if (bad || !(m > -INFINITY)) {
         bad_out = true;
         return -1;
     }
     bad_out = false;
+    __syncthreads();  // every warp has read the maxima
     // tile_m becomes the factor exp((m_t - m)/T) of its tile
     for (int t = tid; t < s.ntiles; t += nthreads) tile_m[t] = (tile_m[t] > -INFINITY) ? expo(tile_m[t], m, s.scale) : 0.0f;
     __syncthreads();

@@ -419,9 +419,10 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
         const double inv_Zq = 1.0 / ri.Zq;
         const double Rr = W_s[n] * inv_Zq;
         const double la = prefix(la_s + k * (g + 1), i), lb = prefix(lb_s + k * (g + 1), i);
-        if (out_resmass) out_resmass[(size_t)b * KG + n] = invalid ? NAN : exp_short(la) * Rr;
+        const double a = exp_flat(la);
+        if (out_resmass) out_resmass[(size_t)b * KG + n] = invalid ? NAN : a * Rr;
         if (i >= 1) {
-            const double hv = weight_sub(la, lb, Rr, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, ri.c < 1.0f, true);
+            const double hv = weight_sub(a, la, lb, Rr, D_s[n] * inv_Zq, M_s[n] * inv_Zq, K, ri.c < 1.0f, true);
             if ((double)u_s[k * g + i - 1] < hv) set_bit(&pass_s[k], i - 1);
             if (out_h) out_h[(size_t)b * KG + k * g + i - 1] = invalid ? NAN : hv;
         }

@@ -7,15 +7,15 @@
 namespace sgbv {
 
 // 1 - (1-u)^K as the geometric sum u (1 + (1-u) + ... + (1-u)^(K-1)): all terms are positive, so
-// a tiny u keeps its full relative accuracy, and no transcendental function is needed.
-__device__ __forceinline__ double gfun(double u, int K) {
-    if (u >= 1.0) return 1.0;
-    if (!(u > 0.0)) return 0.0;
-    const double v = 1.0 - u;
+// a tiny u keeps its full relative accuracy, and no transcendental function is needed.  gsum: the sum, that is (1 - (1-u)^K) / u.
+__device__ __forceinline__ double gsum(double u, int K) {
+    const double v = 1.0 - fmin(fmax(u, 0.0), 1.0);
     double sum = 1.0;
+#pragma unroll 1
     for (int j = 1; j < K; ++j) sum = fma(sum, v, 1.0);
-    return u * sum;
+    return sum;
 }
+__device__ __forceinline__ double gfun(double u, int K) { return fmin(fmax(u, 0.0), 1.0) * gsum(u, K); }
 
 __device__ __forceinline__ double clamp01(double x) {
     if (!(x > 0.0)) return 0.0;
@@ -28,23 +28,24 @@ __device__ __forceinline__ double clamp01(double x) {
 //               = M + K (1-c)^(K-1) Dp               (c <  1, `exact`; equals R - (1-c)^K term by term)
 //               = R - (1-c)^K                        (c <  1, not `exact`: only where plain_form_is_safe says so)
 // denominator/a = numerator/a + g(b)/a - g(min(c,1))
-static __device__ double weight_sub(double la, double lb, double R, double Dp, double M, int K, bool below_one, bool exact) {
-    const double a = exp_short(la), b = exp_short(lb), c = exp_short(lb - la);
-    const double gb = gfun(b, K);
-    if (!(a > 0.0)) return gb > 0.0 ? 0.0 : 1.0;
-    double num, extra;
-    if (below_one) {  // decided on the float32 c the reduction pass used
-        double pw = 1.0;
-        for (int j = 1; j < K; ++j) pw *= (1.0 - c);
-        num = exact ? M + (double)K * pw * Dp : fmax(R - pw * (1.0 - c), 0.0);
-        extra = (K == 1) ? 0.0 : gb / a - gfun(c, K);
-    } else {
-        num = R;
-        extra = gb / a - 1.0;
+// with g(b)/a = c (g(b)/b).  a = exp(la).  Hardly a branch: the kernels run this once per CTA, on code that no cache holds yet and
+// with lanes that take every way (5,500 cycles with branches, three divisions and serial exponentials).
+static __device__ double weight_sub(double a, double la, double lb, double R, double Dp, double M, int K, bool below_one, bool exact) {
+    const double b = exp_flat(lb), c = exp_flat(lb - la);
+    const double gba = c * gsum(b, K);
+    // (1-c)^(K-1) and g(c)/c side by side; below_one was decided on the float32 c that the reduction pass used
+    const double v = 1.0 - c, v01 = 1.0 - fmin(c, 1.0);
+    double pw = 1.0, sum = 1.0;
+#pragma unroll 1
+    for (int j = 1; j < K; ++j) {
+        pw *= v;
+        sum = fma(sum, v01, 1.0);
     }
-    if (extra < 0.0) extra = 0.0;
-    const double den = num + extra;
-    if (!(den > 1e-12 * (gb / a + 1.0))) return 1.0;  // 0/0: accept, as single-draft GBV does
+    const double num = !below_one ? R : exact ? fma((double)K * pw, Dp, M) : fmax(fma(-pw, v, R), 0.0);
+    const double extra = !below_one ? gba - 1.0 : K == 1 ? 0.0 : gba - fmin(c, 1.0) * sum;
+    const double den = num + fmax(extra, 0.0);
+    if (!(a > 0.0)) return b > 0.0 ? 0.0 : 1.0;
+    if (!(den > 1e-12 * (gba + 1.0))) return 1.0;  // 0/0: accept, as single-draft GBV does
     return clamp01(num / den);
 }
 
@@ -60,8 +61,8 @@ static __device__ bool plain_form_is_safe(double R, double c, int K) {
 
 // Eq. 3.
 static __device__ double weight_full(double la, double lb, int K) {
-    const double a = exp_short(la), b = exp_short(lb);
-    double c = exp_short(lb - la);
+    const double a = exp_flat(la), b = exp_flat(lb);
+    double c = exp_flat(lb - la);
     if (!(a > 0.0) || c > 1.0) c = 1.0;
     const double den = gfun(b, K);
     if (!(den > 0.0)) return 0.0;
