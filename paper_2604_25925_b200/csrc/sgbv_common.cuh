@@ -89,12 +89,51 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// 2^x without a flush to 0 below 2^-126.
+__device__ __forceinline__ float ex2_wide(float x) {
+    float y;
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// x y clamped to [0, 1]; NaN gives 0.
+__device__ __forceinline__ float mul_sat(float x, float y) {
+    float r;
+    asm("mul.ftz.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+    return r;
+}
 __device__ __forceinline__ float max3(float a, float b, float c) {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 __device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
+
+// r^K for both halves of r, r in [0,1]; KT > 1 is a compile-time K, KT = 0 takes K at run time.
+template <int KT>
+__device__ __forceinline__ float2 ipow2(float2 r, int K) {
+    if (KT > 1) {
+        float2 acc = r, sq = r;  // acc is only read once it has been assigned
+        bool have = (KT & 1) != 0;
+#pragma unroll
+        for (int k = KT >> 1; k > 0; k >>= 1) {
+            sq = __fmul2_rn(sq, sq);
+            if (k & 1) {
+                acc = have ? __fmul2_rn(acc, sq) : sq;
+                have = true;
+            }
+        }
+        return acc;
+    }
+    float2 acc = r;
+    for (int t = 1; t < K; ++t) acc = __fmul2_rn(acc, r);
+    return acc;
+}
 
 // exp((z - m)/T) as 2^((z-m)*scale).
 __device__ __forceinline__ float expo(float z, float m, float scale) { return exp2f((z - m) * scale); }

@@ -140,24 +140,6 @@ __device__ __forceinline__ void push_f4(void *local, uint32_t local_bar, uint32_
                  "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
                  : "memory");
 }
-__device__ __forceinline__ float rcp(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// 2^x without a flush to 0 below 2^-126.
-__device__ __forceinline__ float ex2_wide(float x) {
-    float y;
-    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// x y clamped to [0, 1]; NaN gives 0.
-__device__ __forceinline__ float mul_sat(float x, float y) {
-    float r;
-    asm("mul.ftz.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
-    return r;
-}
 // This thread's asynchronous copies of 16 bytes, in groups that complete in order.
 template <int kDst, int kSrc>
 __device__ __forceinline__ void copy16(uint32_t dst, const void *src) {
@@ -272,27 +254,6 @@ __device__ __forceinline__ float warp_max_redux(float v) {
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
-// r^K for both halves of r, r in [0,1]; KT > 1 is a compile-time K, KT = 0 takes K at run time.
-template <int KT>
-__device__ __forceinline__ float2 ipow2(float2 r, int K) {
-    if (KT > 1) {
-        float2 acc = r, sq = r;  // acc is only read once it has been assigned
-        bool have = (KT & 1) != 0;
-#pragma unroll
-        for (int k = KT >> 1; k > 0; k >>= 1) {
-            sq = __fmul2_rn(sq, sq);
-            if (k & 1) {
-                acc = have ? __fmul2_rn(acc, sq) : sq;
-                have = true;
-            }
-        }
-        return acc;
-    }
-    float2 acc = r;
-    for (int t = 1; t < K; ++t) acc = __fmul2_rn(acc, r);
-    return acc;
-}
-
 // Sums P values over the 32 lanes of a warp at once ("transposed" butterfly: at every step a lane
 // hands half of its values to its partner and keeps the other half).  P is a power of two (<= 8).
 // On return v[0] of lane l is the warp total of value number owner_index<P>(l).

@@ -278,10 +278,13 @@ __device__ RowStats combine_stats(const float *__restrict__ stats_all, int R, si
         o.flags |= (int)rec[6];
     }
     o.Zq = o.Zp = 0.0;
+#pragma unroll 2
     for (int r = 0; r < R; ++r) {
         const float *rec = stats_all + ((size_t)r * nrows + row) * kRec;
-        if (rec[0] > -INFINITY) o.Zq += (double)rec[1] * exp2((double)(rec[0] - o.mq) * (double)scale);
-        if (rec[2] > -INFINITY) o.Zp += (double)rec[3] * exp2((double)(rec[2] - o.mp) * (double)scale);
+        // (without branches, so that the shards' exponentials overlap)
+        const double fq = exp2_flat((double)(rec[0] - o.mq) * (double)scale), fp = exp2_flat((double)(rec[2] - o.mp) * (double)scale);
+        o.Zq += rec[0] > -INFINITY ? (double)rec[1] * fq : 0.0;
+        o.Zp += rec[2] > -INFINITY ? (double)rec[3] * fp : 0.0;
     }
     return o;
 }
@@ -376,6 +379,8 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
     unsigned char *lcp_s = reinterpret_cast<unsigned char *>(u_s + KG + 1);
     __shared__ int sh_i[2];
     __shared__ int sh_flags;
+    __shared__ double share_s[kMaxRanks];
+    __shared__ float m_s[kMaxRanks];
 
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = warp_index();
     const size_t NR = (size_t)s.B * KG;
@@ -450,6 +455,31 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
     __syncthreads();
     int tau = invalid ? -1 : sh_i[0], f = invalid ? -1 : sh_i[1];
     int status = status_in;
+    // the shards' shares of the mass that the token is drawn from, one thread per shard
+    const int kk = (tau <= 0) ? 0 : f;
+    const bool residual = !invalid && tau < g && W_s[kk * g + tau] > 0.0;
+    const size_t nrows = (size_t)s.B * K * (g + 1);
+    const size_t qrow = ((size_t)b * K + kk) * (g + 1) + (invalid ? 0 : tau);
+    int badrow = 0;
+    float rec_m = -INFINITY, rec_s = 0.0f;
+    if (tid < R && !invalid) {
+        if (residual) {
+            share_s[tid] = sums_all[((size_t)tid * NR + (size_t)b * KG + kk * g + tau) * 3];
+        } else {
+            const float *rec = stats_all + ((size_t)tid * nrows + qrow) * kRec;
+            rec_m = rec[0];
+            rec_s = rec[1];
+            badrow = ((int)rec[6] & SGBV_STATUS_NONFINITE_LOGIT) != 0;
+            m_s[tid] = rec_m;
+        }
+    }
+    const bool bad = __syncthreads_or(badrow);
+    if (tid < R && !invalid && !residual) {
+        float m = -INFINITY;
+        for (int q = 0; q < R; ++q) m = fmaxf(m, m_s[q]);
+        share_s[tid] = rec_m > -INFINITY ? (double)rec_s * exp2_flat((double)(rec_m - m) * (double)s.scale) : 0.0;
+    }
+    __syncthreads();
     if (tid == 0) {
         Plan pl;
         pl.owner = -1;
@@ -457,32 +487,14 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
         pl.k = pl.i = 0;
         pl.frac = 0.0;
         if (!invalid) {
-            const int kk = (tau == 0) ? 0 : f;
             const double us = (double)u_s[KG];
-            const bool residual = tau < g && W_s[kk * g + tau] > 0.0;
             if (tau < g && !residual) status |= SGBV_STATUS_DEGENERATE_RESIDUAL;
             pl.mode = residual ? 0 : 1;
             pl.k = kk;
             pl.i = tau;
-            // the shards' shares of the mass the token is drawn from, in vocabulary (= rank) order
-            const size_t nrows = (size_t)s.B * K * (g + 1);
-            const size_t qrow = ((size_t)b * K + kk) * (g + 1) + tau;
-            const size_t rrow = (size_t)b * KG + kk * g + (residual ? tau : 0);
-            float m = -INFINITY;
-            bool bad = false;
-            if (!residual)
-                for (int q = 0; q < R; ++q) {
-                    const float *rec = stats_all + ((size_t)q * nrows + qrow) * kRec;
-                    m = fmaxf(m, rec[0]);
-                    bad |= ((int)rec[6] & SGBV_STATUS_NONFINITE_LOGIT) != 0;
-                }
-            auto share = [&](int q) {
-                if (residual) return sums_all[((size_t)q * NR + rrow) * 3];
-                const float *rec = stats_all + ((size_t)q * nrows + qrow) * kRec;
-                return rec[0] > -INFINITY ? (double)rec[1] * exp2((double)(rec[0] - m) * (double)s.scale) : 0.0;
-            };
+            // in vocabulary (= rank) order
             double total = 0.0;
-            for (int q = 0; q < R; ++q) total += share(q);
+            for (int q = 0; q < R; ++q) total += share_s[q];
             if (bad || !(total > 0.0)) {  // the row a token would be drawn from is unusable
                 status |= SGBV_STATUS_NONFINITE_LOGIT;
                 tau = f = -1;
@@ -491,7 +503,7 @@ shard_decide_kernel(const int32_t *__restrict__ tok_all, const float *__restrict
                 double cum = 0.0;
                 int last = -1;
                 for (int q = 0; q < R; ++q) {
-                    const double v = share(q);
+                    const double v = share_s[q];
                     if (v > 0.0) last = q;
                     if (pl.owner < 0 && cum + v > target) {
                         pl.owner = q;

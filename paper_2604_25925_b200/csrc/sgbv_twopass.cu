@@ -163,49 +163,89 @@ __device__ __forceinline__ void reduce_tiles(const T *zq, const T *zp, const Sha
     }
 }
 
-// The same sums for rows that can be read in 16-byte pieces: a lane takes 8 entries of a cell of each tensor, two
-// cells per warp are in flight.
-template <typename T, bool kNeedAux, bool kStoreW = true>
+// The same sums for rows that can be read in 16-byte pieces: a lane takes 8 entries of a cell of each tensor, two entries per
+// instruction; the pieces of the warp's next cell are on their way meanwhile.  (One entry at a time, the power by K - 1 products and the
+// loads of two cells at a time, which the compiler took one after the other, bound it before: 65 us for the sums of 32 x 8 x 8 x 18992
+// float32, 311 MB, whose floor is 48; the whole call of one rank of eight 167 us then, 153 now.)
+template <typename T>
+struct Pieces;
+template <>
+struct Pieces<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float *row, int tile, bool in, int V, int lane) {
+        const float ninf = -INFINITY;
+        const int xa = tile * kTile + lane * 4, xb = xa + kTile / 2;
+        a = (in && xa < V) ? __ldg(reinterpret_cast<const float4 *>(row + xa)) : make_float4(ninf, ninf, ninf, ninf);
+        b = (in && xb < V) ? __ldg(reinterpret_cast<const float4 *>(row + xb)) : make_float4(ninf, ninf, ninf, ninf);
+    }
+    __device__ __forceinline__ float2 pair(int e) const {
+        return e == 0 ? make_float2(a.x, a.y) : e == 1 ? make_float2(a.z, a.w) : e == 2 ? make_float2(b.x, b.y) : make_float2(b.z, b.w);
+    }
+};
+template <>
+struct Pieces<uint16_t> {
+    uint4 a;
+    __device__ __forceinline__ void load(const uint16_t *row, int tile, bool in, int V, int lane) {
+        const uint32_t ninf2 = 0xff80ff80u;  // two bf16 -inf
+        const int xa = tile * kTile + lane * 8;
+        a = (in && xa < V) ? __ldg(reinterpret_cast<const uint4 *>(row + xa)) : make_uint4(ninf2, ninf2, ninf2, ninf2);
+    }
+    __device__ __forceinline__ float2 pair(int e) const {
+        const uint32_t w = e == 0 ? a.x : e == 1 ? a.y : e == 2 ? a.z : a.w;
+        return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    }
+};
+template <typename T, int KT, bool kNeedAux, bool kStoreW = true>
 __device__ __forceinline__ void reduce_tiles_pieces(const T *zq, const T *zp, const Shape &s, const RowInfo &ri, int K,
                                                     int t0, int t1, float *wpart, float *dpart, float *mpart) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int t = t0 + 2 * wid; t < t1; t += 2 * (kThreads / 32)) {
-        float a[2][kTile / 32], b[2][kTile / 32];
+    const int lane = threadIdx.x & 31, wid = warp_index();
+    constexpr int kWarps = kThreads / 32;
+    const float2 nmq = splat(-ri.mq), nmp = splat(-ri.mp), sc = splat(s.scale), nk = splat(-ri.kappa), nv = splat(ri.c - 1.0f);
+    Pieces<T> q, p, nq, np;
+    nq.load(zq, t0 + wid, t0 + wid < t1, s.V, lane);
+    np.load(zp, t0 + wid, t0 + wid < t1, s.V, lane);
+    for (int t = t0 + wid; t < t1; t += kWarps) {
+        q = nq;
+        p = np;
+        nq.load(zq, t + kWarps, t + kWarps < t1, s.V, lane);
+        np.load(zp, t + kWarps, t + kWarps < t1, s.V, lane);
+        float2 sw = splat(0.0f), sd = splat(0.0f), sm = splat(0.0f);
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            load_tile_pieces<T>(zq, t + e, t + e < t1, s.V, lane, a[e]);
-            load_tile_pieces<T>(zp, t + e, t + e < t1, s.V, lane, b[e]);
+        for (int e = 0; e < 4; ++e) {  // (entries past the row hold -inf and add nothing)
+            const float2 xq = __fmul2_rn(__fadd2_rn(q.pair(e), nmq), sc), xp = __fmul2_rn(__fadd2_rn(p.pair(e), nmp), sc);
+            const float2 eq = make_float2(ex2_wide(xq.x), ex2_wide(xq.y)), ep = make_float2(ex2_wide(xp.x), ex2_wide(xp.y));
+            const float2 diff = __ffma2_rn(nk, ep, eq);  // q - c p in units of the target row
+            if (KT == 1) {
+                if (kStoreW) sw = __fadd2_rn(sw, make_float2(fmaxf(diff.x, 0.0f), fmaxf(diff.y, 0.0f)));
+            } else {
+                const float2 r = make_float2(mul_sat(diff.x, rcp(eq.x)), mul_sat(diff.y, rcp(eq.y)));  // 1 - min{c p/q, 1}; q = 0 gives 0
+                if (kStoreW) sw = __ffma2_rn(eq, ipow2<KT>(r, K), sw);
+                if (kNeedAux) {
+                    const float v = 1.0f - ri.c;
+                    float2 acc = splat(K >= 2 ? 1.0f : 0.0f);
+                    float vj = 1.0f;
+#pragma unroll
+                    for (int j = 1; j <= K - 2; ++j) {
+                        vj *= v;
+                        acc = __ffma2_rn(acc, r, splat((float)(j + 1) * vj));
+                    }
+                    const float2 ct = __fadd2_rn(r, nv);  // c - t
+                    sm = __ffma2_rn(__fmul2_rn(eq, __fmul2_rn(ct, ct)), acc, sm);
+                }
+            }
+            if (kNeedAux) sd = __fadd2_rn(sd, make_float2(fmaxf(-diff.x, 0.0f), fmaxf(-diff.y, 0.0f)));
         }
-        float sw[2] = {0.0f, 0.0f}, sd[2] = {0.0f, 0.0f}, sm[2] = {0.0f, 0.0f};
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-#pragma unroll
-            for (int j = 0; j < kTile / 32; ++j) {  // entries past the row hold -inf and add nothing
-                const float eq = expo(a[e][j], ri.mq, s.scale), ep = expo(b[e][j], ri.mp, s.scale);
-                float w, dp = 0.0f, m2 = 0.0f;
-                element_terms<kNeedAux>(eq, ep, ri.kappa, ri.c, K, w, dp, m2);
-                sw[e] += w;
-                sd[e] += dp;
-                sm[e] += m2;
-            }
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            sw[e] = warp_sum(sw[e]);
-            if (kNeedAux) {
-                sd[e] = warp_sum(sd[e]);
-                sm[e] = warp_sum(sm[e]);
-            }
-            if (lane == 0 && t + e < t1) {
-                if (kStoreW) wpart[t + e] = sw[e];
-                dpart[t + e] = sd[e];
-                mpart[t + e] = sm[e];
-            }
+        const float w = kStoreW ? warp_sum(sw.x + sw.y) : 0.0f;
+        const float d = kNeedAux ? warp_sum(sd.x + sd.y) : 0.0f, m2 = kNeedAux ? warp_sum(sm.x + sm.y) : 0.0f;
+        if (lane == 0) {
+            if (kStoreW) wpart[t] = w;
+            dpart[t] = d;
+            mpart[t] = m2;
         }
     }
 }
 
-// KT: the number of drafts as a compile-time constant (the power in Eq. 2 then unrolls, in the same order of
-// multiplications as the run-time loop), or 0 for the run-time value.
+// KT: the number of drafts as a compile-time constant, or 0 for the run-time value.
 template <typename T, int KT>
 __global__ void __launch_bounds__(kThreads)
 otreduce_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shape s,
@@ -224,10 +264,10 @@ otreduce_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shap
     const bool pieces = (reinterpret_cast<uintptr_t>(zq) % 16 == 0) && (reinterpret_cast<uintptr_t>(zp) % 16 == 0) &&
                         (s.V % (16 / (int)sizeof(T)) == 0);
     if (ri.c < 1.0f) {
-        if (pieces) reduce_tiles_pieces<T, true>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
+        if (pieces) reduce_tiles_pieces<T, KT, true>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
         else reduce_tiles<T, true>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
     } else {
-        if (pieces) reduce_tiles_pieces<T, false>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
+        if (pieces) reduce_tiles_pieces<T, KT, false>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
         else reduce_tiles<T, false>(zq, zp, s, ri, K, t0, t1, wp, dp, mp);
     }
 }
@@ -284,7 +324,7 @@ auxwork_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Shape
         float *dp = dpart + (size_t)r * s.ntiles, *mp = mpart + (size_t)r * s.ntiles;
         const bool pieces = (reinterpret_cast<uintptr_t>(zq) % 16 == 0) && (reinterpret_cast<uintptr_t>(zp) % 16 == 0) &&
                             (s.V % (16 / (int)sizeof(T)) == 0);
-        if (pieces) reduce_tiles_pieces<T, true, false>(zq, zp, s, ri, K, t0, t1, nullptr, dp, mp);
+        if (pieces) reduce_tiles_pieces<T, KT, true, false>(zq, zp, s, ri, K, t0, t1, nullptr, dp, mp);
         else reduce_tiles<T, true, false>(zq, zp, s, ri, K, t0, t1, nullptr, dp, mp);
     }
 }
