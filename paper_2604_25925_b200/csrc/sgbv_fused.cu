@@ -1309,6 +1309,22 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
         plan.row_mode = 1;
         C = Crow;
     }
+    // A few rounds of rows: what counts is the number of rounds times the time of a row, some 3 us and 48 ns for each of a CTA's
+    // cells.  (64 rows of 594 cells: clusters of five 26 at a time, three rounds, of six 24, three shorter ones: 39.6 -> 36.8 us.  Long
+    // walks are bound by throughput, and the smallest cluster is best: 64 x 8 x 8 rows of that length 818 us, of six 932.)
+    if (!g_opt_cluster && !plan.row_mode && fits(C) && g_opt_max_clusters == 0) {
+        auto cost = [&](int c) {
+            const long side_by_side = std::min<long>(resident(c, false), nchains);
+            return side_by_side < 1 ? 1e30 : (double)((units + side_by_side - 1) / side_by_side) * (62.0 + (double)((cells + c - 1) / c));
+        };
+        const double base = cost(C);
+        if (units <= 4L * std::min<long>(resident(C, false), nchains)) {
+            int best = C;
+            for (int c = C + 1; c <= kMaxCluster && c < 2 * C; ++c)
+                if (cost(c) < 0.95 * base && cost(c) < cost(best)) best = c;
+            C = best;
+        }
+    }
     if (!fits(C)) return g_opt_cluster ? SGBV_ERR_SHAPE : 0;
     plan.cluster = C;
     plan.slice_cells = slice_cells_of(cells, C);
@@ -1326,7 +1342,10 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
     // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed; rows that start
     // anywhere included: error of the weights against 64 bits with the sums here / apart 4.1e-8 / 5.7e-8 at 64 x 8 x 6 x 50257
     // bfloat16, 5.9e-8 / 1.0e-7 at 64 x 2 x 12 x 100003, where the two-sweep path has 1.6e-7 and 4.0e-7)
-    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (bytes < kAuxApartMinBytes || s.K == 1));
+    // (bfloat16 with many drafts: the sums cost most there, and memory hides none of it.  In this kernel / apart, us: 16 x 8 x 4 x 151936
+    // 160 / 146, 64 x 8 x 4 x 32000 117 / 107; float32 32 x 8 x 12 x 32000 158 / 158; K = 4 bfloat16 16 x 4 x 5 x 128256 87 / 90.)
+    const bool apart = bytes >= kAuxApartMinBytes || (sizeof(T) == 2 && s.K >= 6 && bytes >= kAuxApartMinBytes / 10);
+    const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (!apart || s.K == 1));
     *aux_apart = !aux_here;
     return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true, *words_used)
                          : launch_as<T, false, KT, kAny>(L, plan, error_flag, clusters, aux_here, *words_used);
