@@ -367,13 +367,14 @@ __device__ __forceinline__ void set_references(FirstSweep &f, int j, float m1, f
         f.bp = warp_max_redux(m2);
         return;
     }
-    if (!__any_sync(0xffffffffu, m1 > f.bq + rise || m2 > f.bp + rise)) return;
+    // (the difference is what the exponent takes; b + rise would be rounded to a multiple of b's ulp, which may be as much as rise)
+    if (!__any_sync(0xffffffffu, m1 - f.bq > rise || m2 - f.bp > rise)) return;
     if ((threadIdx.x & 31) == 0)
         for (int i = f.moved; i < j; ++i) refs[i] = make_float2(f.bq, f.bp);
     f.moved = j;
     auto raise = [&](float m, float &b, float2 &sum) {
         m = warp_max_redux(m);
-        if (!(m > b + rise)) return;
+        if (!(m - b > rise)) return;
         const float move = ex2((b - m) * scale);
         sum.x *= move;
         sum.y *= move;
@@ -1233,7 +1234,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
     fp.error_flag = error_flag;
     fp.poll_limit = g_opt_poll_us > 0 ? (long long)g_opt_poll_us * 2000ll : kWaitLimitCycles;
     fp.withhold = g_opt_withhold;
-    fp.rise = kRise / L.s.scale;
+    fp.rise = std::min(kRise / L.s.scale, FLT_MAX / 2.0f);  // (-FLT_MAX stands for "no finite logit so far": what follows has to lie above it)
     fp.aux_here = aux_here ? 1 : 0;
 
     cudaLaunchConfig_t cfg = {};

@@ -330,6 +330,43 @@ def test_logits_far_from_the_first_ones_of_a_row(V, K, dtype, kind):
     assert rep.h_violations == 0 and rep.S_violations == 0, rep.detail
 
 
+@pytest.mark.parametrize("V,base,T,walk", [(124 * 256, 6e5, 0.01, 1), (124 * 256, 1e8, 1.0, 1), (128 * 256, -1e8, 1.0, 1), (124 * 256, 6e5, 0.01, 2),
+                                           (124 * 256 + 1, 6e5, 0.01, 1), (124 * 256, 0.0, 1e38, 1)])
+def test_references_move_by_differences_that_a_sum_rounds_away(V, base, T, walk):
+    """Rows of two neighbouring float32 numbers, so large that one step between them is more than the references' rise while their
+    sum with it rounds to the next number: every warp's first cell holds the lower one, the cells behind it the upper one, which is
+    2^9 to 2^12 times as likely.  (At a temperature near the largest float32 the rise itself is infinite.)  Against the two-sweep
+    path, at twice the tolerance against the oracle: every draft token is likely under both rows."""
+    cfg = workloads.VerifyConfig("steps", B=3, K=2, gamma=3, V=V, temperature=T, alpha=0.9, seed=3)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    x = torch.arange(V, device="cuda")
+    low = torch.tensor(base, device="cuda")
+    high = torch.nextafter(low, low + 1e9)
+    first = x % 1024 < 256
+    inp.target_logits.copy_(torch.where(first, low, high))
+    inp.draft_logits.copy_(torch.where(first | (x % 3 == 0), low, high))
+    if T > 1e30:  # masked first cells
+        inp.target_logits[..., first] = float("-inf")
+        inp.draft_logits[..., first] = float("-inf")
+    inp.draft_tokens.copy_(256 + 1024 * (inp.draft_tokens % 30) + inp.draft_tokens % 256 * 3)
+    inp.draft_tokens.add_((inp.draft_tokens % 3 == 0).int())
+    outs = []
+    for options in ({"walk": walk, "cluster": 1}, {"path": 1}):
+        for name, value in options.items():
+            binding.set_option(name, value)
+        try:
+            outs.append(binding.sgbv_verify_ex(inp.target_logits, inp.draft_logits, inp.draft_tokens, inp.uniforms, T))
+            torch.cuda.synchronize()
+            assert binding.last_main_kernel() == ("otreduce_kernel" if "path" in options else "fused_chain_kernel")
+        finally:
+            for name in options:
+                binding.set_option(name, 0)
+    a, b = outs
+    assert (a.status == 0).all() and torch.equal(a.status, b.status)
+    torch.testing.assert_close(a.h, b.h, rtol=2e-5, atol=2e-9)
+    torch.testing.assert_close(a.resmass, b.resmass, rtol=2e-5, atol=0)
+
+
 def test_unaligned_views_and_repeated_calls_are_deterministic():
     cfg = workloads.VerifyConfig("unaligned", B=3, K=2, gamma=3, V=4099, alpha=0.8, seed=99)
     inp = workloads.make_inputs(cfg, device="cuda")
