@@ -45,6 +45,7 @@ static __device__ double weight_sub(double a, double la, double lb, double R, do
     const double extra = !below_one ? gba - 1.0 : K == 1 ? 0.0 : gba - fmin(c, 1.0) * sum;
     const double den = num + fmax(extra, 0.0);
     if (!(a > 0.0)) return b > 0.0 ? 0.0 : 1.0;
+    if (!(gba < (double)INFINITY)) return 0.0;  // c beyond the largest double, a beyond the smallest normal one: num / den without a number
     if (!(den > 1e-12 * (gba + 1.0))) return 1.0;  // 0/0: accept, as single-draft GBV does
     return clamp01(num / den);
 }

@@ -367,6 +367,28 @@ def test_references_move_by_differences_that_a_sum_rounds_away(V, base, T, walk)
     torch.testing.assert_close(a.resmass, b.resmass, rtol=2e-5, atol=0)
 
 
+def _all_but_excluded(T=0.05):
+    """Draft blocks whose first token has a target log-probability from -700 to -760 and a draft probability near 1: a = q(x^i) goes
+    through the smallest normal float64 number, the denormal ones (where c = p/q overflows) and 0.  Other rows are flat."""
+    cfg = workloads.VerifyConfig("excluded", B=31, K=2, gamma=3, V=3000, temperature=T, alpha=0.9, seed=5)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    for t in (inp.target_logits, inp.draft_logits):
+        t.mul_(0.1).clamp_(-0.5, 0.5)
+    first = inp.draft_tokens[:, :, :1].long()
+    b = torch.arange(cfg.B, device="cuda", dtype=torch.float32)
+    inp.target_logits[:, :, 0].scatter_(2, first, (-34.5 - 0.1 * b).view(-1, 1, 1).expand(-1, cfg.K, 1))
+    inp.draft_logits[:, :, 0].scatter_(2, first, 3.0)
+    inp.uniforms.fill_(0.5)
+    return inp
+
+
+def test_a_block_that_the_target_all_but_excludes_is_not_accepted():
+    inp = _all_but_excluded()
+    rep, out, ref = run_both(inp)
+    assert_parity(rep)
+    assert (ref.tau == 0).all() and out.h[:, :, 0].max() < 1e-290
+
+
 def test_unaligned_views_and_repeated_calls_are_deterministic():
     cfg = workloads.VerifyConfig("unaligned", B=3, K=2, gamma=3, V=4099, alpha=0.8, seed=99)
     inp = workloads.make_inputs(cfg, device="cuda")

@@ -8,7 +8,7 @@ import torch
 import oracle
 from oracle.compare import compare
 from paper_2604_25925_b200 import binding, sharded, workloads
-from test_gpu_parity import assert_parity, _to_np32
+from test_gpu_parity import assert_parity, _all_but_excluded, _to_np32
 
 pytestmark = pytest.mark.gpu
 
@@ -115,6 +115,13 @@ def test_degenerate_and_flagged_rows_sharded():
     assert (out.tokens[2:5].cpu().numpy() == -1).all() and (out.accept_len[2:5].cpu().numpy() == -1).all()
     y6 = int(out.tokens[6, int(out.accept_len[6])])
     assert 0 <= y6 < 300 and not (100 <= y6 < 200)
+
+
+def test_a_block_that_the_target_all_but_excludes_is_not_accepted_by_any_rank():
+    inp = _all_but_excluded()
+    rep, out, _ = run_sharded(inp, sharded.shard_bounds(inp.cfg.V, 3))
+    assert_parity(rep)
+    assert (out.accept_len == 0).all()
 
 
 def test_argument_checks():
