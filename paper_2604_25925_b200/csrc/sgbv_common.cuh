@@ -21,6 +21,9 @@ constexpr int kMaxK = 64;
 constexpr int kMaxGamma = 64;
 constexpr int kMaxV = 1 << 22;
 constexpr float kLog2e = 1.4426950408889634f;
+// Dynamic shared memory that a kernel gets without cudaFuncSetAttribute: 48 KB less what it declares itself (at most 2 KB in the
+// kernels that compare with this).
+constexpr size_t kSmemWithoutAsking = 46 * 1024;
 
 // Per (b,k,i) row pair, i < gamma.  Written by the statistics pass, read by the reduction pass
 // and by the finishing kernel.

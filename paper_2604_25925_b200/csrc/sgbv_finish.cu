@@ -394,7 +394,7 @@ int run(const Launch &L) {
     const size_t tiles = 2 * (size_t)s.ntiles * sizeof(float);
     ws.bonus_in_smem = (s.ntiles <= kTilesInSmem && smem + tiles <= 160 * 1024) ? 1 : 0;
     if (ws.bonus_in_smem) smem += tiles;
-    if (smem > 48 * 1024) {
+    if (smem > kSmemWithoutAsking) {
         cudaError_t e = cudaFuncSetAttribute(finish_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return SGBV_ERR_CUDA;
     }

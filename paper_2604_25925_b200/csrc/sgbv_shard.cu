@@ -689,7 +689,7 @@ int sgbv_shard_decide(const int32_t *draft_tokens, const float *uniforms, int B,
     const size_t smem = 3 * KG * sizeof(double) + 2 * (size_t)K * (gamma + 1) * sizeof(double) +
                         K * sizeof(unsigned long long) + KG * sizeof(int32_t) + (KG + 1) * sizeof(float) +
                         ((size_t)K * K + 15) / 16 * 16;
-    if (smem > 48 * 1024 &&
+    if (smem > kSmemWithoutAsking &&
         cudaFuncSetAttribute(shard_decide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return SGBV_ERR_CUDA;
     shard_decide_kernel<<<B, kThreads, smem, (cudaStream_t)stream>>>(draft_tokens, uniforms, s, stats_all, sums_all,

@@ -1,6 +1,10 @@
 """GPU parity: the CUDA path (through the C ABI) against the float64 oracle on the same seeded
 inputs.  Rules are those of ``oracle/compare.py``: decisions bit-exact except rows within 1e-6 of
 a threshold (counted), weights and residual masses within 1e-5 relative."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -11,6 +15,7 @@ from paper_2604_25925_b200 import binding, workloads
 from treemodel import chi_square, gbv_single_draft, np_softmax
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def _to_np32(t):
@@ -387,6 +392,31 @@ def test_a_block_that_the_target_all_but_excludes_is_not_accepted():
     rep, out, ref = run_both(inp)
     assert_parity(rep)
     assert (ref.tau == 0).all() and out.h[:, :, 0].max() < 1e-290
+
+
+_IN_A_PROCESS_OF_ITS_OWN = """
+import sys, torch
+sys.path.insert(0, {root!r})
+from paper_2604_25925_b200 import binding, sharded, workloads
+inp = workloads.make_inputs(workloads.VerifyConfig("window", B=2, K={K}, gamma={gamma}, V={V}, seed=1), device="cuda")
+if {ranks} > 1:
+    parts = [(inp.target_logits[..., lo:hi].contiguous(), inp.draft_logits[..., lo:hi].contiguous(), lo)
+             for lo, hi in sharded.shard_bounds({V}, {ranks})]
+    out = sharded.verify_all_ranks_on_one_device(parts, inp.draft_tokens, inp.uniforms, 1.0, {V})[0]
+else:
+    out = binding.sgbv_verify_ex(inp.target_logits, inp.draft_logits, inp.draft_tokens, inp.uniforms, 1.0)
+torch.cuda.synchronize()
+assert (out.status == 0).all()
+"""
+
+
+@pytest.mark.parametrize("K,gamma,V,ranks", [(17, 58, 256, 1), (41, 23, 256, 1), (16, 63, 600, 2), (35, 28, 600, 2), (40, 24, 600, 2)])
+def test_shared_memory_just_below_what_a_kernel_gets_without_asking(K, gamma, V, ranks):
+    """Draft counts and lengths for which the finishing kernel's or the sharded decision's dynamic shared memory is below 48 KB and
+    the sum with what the kernel declares itself above.  In a process of its own: one larger call asks for all later ones."""
+    code = _IN_A_PROCESS_OF_ITS_OWN.format(root=ROOT, K=K, gamma=gamma, V=V, ranks=ranks)
+    run = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr[-1500:]
 
 
 def test_unaligned_views_and_repeated_calls_are_deterministic():
