@@ -265,8 +265,11 @@ finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, const 
             };
             Pick p = pick_in_tile(x0, x1, sh_d[0], sh_d[1], wfun, sh_warp, sh_pick);
             y = (p.first != INT_MAX) ? p.first : p.last;
-        } else {
-            from_q = true;  // zero residual mass: draw from q of the same row
+        }
+        // Zero residual mass: draw from q of the same row.  So too where the mass is the rounding of q - c p and nothing of it is left
+        // when the cell is worked out again, relative to the row's references and not to the warp's.
+        if (uniform(y) < 0) {
+            from_q = true;
             flags |= SGBV_STATUS_DEGENERATE_RESIDUAL;
         }
     }
@@ -343,7 +346,8 @@ modify_finish_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all,
         };
         Pick pk = pick_in_tile(x0, x1, sc.d[0], sc.d[1], wfun, sc.warp, sc.pick);
         y = (pk.first != INT_MAX) ? pk.first : pk.last;
-    } else {  // no residual mass at all: the draw comes from q(.|s) itself
+    }
+    if (uniform(y) < 0) {  // no residual mass at all, or none that can be told from rounding: the draw comes from q(.|s) itself
         flags |= SGBV_STATUS_DEGENERATE_RESIDUAL;
         bool bad = false;
         float *tile_s = ws.bonus + (size_t)b * 2 * s.ntiles;

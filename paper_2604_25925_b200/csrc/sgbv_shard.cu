@@ -562,7 +562,8 @@ shard_draw_kernel(const T *__restrict__ zq_all, const T *__restrict__ zp_all, Sh
         };
         const Pick p = pick_in_tile(x0, x1, sc.d[0], sc.d[1], wfun, sc.warp, sc.pick);
         y = (p.first != INT_MAX) ? p.first : p.last;
-    } else {
+    }
+    if (uniform(y) < 0) {  // (also where the shard's residual mass is rounding, of which nothing is left when the cell is worked out again)
         bool bad = false;
         float *tile_s = bonus + (size_t)b * 2 * s.ntiles;
         y = draw_from_row<T>(zq, s, pl.frac, tile_s, tile_s + s.ntiles, &sc, bad);

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 import oracle
-from paper_2604_25925_b200 import binding, workloads
+from paper_2604_25925_b200 import binding, sharded, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -59,6 +59,39 @@ def test_modify_flags_and_degenerate_rows():
     assert (st == ref.status).all()
     assert st[1] & binding.STATUS_DEGENERATE_RESIDUAL and st[2] & binding.STATUS_NONFINITE_LOGIT
     assert out.token[2].item() == -1 and (out.token.cpu().numpy()[[0, 1, 3]] == ref.token[[0, 1, 3]]).all()
+
+
+@pytest.mark.parametrize("entry", ["modify", "verify", "sharded"])
+def test_a_residual_of_nothing_but_rounding_still_gives_a_token(entry):
+    """Rows of two entries in cells of their own, the draft's logits the target's plus 0.1 rounded to float32: q and p differ by
+    rounding, and what one kernel sees of max(q - p, 0) in a cell need not be there when the cell is worked out again.
+    Whatever is drawn is one of the two entries, and flagged if it came from q."""
+    B, V = 1 << 16, 512
+    g = torch.Generator().manual_seed(1)
+    q = torch.full((B, V), float("-inf"))
+    q[:, 3] = torch.randn(B, generator=g)
+    q[:, 300] = q[:, 3] - 3 * torch.rand(B, generator=g)
+    p, u = (q + 0.1).cuda(), torch.rand(B, 2, generator=g).cuda()
+    q = q.cuda()
+    zero = torch.zeros(B, dtype=torch.float64, device="cuda")
+    if entry == "modify":
+        out = binding.sgbv_modify(q, p, zero, zero, u[:, 1].contiguous(), 1, 1.0)
+        drawn, status = out.token, out.status
+    else:
+        target, draft = torch.stack([q, q], 1).view(B, 1, 2, V), p.view(B, 1, 1, V)
+        u[:, 0] = 1.0 - 2.0 ** -24                            # rejects whatever is not certain
+        tok = torch.where(q[:, 3:4] < -5.0, 3, 300).int().view(B, 1, 1)
+        tok[::2] = 3
+        if entry == "verify":
+            out = binding.sgbv_verify_ex(target, draft, tok, u, 1.0)
+        else:
+            parts = [(target[..., lo:lo + 256].contiguous(), draft[..., lo:lo + 256].contiguous(), lo) for lo in (0, 256)]
+            out = sharded.verify_all_ranks_on_one_device(parts, tok, u, 1.0, V)[0]
+        rejected = out.accept_len == 0
+        assert rejected.sum() > 100
+        drawn, status = out.tokens[rejected, 0], out.status[rejected]
+    assert ((drawn == 3) | (drawn == 300)).all(), int((drawn < 0).sum())
+    assert ((status & ~binding.STATUS_DEGENERATE_RESIDUAL) == 0).all()
 
 
 @pytest.mark.parametrize("V,dtype,shift", [(701, "fp32", 0), (40001, "bf16", 1), (40000, "fp32", 3), (151937, "bf16", 0)])
