@@ -369,6 +369,7 @@ __device__ __forceinline__ void set_references(FirstSweep &f, int j, float m1, f
     }
     // (the difference is what the exponent takes; b + rise would be rounded to a multiple of b's ulp, which may be as much as rise)
     if (!__any_sync(0xffffffffu, m1 - f.bq > rise || m2 - f.bp > rise)) return;
+    __syncwarp();  // (other lanes have read the words of the row before)
     if ((threadIdx.x & 31) == 0)
         for (int i = f.moved; i < j; ++i) refs[i] = make_float2(f.bq, f.bp);
     f.moved = j;
@@ -1108,6 +1109,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
                 const float2 own = lane < f.moved ? refs[lane] : make_float2(f.bq, f.bp);
                 refs[lane] = make_float2((own.x - f.bq) * s.scale, (own.y - f.bp) * s.scale);
             }
+            __syncwarp();  // (the combining warp comes to no block barrier before all its lanes read them)
         }
         const float bq_b = f.bq, bp_b = f.bp;
         fresh_row();

@@ -298,6 +298,25 @@ def test_extra_sums_in_kernels_of_their_own(K, dtype, alpha, T):
     np.testing.assert_allclose(res[2], res[1], rtol=2e-5, atol=1e-9)
 
 
+def _far_rows(B, V, K, dtype, kind):
+    cfg = workloads.VerifyConfig(f"far_{V}_{kind}", B=B, K=K, gamma=4, V=V, dtype=dtype, temperature=0.8, alpha=0.9, seed=V + K)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    x = torch.arange(V, device="cuda")
+    for t in (inp.target_logits, inp.draft_logits):
+        if kind == "ramp":
+            t += (5.0 * (x // 256)).to(t.dtype)
+        elif kind == "far":
+            t += 1.0e6
+        else:
+            for b, value in enumerate((float("-inf"), -1e9, torch.finfo(t.dtype).min)):
+                t[b::3, :, :, (x < V // 3 * (b + 1) // 2) & (x % 97 != 5)] = value
+    if kind == "ramp":
+        inp.draft_tokens.copy_(V - 1 - inp.draft_tokens % min(V, 150))
+    elif kind == "masked":
+        inp.draft_tokens.copy_((inp.draft_tokens % (V // 97)) * 97 + 5)
+    return inp
+
+
 @pytest.mark.parametrize("V,K,dtype,kind", [
     (200, 4, "fp32", "ramp"), (31 * 256, 1, "fp32", "ramp"), (31 * 256 + 1, 3, "bf16", "masked"), (32 * 256 + 8, 8, "bf16", "ramp"),
     (124 * 256, 4, "fp32", "masked"), (124 * 256 + 4, 2, "fp32", "ramp"), (125 * 256, 1, "bf16", "masked"), (128 * 256, 8, "fp32", "far"),
@@ -308,21 +327,7 @@ def test_logits_far_from_the_first_ones_of_a_row(V, K, dtype, kind):
     lowest value) but for an entry here and there, or a million from 0.  Two clusters walk all rows, so that every cell of a warp takes
     every place it can have, at the sizes where the cells per warp change.  Both tensors get the same offsets, and the
     draft tokens are entries that they leave likely."""
-    cfg = workloads.VerifyConfig(f"far_{V}_{kind}", B=3, K=K, gamma=4, V=V, dtype=dtype, temperature=0.8, alpha=0.9, seed=V + K)
-    inp = workloads.make_inputs(cfg, device="cuda")
-    x = torch.arange(V, device="cuda")
-    for t in (inp.target_logits, inp.draft_logits):
-        if kind == "ramp":
-            t += (5.0 * (x // 256)).to(t.dtype)
-        elif kind == "far":
-            t += 1.0e6
-        else:
-            for b, value in enumerate((float("-inf"), -1e9, torch.finfo(t.dtype).min)):
-                t[b, :, :, (x < V // 3 * (b + 1) // 2) & (x % 97 != 5)] = value
-    if kind == "ramp":
-        inp.draft_tokens.copy_(V - 1 - inp.draft_tokens % min(V, 150))
-    elif kind == "masked":
-        inp.draft_tokens.copy_((inp.draft_tokens % (V // 97)) * 97 + 5)
+    inp = _far_rows(3, V, K, dtype, kind)
     binding.set_option("walk", 1)
     binding.set_option("max_clusters", 2)
     try:
@@ -333,6 +338,28 @@ def test_logits_far_from_the_first_ones_of_a_row(V, K, dtype, kind):
         binding.set_option("max_clusters", 0)
     assert rep.decision_mismatches == 0 and rep.status_mismatches == 0, rep.detail
     assert rep.h_violations == 0 and rep.S_violations == 0, rep.detail
+
+
+@pytest.mark.parametrize("walk,aux", [(2, 0), (1, 1), (1, 2)])
+@pytest.mark.parametrize("V,K,dtype,kind", [
+    (31 * 256, 4, "fp32", "ramp"), (33 * 256, 1, "bf16", "masked"), (64 * 256 + 4, 2, "fp32", "ramp"), (128 * 256, 3, "fp32", "masked"),
+    (125 * 256, 8, "bf16", "ramp"), (97 * 256 + 8, 5, "bf16", "masked"), (40001, 4, "fp32", "masked"), (70001, 8, "fp32", "ramp"),
+])
+def test_references_that_move_in_both_walks_and_with_the_extra_sums(V, K, dtype, kind, walk, aux):
+    """The same kinds of rows in the row walk, where the combining warp has its share of the cells, and in the chain walk with the
+    extra sums of rows with c < 1 in the kernel and behind it."""
+    inp = _far_rows(6, V, K, dtype, kind)
+    options = {"walk": walk, "aux": aux, "cluster": 1 if V <= 128 * 256 else 0}
+    for name, value in options.items():
+        binding.set_option(name, value)
+    try:
+        rep, _, _ = run_both(inp)
+        assert binding.last_main_kernel() == "fused_chain_kernel"
+        assert binding.last_launch_count() == (4 if aux == 2 else 2)
+    finally:
+        for name in options:
+            binding.set_option(name, 0)
+    assert_parity(rep)
 
 
 @pytest.mark.parametrize("V,base,T,walk", [(124 * 256, 6e5, 0.01, 1), (124 * 256, 1e8, 1.0, 1), (128 * 256, -1e8, 1.0, 1), (124 * 256, 6e5, 0.01, 2),
