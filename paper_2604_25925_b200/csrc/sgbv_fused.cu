@@ -369,7 +369,6 @@ __device__ __forceinline__ void set_references(FirstSweep &f, int j, float m1, f
     }
     // (the difference is what the exponent takes; b + rise would be rounded to a multiple of b's ulp, which may be as much as rise)
     if (!__any_sync(0xffffffffu, m1 - f.bq > rise || m2 - f.bp > rise)) return;
-    __syncwarp();  // (other lanes have read the words of the row before)
     if ((threadIdx.x & 31) == 0)
         for (int i = f.moved; i < j; ++i) refs[i] = make_float2(f.bq, f.bp);
     f.moved = j;
@@ -504,12 +503,18 @@ __device__ __forceinline__ double unit_factor(float m, float row, float scale) {
     const double lo = fma(t2, c1, c0), mid = fma(t2, c3, c2), hi = fma(t2, c5, c4);
     return fma(t4, fma(t4, hi, mid), lo) * __hiloint2double((__double2loint(y) + 1023) << 20, 0);
 }
-// The same in float32: the difference and the product with what they were rounded by, so that what is left is the error of
-// ex2.approx, 2^-22, in factors other than 1.
+// (m - row) scale in float32, m <= row, and what the difference and the product were rounded by.
+__device__ __forceinline__ float unit_exponent(float m, float row, float scale, float &lost) {
+    const float d = row - m, x = d * -scale;
+    lost = fmaf(d, -scale, -x) - ((row - d) - m) * scale;
+    return x;
+}
+// unit_factor in float32, with what the exponent was rounded by, so that what is left is the error of ex2.approx, 2^-22, in factors
+// other than 1.
 __device__ __forceinline__ float unit_factor_f32(float m, float row, float scale) {
-    const float d = row - m, lost = (row - d) - m, x = d * -scale;
-    const float f = ex2(x);
-    return f > 0.0f ? fmaf(f, (fmaf(d, -scale, -x) - lost * scale) * 0.69314718f, f) : 0.0f;  // (0 x inf where m is -FLT_MAX)
+    float lost;
+    const float f = ex2(unit_exponent(m, row, scale, lost));
+    return f > 0.0f ? fmaf(f, lost * 0.69314718f, f) : 0.0f;  // (0 x inf where m is -FLT_MAX)
 }
 // Sum over the warp of values in [0, 2^17), rounded to multiples of 2^-28 (of 32 multiples each, which add up exactly): the parts above
 // and below 2^-5 as integers.  NaN if a lane's value is not in the range.
@@ -1122,11 +1127,16 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             rowv = ctl->rs;  // (the barrier statement is a compiler barrier for memory)
         }
         // this warp's units -> the row's; row B becomes row A
-        const float ref_q = (bq_b - rowv.x) * s.scale, ref_p = (bp_b - rowv.y) * s.scale;
-        rs.Fq = ex2_wide(ref_q);  // (not flushed below 2^-126: the warp's exponentials may be up to 2^kRise)
+        // (a factor is common to all of the warp's cells: its exponent's rounding, up to 2^-24 of the exponent, stays in their sums
+        // where that of single entries averages out)
+        float lost_q, lost_p;
+        const float ref_q = unit_exponent(bq_b, rowv.x, s.scale, lost_q), ref_p = unit_exponent(bp_b, rowv.y, s.scale, lost_p);
+        const float f_q = ex2_wide(ref_q);  // (not flushed below 2^-126: the warp's exponentials may be up to 2^kRise)
+        rs.Fq = f_q > 0.0f ? fmaf(f_q, lost_q * 0.69314718f, f_q) : 0.0f;
         // equal references (identical rows above all) must give kappa itself: p = q everywhere then leaves an
         // exactly zero residual.  Finite: 0 x inf would take the weight of an entry with p = 0
-        rs.KF = fminf(rowv.z * ex2(ref_p - ref_q), FLT_MAX);
+        const float ref_pq = ref_p - ref_q, f_pq = ex2(ref_pq), lost_pq = (ref_p - (ref_q + ref_pq)) + (lost_p - lost_q);
+        rs.KF = f_pq > 0.0f ? fminf(rowv.z * fmaf(f_pq, lost_pq * 0.69314718f, f_pq), FLT_MAX) : 0.0f;
         rs.kFp = p.aux_here ? rowv.z * ex2(ref_p) : 0.0f;
         rs.c = rowv.w;
         r_a = r_b;

@@ -399,6 +399,34 @@ def test_references_move_by_differences_that_a_sum_rounds_away(V, base, T, walk)
     torch.testing.assert_close(a.resmass, b.resmass, rtol=2e-5, atol=0)
 
 
+@pytest.mark.parametrize("V", [31 * 256, 31 * 256 + 1])
+def test_factors_between_units_far_apart(V):
+    """One entry D nats above all others, which the draft covers: the residual mass lies in warps whose references are 21 to 65 powers
+    of two below the row's.  A float32 exponent of that size is rounded by up to 2^-19 (2.6e-6 of the factor); ex2.approx itself and
+    the float32 scalars of a row are good to 2^-22 each (2.4e-7): 6e-7 for the mass, whose terms carry three of them.  scale is
+    the float32 that the kernels are given."""
+    B, K = 48, 4
+    g = torch.Generator().manual_seed(7)
+    zq = torch.randn(B, V, generator=g)
+    zp = zq + 0.7 * torch.randn(B, V, generator=g)
+    zq[:, 5] = zp[:, 5] = torch.linspace(15.0, 45.0, B) + 0.01 * torch.randn(B, generator=g)
+    binding.set_option("path", 2)
+    binding.set_option("cluster", 1)
+    try:
+        target = torch.stack([zq, zq], 1).view(B, 1, 2, V).expand(B, K, 2, V).contiguous().cuda()
+        draft = zp.view(B, 1, 1, V).expand(B, K, 1, V).contiguous().cuda()
+        out = binding.sgbv_verify_ex(target, draft, torch.full((B, K, 1), 5, dtype=torch.int32, device="cuda"),
+                                     torch.full((B, K + 1), 0.5, device="cuda"), 1.0)
+    finally:
+        binding.set_option("path", 0)
+        binding.set_option("cluster", 0)
+    scale = np.float64(np.float32(1.4426950408889634))
+    q, p = (np.exp2((z.numpy().astype(np.float64) - z.numpy().max(1, keepdims=True)) * scale) for z in (zq, zp))
+    q, p = q / q.sum(1, keepdims=True), p / p.sum(1, keepdims=True)
+    want = (q * np.maximum(1.0 - p / q, 0.0) ** K).sum(1)
+    np.testing.assert_allclose(out.resmass[:, 0, 0].cpu().numpy(), want, rtol=6e-7)
+
+
 def _all_but_excluded(T=0.05):
     """Draft blocks whose first token has a target log-probability from -700 to -760 and a draft probability near 1: a = q(x^i) goes
     through the smallest normal float64 number, the denormal ones (where c = p/q overflows) and 0.  Other rows are flat."""
