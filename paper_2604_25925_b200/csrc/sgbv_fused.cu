@@ -1355,9 +1355,10 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
     // (with one draft the extra sum costs the kernel next to nothing, and most rows with c < 1 would be listed; rows that start
     // anywhere included: error of the weights against 64 bits with the sums here / apart 4.1e-8 / 5.7e-8 at 64 x 8 x 6 x 50257
     // bfloat16, 5.9e-8 / 1.0e-7 at 64 x 2 x 12 x 100003, where the two-sweep path has 1.6e-7 and 4.0e-7)
-    // (bfloat16 with many drafts: the sums cost most there, and memory hides none of it.  In this kernel / apart, us: 16 x 8 x 4 x 151936
-    // 160 / 146, 64 x 8 x 4 x 32000 117 / 107; float32 32 x 8 x 12 x 32000 158 / 158; K = 4 bfloat16 16 x 4 x 5 x 128256 87 / 90.)
-    const bool apart = bytes >= kAuxApartMinBytes || (sizeof(T) == 2 && s.K >= 6 && bytes >= kAuxApartMinBytes / 10);
+    // (Apart, rows whose numerator does not cancel take its plain form, which costs them up to a bit, and some of the error: bfloat16 with
+    // many drafts would be faster apart from 100 MB on, 16 x 8 x 4 x 151936 148 / 140 us, 64 x 6 x 8 x 32000 220 / 170, but the 2-norm of the
+    // weights' error there is 5.5e-8 / 6.5e-8 and 6.9e-8 / 7.4e-8.)
+    const bool apart = bytes >= kAuxApartMinBytes;
     const bool aux_here = plan.row_mode || g_opt_aux == 1 || (g_opt_aux == 0 && (!apart || s.K == 1));
     *aux_apart = !aux_here;
     return plan.row_mode ? launch_as<T, true, KT, kAny>(L, plan, error_flag, clusters, true, *words_used)

@@ -298,6 +298,24 @@ def test_extra_sums_in_kernels_of_their_own(K, dtype, alpha, T):
     np.testing.assert_allclose(res[2], res[1], rtol=2e-5, atol=1e-9)
 
 
+@pytest.mark.parametrize("B,K,gamma,V,dtype,launches", [
+    (16, 8, 4, 98304, "bf16", 2), (64, 6, 2, 50304, "bf16", 2), (64, 7, 1, 100352, "bf16", 2), (16, 8, 4, 98304, "fp32", 2),
+    (43, 8, 8, 98304, "bf16", 4), (43, 4, 8, 98304, "fp32", 4),     # 1.08e9 bytes: just above 2^30
+    (42, 8, 8, 98304, "bf16", 2), (42, 4, 8, 98304, "fp32", 2),     # 1.06e9
+    (86, 1, 16, 98304, "fp32", 2),                                  # one draft: in the kernel at any size
+])
+def test_where_the_extra_sums_are_worked_out(B, K, gamma, V, dtype, launches):
+    """Kernels of their own (two more launches) for the extra sums of rows with c < 1: from 1 GB of logits on and not below, at any
+    type and number of drafts but one."""
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    target = torch.zeros(B, K, gamma + 1, V, dtype=dt, device="cuda")
+    draft = torch.zeros(B, K, gamma, V, dtype=dt, device="cuda")
+    binding.sgbv_verify_ex(target, draft, torch.zeros(B, K, gamma, dtype=torch.int32, device="cuda"),
+                           torch.full((B, K * gamma + 1), 0.5, device="cuda"), 1.0)
+    torch.cuda.synchronize()
+    assert binding.last_main_kernel() == "fused_chain_kernel" and binding.last_launch_count() == launches
+
+
 def _far_rows(B, V, K, dtype, kind):
     cfg = workloads.VerifyConfig(f"far_{V}_{kind}", B=B, K=K, gamma=4, V=V, dtype=dtype, temperature=0.8, alpha=0.9, seed=V + K)
     inp = workloads.make_inputs(cfg, device="cuda")
