@@ -30,9 +30,9 @@ constexpr size_t kSmemWithoutAsking = 46 * 1024;
 struct RowInfo {
     double Zq;      // sum_x exp((zq_x - mq)/T)
     double Zp;
-    float mq;       // row maxima of the raw logits
-    float mp;
-    float kappa;    // c * Zq / Zp with c = b/a: ratio c*p(x)/q(x) = kappa * ep/eq in row-max units
+    float mq;       // the rows' references: their largest logits on the two-sweep and the sharded path; on the streaming path the
+    float mp;       // largest reference of a warp, which a row's maximum may exceed by a factor of 2^kRise in the exponentials
+    float kappa;    // c * Zq / Zp with c = b/a: ratio c*p(x)/q(x) = kappa * ep/eq in units of the references
     float c;        // c = p(x_k^i)/q(x_k^i), ratio of the joint prefix probabilities (c < 1 selects
                     // the cancellation-free numerator)
     int32_t flags;  // SGBV_STATUS_NONFINITE_LOGIT if the streaming pass found the row pair unusable
@@ -141,7 +141,7 @@ __device__ __forceinline__ float2 ipow2(float2 r, int K) {
 // exp((z - m)/T) as 2^((z-m)*scale).
 __device__ __forceinline__ float expo(float z, float m, float scale) { return exp2f((z - m) * scale); }
 
-// One vocabulary element of the coupling sums, in row-max units (eq = exp((zq-mq)/T) etc.).
+// One vocabulary element of the coupling sums, in units of the row's references (eq = exp((zq-mq)/T) etc., which may be above 1: RowInfo).
 //   w  = eq * max(1 - kappa*ep/eq, 0)^K       -> sum/Zq = R_i, and w is Eq. 4's weight
 //   dp = max(kappa*ep - eq, 0)                 -> sum/Zq = sum_x max(c p - q, 0)
 //   m2 = eq * (c - t)^2 * Q(t), t = min(kappa*ep/eq, 1),

@@ -1,6 +1,6 @@
 // Finishing kernel: one CTA of 1024 threads per batch row.
 //   0. log a_i = log q(x_k^i), log b_i = log p(x_k^i) of every draft by running sums of the token
-//      log-probabilities (row maxima and normalisers come from the streaming pass);
+//      log-probabilities (the rows' references and normalisers come from the streaming pass);
 //   1. combine the cached per-tile sums of every (k,i) row into S_i and the acceptance weights
 //      (Eq. 2 for proper sub-blocks, Eq. 3 for the whole block), in float64;
 //   2. the scan of Algorithm 1 over drafts and positions with the pre-drawn uniforms;

@@ -194,7 +194,7 @@ __device__ __forceinline__ void tmem_wait_ld(float2 (&a)[4], float2 (&b)[4]) {
 // [rings: 32 warps x slots x (cell of zq, cell of zp)] [full barriers: 32 warps x slots] [Control]
 struct Control {
     uint64_t xbar[2];                    // by row parity: "the partials of all CTAs of the cluster are here"
-    // partials (maximum of zq, sum eq, maximum of zp, sum ep): of this CTA's warps, and, double-buffered by
+    // partials (reference of zq, sum eq, reference of zp, sum ep): of this CTA's warps, and, double-buffered by
     // row parity, of every CTA of the cluster (pushed by their owners)
     float4 wslots[kMaxWarps];
     float4 slots[2][kMaxCluster];
@@ -491,7 +491,7 @@ __device__ __forceinline__ void second_sweep_cell(uint32_t taddr_cell, bool park
     }
 }
 
-// 2^((m - row) scale), m <= row: the factor that moves a sum from units of the maximum m to units of the row's, in float64.
+// 2^((m - row) scale), m <= row: the factor that moves a sum from units of the reference m to units of the row's, in float64.
 __device__ __forceinline__ double unit_factor(float m, float row, float scale) {
     // e^(f ln 2), |f| <= 1/2, by its Taylor series to degree 11 (remainder below 7e-15), in pairs and without a branch: behind
     // exp2_short's the lanes ran apart and the shuffles of the sums took 1.1 us more per row
@@ -526,8 +526,8 @@ __device__ __forceinline__ double warp_sum_fixed(float v) {
     const double sum = fma((double)h, 1.0 / 32.0, (double)l * (1.0 / 268435456.0));
     return __any_sync(0xffffffffu, !(v < 131072.0f)) ? (double)NAN : sum;
 }
-// 1/x for x in the range of normal float32 numbers: the hardware's float32 reciprocal and one step of Newton's method (relative
-// error below 2e-14).  NaN for 0 and inf.
+// 1/x for x in the range of normal float32 numbers: the hardware's float32 reciprocal and one step of Newton's method, which squares
+// its error: at most 2^-24 from x's conversion and 2^-23 from rcp.approx, 1.8e-7, so 3.2e-14 is left.  NaN for 0 and inf.
 __device__ __forceinline__ double reciprocal(double x) {
     const double r = (double)rcp((float)x);
     return fma(r, fma(-x, r, 1.0), r);
@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
             }
         }
         if (lane == 0 && rank == 0) {
-            // nonfinite logits: NaN poisons Z, +inf shows up as an infinite maximum, a row of
+            // nonfinite logits: NaN poisons Z, +inf shows up as an infinite reference, a row of
             // -inf only has Z = 0
             const bool bad = !(Zq > 0.0f) || !(Zp > 0.0f) || !(Zq < (double)INFINITY) || !(Zp < (double)INFINITY) ||
                              !(bq_row < INFINITY) || !(bp_row < INFINITY);
