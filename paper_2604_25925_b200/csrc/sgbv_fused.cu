@@ -39,17 +39,15 @@ namespace sgbv {
 
 namespace {
 
-constexpr int kMaxWarps = 32;              // warps per CTA: 32 (64 registers each) or 16 (128 registers each)
 constexpr int kCell = kTile;               // 256 contiguous entries: the unit a warp works on
-constexpr int kCtasPerSm = 1;              // CTAs that share an SM (1 or 2): two are in different phases of their rows
-                                           // most of the time, so that one's exponentials overlap the other's sums
-constexpr int kWarps = 32;                 // warps per CTA (16 warps of 128 registers measured a third slower)
-constexpr int kCtaCells = 128 / kCtasPerSm;  // cells of a row per CTA: 16 tensor-memory columns per cell in each of the 4
+constexpr int kWarps = 32;                 // warps per CTA, one CTA per SM (16 warps of 128 registers, or two CTAs of 16, measured slower)
+constexpr int kCtaThreads = kWarps * 32;
+constexpr int kCtaCells = 128;             // cells of a row per CTA: 16 tensor-memory columns per cell in each of the 4
                                            // lane quarters, 512 columns per SM: 128 cells = 32,768 entries per SM
 constexpr int kSlack = 16;  // extra bytes per cell and tensor in a slot when rows start anywhere: a copy then begins at the
                            // 16-byte boundary before the cell and ends behind it
 constexpr int kParkBytes = kCell * 2 * (int)sizeof(float);  // the exponentials of one cell of both tensors, a warp's parked first cell
-constexpr int kTmemCols = 512 / kCtasPerSm;  // this CTA's share of the SM's tensor memory
+constexpr int kTmemCols = 512;             // all of the SM's tensor memory
 constexpr int kMaxCluster = 8;  // CTAs per cluster (beyond 8 the size is not portable, which sm_100 allows)
 constexpr long long kWaitLimitCycles = 2000000000ll;  // about one second of SM clock
 constexpr uint32_t kPollNs = 100u;                    // sleep between two tests of a barrier that is not ready
@@ -196,7 +194,7 @@ struct Control {
     uint64_t xbar[2];                    // by row parity: "the partials of all CTAs of the cluster are here"
     // partials (reference of zq, sum eq, reference of zp, sum ep): of this CTA's warps, and, double-buffered by
     // row parity, of every CTA of the cluster (pushed by their owners)
-    float4 wslots[kMaxWarps];
+    float4 wslots[kWarps];
     float4 slots[2][kMaxCluster];
     float4 low[2][kMaxCluster];          // what the sums in `slots` were rounded by (y, w)
     float4 rs;                           // the row's scalars for the second sweep: rq, rp, kappa, c
@@ -540,12 +538,12 @@ __device__ __forceinline__ double reciprocal(double x) {
 // (fused_outrun): 16 prompts, K = 4, gamma = 4, V = 50257 bfloat16 105 us against 63 here, one prompt at V = 32001 float32 68 and 20,
 // 64 prompts, K = 2 at V = 128255 float32 510 and 200.
 // Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4, and mbarriers for its copies.
-// W warps per CTA; NS ring slots per warp (the cells per warp and row, kCtaCells / W, are a multiple of it, so
+// NS: ring slots per warp (the cells per warp and row, kCtaCells / kWarps, are a multiple of it, so
 // that cell j of a row always sits in slot j % NS); KT: the number of drafts K when it has a specialised
 // second sweep (1, 2, 3, 4, 8), else 0 (any K, loops).
-template <typename T, bool kRow, int W, int NS, int KT, bool kAny>
-__global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const FusedParams p) {
-    constexpr int kFWarps = W, kFThreads = W * 32, kCellsPerWarp = kCtaCells / W;
+template <typename T, bool kRow, int NS, int KT, bool kAny>
+__global__ void __launch_bounds__(kCtaThreads, 1) fused_chain_kernel(const FusedParams p) {
+    constexpr int kCellsPerWarp = kCtaCells / kWarps;
     static_assert(kCellsPerWarp % NS == 0, "cell j of a row must always land in slot j % NS");
     extern __shared__ __align__(1024) unsigned char smem[];
     const Shape &s = p.s;
@@ -558,16 +556,16 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     constexpr int kHalfBytes = kCell * (int)sizeof(T);  // one tensor's cell
     constexpr int kHalfSlot = kHalfBytes + (kAny ? kSlack : 0);
     constexpr int kSlotBytes = 2 * kHalfSlot;           // the cell of zq, then the same cell of zp
-    constexpr int kStride = kAny ? kFWarps : 1;  // from one cell of a warp to its next, in a row
-    constexpr int kRingBytes = kFWarps * NS * kSlotBytes;
+    constexpr int kStride = kAny ? kWarps : 1;  // from one cell of a warp to its next, in a row
+    constexpr int kRingBytes = kWarps * NS * kSlotBytes;
     // [rings][full barriers][references of the cells][parked first cells][Control]
     const unsigned char *ring = smem + (size_t)warp * NS * kSlotBytes;
     const uint32_t ring_u32 = smem_u32(ring);
     uint32_t pieces_u32 = ring_u32 + (uint32_t)lane * 16u;
     const uint32_t full_u32 = smem_u32(smem) + (uint32_t)(kRingBytes + warp * NS * 8);
-    float2 *refs = reinterpret_cast<float2 *>(smem + kRingBytes + kFWarps * NS * 8) + warp * kCellsPerWarp;
-    float4 *park = reinterpret_cast<float4 *>(smem + kRingBytes + kFWarps * NS * 8 + kCtaCells * (int)sizeof(float2)) + warp * 128 + lane;  // stride 32
-    Control *ctl = reinterpret_cast<Control *>(smem + kRingBytes + kFWarps * NS * 8 + kCtaCells * (int)sizeof(float2) + kFWarps * kParkBytes);
+    float2 *refs = reinterpret_cast<float2 *>(smem + kRingBytes + kWarps * NS * 8) + warp * kCellsPerWarp;
+    float4 *park = reinterpret_cast<float4 *>(smem + kRingBytes + kWarps * NS * 8 + kCtaCells * (int)sizeof(float2)) + warp * 128 + lane;  // stride 32
+    Control *ctl = reinterpret_cast<Control *>(smem + kRingBytes + kWarps * NS * 8 + kCtaCells * (int)sizeof(float2) + kWarps * kParkBytes);
     const uint32_t xbar_u32 = smem_u32(&ctl->xbar[0]);
 
     // This CTA's slice of the vocabulary, and this warp's cells in it: a few neighbours each.  The last warp, which does the exchange
@@ -575,18 +573,18 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
     const int cell_begin = rank * p.slice_cells;
     const int ncells_cta = max(0, min(s.ntiles, cell_begin + p.slice_cells) - cell_begin);
     // (In the row walk, where one row is all that most clusters have, the cells are shared out evenly.)
-    const int most = kRow ? (ncells_cta + kFWarps - 1) / kFWarps : kCellsPerWarp;
-    const int rest = max(0, ncells_cta - most * (kFWarps - 1));  // of the last warp
-    const int each = (ncells_cta - rest) / (kFWarps - 1), more_by_one = (ncells_cta - rest) % (kFWarps - 1);
+    const int most = kRow ? (ncells_cta + kWarps - 1) / kWarps : kCellsPerWarp;
+    const int rest = max(0, ncells_cta - most * (kWarps - 1));  // of the last warp
+    const int each = (ncells_cta - rest) / (kWarps - 1), more_by_one = (ncells_cta - rest) % (kWarps - 1);
     // (rows that start anywhere: cells w, w + 32, ... of the slice for warp w; of the last warp's, those that fit go one each to
     // the first warps that would have one cell fewer than others)
-    const int columns = ncells_cta / kFWarps, odd = ncells_cta % kFWarps, given = odd > 0 ? min(columns, kFWarps - 1 - odd) : 0;
+    const int columns = ncells_cta / kWarps, odd = ncells_cta % kWarps, given = odd > 0 ? min(columns, kWarps - 1 - odd) : 0;
     const int own_cells = columns + (warp < odd), extra = kAny && warp >= odd && warp < odd + given ? warp - odd : -1;
-    int ncw = !kAny ? (warp == kFWarps - 1 ? rest : each + (warp < more_by_one))  // cells of this warp per row
-                    : warp == kFWarps - 1 ? columns - given : own_cells + (extra >= 0);
-    const int first_cell = cell_begin + (kAny ? (warp == kFWarps - 1 ? warp + given * kFWarps : warp) : warp == kFWarps - 1 ? ncells_cta - rest : warp * each + min(warp, more_by_one));
+    int ncw = !kAny ? (warp == kWarps - 1 ? rest : each + (warp < more_by_one))  // cells of this warp per row
+                    : warp == kWarps - 1 ? columns - given : own_cells + (extra >= 0);
+    const int first_cell = cell_begin + (kAny ? (warp == kWarps - 1 ? warp + given * kWarps : warp) : warp == kWarps - 1 ? ncells_cta - rest : warp * each + min(warp, more_by_one));
     // cell j of this warp, counted from its first one
-    const int extra_j = extra >= 0 ? own_cells : -1, extra_at = kFWarps - 1 + extra * kFWarps - warp;
+    const int extra_j = extra >= 0 ? own_cells : -1, extra_at = kWarps - 1 + extra * kWarps - warp;
     auto cell_at = [&](int j) { return kAny && j == extra_j ? extra_at : j * kStride; };
     // the row's last cell may be a partial one: which of this warp's cells it is (-1: none), and its entries
     const int tail_valid = s.V - (s.ntiles - 1) * kCell;
@@ -739,7 +737,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
 
     // The last warp of this CTA combines the partials, carries c_i and fetches the token logits of a row ahead of its exchange
     // (every lane the same words).
-    const bool combiner = warp == kFWarps - 1;
+    const bool combiner = warp == kWarps - 1;
     // c at the start of chain bk: 1, or exp(log p(s) - log q(s)) of what Algorithm 2 carries in
 #define SGBV_C0(BK) (p.carry_loga ? exp_short(p.carry_logb[BK] - p.carry_loga[BK]) : 1.0)
     double c_carry = 1.0;  // chain walk: c of the row whose exchange comes next (the first row of the walk starts a chain)
@@ -759,8 +757,8 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         const int par = pos & 1;
         const uint32_t xph = (uint32_t)(pos >> 1) & 1u;
         const uint32_t xbar = xbar_u32 + 8u * (uint32_t)par;
-        bar_sync(1, kFThreads);
-        const float4 v = lane < kFWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+        bar_sync(1, kCtaThreads);
+        const float4 v = lane < kWarps ? ctl->wslots[lane] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
         float bq_row = warp_max_redux(v.x), bp_row = warp_max_redux(v.z);
         float rq_row = (bq_row > -INFINITY) ? bq_row : 0.0f, rp_row = (bp_row > -INFINITY) ? bp_row : 0.0f;
         // The sum over the lanes of z, each moved from units of m to units of `row` (-inf: a lane without a share).  Every cycle from
@@ -853,7 +851,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         const float4 rowv = make_float4(rq_row, rp_row, (float)(cd * Zratio), (float)cd);
         if (lane == 0) ctl->rs = rowv;
         __syncwarp();
-        bar_arrive(2, kFThreads);
+        bar_arrive(2, kCtaThreads);
         // off the critical path: c of the next row of the chain walk (c_{i+1} = c_i ratio, and 1 at the start of
         // the next chain), and the row's record for the finishing kernel
         if (!row_mode) {
@@ -1102,7 +1100,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         __syncwarp();
         float4 rowv;  // rq, rp, kappa, c
         if (!combiner) {
-            bar_arrive(1, kFThreads);
+            bar_arrive(1, kCtaThreads);
         } else {
             rowv = exchange(n + 1, r_b, i_b, has_d, r_d, i_d, chains_on);
         }
@@ -1123,7 +1121,7 @@ __global__ void __launch_bounds__(W * 32, kCtasPerSm) fused_chain_kernel(const F
         tmem_wait_st();
         next_place();  // of row B's first cell
         if (!combiner) {
-            bar_sync(2, kFThreads);
+            bar_sync(2, kCtaThreads);
             rowv = ctl->rs;  // (the barrier statement is a compiler barrier for memory)
         }
         // this warp's units -> the row's; row B becomes row A
@@ -1176,14 +1174,14 @@ int g_opt_withhold = 0;
 int g_opt_aux = 0;         // 0 = automatic, 1 = the extra sums of rows with c < 1 in the streaming kernel, 2 = in kernels of their own
 constexpr double kAuxApartMinBytes = 1024.0 * 1024 * 1024;
 
-constexpr int kSmemPerCta = (228 * 1024) / kCtasPerSm - 1024;  // largest dynamic shared memory of one CTA
+constexpr int kSmemPerCta = 227 * 1024;  // largest dynamic shared memory of one CTA
 constexpr int kDevices = 64;
 std::mutex g_plan_mu;      // guards the options and the per-device caches below
 
-constexpr int kCtaSlots = 148 * kCtasPerSm;  // CTAs the device holds
+constexpr int kCtaSlots = 148;  // CTAs the device holds
 // ring slots per warp: half a row's cells for float32 (128 KB of copies under way per SM), all of them for bfloat16
 template <typename T>
-constexpr int slots_for() { return (sizeof(T) == 4 ? 2 : 4) * 32 / kWarps / kCtasPerSm; }
+constexpr int slots_for() { return sizeof(T) == 4 ? 2 : 4; }
 template <typename T, bool kAny>
 constexpr size_t smem_bytes() {
     return (size_t)kWarps * slots_for<T>() * (2 * (kCell * sizeof(T) + (kAny ? kSlack : 0)) + 8) + (size_t)kCtaCells * sizeof(float2) + (size_t)kWarps * kParkBytes + sizeof(Control);
@@ -1194,9 +1192,9 @@ template <typename T, bool kRow, int KT, bool kAny>
 cudaError_t prepare(int dev) {
     static bool attr_done[kDevices];
     if (!attr_done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
+        cudaError_t e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, slots_for<T>(), KT, kAny>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerCta);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        e = cudaFuncSetAttribute(fused_chain_kernel<T, kRow, slots_for<T>(), KT, kAny>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         attr_done[dev] = true;
     }
@@ -1210,7 +1208,7 @@ int resident_clusters(int dev, int C) {
     int &slot = cached[dev][C];
     if (slot == 0) {
         cudaLaunchConfig_t cfg = {};
-        cfg.blockDim = dim3(kWarps * 32);
+        cfg.blockDim = dim3(kCtaThreads);
         cfg.dynamicSmemBytes = smem_bytes<T, kAny>();
         cfg.gridDim = dim3(C * (kCtaSlots / C));
         cudaLaunchAttribute attr[1];
@@ -1221,7 +1219,7 @@ int resident_clusters(int dev, int C) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int nmax = 0;
-        if (cudaOccupancyMaxActiveClusters(&nmax, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, &cfg) != cudaSuccess || nmax < 1) {
+        if (cudaOccupancyMaxActiveClusters(&nmax, fused_chain_kernel<T, kRow, slots_for<T>(), KT, kAny>, &cfg) != cudaSuccess || nmax < 1) {
             cudaGetLastError();
             return 0;
         }
@@ -1250,7 +1248,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
     fp.aux_here = aux_here ? 1 : 0;
 
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kWarps * 32);
+    cfg.blockDim = dim3(kCtaThreads);
     cfg.dynamicSmemBytes = smem_bytes<T, kAny>();
     cfg.stream = L.stream;
     cudaLaunchAttribute attr[2];
@@ -1275,7 +1273,7 @@ int launch_as(const Launch &L, const Plan &plan, int *error_flag, int clusters, 
         cudaMemsetAsync(L.ws.ratio, 0xff, (size_t)words_used * sizeof(double), L.stream) != cudaSuccess)
         return SGBV_ERR_CUDA;
     if (L.ev_begin) cudaEventRecord(L.ev_begin, L.stream);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_chain_kernel<T, kRow, kWarps, slots_for<T>(), KT, kAny>, fp);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_chain_kernel<T, kRow, slots_for<T>(), KT, kAny>, fp);
     if (L.ev_end) cudaEventRecord(L.ev_end, L.stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
