@@ -18,10 +18,11 @@
 // The joint likelihood ratio c_i = p(x^i)/q(x^i) is carried as a running product by the last warp, which works c_{i+1} out
 // right after the release of row i.  The finishing kernel (weights, scan, extra token) consumes the cell sums.
 //
-// What bounds it: the special-function unit (3.1 of its instructions per pair, 62 % of its rate at 16 x 8 x 8 x 151936 float32) and
-// the exchange, during which most of the SM waits; up to there float32 rows, HBM.  Steps, us, before / now (one B200, streaming
-// kernel and the kernels behind it): 64 x 8 x 8 x 151936 float32 1087 / 818, 256 x 8 x 4 x 32000 float32 396 / 360,
-// 32 x 4 x 5 x 128256 bfloat16 169 / 128, 256 x 1 x 4 x 32000 float32 81 / 70.  Warp instructions per 32 pairs 34 / 25.6.
+// What bounds it: the special-function unit (3.1 of its instructions per pair, 63 % of its rate at 16 x 8 x 8 x 151936 float32) and
+// the exchange, during which most of the SM waits; up to there float32 rows, HBM.  Whole calls one after the other, us, with references
+// per thread and cell / per warp (one B200): 64 x 8 x 8 x 151936 float32 1140 / 951 (bursts of 140 calls, before the power limit counts:
+// 820), 256 x 8 x 4 x 32000 float32 437 / 376, 32 x 4 x 5 x 128256 bfloat16 180 / 138, 256 x 1 x 4 x 32000 float32 80 / 68.  Warp
+// instructions per 32 pairs 34.1 / 26.3 (16 x 8 x 8 x 151936 float32).
 //
 // Every wait on an mbarrier or on a word in global memory is bounded; on expiry the warp records
 // an error flag and keeps executing the protocol, so a lost copy cannot hang the kernel, and the
@@ -535,8 +536,8 @@ __device__ __forceinline__ double reciprocal(double x) {
 // 16-byte pieces that hold the cell, and the reads from shared memory start at the remainder.  The few cells at the ends of the
 // tensors whose pieces reach past them are loaded directly.
 // Two sweeps over such rows (three scalar reads of every logit, four kernels) take longer, unless the rows are short and many
-// (fused_outrun): 16 prompts, K = 4, gamma = 4, V = 50257 bfloat16 105 us against 63 here, one prompt at V = 32001 float32 68 and 20,
-// 64 prompts, K = 2 at V = 128255 float32 510 and 200.
+// (fused_outrun): 16 prompts, K = 4, gamma = 4, V = 50257 bfloat16 93 us against 55 here, one prompt, K = 3, gamma = 12, V = 32001
+// float32 104 and 26, 64 prompts, K = 2, gamma = 4, V = 128255 float32 499 and 190.
 // Against rows that start on the boundaries it costs 16 loads per lane and cell instead of 2 or 4, and mbarriers for its copies.
 // NS: ring slots per warp (the cells per warp and row, kCtaCells / kWarps, are a multiple of it, so
 // that cell j of a row always sits in slot j % NS); KT: the number of drafts K when it has a specialised
@@ -1322,7 +1323,7 @@ int plan_and_launch(const Launch &L, int *error_flag, int *words_used, bool *aux
     }
     // A few rounds of rows: what counts is the number of rounds times the time of a row, some 3 us and 48 ns for each of a CTA's
     // cells.  (64 rows of 594 cells: clusters of five 26 at a time, three rounds, of six 24, three shorter ones: 39.6 -> 36.8 us.  Long
-    // walks are bound by throughput, and the smallest cluster is best: 64 x 8 x 8 rows of that length 818 us, of six 932.)
+    // walks are bound by throughput, and the smallest cluster is best: 64 x 8 x 8 rows of that length 821 us, of six 996.)
     if (!g_opt_cluster && !plan.row_mode && fits(C) && g_opt_max_clusters == 0) {
         auto cost = [&](int c) {
             const long side_by_side = std::min<long>(resident(c, false), nchains);
@@ -1387,11 +1388,12 @@ bool fused_supported(const Launch &L) { return L.s.ntiles <= kMaxCluster * kCtaC
 // Whether the two-sweep kernels are the faster ones: many short rows that start anywhere.  A row costs a cluster some 2.5 us
 // however short it is, and a cluster walks its rows one after the other, where the two-sweep kernels run all rows side by side
 // and pay by the entry (three scalar reads, and the power of Eq. 2 in a loop where K has no kernel of its own).  Two sweeps :
-// streaming, us, bfloat16 (float32): 1024 rows (64 x 4 x 4) of 4 cells 40 : 43 (38 : 43), of 17 cells 50 : 47 (47 : 45); 8192 rows
-// (256 x 8 x 4) of 4 cells 82 : 222 (82 : 220), 17 cells 182 : 247 (189 : 245), 25 cells 243 : 264 (257 : 261), 32 cells 308 : 295
-// (327 : 285).  One position (1024 x 1 x 1): 4 cells 40 : 51 (41 : 49), 17 cells 49 : 54 (48 : 52), 29 cells 58 : 58 (60 : 57);
-// 512 rows (64 x 8 x 1) of 4 cells 32 : 33 (30 : 33), of 13 cells 36 : 34 (34 : 34).  K = 5, 3840 rows of 7 cells 85 : 119
-// (87 : 117), of 13 cells 106 : 124 (152 : 129).  Rows on the boundaries (16-byte reads) stay with the streaming kernel at any
+// streaming, us, bfloat16 (float32): 1024 rows (64 x 4 x 4) of 4 cells 43 : 49 (44 : 47), of 12 cells 51 : 50 (47 : 48), of 17 cells
+// 53 : 51 (51 : 49); 8192 rows (256 x 8 x 4) of 4 cells 85 : 245 (86 : 218), 17 cells 196 : 267 (215 : 252), 24 cells 249 : 274
+// (270 : 262), 29 cells 286 : 285 (318 : 276).  One position (1024 x 1 x 1): 4 cells 40 : 51 (40 : 50), 20 cells 54 : 55 (54 : 53), 25
+// cells 57 : 56 (59 : 55); 512 rows (64 x 8 x 1) of 4 cells 34 : 36 (34 : 34), of 9 cells 37 : 36 (35 : 34), of 17 cells 41 : 37 (39 : 36).
+// K = 5, 3840 rows of 7 cells 69 : 134 (72 : 124), of 13 cells 92 : 138 (138 : 145), of 17 cells 110 : 142 (176 : 152): the line lies at
+// 9 cells there, which leaves up to 12 cells of bfloat16 something to gain.  Rows on the boundaries (16-byte reads) stay with the streaming kernel at any
 // length, as before.
 bool fused_outrun(const Launch &L) {
     const Shape &s = L.s;

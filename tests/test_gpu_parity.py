@@ -421,8 +421,8 @@ def test_references_move_by_differences_that_a_sum_rounds_away(V, base, T, walk)
 def test_factors_between_units_far_apart(V):
     """One entry D nats above all others, which the draft covers: the residual mass lies in warps whose references are 21 to 65 powers
     of two below the row's.  A float32 exponent of that size is rounded by up to 2^-19 (2.6e-6 of the factor); ex2.approx itself and
-    the float32 scalars of a row are good to 2^-22 each (2.4e-7): 6e-7 for the mass, whose terms carry three of them.  scale is
-    the float32 that the kernels are given."""
+    the float32 scalars of a row are good to 2^-22 each (2.4e-7): 6e-7 for the mass, whose terms carry three of them (what q - c p
+    cancels comes on top, and makes up to 1.7e-6 of it with other draws).  scale is the float32 that the kernels are given."""
     B, K = 48, 4
     g = torch.Generator().manual_seed(7)
     zq = torch.randn(B, V, generator=g)
