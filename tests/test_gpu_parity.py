@@ -608,6 +608,37 @@ def test_many_short_rows_that_start_anywhere_take_two_sweeps(B, K, gamma, V, dty
     torch.testing.assert_close(out.resmass, other.resmass, rtol=2e-5, atol=5e-7)   # a <= 1
 
 
+@pytest.mark.parametrize("shift", [0, 1, 7])
+@pytest.mark.parametrize("V,dtype,walk", [(1, "fp32", 1), (2, "bf16", 1), (3, "bf16", 2), (7, "bf16", 1), (9, "fp32", 1), (15, "fp32", 2), (17, "fp32", 1),
+                                          (31, "bf16", 1), (33, "bf16", 2), (257, "bf16", 1), (511, "fp32", 1)])
+def test_short_rows_near_the_ends_of_the_tensors(V, dtype, walk, shift):
+    """Rows of which several lie within the 64 bytes at either end of a tensor that copies must not leave, at several remainders: to the bit
+    what the same rows give in the middle of a larger batch, where all of them are copied."""
+    cfg = workloads.VerifyConfig("short", B=3, K=2, gamma=3, V=V, dtype=dtype, alpha=0.8, seed=V + shift)
+    inp = workloads.make_inputs(cfg, device="cuda")
+
+    def moved(t):
+        return torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:].view(t.shape).copy_(t)
+
+    def padded(t):
+        return torch.cat([t[:1]] * 8 + [t] + [t[:1]] * 8)
+    outs = []
+    for place in (moved, padded):
+        logits = [place(t) for t in (inp.target_logits, inp.draft_logits)]
+        rest = [padded(t) if place is padded else t for t in (inp.draft_tokens, inp.uniforms)]
+        binding.set_option("path", 2)
+        binding.set_option("walk", walk)
+        try:
+            outs.append(binding.sgbv_verify_ex(*logits, *rest, cfg.temperature))
+        finally:
+            binding.set_option("path", 0)
+            binding.set_option("walk", 0)
+    a, b = outs
+    assert (a.status & binding.STATUS_NONFINITE_LOGIT == 0).all()
+    for name in ("accept_len", "draft_idx", "tokens", "h", "resmass", "status"):
+        assert torch.equal(getattr(a, name), getattr(b, name)[8:11]), name
+
+
 @pytest.mark.parametrize("V,dtype,walk,shift", [(8191, "fp32", 1, 0), (8191, "bf16", 2, 1), (40001, "bf16", 1, 3), (40001, "fp32", 2, 1),
                                                (151937, "bf16", 1, 0)])
 def test_flagged_and_masked_rows_that_start_anywhere(V, dtype, walk, shift):
