@@ -608,6 +608,27 @@ def test_many_short_rows_that_start_anywhere_take_two_sweeps(B, K, gamma, V, dty
     torch.testing.assert_close(out.resmass, other.resmass, rtol=2e-5, atol=5e-7)   # a <= 1
 
 
+@pytest.mark.parametrize("walk", [1, 2])
+@pytest.mark.parametrize("cells,K,dtype", [(1, 4, "fp32"), (31, 2, "bf16"), (32, 4, "bf16"), (32, 1, "fp32"), (33, 3, "fp32"), (62, 8, "bf16"), (63, 4, "fp32"),
+                                           (64, 4, "bf16"), (65, 2, "fp32"), (95, 4, "bf16"), (96, 4, "fp32"), (97, 3, "bf16"), (126, 8, "fp32"), (127, 5, "bf16"),
+                                           (128, 4, "fp32")])
+def test_cells_of_a_slice_among_its_warps_on_rows_that_start_anywhere(cells, K, dtype, walk):
+    """One CTA per row and slices around the multiples of 32 cells, where the number of cells per warp changes and whether the combining
+    warp has any."""
+    cfg = workloads.VerifyConfig(f"cells_{cells}", B=3, K=K, gamma=3, V=256 * cells - 3, dtype=dtype, alpha=0.85, seed=cells)
+    inp = workloads.make_inputs(cfg, device="cuda")
+    options = {"walk": walk, "cluster": 1, "max_clusters": 2 if walk == 1 else 0}
+    for name, value in options.items():
+        binding.set_option(name, value)
+    try:
+        rep, _, _ = run_both(inp)
+        assert binding.last_main_kernel() == "fused_chain_kernel"
+    finally:
+        for name in options:
+            binding.set_option(name, 0)
+    assert_parity(rep)
+
+
 @pytest.mark.parametrize("shift", [0, 1, 7])
 @pytest.mark.parametrize("V,dtype,walk", [(1, "fp32", 1), (2, "bf16", 1), (3, "bf16", 2), (7, "bf16", 1), (9, "fp32", 1), (15, "fp32", 2), (17, "fp32", 1),
                                           (31, "bf16", 1), (33, "bf16", 2), (257, "bf16", 1), (511, "fp32", 1)])
