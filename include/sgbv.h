@@ -53,7 +53,7 @@ extern "C" {
 
 #define SGBV_STATUS_TOKEN_RANGE 1         /* a draft token of the row is outside [0,V) */
 #define SGBV_STATUS_NONFINITE_LOGIT 2     /* NaN/+inf logit, or a row with no finite logit, among the rows read */
-#define SGBV_STATUS_DEGENERATE_RESIDUAL 4 /* Eq. 4 had zero total mass; y was drawn from q of that row */
+#define SGBV_STATUS_DEGENERATE_RESIDUAL 4 /* Eq. 4 had no mass (beyond rounding); y was drawn from q of that row */
 
 #define SGBV_STATUS_TIMEOUT 8             /* a bounded device-side wait expired; the row's outputs are -1 */
 
